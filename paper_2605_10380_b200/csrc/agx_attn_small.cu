@@ -9,7 +9,7 @@
 //
 // Work item = (sequence, KV head, KV split).  A CTA of KW * MT warps (KW = 4 or 8 KV groups): warp (mt, kg)
 // owns query rows [16 mt, 16 mt + 16) and, in every stage of KW pages, page kg.  K/V pages stream through a
-// 3-stage ring filled by TMA (per page two [16 tokens][64 dims] boxes for K and for V, SWIZZLE_128B so
+// 3-stage ring filled by TMA (per page one 4 KB box for K and one for V, SWIZZLE_128B so
 // ldmatrix is conflict-free; page ids come from the page table, prefetched 32 at a time) and handed over
 // with full/empty mbarriers, so no thread spends instructions on addresses.  Per stage the KV groups of an
 // m-tile meet twice at a named barrier: once to agree on the rows' running maximum (page maxima through
@@ -173,21 +173,32 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         const int pi0 = stage * kKW;
         if ((pi0 >> 5) != group_cur) { ids_cur = ids_next; group_cur = pi0 >> 5; ids_next = fetch_ids(group_cur + 1); }
         const int npg = min(kKW, n_pages - pi0);
-        const int my_id = __shfl_sync(0xFFFFFFFFu, ids_cur, (pi0 + lane) & 31);   // lane pg < npg: the id of the stage's page pg
         if (stage == p.drop_stage) return;   // test hook: this stage never arrives, its consumers' waits run out
-        if (lane == 0) {
-            mbar_arrive_expect_tx(full_bar(slot), npg * 8192u);
-            last_armed = stage;
-        }
-        __syncwarp();   // the barrier is armed before any lane's copies can complete on it
-        // lane pg copies page pg: one lane issuing a stage's 32 boxes of 2 KB takes ~60 ns per box, eight lanes ~40 (measured)
-        if (lane < npg) {
-            const int y = (my_id * p.hkv + g) * kPage;
-            const uint32_t dk = smem_base + slot * kStageBytes + lane * 4096, dv = dk + kStageTokens * kRowBytes;
-            tma_load_2d(dk, &map_k, 0, y, full_bar(slot));
-            tma_load_2d(dk + 2048, &map_k, 64, y, full_bar(slot));
-            tma_load_2d(dv, &map_v, 0, y, full_bar(slot));
-            tma_load_2d(dv + 2048, &map_v, 64, y, full_bar(slot));
+        if (lane == 0) last_armed = stage;
+        if constexpr (MW == 2) {
+            // lane pg copies page pg of K, lane KW + pg that of V
+            const int id = __shfl_sync(0xFFFFFFFFu, ids_cur, (pi0 + (lane & (kKW - 1))) & 31);
+            if (lane == 0) mbar_arrive_expect_tx(full_bar(slot), npg * 8192u);
+            __syncwarp();   // the barrier is armed before any lane's copies can complete on it
+            if (lane < 2 * kKW && (lane & (kKW - 1)) < npg)
+                tma_load_page(smem_base + slot * kStageBytes + lane * 4096, lane < kKW ? &map_k : &map_v, (id * p.hkv + g) * (kPage / 8), full_bar(slot));
+        } else {
+            // One elected thread issues all copies of the stage: 4 x 4096 verify 18.9 -> 18.5 us, decode over 300 tokens 5.50 -> 5.37
+            // (with two m-tiles per warp this form costs decode verify 9.83 -> 10.08, hence the other branch).
+            int group[kKW];   // first row group of each page
+#pragma unroll
+            for (int pg = 0; pg < kKW; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids_cur, (pi0 + pg) & 31) * p.hkv + g) * (kPage / 8);
+            if (elect_one()) {
+                mbar_arrive_expect_tx(full_bar(slot), npg * 8192u);
+                const uint32_t dk = smem_base + slot * kStageBytes, dv = dk + kStageTokens * kRowBytes;
+#pragma unroll
+                for (int pg = 0; pg < kKW; ++pg)
+                    if (pg < npg) {
+                        tma_load_page(dk + pg * 4096, &map_k, group[pg], full_bar(slot));
+                        tma_load_page(dv + pg * 4096, &map_v, group[pg], full_bar(slot));
+                    }
+            }
+            __syncwarp();
         }
     };
     // A CTA with block rows of its own stores them first (fused append, one row chunk per sequence); its producer warp
@@ -263,16 +274,19 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         limit[w][0] = P + min(rA / G, q - 1);
         limit[w][1] = P + min((rA + 8) / G, q - 1);
     }
-    // Per-lane ldmatrix offsets inside one page of the TMA layout [half 2][16 rows][128 B], where the
+    // Per-lane ldmatrix offsets inside one page of the TMA layout [row group 2][half 2][8 rows][128 B], where the
     // 16-byte unit u of row r sits at ((u ^ (r & 7)) << 4).  K (x4): row = nt*8 + lane%8, unit = (kp&1)*4 + lane/8.
     // V (x4.trans): row = lane%8 + 8*((lane/8)&1), unit = (cp&3)*2 + lane/16.
     const uint32_t k_x = ((lane >> 3) ^ (lane & 7));
     const uint32_t k_off[2] = {(uint32_t)((lane & 7) * 128 + (k_x << 4)), (uint32_t)((lane & 7) * 128 + ((k_x ^ 4u) << 4))};
     const uint32_t v_row = (lane & 7) + ((lane >> 3) & 1) * 8;
     const uint32_t v_x = (lane >> 4) ^ (lane & 7);
-    uint32_t v_off[4];
+    uint32_t v_off[kCG];   // of this warp's 16-column groups cp = kg * kCG + c
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v_off[j] = v_row * 128 + ((v_x ^ (uint32_t)(j << 1)) << 4);
+    for (int c = 0; c < kCG; ++c) {
+        const uint32_t cp = (uint32_t)(kg * kCG + c);
+        v_off[c] = (v_row >> 3) * 2048 + (cp >> 2) * 1024 + (v_row & 7) * 128 + ((v_x ^ ((cp & 3) << 1)) << 4);
+    }
 
     const int rg = lane >> 2;                      // this lane's rows in an m-tile: rg and rg + 8
     float* my_max = x_max + (mt0 * 16 + rg) * KW;  // x_max[mt][row][kg]; m-tile mt0 + w: + w * 16 * KW
@@ -304,7 +318,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 const int valid_rows = L - tok0;
                 for (int idx = lane; idx < (kPage - valid_rows) * 16; idx += 32) {
                     const int r = valid_rows + (idx >> 4), ch = idx & 15;
-                    *(uint4*)(ring + (v_base - smem_base) + (ch >> 3) * 2048 + r * 128 + (((ch & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+                    *(uint4*)(ring + (v_base - smem_base) + (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
                 }
                 __syncwarp();
             }
@@ -324,7 +338,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) {
                     uint32_t b0, b1, b2, b3;
-                    ldmatrix_x4(b0, b1, b2, b3, k_base + (kp >> 1) * 2048 + nt * 1024 + k_off[kp & 1]);
+                    ldmatrix_x4(b0, b1, b2, b3, k_base + (kp >> 1) * 1024 + nt * 2048 + k_off[kp & 1]);
 #pragma unroll
                     for (int w = 0; w < MW; ++w) {
                         mma_bf16(s[w][nt], qa[w][2 * kp], b0, b1);
@@ -419,9 +433,8 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 const uint32_t v_base = stage_base + kStageTokens * kRowBytes + k * 4096;
 #pragma unroll
                 for (int c = 0; c < kCG; ++c) {
-                    const int cp = kg * kCG + c;
                     uint32_t b0, b1, b2, b3;
-                    ldmatrix_x4_trans(b0, b1, b2, b3, v_base + (cp >> 2) * 2048 + v_off[cp & 3]);
+                    ldmatrix_x4_trans(b0, b1, b2, b3, v_base + v_off[c]);
 #pragma unroll
                     for (int w = 0; w < MW; ++w) {
                         const uint32_t a[4] = {pk[w].x, pk[w].y, pk[w].z, pk[w].w};

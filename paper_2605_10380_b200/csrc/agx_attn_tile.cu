@@ -7,9 +7,12 @@
 // Work item = (sequence, KV head g, chunk of 256 query rows, KV split).  The q * G rows of one KV
 // head (row r = i * G + h % G) are cut into two 128-row tiles A and B that share every K/V tile.
 // CTA = 12 warps:
-//   warp 0      TMA producer: per 128-token tile, 8 pages x 2 boxes of [16 tokens][64 dims] for K and
-//               for V (SWIZZLE_128B), page ids read through the page table; 2-stage rings.
-//   warp 1      MMA issuer (one lane) and TMEM owner.  Order on the tensor pipe:
+//   warp 0      TMA producer (one elected thread): per 128-token tile, 8 pages x one 4 KB box for K and
+//               for V (SWIZZLE_128B), page ids read through the page table.  One box per page instead of two
+//               of 64 dims, issued without a loop over lanes: 4 x 32768 verify 107 -> 100 us, 16 x 8192 verify
+//               116 -> 92 us, 16 decode blocks over 2k-14k tokens 83 -> 76 us.
+//   warp 1      MMA issuer (one elected thread: with `lane == 0` the issue of eight tcgen05.mma took up to
+//               570 cycles, with elect.sync about 300) and TMEM owner.  Order on the tensor pipe:
 //               S_A(0) S_B(0) | O_A+=P_A V(t)  S_A(t+1)  O_B+=P_B V(t)  S_B(t+1) | ...
 //               so the softmax of one tile overlaps the MMAs of the other.
 //   warps 4-7   softmax of tile A, warps 8-11 softmax of tile B: one thread per query row (TMEM lane).
@@ -48,7 +51,8 @@ template <bool kStreams> struct Sched {
 };
 constexpr int kThreads = 384;
 constexpr uint32_t kTileBytes = 128 * 256;  // one operand tile: [2 halves of 64 dims][128 rows][128 B]
-constexpr uint32_t kHalfBytes = 128 * 128;
+constexpr uint32_t kHalfBytes = 128 * 128;  // (Q tiles: [2 halves][128 rows][128 B])
+constexpr uint32_t kPageBytes = kPage * 256; // K/V tiles: 8 pages of [2 row groups][2 halves of 64 dims][8 rows][128 B], as TMA writes them
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffK = 2 * kTileBytes;
 constexpr uint32_t kOffV = kOffK + kStagesK * kTileBytes;
@@ -426,7 +430,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // ---- setup: barriers, TMEM, Q tiles
     if (tid == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1) ? 128u : (i == BAR_Q_FULL) ? (uint32_t)kQLoadThreads : 1u);
+            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1) ? 4u : (i == BAR_Q_FULL) ? (uint32_t)kQLoadThreads : 1u);
         *abort_flag = 0;
         *(long long*)(smem + kOffBar + BAR_COUNT * 8 + 16) = p.wait_limit_cycles;   // for the out-of-line epilogue
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -504,20 +508,22 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             const int ks = t % kStagesK, kph = (t / kStagesK) & 1;
             const int vs = t % kStagesV, vph = (t / kStagesV) & 1;
             const int npg = pages_in_tile(t);
-            const int pg = lane - (t & 3) * 8;              // this lane's page of the tile
-            const bool mine = pg >= 0 && pg < npg;
-            const int y = (ids * p.hkv + g) * kPage;
+            int group[8];                                   // first row group of each page of the tile
+#pragma unroll
+            for (int pg = 0; pg < 8; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids, (t & 3) * 8 + pg) * p.hkv + g) * (kPage / 8);
             // ---- K
             ok = mbar_wait(bar(BAR_K_EMPTY + ks), kph ^ 1, abort_flag, p.status, p.wait_limit_cycles);
             if (!ok) break;
-            if (lane == 0) mbar_arrive_expect_tx(bar(BAR_K_FULL + ks), npg * 4096u);
+            __syncwarp();
+            if (elect_one()) {
+                mbar_arrive_expect_tx(bar(BAR_K_FULL + ks), npg * kPageBytes);
+                const uint32_t dst = smem_base + kOffK + ks * kTileBytes;
+#pragma unroll
+                for (int pg = 0; pg < 8; ++pg)
+                    if (pg < npg) tma_load_page(dst + pg * kPageBytes, &map_k, group[pg], bar(BAR_K_FULL + ks));
+            }
             __syncwarp();
             last_k = t;
-            if (mine) {
-                const uint32_t dst = smem_base + kOffK + ks * kTileBytes + pg * 2048;
-                tma_load_2d(dst, &map_k, 0, y, bar(BAR_K_FULL + ks));
-                tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(BAR_K_FULL + ks));
-            }
             // ---- V (the page that holds token L, if L is not page-aligned, is copied by hand so that
             //      slots past the end of the sequence are zeros whatever the pool holds there)
             if (!waited && !(stable && t < kStagesV)) { pdl_wait(); waited = true; }
@@ -532,19 +538,21 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                     const int r = idx >> 4, ch = idx & 15, half = ch >> 3, u = ch & 7;
                     uint4 v = make_uint4(0, 0, 0, 0);
                     if (r < valid_rows) v = __ldcg((const uint4*)(src + r * 256 + ch * 16));   // (rows a fused append may just have written)
-                    *(uint4*)(smem + v_stage_off(vs) + half * kHalfBytes + ragged_pg * 2048 + r * 128 + ((u ^ (r & 7)) << 4)) = v;
+                    *(uint4*)(smem + v_stage_off(vs) + ragged_pg * kPageBytes + (r >> 3) * 2048 + half * 1024 + (r & 7) * 128 + ((u ^ (r & 7)) << 4)) = v;
                 }
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 __syncwarp();
             }
-            if (lane == 0) mbar_arrive_expect_tx(bar(BAR_V_FULL + vs), (npg - (ragged_pg >= 0 ? 1 : 0)) * 4096u);
+            __syncwarp();
+            if (elect_one()) {
+                mbar_arrive_expect_tx(bar(BAR_V_FULL + vs), (npg - (ragged_pg >= 0 ? 1 : 0)) * kPageBytes);
+                const uint32_t dst = smem_base + v_stage_off(vs);
+#pragma unroll
+                for (int pg = 0; pg < 8; ++pg)
+                    if (pg < npg && pg != ragged_pg) tma_load_page(dst + pg * kPageBytes, &map_v, group[pg], bar(BAR_V_FULL + vs));
+            }
             __syncwarp();
             last_v = t;
-            if (mine && pg != ragged_pg) {
-                const uint32_t dst = smem_base + v_stage_off(vs) + pg * 2048;
-                tma_load_2d(dst, &map_v, 0, y, bar(BAR_V_FULL + vs));
-                tma_load_2d(dst + kHalfBytes, &map_v, 64, y, bar(BAR_V_FULL + vs));
-            }
         }
         // drain: the copies this warp started must land before the CTA's shared memory goes away.  Bounded by the
         // clock alone: after a time-out elsewhere in the CTA the abort flag is up, and the copies still have to land.
@@ -556,37 +564,38 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t tS[2] = {tmem_base + kColS, tmem_base + kColS + 128};
             const uint32_t tO[2] = {tmem_base + kColO, tmem_base + kColO + 128};
             // descriptors differ only in the start address: add (byte offset >> 4) to a base descriptor
             const uint64_t q_desc[2] = {make_desc(smem_base + kOffQ, 16, 1024), make_desc(smem_base + kOffQ + kTileBytes, 16, 1024)};
-            const uint64_t k_desc0 = make_desc(smem_base + kOffK, 16, 1024);
+            const uint64_t k_desc0 = make_desc(smem_base + kOffK, 16, 2048);
             auto issue_qk = [&](int qt, int stage, int x) {   // S_x = Q_qt K^T : 8 k-steps of 16 dims
                 const uint64_t kd = k_desc0 + (uint64_t)((stage * kTileBytes) >> 4);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-                    umma_ss(tS[x], q_desc[qt] + off, kd + off, kIdescQK, ks > 0);
+                    const uint64_t q_off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
+                    const uint64_t k_off = (uint64_t)(((ks >> 2) * 1024 + (ks & 3) * 32) >> 4);
+                    umma_ss(tS[x], q_desc[qt] + q_off, kd + k_off, kIdescQK, ks > 0);
                 }
             };
             // O_x += P_x V, one k-step per page: the head part (pages 0 .. kPvHeadSteps-1) once P_READY says those columns
             // of P are stored, the tail part after P_TAIL
             auto issue_pv = [&](int x, int stage, int npg, bool first, bool tail) {
-                const uint64_t vd = make_desc(smem_base + v_stage_off(stage), kHalfBytes, 1024);
+                const uint64_t vd = make_desc(smem_base + v_stage_off(stage), 1024, 2048);
                 if (npg == 8) {
                     if (!tail) {
 #pragma unroll
                         for (int ks = 0; ks < kPvHeadSteps; ++ks)
-                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), kIdescPV, !(first && ks == 0));
+                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, !(first && ks == 0));
                     } else {
 #pragma unroll
                         for (int ks = kPvHeadSteps; ks < 8; ++ks)
-                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), kIdescPV, true);
+                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, true);
                     }
                 } else {
                     for (int ks = tail ? kPvHeadSteps : 0; ks < (tail ? npg : min(npg, kPvHeadSteps)); ++ks)
-                        umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), kIdescPV, !(first && ks == 0));
+                        umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, !(first && ks == 0));
                 }
             };
             bool ok = mbar_wait(bar(BAR_Q_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
@@ -700,7 +709,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         if (!warp_has_rows) {   // keep S_FULL / P_READY in step, nothing else
             for (int t = t_first; t < n_tiles && ok; t += kStep) {
                 ok = mbar_wait(bar(BAR_S_FULL + x), ((t - t_first) / kStep) & 1, abort_flag, p.status, p.wait_limit_cycles);
-                if (ok) { mbar_arrive(bar(BAR_P_READY + x)); mbar_arrive(bar(BAR_P_TAIL + x)); }
+                __syncwarp();
+                if (ok && lane == 0) { mbar_arrive(bar(BAR_P_READY + x)); mbar_arrive(bar(BAR_P_TAIL + x)); }
             }
         } else
         for (int t = t_first; t < n_tiles; t += kStep) {
@@ -777,13 +787,15 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             tmem_st_x16(tS + 32, sreg + 32);
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(bar(BAR_P_READY + x));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_P_READY + x));   // (one arrival per warp: 32 on one barrier take turns)
             sweep(kHeadCols, 128);
             l_run += (lt0 + lt1) + (lt2 + lt3);
             tmem_st_x16(tS + 48, sreg + 48);
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(bar(BAR_P_TAIL + x));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_P_TAIL + x));
         }
         if (ok) ok = mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
         if (ok || kStreams) tile_epilogue<kStreams>(smem, tO, m_ref, l_run, ok);
@@ -813,15 +825,16 @@ EncodeTiledFn get_encode_fn() {
     }
     return fn;
 }
-// 2-D view of a pool: [num_pages * Hkv * 16 rows][128 dims] bf16; box = 16 rows x 64 dims, 128-byte swizzle
+// View of a pool [num_pages * Hkv * 16 rows][128 dims] bf16 as [row groups of 8][halves of 64 dims][8 rows][64 dims]; a box is two row
+// groups = the 4 KB of one page and KV head, 128-byte swizzle
 bool make_pool_map_impl(CUtensorMap* map, const void* pool, long long num_pages, int hkv) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)kD, (cuuint64_t)num_pages * hkv * kPage};
-    const cuuint64_t strides[1] = {(cuuint64_t)kD * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kPage};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(pool), dims, strides, box, estr,
+    const cuuint64_t dims[4] = {64, 8, 2, (cuuint64_t)num_pages * hkv * (kPage / 8)};
+    const cuuint64_t strides[3] = {(cuuint64_t)kD * 2, 128, (cuuint64_t)kD * 2 * 8};
+    const cuuint32_t box[4] = {64, 8, 2, (cuuint32_t)(kPage / 8)};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(pool), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -14,7 +14,7 @@ constexpr int kMaxSeqs = 48;       // sequences per attention launch (plans trav
 constexpr int kSmallRowsMax = 64;  // q_len * G above this goes to the tile kernel
 constexpr long long kWaitLimitCycles = 4000000000ll;  // ~2 s at 1.9 GHz: default limit of every in-kernel wait
 
-// 2-D TMA view of a KV pool: [num_pages * Hkv * 16 rows][128 dims] bf16, box = 16 rows x 64 dims, SWIZZLE_128B.
+// TMA view of a KV pool (head_dim 128, bf16): one box is the 16 rows of one page and KV head, see tma_load_page.
 bool make_pool_map(CUtensorMap* map, const void* pool, long long num_pages, int hkv);
 
 // Per-sequence launch plan, built on the host from the host lengths.

@@ -57,9 +57,19 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, long l
     return true;
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+// One page of one KV head (16 tokens x 256 B, 4 KB in HBM and in shared memory) through the pool's tensor map; `group` = row / 8 of
+// the page's first row.  Layout in shared memory: [row group of 8][half of 64 dims][8 rows][128 B], 128-byte swizzled.
+__device__ __forceinline__ void tma_load_page(uint32_t dst, const CUtensorMap* map, int group, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %2, %2, %3}], [%4];\n"
+                 ::"r"(dst), "l"(map), "r"(0), "r"(group), "r"(bar) : "memory");
+}
+
+// One lane of a converged warp.  Unlike `lane == 0` this tells the compiler that a single thread takes the branch, so the
+// instructions that want their operands in uniform registers (tcgen05.mma, TMA copies) are issued without a loop over lanes.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xFFFFFFFF;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
 }
 
 // Programmatic dependent launch: a kernel lets the next launch in the stream start early (its CTAs then run
