@@ -213,12 +213,16 @@ __device__ __forceinline__ TileItem locate_item(const AttnParams& p, int block) 
     const int si = find_seq(p, block);
     const SeqPlan& sp = p.seq[si];
     TileItem it;
-    int local = block - sp.item0;  // ((g * row_chunks) + rc) * nsplit + split
+    // work items reach the SMs in block order: the row chunks that see the most tokens (the last ones) go first.
+    // block - item0 = ((g * row_chunks) + last - rc) * nsplit + split, or (((last - rc) * hkv) + g) * nsplit + split
+    int local = block - sp.item0;
     it.nsplit = sp.nsplit;
     it.split = local % sp.nsplit;
     local /= sp.nsplit;
-    const int rc = local % sp.row_chunks;
-    it.g = local / sp.row_chunks;
+    const int inner = sp.chunk_major ? p.hkv : sp.row_chunks;
+    const int outer_idx = local / inner, inner_idx = local - outer_idx * inner;
+    it.g = sp.chunk_major ? inner_idx : outer_idx;
+    const int rc = sp.row_chunks - 1 - (sp.chunk_major ? outer_idx : inner_idx);
     it.G = p.hq / p.hkv;
     it.P = sp.prefix_len; it.q = sp.q_len;
     it.rows = it.q * it.G;

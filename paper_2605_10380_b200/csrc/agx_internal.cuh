@@ -28,6 +28,7 @@ struct SeqPlan {
     int split_tokens;  // tokens per split (multiple of the kernel's KV tile)
     int item0;         // first work item of this sequence in the launch
     int part_base;     // first partial entry; entry = part_base + (i*Hq + h)*nsplit + split
+    int chunk_major;   // order of the work items: 0 = KV head outermost, 1 = row chunk outermost (row chunks last to first in both)
 };
 
 struct AttnParams {
