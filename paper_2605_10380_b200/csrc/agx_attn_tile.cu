@@ -63,14 +63,10 @@ constexpr uint32_t kOffPark = kOffK + 2 * kTileBytes;   // kStreams epilogue: st
 constexpr uint32_t kOffCtx = kOffBar + 256;            // what the epilogue needs to know, parked at kernel start
 constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;  // + barriers + epilogue context + alignment slack
 constexpr float kRescaleThreshold = 8.0f;              // log2 units
-// Of every 8 column pairs, this many take the polynomial 2^x instead of the special-function unit.
-// Measured on B200 (P = 30720, q = 2048): 0 -> 950 us, 1 -> 957, 2 -> 964, 4 -> 982: the extra FMA-pipe
-// instructions cost more issue slots (shared with the MMA-issuing warp) than the special-function unit
-// gives back, so the default is 0 and the option only remains for experiments.
-#ifndef AGX_POLY_PAIRS
-#define AGX_POLY_PAIRS 0
-#endif
-constexpr int kPolyPairsOf8 = AGX_POLY_PAIRS;
+// Of every 8 column pairs, this many take the polynomial 2^x instead of the special-function unit (16 exponentials per clock
+// and SM: the two Q tiles' 2 x 128 x 128 take as long as their MMAs).  0 / 1 / 2: c3 30.2 / 29.5 / 30.6 us, 3584 uncached
+// tokens 89.5 / 88.7 / 91.5, 8000 + 700 tokens 107.2 / 106.8 / 109.2, the long prefill 1012 / 974 / 990 at the power cap.
+constexpr int kPolyPairsOf8 = 1;
 
 // barrier slots (8 bytes each)
 enum { BAR_K_FULL = 0, BAR_K_EMPTY = 3, BAR_V_FULL = 6, BAR_V_EMPTY = 9, BAR_S_FULL = 12, BAR_P_READY = 14,
@@ -146,9 +142,9 @@ __device__ __forceinline__ uint64_t add2p(uint64_t a, uint64_t b) {
     return d;
 }
 // 2^x for a packed pair on the FMA pipes instead of the special-function unit: n = round(x) by the
-// 1.5 * 2^23 trick, f = x - n in [-0.5, 0.5], 2^f by a cubic fitted to minimise the maximum relative
-// error on that interval (7.5e-5, far below the 2^-9 rounding of P to bfloat16), then n is added
-// into the exponent field.  x is clamped at -126 so the exponent cannot wrap.
+// 1.5 * 2^23 trick, f = x - n in [-0.5, 0.5], 2^f by a polynomial of degree 5 fitted (Lawson's
+// iteration) to minimise the maximum relative error on that interval (2.1e-7 evaluated in fp32, no more than the
+// special-function unit's), then n is added into the exponent field.  x is clamped at -126 so the exponent cannot wrap.
 __device__ __forceinline__ void ex2_poly2(uint64_t x, float& p0, float& p1) {
     float x0, x1;
     upk2(x, x0, x1);
@@ -157,9 +153,12 @@ __device__ __forceinline__ void ex2_poly2(uint64_t x, float& p0, float& p1) {
     const uint64_t t = add2p(x, magic);
     const uint64_t n = add2p(t, neg_magic);
     const uint64_t f = fma2p(n, pk2(-1.f, -1.f), x);
-    uint64_t q = fma2p(f, pk2(0.0551716648042202f, 0.0551716648042202f), pk2(0.2426111251115799f, 0.2426111251115799f));
-    q = fma2p(q, f, pk2(0.6932609677314758f, 0.6932609677314758f));
-    q = fma2p(q, f, pk2(0.9999280571937561f, 0.9999280571937561f));
+    auto c2 = [](float c) { return pk2(c, c); };
+    uint64_t q = fma2p(f, c2(1.32764725e-3f), c2(9.67554096e-3f));
+    q = fma2p(q, f, c2(5.55071309e-2f));
+    q = fma2p(q, f, c2(2.40221202e-1f));
+    q = fma2p(q, f, c2(6.93146944e-1f));
+    q = fma2p(q, f, c2(1.00000012f));
     float q0, q1, t0, t1;
     upk2(q, q0, q1);
     upk2(t, t0, t1);
