@@ -8,6 +8,7 @@ library is missing or fails to load, importing a symbol raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 from pathlib import Path
 from typing import Optional
 
@@ -21,6 +22,7 @@ DTYPES = {"bf16": AGX_BF16, "f32": AGX_F32}
 
 _LIB_PATH = Path(__file__).resolve().parent / "lib" / "libagx.so"
 _lib = None
+_native = None
 
 EXPORTS = (
     "agx_create", "agx_destroy", "agx_status_string", "agx_last_error", "agx_kv_append",
@@ -160,6 +162,26 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+def _binding():
+    """The compiled argument marshalling (``csrc/agx_torch.cpp``) for the calls a model makes per layer or per step, bound to
+    the functions of ``load()``'s library; raises if it was not built."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries have to be in the process first)
+        lib = load()
+        path = Path(__file__).resolve().parent / "lib" / "agx_torch.so"
+        if not path.exists():
+            raise RuntimeError(f"{path} is missing: build the library first (python -m paper_2605_10380_b200.build)")
+        spec = importlib.util.spec_from_file_location("agx_torch", path)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+        native.bind(_h_i32, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in (
+            "agx_kv_append", "agx_attn_prefixed", "agx_attn_prefixed_append", "agx_accept_greedy", "agx_verify_step_host",
+            "agx_verify_step_host_enqueue", "agx_ngram_build", "agx_ngram_draft", "agx_kv_copy_pages")))
+        _native = native
+    return _native
+
+
 def status_string(status: int) -> str:
     return load().agx_status_string(int(status)).decode()
 
@@ -210,11 +232,12 @@ class Handle:
         st = self._lib.agx_create(ctypes.byref(self.cfg), ctypes.byref(self._h))
         if st != AGX_OK:
             raise AgxError(st, "agx_create")
+        self._n, self._p = _binding(), self._h.value
 
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
             self._lib.agx_destroy(self._h)
-            self._h = None   # (at interpreter shutdown the ctypes module may already be gone)
+            self._h, self._p = None, 0   # (at interpreter shutdown the ctypes module may already be gone)
 
     __del__ = close
 
@@ -231,12 +254,9 @@ class Handle:
 
     # -- agx_kv_append
     def kv_append(self, k_pool, v_pool, k_new, v_new, page_table, prefix_len, cu_q, stream=None):
-        B = int(prefix_len.shape[0])
-        total_q = int(k_new.shape[0])
-        st = self._lib.agx_kv_append(self._h, _ptr(k_pool), _ptr(v_pool), int(k_pool.shape[0]), _ptr(k_new),
-                                     _ptr(v_new), _ptr(page_table), int(page_table.shape[1]), _ptr(prefix_len),
-                                     _ptr(cu_q), B, total_q, _stream_ptr(stream))
-        self._check(st, "agx_kv_append")
+        st = self._n.kv_append(self._p, k_pool, v_pool, k_new, v_new, page_table, prefix_len, cu_q, stream)
+        if st:
+            self._check(st, "agx_kv_append")
 
     # -- agx_attn_workspace_bytes
     def attn_workspace_bytes(self, h_prefix_len, h_q_len) -> int:
@@ -249,24 +269,18 @@ class Handle:
     # -- agx_attn_prefixed
     def attn_prefixed(self, q_block, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse=None,
                       workspace=None, stream=None):
-        P, Q = _h_i32(h_prefix_len), _h_i32(h_q_len)
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        st = self._lib.agx_attn_prefixed(self._h, _ptr(q_block), _ptr(k_pool), _ptr(v_pool), int(k_pool.shape[0]),
-                                         _ptr(page_table), int(page_table.shape[1]), _ptr(P), _ptr(Q),
-                                         int(P.shape[0]), _ptr(out), _ptr(lse), _ptr(workspace), ws_bytes,
-                                         _stream_ptr(stream))
-        self._check(st, "agx_attn_prefixed")
+        st = self._n.attn(self._p, q_block, None, None, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse, workspace, stream)
+        if st:
+            self._check(st, "agx_attn_prefixed")
 
     # -- agx_attn_prefixed_append
     def attn_prefixed_append(self, q_block, k_new, v_new, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse=None,
                              workspace=None, stream=None):
-        P, Q = _h_i32(h_prefix_len), _h_i32(h_q_len)
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        st = self._lib.agx_attn_prefixed_append(self._h, _ptr(q_block), _ptr(k_new), _ptr(v_new), _ptr(k_pool), _ptr(v_pool),
-                                                int(k_pool.shape[0]), _ptr(page_table), int(page_table.shape[1]), _ptr(P),
-                                                _ptr(Q), int(P.shape[0]), _ptr(out), _ptr(lse), _ptr(workspace), ws_bytes,
-                                                _stream_ptr(stream))
-        self._check(st, "agx_attn_prefixed_append")
+        if k_new is None:   # (None there would select the call without an append)
+            raise AgxError(-1, "agx_attn_prefixed_append", "null pointer")
+        st = self._n.attn(self._p, q_block, k_new, v_new, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse, workspace, stream)
+        if st:
+            self._check(st, "agx_attn_prefixed_append")
 
     # -- agx_accept_workspace_bytes
     def accept_workspace_bytes(self, total_q: int, vocab: int) -> int:
@@ -278,20 +292,16 @@ class Handle:
     # -- agx_accept_greedy
     def accept_greedy(self, logits, logits_dtype: str, vocab: int, drafts, cu_q, accept_len, next_token,
                       argmax=None, seq_lens=None, workspace=None, stream=None):
-        B = int(cu_q.shape[0]) - 1
-        total_q = int(logits.shape[0])
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        st = self._lib.agx_accept_greedy(self._h, _ptr(logits), DTYPES[logits_dtype], int(logits.stride(0)),
-                                         int(vocab), _ptr(drafts), _ptr(cu_q), B, total_q, _ptr(accept_len),
-                                         _ptr(next_token), _ptr(argmax), _ptr(seq_lens), _ptr(workspace), ws_bytes,
-                                         _stream_ptr(stream))
-        self._check(st, "agx_accept_greedy")
+        st = self._n.accept(self._p, logits, DTYPES[logits_dtype], vocab, drafts, cu_q, accept_len, next_token, argmax, seq_lens,
+                            workspace, stream)
+        if st:
+            self._check(st, "agx_accept_greedy")
 
     # -- agx_kv_copy_pages (src, dst: device int32 tensors)
     def kv_copy_pages(self, k_pool, v_pool, src, dst, stream=None):
-        st = self._lib.agx_kv_copy_pages(self._h, _ptr(k_pool), _ptr(v_pool), int(k_pool.shape[0]), _ptr(src), _ptr(dst),
-                                         int(src.numel()), _stream_ptr(stream))
-        self._check(st, "agx_kv_copy_pages")
+        st = self._n.copy_pages(self._p, k_pool, v_pool, src, dst, stream)
+        if st:
+            self._check(st, "agx_kv_copy_pages")
 
     # -- agx_kv_import_pages (h_k, h_v: pinned host tensors or numpy arrays; dst_pages: device int32; staging: device uint8)
     def kv_import_staging_bytes(self, count: int) -> int:
@@ -305,15 +315,14 @@ class Handle:
 
     # -- agx_ngram_build / agx_ngram_draft (device int32 tensors; lut and workspace are uint8 tensors)
     def ngram_build(self, stream_tokens, n: int, lut, workspace, stream=None):
-        st = self._lib.agx_ngram_build(self._h, _ptr(stream_tokens), int(stream_tokens.numel()), int(n), _ptr(lut),
-                                       lut.numel() * lut.element_size(), _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-        self._check(st, "agx_ngram_build")
+        st = self._n.ngram_build(self._p, stream_tokens, n, lut, workspace, stream)
+        if st:
+            self._check(st, "agx_ngram_build")
 
     def ngram_draft(self, lut, context, fill, k: int, drafts, has_draft, stream=None):
-        st = self._lib.agx_ngram_draft(self._h, _ptr(lut), _ptr(context), _ptr(fill), int(has_draft.shape[0]), int(k),
-                                       _ptr(drafts), _ptr(has_draft), _stream_ptr(stream))
-        self._check(st, "agx_ngram_draft")
+        st = self._n.ngram_draft(self._p, lut, context, fill, k, drafts, has_draft, stream)
+        if st:
+            self._check(st, "agx_ngram_draft")
 
     # -- agx_get_status
     def get_status(self, stream=None, raise_on_error: bool = False) -> int:
@@ -366,13 +375,7 @@ class Handle:
         """agx_verify_step_host, or agx_verify_step_host_enqueue when ``enqueue_only`` (the caller then
         synchronises the stream before reading the host outputs and keeps ``h_prefix_len``/``h_q_len`` and the
         pinned inputs alive until then)."""
-        P, Q = _h_i32(h_prefix_len), _h_i32(h_q_len)
-        ws_bytes = workspace.numel() * workspace.element_size()
-        fn = self._lib.agx_verify_step_host_enqueue if enqueue_only else self._lib.agx_verify_step_host
-        st = fn(self._h, _ptr(k_pool), _ptr(v_pool), int(k_pool.shape[0]),
-                _ptr(page_table), int(page_table.shape[1]), _ptr(P), _ptr(Q),
-                int(P.shape[0]), _ptr(h_q_block), _ptr(h_k_new), _ptr(h_v_new),
-                _ptr(h_logits), DTYPES[logits_dtype], int(row_stride), int(vocab),
-                _ptr(h_drafts), _ptr(h_out), _ptr(h_accept_len), _ptr(h_next_token),
-                _ptr(h_seq_lens), _ptr(workspace), ws_bytes, _stream_ptr(stream))
+        st = self._n.step(self._p, not enqueue_only, k_pool, v_pool, page_table, h_prefix_len, h_q_len, h_q_block, h_k_new, h_v_new,
+                          h_logits, DTYPES[logits_dtype], row_stride, vocab, h_drafts, h_out, h_accept_len, h_next_token,
+                          h_seq_lens, workspace, stream)
         self._check(st, "agx_verify_step_host_enqueue" if enqueue_only else "agx_verify_step_host")

@@ -1,4 +1,5 @@
-"""Build the agx CUDA library (sm_100a only) into ``paper_2605_10380_b200/lib/libagx.so``.
+"""Build the agx CUDA library (sm_100a only) into ``paper_2605_10380_b200/lib/libagx.so``, and the CPython module that marshals
+its calls' arguments (``csrc/agx_torch.cpp``, host code only) into ``lib/agx_torch.so``.
 
 Usage: ``python -m paper_2605_10380_b200.build [--force] [--verbose]``.  nvcc cross-compiles
 without a GPU.  Objects are cached under ``_build/`` and rebuilt when a source or header is newer.
@@ -8,6 +9,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -15,6 +17,7 @@ PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 CSRC = PKG / "csrc"
 OUT = PKG / "lib" / "libagx.so"
+BINDING = PKG / "lib" / "agx_torch.so"
 OBJ_DIR = PKG / "_build"
 
 NVCC_FLAGS = [
@@ -42,6 +45,18 @@ def _stale(target: Path, deps) -> bool:
     return any(Path(d).stat().st_mtime > t for d in deps)
 
 
+def _binding_command(out: Path):
+    """g++ command of the argument-marshalling module (torch's headers give the tensors' addresses and the current stream)."""
+    import torch
+    base = Path(torch.__file__).resolve().parent
+    cuda = Path(_nvcc()).resolve().parent.parent
+    inc = [base / "include", base / "include" / "torch" / "csrc" / "api" / "include", cuda / "include",
+           sysconfig.get_paths()["include"], ROOT / "include"]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{i}" for i in inc),
+            str(CSRC / "agx_torch.cpp"), "-o", str(out), f"-L{base / 'lib'}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
     srcs = sources()
     headers = list(CSRC.glob("*.cuh")) + list((ROOT / "include").glob("*.h"))
@@ -58,15 +73,21 @@ def build(force: bool = False, verbose: bool = False) -> Path:
                 cmd.insert(2, "-v")
             jobs.append(cmd)
 
+    binding_tmp = BINDING.with_suffix(f".tmp{os.getpid()}.so")
+    if force or _stale(BINDING, [CSRC / "agx_torch.cpp", ROOT / "include" / "agx.h"]):
+        jobs.append(_binding_command(binding_tmp))
+
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or r.returncode != 0:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode != 0:
-            raise RuntimeError(f"nvcc failed on {cmd[-3]}")
+            raise RuntimeError("compilation failed: " + " ".join(cmd))
 
     with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
         list(ex.map(run, jobs))
+    if binding_tmp.exists():
+        os.replace(binding_tmp, BINDING)
     objs = [OBJ_DIR / (s.stem + ".o") for s in srcs]
     if force or jobs or _stale(OUT, objs):
         tmp = OUT.with_suffix(f".tmp{os.getpid()}.so")
