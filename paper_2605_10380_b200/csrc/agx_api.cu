@@ -6,7 +6,6 @@
 
 #include <algorithm>
 #include <new>
-#include <unordered_map>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -21,12 +20,6 @@ struct CallRange {
     ~CallRange() { nvtxRangePop(); }
 };
 struct Plan;
-// TMA view of one KV pool, kept per pool address: encoding a tensor map costs about as much host time as a launch.
-struct PoolMap {
-    alignas(64) CUtensorMap map;
-    long long num_pages;
-    int hkv;
-};
 }  // namespace
 
 struct agx_handle {
@@ -52,7 +45,6 @@ struct agx_handle {
     long long wait_limit_cycles;   // AGX_OPT_WAIT_LIMIT_CYCLES
     int early_prefix;       // AGX_OPT_EARLY_PREFIX_LOADS
     int drop_stage;         // AGX_OPT_TEST_DROP_STAGE (-1 = none)
-    std::unordered_map<const void*, PoolMap> pool_maps;
     std::vector<int32_t> cu_host;  // staging for agx_verify_step_host (lives until its final sync)
     // Large attention-only host steps run as a pipeline of row chunks: uploads on one stream of the handle's own, the
     // attention calls on the caller's stream, downloads on a third (env AGX_HOST_PIPELINE_ROWS: rows per chunk, 0 = off).
@@ -85,18 +77,6 @@ agx_status cuda_fail(agx_handle* h, cudaError_t e, const char* what) {
 
 inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
-// The handle's tensor map of a pool (encoded on first use of that address with that geometry).
-const CUtensorMap* pool_map(agx_handle* h, const void* pool, long long num_pages, int hkv) {
-    auto it = h->pool_maps.find(pool);
-    if (it != h->pool_maps.end() && it->second.num_pages == num_pages && it->second.hkv == hkv) return &it->second.map;
-    if (h->pool_maps.size() >= 4096) h->pool_maps.clear();
-    PoolMap& pm = h->pool_maps[pool];
-    pm.num_pages = -1;
-    if (!make_pool_map(&pm.map, pool, num_pages, hkv)) { h->pool_maps.erase(pool); return nullptr; }
-    pm.num_pages = num_pages;
-    pm.hkv = hkv;
-    return &pm.map;
-}
 inline int round_up(long long v, int m) { return (int)((v + m - 1) / m * m); }
 inline int elem_size(int dtype) { return dtype == AGX_BF16 ? 2 : 4; }
 
@@ -116,6 +96,7 @@ struct Plan {
     std::vector<Launch> launches;
     long long part_entries = 0;  // (row, head, split) partial slots
     bool any_split = false;
+    long long total_rows = 0;    // block rows of the whole batch
 };
 
 // Decide kernel kind, KV splits and partial slots for every sequence (host lengths only).
@@ -131,6 +112,7 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         if ((long long)row0[s] + Q[s] > (1 << 30)) return fail(h, AGX_E_RANGE, "too many rows");
         row0[s + 1] = row0[s] + Q[s];
     }
+    plan.total_rows = row0[B];
     // Blocks of at most 32 rows: measured on B200 (GQA 32/8, equal sequences), what decides is the batch's total
     // context, not each sequence's: from ~24k tokens in all (two sequences or more) the tensor-core stream schedule
     // wins whatever the single lengths; below that the warp-MMA kernel, with 4-page stages and two CTAs per SM from
@@ -483,9 +465,9 @@ int64_t agx_attn_workspace_bytes(agx_handle* h, int32_t B, const int32_t* P, con
     return (int64_t)(part_ml_bytes(plan.part_entries) + (size_t)plan.part_entries * h->cfg.head_dim * sizeof(float));
 }
 
-// Attention, optionally preceded by the append of the block's own K/V rows (k_new != NULL).  Launches whose
-// sequences all fit one row chunk write those rows in the attention kernel's prologue (each CTA the rows of its own
-// KV split and head); the others (blocks of more than 256 rows, fp32 handles) get a separate append launch in front.
+// Attention, optionally with the append of the block's own K/V rows (k_new != NULL): the attention kernels take the block's rows from
+// k_new / v_new and store them into the pages on the side.  Launches of the scalar kernel (and of the warp-MMA kernel with more than
+// one row chunk, which only AGX_FORCE_MMA_SYNC makes) get a separate append launch in front.
 static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_new, const void* v_new, const void* k_pool,
                             const void* v_pool, int64_t num_pages, const int32_t* page_table, int32_t pt_stride,
                             const int32_t* P, const int32_t* Q, int32_t B, void* out, float* lse, void* workspace,
@@ -520,6 +502,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.part_o = need ? (float*)((char*)workspace + part_ml_bytes(plan.part_entries)) : nullptr;
     p.status = h->d_status;
     p.num_pages = num_pages;
+    p.total_rows = (int)plan.total_rows;
     p.pt_stride = pt_stride;
     p.hq = h->cfg.num_q_heads; p.hkv = h->cfg.num_kv_heads; p.head_dim = h->cfg.head_dim;
     p.scale_log2 = h->scale * 1.4426950408889634f;
@@ -527,12 +510,14 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.wait_limit_cycles = h->wait_limit_cycles;
     p.early_prefix = h->early_prefix;
     p.drop_stage = h->drop_stage;
-    const CUtensorMap *map_k = nullptr, *map_v = nullptr;
+    alignas(64) CUtensorMap map_k, map_v;   // (encoding one takes 0.05 us)
+    RowsMaps maps_new;
     if (h->cfg.dtype == AGX_BF16 && h->cfg.head_dim == 128) {
         if ((long long)num_pages * p.hkv * kPage > 0x7FFFFFFFll) return fail(h, AGX_E_RANGE, "pool too large for one tensor map");
-        map_k = pool_map(h, k_pool, num_pages, p.hkv);
-        map_v = pool_map(h, v_pool, num_pages, p.hkv);
-        if (!map_k || !map_v) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
+        bool ok = make_pool_map(&map_k, k_pool, num_pages, p.hkv) && make_pool_map(&map_v, v_pool, num_pages, p.hkv);
+        if (ok && k_new) ok = make_rows_maps(&maps_new, k_new, v_new, plan.total_rows, p.hkv);
+        else memset(&maps_new, 0, sizeof maps_new);
+        if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
     for (const Launch& ln : plan.launches) {
         p.num_seqs = (int)ln.seqs.size();
@@ -550,7 +535,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         p.k_new = p.v_new = nullptr;
         if (k_new) {
             p.k_new = k_new; p.v_new = v_new;
-            if (ln.kind == KIND_SIMT || !one_chunk) {
+            if (ln.kind == KIND_SIMT || (!one_chunk && ln.kind != KIND_TILE && ln.kind != KIND_STREAM)) {
                 e = launch_kv_append_plan(p, h->cfg.dtype, ln.total_rows, stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "append launch");
                 h->last_launches++;
@@ -558,12 +543,12 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
             }
         }
         switch (ln.kind) {
-            case KIND_SMALL1: e = launch_attn_small_bf16(p, 1, ln.kw, *map_k, *map_v, stream); break;
-            case KIND_SMALL2: e = launch_attn_small_bf16(p, 2, ln.kw, *map_k, *map_v, stream); break;
-            case KIND_SMALL4: e = launch_attn_small_bf16(p, 4, 4, *map_k, *map_v, stream); break;
+            case KIND_SMALL1: e = launch_attn_small_bf16(p, 1, ln.kw, map_k, map_v, stream); break;
+            case KIND_SMALL2: e = launch_attn_small_bf16(p, 2, ln.kw, map_k, map_v, stream); break;
+            case KIND_SMALL4: e = launch_attn_small_bf16(p, 4, 4, map_k, map_v, stream); break;
             case KIND_SIMT: e = launch_attn_simt(p, h->cfg.dtype, stream); break;
-            case KIND_TILE: e = launch_attn_tile_bf16(p, false, *map_k, *map_v, stream); break;
-            case KIND_STREAM: e = launch_attn_tile_bf16(p, true, *map_k, *map_v, stream); break;
+            case KIND_TILE: e = launch_attn_tile_bf16(p, false, map_k, map_v, maps_new, stream); break;
+            case KIND_STREAM: e = launch_attn_tile_bf16(p, true, map_k, map_v, maps_new, stream); break;
             default: return fail(h, AGX_E_UNSUPPORTED, "unknown kernel kind");
         }
         if (e != cudaSuccess) return cuda_fail(h, e, "attention launch");

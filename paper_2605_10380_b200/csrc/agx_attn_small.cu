@@ -144,20 +144,55 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
     const int page0 = tok_begin / kPage;
     const int n_pages = (tok_end - tok_begin + kPage - 1) / kPage;
-    // A CTA whose KV split holds block rows stores them itself first (fused append) and keeps its copies back until
-    // they are in place.  Any other CTA may, with p.early_prefix (the caller vouches that the page table and the pages
-    // below the cached-prefix length are not written by a launch still in flight), fetch page ids and K/V stages that
-    // lie wholly inside the cached prefix before the dependency wait, i.e. while the launch in front drains.
-    const bool own_rows = p.k_new && tok_begin < L && tok_begin + sp.split_tokens > P;
-    const bool pre = p.early_prefix && !own_rows;
+    // With p.early_prefix (the caller vouches that the page table and the pages below the cached-prefix length are not written by a
+    // launch still in flight) the producer warp fetches page ids and K/V stages that lie wholly inside the cached prefix before
+    // the dependency wait, i.e. while the launch in front drains.
+    const bool pre = p.early_prefix;
+    // The pages from own_pg on (counted from the split's first page) are put together by hand, beside the Q tile: with a fused append
+    // those that hold block rows, which come from k_new / v_new and go into the pool on the way; otherwise a last page that is only partly
+    // valid (what lies behind the last token may be anything, and V has to be zero there).  They are at the end of the sequence, and a
+    // split's stages are worked off from its end, so they are always among the first in the ring.
+    const int pool_end = p.k_new ? P : L;
+    const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
+    const int own_units = (n_pages - own_pg) * 512;   // 16-byte units, [page][K, V][16 rows][16 units]
+    constexpr int kLoaders = kThreads - 32;           // all warps but the producer's
+    constexpr int kOwn = (512 + kLoaders - 1) / kLoaders;   // a thread's units of the first own page
+    auto own_id = [&](int u) { const int slot = page0 + own_pg + (u >> 9); return slot < p.pt_stride ? __ldg(pt_row + slot) : -1; };
+    auto own_load = [&](int u, int id) {
+        const int tok = tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15), is_v = (u >> 8) & 1, ch = u & 15;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (tok < pool_end) {
+            const long long page = (id < 0 || id >= p.num_pages) ? 0 : id;   // (reported by fetch_ids)
+            v = __ldcg((const uint4*)((const unsigned char*)(is_v ? p.v_pool : p.k_pool) + ((page * p.hkv + g) * kPage + (tok & 15)) * kRowBytes + ch * 16));
+        } else if (tok < L) {
+            v = __ldg((const uint4*)((const unsigned char*)(is_v ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * kRowBytes + ch * 16));
+        }
+        return v;
+    };
+    auto own_store = [&](int u, int id, const uint4 v) {
+        const int pg = own_pg + (u >> 9), r = (u >> 4) & 15, is_v = (u >> 8) & 1, ch = u & 15, tok = tok_begin + pg * kPage + r;
+        const int stage = pg / kKW;
+        *(uint4*)(ring + ((n_stages - 1 - stage) % NS) * kStageBytes + is_v * (kStageTokens * kRowBytes) + (pg - stage * kKW) * 4096 +
+                  (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v;
+        if (tok >= pool_end && tok < L && id >= 0 && id < p.num_pages)
+            *(uint4*)((unsigned char*)(is_v ? p.v_pool : p.k_pool) + (((long long)id * p.hkv + g) * kPage + (tok & 15)) * kRowBytes + ch * 16) = v;
+    };
+    int first_id[kOwn];
+    auto fetch_own_ids = [&]() {
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j)
+            if (tid >= 32 && tid - 32 + j * kLoaders < own_units) first_id[j] = own_id(tid - 32 + j * kLoaders);
+    };
+    if (pre) fetch_own_ids();         // (the caller vouches for the page table too)
     if (!(warp == 0 && pre)) pdl_wait();   // from here on global memory written by the launch before this one is read
+    if (!pre) fetch_own_ids();
     // ---- producer state (warp 0; lane 0 issues the TMA copies).  Page ids are fetched 32 at a time,
     //      one group ahead, so the page-table latency never sits in front of a copy.
-    int ids_cur = 0, ids_next = 0, group_cur = 0;
+    int ids_cur = 0, ids_next = 0, group_cur = max(0, (n_stages - 1) * kKW) >> 5;
     auto fetch_ids = [&](int group) {
         const int pi = group * 32 + lane;
         long long id = 0;
-        if (pi < n_pages) {
+        if (pi >= 0 && pi < n_pages) {
             id = __ldg(pt_row + page0 + pi);
             if (id < 0 || id >= p.num_pages) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
         }
@@ -165,22 +200,23 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     };
     bool alive = true;
     int last_armed = -1;              // last stage whose copies were armed (lane 0 of warp 0)
-    auto produce = [&](int stage) {   // called by all lanes of warp 0
+    auto produce = [&](int stage) {   // called by all lanes of warp 0; `stage` counts from the end of the split
         if (stage >= n_stages || !alive) return;
         const int slot = stage % NS;
         alive = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar(slot), ((stage / NS) & 1) ^ 1, abort_flag, p.status, p.wait_limit_cycles));
         if (!alive) return;   // (the same answer in every lane: the lanes stay together for the shuffles and copies below)
-        const int pi0 = stage * kKW;
-        if ((pi0 >> 5) != group_cur) { ids_cur = ids_next; group_cur = pi0 >> 5; ids_next = fetch_ids(group_cur + 1); }
+        const int pi0 = (n_stages - 1 - stage) * kKW;
+        if ((pi0 >> 5) != group_cur) { ids_cur = ids_next; group_cur = pi0 >> 5; ids_next = fetch_ids(group_cur - 1); }
         const int npg = min(kKW, n_pages - pi0);
+        const int npool = min(npg, max(0, own_pg - pi0));   // pages that come from the pool
         if (stage == p.drop_stage) return;   // test hook: this stage never arrives, its consumers' waits run out
         if (lane == 0) last_armed = stage;
         if constexpr (MW == 2) {
             // lane pg copies page pg of K, lane KW + pg that of V
             const int id = __shfl_sync(0xFFFFFFFFu, ids_cur, (pi0 + (lane & (kKW - 1))) & 31);
-            if (lane == 0) mbar_arrive_expect_tx(full_bar(slot), npg * 8192u);
+            if (lane == 0) mbar_arrive_expect_tx(full_bar(slot), npool * 8192u);
             __syncwarp();   // the barrier is armed before any lane's copies can complete on it
-            if (lane < 2 * kKW && (lane & (kKW - 1)) < npg)
+            if (lane < 2 * kKW && (lane & (kKW - 1)) < npool)
                 tma_load_page(smem_base + slot * kStageBytes + lane * 4096, lane < kKW ? &map_k : &map_v, (id * p.hkv + g) * (kPage / 8), full_bar(slot));
         } else {
             // One elected thread issues all copies of the stage: 4 x 4096 verify 18.9 -> 18.5 us, decode over 300 tokens 5.50 -> 5.37
@@ -189,11 +225,11 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 #pragma unroll
             for (int pg = 0; pg < kKW; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids_cur, (pi0 + pg) & 31) * p.hkv + g) * (kPage / 8);
             if (elect_one()) {
-                mbar_arrive_expect_tx(full_bar(slot), npg * 8192u);
+                mbar_arrive_expect_tx(full_bar(slot), npool * 8192u);
                 const uint32_t dk = smem_base + slot * kStageBytes, dv = dk + kStageTokens * kRowBytes;
 #pragma unroll
                 for (int pg = 0; pg < kKW; ++pg)
-                    if (pg < npg) {
+                    if (pg < npool) {
                         tma_load_page(dk + pg * 4096, &map_k, group[pg], full_bar(slot));
                         tma_load_page(dv + pg * 4096, &map_v, group[pg], full_bar(slot));
                     }
@@ -201,24 +237,18 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
             __syncwarp();
         }
     };
-    // A CTA with block rows of its own stores them first (fused append, one row chunk per sequence); its producer warp
-    // waits on a named barrier until every thread's rows are in the pages, the other warps only arrive there and go on.
-    if (own_rows) {
-        append_rows_bf16(p, sp, g, tok_begin, tok_begin + sp.split_tokens, tid, kThreads);
-        if (warp != 0) asm volatile("bar.arrive 8, %0;\n" ::"n"(kThreads) : "memory");
-    }
     // The producer lane set the barriers up itself, so it needs nothing else from the other warps: it fetches the page
     // ids and issues the first copies at once, while the others bring the Q tile in.
     if (warp == 0) {
         __syncwarp();   // lane 0's barrier initialisation, before the other lanes poll those barriers
-        ids_cur = fetch_ids(0);
-        ids_next = fetch_ids(1);
+        ids_cur = fetch_ids(group_cur);
+        ids_next = fetch_ids(group_cur - 1);
         bool waited = !pre;
-        if (own_rows) asm volatile("bar.sync 8, %0;\n" ::"n"(kThreads) : "memory");
         const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
 #pragma unroll 1
         for (int s = 0; s < NS - 1; ++s) {
-            if (!waited && tok_begin + (s + 1) * kStageTokens > stable_end) { pdl_wait(); waited = true; }
+            // (with a fused append only pages below stable_end come from the pool)
+            if (!waited && !p.k_new && tok_begin + (n_stages - s) * kStageTokens > stable_end) { pdl_wait(); waited = true; }
             produce(s);
         }
         if (!waited) pdl_wait();
@@ -226,7 +256,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     // ---- Q tile -> shared (rows beyond q*G are zero), by the warps other than the producer's
     //      (a thread's loads are all issued before its first store: one trip to memory, not one per 16-byte unit)
     if (tid >= 32) {
-        constexpr int kUnits = MT * 16 * 16, kLoaders = kThreads - 32, kPer = (kUnits + kLoaders - 1) / kLoaders;
+        constexpr int kUnits = MT * 16 * 16, kPer = (kUnits + kLoaders - 1) / kLoaders;
         uint4 v[kPer];
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
@@ -238,6 +268,15 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 v[j] = __ldg((const uint4*)((const unsigned char*)p.q + off));
             }
         }
+        // own pages: their loads go out behind Q's, before anything is stored
+        uint4 w[kOwn];
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j)
+            if (tid - 32 + j * kLoaders < own_units) w[j] = own_load(tid - 32 + j * kLoaders, first_id[j]);
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j)
+            if (tid - 32 + j * kLoaders < own_units) own_store(tid - 32 + j * kLoaders, first_id[j], w[j]);
+        for (int u = tid - 32 + kOwn * kLoaders; u < own_units; u += kLoaders) { const int id = own_id(u); own_store(u, id, own_load(u, id)); }
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int c = tid - 32 + j * kLoaders;
@@ -300,7 +339,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         if (warp == 0) produce(stage + NS - 1);
         if (live) live = mbar_wait(full_bar(slot), (stage / NS) & 1, abort_flag, p.status, p.wait_limit_cycles);
 
-        const int stage_tok0 = tok_begin + stage * kStageTokens;
+        const int stage_tok0 = tok_begin + (n_stages - 1 - stage) * kStageTokens;
         const int npg = live ? min(kKW, (tok_end - stage_tok0 + kPage - 1) / kPage) : 0;   // pages of this stage
         const int tok0 = stage_tok0 + kg * kPage;
         const bool has_page = kg < npg;
@@ -311,17 +350,6 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         for (int w = 0; w < MW; ++w) mx[w][0] = mx[w][1] = -INFINITY;
         if (has_page) {
             const uint32_t k_base = stage_base + kg * 4096;
-            const uint32_t v_base = k_base + kStageTokens * kRowBytes;
-            // slots past the end of the sequence may hold anything: zero those V rows (P is 0 there,
-            // but 0 * NaN is not).  Every warp that scores the page writes the same zeros.
-            if (tok0 + kPage > L) {
-                const int valid_rows = L - tok0;
-                for (int idx = lane; idx < (kPage - valid_rows) * 16; idx += 32) {
-                    const int r = valid_rows + (idx >> 4), ch = idx & 15;
-                    *(uint4*)(ring + (v_base - smem_base) + (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
-                }
-                __syncwarp();
-            }
             // S = Q K^T for 16 tokens: two n-tiles of 8 tokens, as four accumulation chains of four MMAs each per m-tile
             // (even and odd k-steps of both n-tiles): a dependent mma.sync is slow to issue.  A K fragment serves every m-tile.
             float s_odd[MW][2][4];
@@ -421,7 +449,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 }
             }
         }
-        group_sync();   // every page's P fragments (and zeroed V rows) are in place
+        group_sync();   // every page's P fragments are in place
 
         // O[:, this warp's columns] += P V over the stage's pages (a V fragment serves every m-tile)
 #pragma unroll

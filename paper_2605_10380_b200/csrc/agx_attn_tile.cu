@@ -394,12 +394,65 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     }
 }
 
+// K or V of a tile that holds block rows or ends inside a page, by the whole producer warp.  Tokens [0, pool_end) come from the pool,
+// with a fused append the block's own from k_new / v_new: pages from the pool; a tile of nothing but block rows as one copy where
+// 128 rows are there; else row groups of 8 tokens from k_new / v_new; and by hand the groups that mix prefix and block or, for V,
+// reach beyond the last token (zeros: P is 0 there, but 0 * NaN is not).  Out of line: inlined twice into the producer's loop it cost the
+// other warps 7 % on a long prefill that never takes it (instruction fetch).
+__device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* pool_map, const CUtensorMap* rows8, const CUtensorMap* rows128,
+                                        const unsigned char* pool, const unsigned char* rows, bool is_v, int g, int P, int L, int q_row0,
+                                        unsigned char* dst, uint32_t full_bar, int tok0, int npg, int id) {
+    const int lane = threadIdx.x & 31, hkv = p.hkv;
+    const int pool_end = rows ? P : L, pool_full = pool_end & ~(kPage - 1);
+    const int pool_pg = min(npg, max(0, (pool_full - tok0) >> 4));        // pages of the tile that come from the pool; lane l holds page l's id
+    const int own0 = tok0 + pool_pg * kPage, own1 = tok0 + npg * kPage;   // tokens of the pages that do not
+    const int rows0 = min(own1, max(own0, (pool_end + 7) & ~7));          // row groups by TMA: [rows0, rows1)
+    const int rows1 = rows ? max(rows0, min(own1, is_v ? (L & ~7) : ((L + 7) & ~7))) : rows0;
+    const int own_id = __shfl_sync(0xFFFFFFFFu, id, pool_pg & 31);
+    // (the whole-tile copy may bring in rows of the next sequence: for V none of them may be met by the MMAs, 16 tokens at a time)
+    const int row0_new = q_row0 + tok0 - P;
+    const bool big = rows && tok0 >= P && row0_new + kBN <= p.total_rows && (!is_v || own1 <= L);
+    bool by_hand = false;
+    for (int base = own0; base < own1 && !big; base += 8) {
+        if (base == rows0) base = rows1;
+        if (base >= own1 || (!is_v && base >= rows1)) break;   // (K rows beyond the last token are masked, whatever they are)
+        by_hand = true;
+        uint4 u[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int tok = base + (lane >> 4) + 2 * j;
+            u[j] = make_uint4(0, 0, 0, 0);
+            if (tok < pool_end) u[j] = __ldcg((const uint4*)(pool + (((long long)own_id * hkv + g) * kPage + (tok & 15)) * 256 + (lane & 15) * 16));
+            else if (tok < L) u[j] = __ldg((const uint4*)(rows + ((long long)(q_row0 + tok - P) * hkv + g) * 256 + (lane & 15) * 16));
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = (lane >> 4) + 2 * j;
+            *(uint4*)(dst + (base - tok0) * 256 + ((lane & 15) >> 3) * 1024 + r * 128 + (((lane & 7) ^ r) << 4)) = u[j];
+        }
+    }
+    if (by_hand) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncwarp();
+    const uint32_t d = smem_u32(dst);
+    if (lane == 0) {
+        mbar_arrive_expect_tx(full_bar, big ? kTileBytes : pool_pg * kPageBytes + (rows1 - rows0) * 256);
+        if (big) tma_load_rows128(d, rows128, row0_new, g, full_bar);
+    }
+    __syncwarp();
+    if (!big) {
+        if (lane < pool_pg) tma_load_page(d + lane * kPageBytes, pool_map, (id * hkv + g) * (kPage / 8), full_bar);
+        const int base = rows0 + lane * 8;
+        if (base < rows1) tma_load_rows8(d + (base - tok0) * 256, rows8, q_row0 + base - P, g, full_bar);
+    }
+    __syncwarp();
+}
+
 }  // namespace
 
 template <bool kStreams>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k,
-                      const __grid_constant__ CUtensorMap map_v) {
+                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ RowsMaps maps_new) {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* smem = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -446,12 +499,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     }
     // Early loads: with p.early_prefix the caller vouches that the page table and the K/V pages below the cached-prefix
     // length are not written by any launch still in flight, so the producer warp may fetch them while the launch in
-    // front of this one drains.  A CTA that first stores block rows of its own (fused append) keeps to the usual order.
-    const bool own_rows = p.k_new && kv_begin < L && kv_begin + sp.split_tokens > P;
-    const bool early_cta = p.early_prefix && !own_rows;
-    if (!(warp == 0 && early_cta)) pdl_wait();   // from here on global memory written by the launch before this one is read (Q, page table, K/V)
-    // fused append (one row chunk per sequence): the block's own K/V rows of this split go into the pages first
-    if (own_rows && warp >= 2) append_rows_bf16(p, sp, g, kv_begin, kv_begin + sp.split_tokens, tid - 64, kQLoadThreads);
+    // front of this one drains.
+    if (!(warp == 0 && p.early_prefix)) pdl_wait();   // from here on global memory written by the launch before this one is read (Q, page table, K/V)
     // Q: 256 rows x 256 B by 16-byte cp.async (all of a thread's copies in flight at once), written in
     // the 128-byte-swizzled K-major operand layout; rows past q * G are zero-filled.
     if (warp >= 2) {
@@ -466,10 +515,17 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cp_async_16(smem_base + kOffQ + tile * kTileBytes + half * kHalfBytes + rt * 128 + ((u ^ (rt & 7)) << 4), src, valid ? 16u : 0u);
         }
     }
+    // fused append: the CTAs of a row chunk store the block rows whose first query row lies in the chunk, each split its share, while the
+    // first K tile and Q are on their way
+    if (p.k_new && warp >= 2) {
+        const int i_lo = (row0 + G - 1) / G, i_n = min(q, (row0 + kRowsPerCta + G - 1) / G) - i_lo;
+        const int parts = (it.vis_end + sp.split_tokens - 1) / sp.split_tokens;   // splits with work (the last ones may have none)
+        store_block_rows(p, sp, g, i_lo + i_n * split / parts, i_lo + i_n * (split + 1) / parts, tid - 64, kQLoadThreads);
+    }
     // Barriers initialised, TMEM address published.  Warp 0 (which set the barriers up and needs nothing
     // from the others) only signals and goes straight to the page table and its first K/V copies.
     tc_fence_before();
-    if (warp == 0 && !own_rows) { __syncwarp(); asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory"); }   // (a fused append must land first)
+    if (warp == 0) { __syncwarp(); asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory"); }
     else asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
     tc_fence_after();
     const uint32_t tmem_base = (warp == 0) ? 0u : *tmem_slot;
@@ -484,14 +540,16 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsLow));
     if (warp == 0) {
-        // ================= TMA producer: lane l of the warp copies page l of the tile =================
+        // ================= TMA producer =================
         const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
         const int page0 = kv_begin / kPage;
         const int n_pages_total = (kv_end - kv_begin + kPage - 1) / kPage;
         int ids = 0;  // page ids of the current group of 4 tiles: lane l holds page (group * 32 + l)
         bool ok = true;
-        bool waited = !early_cta;       // has this warp passed the dependency wait?
+        bool waited = !p.early_prefix;       // has this warp passed the dependency wait?
         const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
+        // tokens [0, pool_end) come from the pool; a tile wholly inside the pool's full pages is eight page copies, see load_mixed for others
+        const int pool_full = (p.k_new ? P : L) & ~(kPage - 1);
         int last_k = -1, last_v = -1;   // last tiles whose copies were armed (for the drain below)
         for (int t = 0; t < n_tiles && ok; ++t) {
             const int tok0 = kv_begin + t * kBN;
@@ -511,14 +569,20 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             const int ks = t % kStagesK, kph = (t / kStagesK) & 1;
             const int vs = t % kStagesV, vph = (t / kStagesV) & 1;
             const int npg = pages_in_tile(t);
+            const bool pure = tok0 + npg * kPage <= pool_full;
             int group[8];                                   // first row group of each page of the tile
+            if (pure) {
 #pragma unroll
-            for (int pg = 0; pg < 8; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids, (t & 3) * 8 + pg) * p.hkv + g) * (kPage / 8);
+                for (int pg = 0; pg < 8; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids, (t & 3) * 8 + pg) * p.hkv + g) * (kPage / 8);
+            }
             // ---- K
             ok = mbar_wait(bar(BAR_K_EMPTY + ks), kph ^ 1, abort_flag, p.status, p.wait_limit_cycles);
             if (!ok) break;
-            __syncwarp();
-            if (elect_one()) {
+            last_k = t;
+            if (!pure)
+                load_mixed(p, &map_k, &maps_new.k8, &maps_new.k128, (const unsigned char*)p.k_pool, (const unsigned char*)p.k_new, false, g, P, L,
+                           sp.q_row0, smem + kOffK + ks * kTileBytes, bar(BAR_K_FULL + ks), tok0, npg, __shfl_sync(0xFFFFFFFFu, ids, ((t & 3) * 8 + lane) & 31));
+            else if (elect_one()) {
                 mbar_arrive_expect_tx(bar(BAR_K_FULL + ks), npg * kPageBytes);
                 const uint32_t dst = smem_base + kOffK + ks * kTileBytes;
 #pragma unroll
@@ -526,36 +590,22 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                     if (pg < npg) tma_load_page(dst + pg * kPageBytes, &map_k, group[pg], bar(BAR_K_FULL + ks));
             }
             __syncwarp();
-            last_k = t;
-            // ---- V (the page that holds token L, if L is not page-aligned, is copied by hand so that
-            //      slots past the end of the sequence are zeros whatever the pool holds there)
+            // ---- V
             if (!waited && !(stable && t < kStagesV)) { pdl_wait(); waited = true; }
             ok = mbar_wait(bar(BAR_V_EMPTY + vs), vph ^ 1, abort_flag, p.status, p.wait_limit_cycles);
             if (!ok) break;
-            const int ragged_pg = ((L & 15) != 0 && (L >> 4) >= (tok0 >> 4) && (L >> 4) < (tok0 >> 4) + npg) ? (L >> 4) - (tok0 >> 4) : -1;
-            if (ragged_pg >= 0) {
-                const int id = __shfl_sync(0xFFFFFFFFu, ids, (t & 3) * 8 + ragged_pg);
-                const unsigned char* src = (const unsigned char*)p.v_pool + ((long long)id * p.hkv + g) * (kPage * 256);
-                const int valid_rows = L & 15;
-                for (int idx = lane; idx < 256; idx += 32) {
-                    const int r = idx >> 4, ch = idx & 15, half = ch >> 3, u = ch & 7;
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (r < valid_rows) v = __ldcg((const uint4*)(src + r * 256 + ch * 16));   // (rows a fused append may just have written)
-                    *(uint4*)(smem + v_stage_off(vs) + ragged_pg * kPageBytes + (r >> 3) * 2048 + half * 1024 + (r & 7) * 128 + ((u ^ (r & 7)) << 4)) = v;
-                }
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                __syncwarp();
-            }
-            __syncwarp();
-            if (elect_one()) {
-                mbar_arrive_expect_tx(bar(BAR_V_FULL + vs), (npg - (ragged_pg >= 0 ? 1 : 0)) * kPageBytes);
+            last_v = t;
+            if (!pure)
+                load_mixed(p, &map_v, &maps_new.v8, &maps_new.v128, (const unsigned char*)p.v_pool, (const unsigned char*)p.v_new, true, g, P, L,
+                           sp.q_row0, smem + v_stage_off(vs), bar(BAR_V_FULL + vs), tok0, npg, __shfl_sync(0xFFFFFFFFu, ids, ((t & 3) * 8 + lane) & 31));
+            else if (elect_one()) {
+                mbar_arrive_expect_tx(bar(BAR_V_FULL + vs), npg * kPageBytes);
                 const uint32_t dst = smem_base + v_stage_off(vs);
 #pragma unroll
                 for (int pg = 0; pg < 8; ++pg)
-                    if (pg < npg && pg != ragged_pg) tma_load_page(dst + pg * kPageBytes, &map_v, group[pg], bar(BAR_V_FULL + vs));
+                    if (pg < npg) tma_load_page(dst + pg * kPageBytes, &map_v, group[pg], bar(BAR_V_FULL + vs));
             }
             __syncwarp();
-            last_v = t;
         }
         // drain: the copies this warp started must land before the CTA's shared memory goes away.  Bounded by the
         // clock alone: after a time-out elsewhere in the CTA the abort flag is up, and the copies still have to land.
@@ -680,14 +730,16 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
         }
         __syncwarp();
-    } else if (tid == 32 * 3) {   // an otherwise idle warp parks the epilogue's context
-        EpiCtx* cx = (EpiCtx*)(smem + kOffCtx);
-        cx->it = locate_item<kStreams>(p, blockIdx.x);
-        cx->part_base = sp.part_base; cx->hq = p.hq;
-        cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->lse = p.lse;
-        cx->magic = p.row_div_magic;
-        cx->part_half = p.part_half;
-        mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
+    } else {   // warps 2 and 3, otherwise idle
+        if (tid == 32 * 3) {   // park the epilogue's context
+            EpiCtx* cx = (EpiCtx*)(smem + kOffCtx);
+            cx->it = locate_item<kStreams>(p, blockIdx.x);
+            cx->part_base = sp.part_base; cx->hq = p.hq;
+            cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->lse = p.lse;
+            cx->magic = p.row_div_magic;
+            cx->part_half = p.part_half;
+            mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
+        }
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kRegsHigh));
@@ -847,9 +899,29 @@ bool make_pool_map(CUtensorMap* map, const void* pool, long long num_pages, int 
     return make_pool_map_impl(map, pool, num_pages, hkv);
 }
 
+// [KV heads][row groups of 8][halves of 64 dims][rows][64 dims]; the row and the row-group dimension overlap (a box of 16 groups from any
+// row on), so the bounds of the map do not protect a box of `groups` > 1: its 8 * groups rows have to exist
+static bool make_rows_map(CUtensorMap* map, const void* rows, long long total_q, int hkv, int groups) {
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)hkv * kD * 2;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)total_q, 2, (cuuint64_t)groups, (cuuint64_t)hkv};
+    const cuuint64_t strides[4] = {row, 128, row * 8, (cuuint64_t)kD * 2};
+    const cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)groups, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(rows), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool make_rows_maps(RowsMaps* m, const void* k_new, const void* v_new, long long total_q, int hkv) {
+    return make_rows_map(&m->k8, k_new, total_q, hkv, 1) && make_rows_map(&m->v8, v_new, total_q, hkv, 1) &&
+           make_rows_map(&m->k128, k_new, total_q, hkv, 16) && make_rows_map(&m->v128, v_new, total_q, hkv, 16);
+}
+
 namespace {
 template <bool kStreams>
-cudaError_t launch_tile(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
+cudaError_t launch_tile(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, const RowsMaps& maps_new,
+                        cudaStream_t stream) {
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
     static bool configured_on[64] = {false};
     int device = 0;
@@ -860,14 +932,14 @@ cudaError_t launch_tile(const AttnParams& p, const CUtensorMap& map_k, const CUt
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_chained(attn_tile_bf16_kernel<kStreams>, dim3(p.num_items), dim3(kThreads), kSmemBytes, stream, p, map_k, map_v);
+    return launch_chained(attn_tile_bf16_kernel<kStreams>, dim3(p.num_items), dim3(kThreads), kSmemBytes, stream, p, map_k, map_v, maps_new);
 }
 }  // namespace
 
 cudaError_t launch_attn_tile_bf16(const AttnParams& p, bool streams, const CUtensorMap& map_k, const CUtensorMap& map_v,
-                                  cudaStream_t stream) {
+                                  const RowsMaps& maps_new, cudaStream_t stream) {
     if (p.num_items == 0) return cudaSuccess;
-    return streams ? launch_tile<true>(p, map_k, map_v, stream) : launch_tile<false>(p, map_k, map_v, stream);
+    return streams ? launch_tile<true>(p, map_k, map_v, maps_new, stream) : launch_tile<false>(p, map_k, map_v, maps_new, stream);
 }
 
 }  // namespace agx

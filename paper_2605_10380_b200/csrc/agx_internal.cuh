@@ -16,6 +16,11 @@ constexpr long long kWaitLimitCycles = 4000000000ll;  // ~2 s at 1.9 GHz: defaul
 
 // TMA view of a KV pool (head_dim 128, bf16): one box is the 16 rows of one page and KV head, see tma_load_page.
 bool make_pool_map(CUtensorMap* map, const void* pool, long long num_pages, int hkv);
+// TMA views of a block's own K and V rows [total_q][hkv][128] bf16: one box is 8 or 128 rows of one KV head, see tma_load_rows8 / 128.
+struct alignas(64) RowsMaps {
+    CUtensorMap k8, v8, k128, v128;
+};
+bool make_rows_maps(RowsMaps* maps, const void* k_new, const void* v_new, long long total_q, int hkv);
 
 // Per-sequence launch plan, built on the host from the host lengths.
 struct SeqPlan {
@@ -48,6 +53,7 @@ struct AttnParams {
     const void* k_new;   // fused append (agx_attn_prefixed_append): the block's K/V rows [total_q][hkv][d], or NULL
     const void* v_new;
     long long num_pages;
+    int total_rows;      // rows of k_new / v_new
     int pt_stride;
     int hq, hkv, head_dim;
     int num_seqs;
@@ -132,8 +138,9 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
 // Tensor-core tile kernel (bf16, d = 128, tcgen05 + TMEM + TMA).  streams = false: 256 query rows per CTA
 // (two Q tiles); streams = true: 128 rows per CTA whose KV tiles alternate between two softmax warpgroups
 // (verify blocks and short suffixes over long contexts).
+// maps_new: views of p.k_new / p.v_new (fused append; unused otherwise).
 cudaError_t launch_attn_tile_bf16(const AttnParams& p, bool streams, const CUtensorMap& map_k, const CUtensorMap& map_v,
-                                  cudaStream_t stream);
+                                  const RowsMaps& maps_new, cudaStream_t stream);
 
 cudaError_t launch_accept(const void* logits, int logits_dtype, long long row_stride, int vocab, const int* drafts,
                           const int* cu_q, int B, int total_q, int* accept_len, int* next_token, int* argmax,

@@ -64,6 +64,16 @@ __device__ __forceinline__ void tma_load_page(uint32_t dst, const CUtensorMap* m
                  ::"r"(dst), "l"(map), "r"(0), "r"(group), "r"(bar) : "memory");
 }
 
+// Eight or 128 rows of one KV head of the block's own K or V ([total_q][hkv][128]) from `row` on (see RowsMaps), in the layout of
+// row groups.  Past the end the 8-row copy brings zeros; the 128 rows must all exist.
+__device__ __forceinline__ void tma_load_rows8(uint32_t dst, const CUtensorMap* map, int row, int head, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %2, %2, %4}], [%5];\n"
+                 ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(head), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_load_rows128(uint32_t dst, const CUtensorMap* map, int row, int head, uint32_t bar) {
+    tma_load_rows8(dst, map, row, head, bar);   // (the map's box is 16 row groups)
+}
+
 // One lane of a converged warp.  Unlike `lane == 0` this tells the compiler that a single thread takes the branch, so the
 // instructions that want their operands in uniform registers (tcgen05.mma, TMA copies) are issued without a loop over lanes.
 __device__ __forceinline__ bool elect_one() {
@@ -78,25 +88,32 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
-// Fused KV append (bf16, d = 128): the CTA that will read tokens [t_lo, t_hi) of KV head g writes the block's own
-// rows in that range into the sequence's pages first (Sec. 2.3: the block's KV joins the cache before it is attended
-// to), then makes them visible to the TMA copies that follow: a generic-proxy fence here, a CTA barrier at the caller.
-__device__ __forceinline__ void append_rows_bf16(const AttnParams& p, const SeqPlan& sp, int g, int t_lo, int t_hi, int tid,
-                                                 int nthreads) {
-    const int lo = max(t_lo, sp.prefix_len), hi = min(t_hi, sp.prefix_len + sp.q_len);
-    if (hi > lo) {
-        const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
-        for (int idx = tid; idx < (hi - lo) * 32; idx += nthreads) {
-            const int tok = lo + (idx >> 5), is_v = (idx >> 4) & 1, c = idx & 15;
-            const long long page = (tok >> 4) < p.pt_stride ? __ldg(pt_row + (tok >> 4)) : -1;
-            if (page < 0 || page >= p.num_pages) { if (c == 0) atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
-            const unsigned char* src = (const unsigned char*)(is_v ? p.v_new : p.k_new) +
-                                       (((long long)(sp.q_row0 + tok - sp.prefix_len) * p.hkv + g) * 256 + c * 16);
-            unsigned char* dst = (unsigned char*)(is_v ? p.v_pool : p.k_pool) + (((page * p.hkv + g) * kPage + (tok & 15)) * 256 + c * 16);
-            *(uint4*)dst = __ldg((const uint4*)src);
+// Fused KV append (bf16, d = 128): the block's rows [i_lo, i_hi) of KV head g go into the sequence's pages (Sec. 2.3: the block's KV
+// joins the cache).  Nothing in the same launch reads them there: the attention CTAs take the block's own rows from k_new / v_new,
+// so there is nothing to wait for.
+__device__ __forceinline__ void store_block_rows(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int tid, int nthreads) {
+    const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
+    const int units = (i_hi - i_lo) * 32;
+    constexpr int kBatch = 4;   // loads in flight per thread
+    for (int idx0 = tid; idx0 < units; idx0 += kBatch * nthreads) {
+        uint4 v[kBatch];
+        int id[kBatch];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int idx = idx0 + j * nthreads, i = i_lo + (idx >> 5), slot = (sp.prefix_len + i) >> 4;
+            id[j] = -2;
+            if (idx < units) {
+                id[j] = slot < p.pt_stride ? __ldg(pt_row + slot) : -1;
+                v[j] = __ldg((const uint4*)((const unsigned char*)((idx & 16) ? p.v_new : p.k_new) + (((long long)(sp.q_row0 + i) * p.hkv + g) * 256 + (idx & 15) * 16)));
+            }
         }
-        __threadfence();
-        asm volatile("fence.proxy.async;\n" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const int idx = idx0 + j * nthreads, tok = sp.prefix_len + i_lo + (idx >> 5);
+            if (id[j] >= 0 && id[j] < p.num_pages)
+                *(uint4*)((unsigned char*)((idx & 16) ? p.v_pool : p.k_pool) + ((((long long)id[j] * p.hkv + g) * kPage + (tok & 15)) * 256 + (idx & 15) * 16)) = v[j];
+            else if (id[j] != -2) atomicOr(p.status, AGX_DEV_BAD_PAGE);
+        }
     }
 }
 
