@@ -471,7 +471,7 @@ int64_t agx_attn_workspace_bytes(agx_handle* h, int32_t B, const int32_t* P, con
 static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_new, const void* v_new, const void* k_pool,
                             const void* v_pool, int64_t num_pages, const int32_t* page_table, int32_t pt_stride,
                             const int32_t* P, const int32_t* Q, int32_t B, void* out, float* lse, void* workspace,
-                            size_t workspace_bytes, void* stream_v) {
+                            size_t workspace_bytes, void* stream_v, bool early_prefix) {
     CallRange range_("agx_attn_prefixed");
     if (!h) return AGX_E_INVAL;
     h->last_launches = 0;
@@ -508,7 +508,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.scale_log2 = h->scale * 1.4426950408889634f;
     p.row_div_magic = (0x100000000ull + (unsigned)(p.hq / p.hkv) - 1) / (unsigned)(p.hq / p.hkv);
     p.wait_limit_cycles = h->wait_limit_cycles;
-    p.early_prefix = h->early_prefix;
+    p.early_prefix = early_prefix;
     p.drop_stage = h->drop_stage;
     alignas(64) CUtensorMap map_k, map_v;   // (encoding one takes 0.05 us)
     RowsMaps maps_new;
@@ -567,7 +567,7 @@ agx_status agx_attn_prefixed(agx_handle* h, const void* q_block, const void* k_p
                              const int32_t* Q, int32_t B, void* out, float* lse, void* workspace,
                              size_t workspace_bytes, void* stream) {
     return attn_impl(h, q_block, nullptr, nullptr, k_pool, v_pool, num_pages, page_table, pt_stride, P, Q, B, out, lse,
-                     workspace, workspace_bytes, stream);
+                     workspace, workspace_bytes, stream, h && h->early_prefix);
 }
 
 agx_status agx_attn_prefixed_append(agx_handle* h, const void* q_block, const void* k_new, const void* v_new, void* k_pool,
@@ -576,7 +576,7 @@ agx_status agx_attn_prefixed_append(agx_handle* h, const void* q_block, const vo
                                     void* workspace, size_t workspace_bytes, void* stream) {
     if (h && B > 0 && (!k_new || !v_new)) return fail(h, AGX_E_INVAL, "null pointer");
     return attn_impl(h, q_block, k_new, v_new, k_pool, v_pool, num_pages, page_table, pt_stride, P, Q, B, out, lse,
-                     workspace, workspace_bytes, stream);
+                     workspace, workspace_bytes, stream, h && h->early_prefix);
 }
 
 static int accept_chunks(const agx_handle* h, int total_q, int vocab, int dtype) {
@@ -927,9 +927,10 @@ static agx_status verify_step_host_impl(agx_handle* h, void* k_pool, void* v_poo
         h2d(L.cu, cu.data(), (size_t)(B + 1) * 4);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "host step: upload");
-    st = agx_attn_prefixed_append(h, ws + L.q, ws + L.k, ws + L.v, k_pool, v_pool, num_pages, page_table, pt_stride, P, Q,
-                                  B, out_dev, nullptr, L.attn_ws_bytes ? ws + L.attn_ws : nullptr, L.attn_ws_bytes,
-                                  stream);
+    // behind the stage-in kernel, which lets this launch start only when everything before it is complete, cached-prefix pages may
+    // always be fetched early
+    st = attn_impl(h, ws + L.q, ws + L.k, ws + L.v, k_pool, v_pool, num_pages, page_table, pt_stride, P, Q, B, out_dev, nullptr,
+                   L.attn_ws_bytes ? ws + L.attn_ws : nullptr, L.attn_ws_bytes, stream, mv || h->early_prefix);
     if (st == AGX_OK) launches += h->last_launches;
     if (logits_done) {   // (also when the attention call failed: the side stream is brought back before the call returns)
         e = cudaStreamWaitEvent(stream, logits_done, 0);

@@ -110,9 +110,11 @@ cudaError_t launch_write_meta(const StepMeta& m, int* prefix, int* seq_lens, int
     return launch_chained(write_meta_kernel, dim3(1), dim3(64), 0, stream, m, prefix, seq_lens, cu_q);
 }
 
+// Bound by the trip across the bus (96 KB: 6.2 us).  The next launch may start only once everything in front of this one is complete, so
+// that the attention kernel behind it may fetch cached-prefix pages, its set-up and its page ids while this kernel waits for the bus.
 __global__ void __launch_bounds__(256) stage_in_kernel(const StageCopies c) {
-    pdl_launch_dependents();
     pdl_wait();   // the launch before this one may still read the destination
+    pdl_launch_dependents();
     const unsigned n0 = c.units[0], n1 = n0 + c.units[1], n2 = n1 + c.units[2];
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += gridDim.x * blockDim.x) {
         const int k = i < n0 ? 0 : i < n1 ? 1 : 2;
