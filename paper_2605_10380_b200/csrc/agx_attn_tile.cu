@@ -4,6 +4,10 @@
 // tensor cores: tcgen05.mma issued by one thread, operands staged in shared memory by TMA,
 // accumulators in tensor memory (TMEM).
 //
+// What bounds it: the tensor pipe and the exponentials (2048 cycles each per KV tile), the instruction issue of the single-thread
+// roles, whose warps share their schedulers with two softmax warps each (a KV tile took the TMA producer 3000 cycles while it
+// divided by run-time stage counts and shuffled page ids; it is now two 16-byte loads and eight copies), and on long runs the power cap.
+//
 // Work item = (sequence, KV head g, chunk of 256 query rows, KV split).  The q * G rows of one KV
 // head (row r = i * G + h % G) are cut into two 128-row tiles A and B that share every K/V tile.
 // CTA = 12 warps:
@@ -11,19 +15,22 @@
 //               for V (SWIZZLE_128B), page ids read through the page table.  One box per page instead of two
 //               of 64 dims, issued without a loop over lanes: 4 x 32768 verify 107 -> 100 us, 16 x 8192 verify
 //               116 -> 92 us, 16 decode blocks over 2k-14k tokens 83 -> 76 us.
-//   warp 1      MMA issuer (one elected thread: with `lane == 0` the issue of eight tcgen05.mma took up to
-//               570 cycles, with elect.sync about 300) and TMEM owner.  Order on the tensor pipe:
-//               S_A(0) S_B(0) | O_A+=P_A V(t)  S_A(t+1)  O_B+=P_B V(t)  S_B(t+1) | ...
-//               so the softmax of one tile overlaps the MMAs of the other.
+//   warps 1, 2  MMA issuers, one elected thread each (elect.sync: behind `lane == 0` the issue of eight tcgen05.mma took up to
+//               570 cycles), warp 1 also TMEM owner.  Warp 1 issues S = Q K^T, warp 2 O += P V:
+//               S(A, 0) | S(B, 0) | S(A, 1)  O_A += P_A V(0) | S(B, 1)  O_B += P_B V(0) | ...
+//               There is one S for both tiles: it is free as soon as the softmax warps hold the scores in registers, so
+//               that S of the next unit is computed under the softmax of this one and under the PV of the one before.
+//               (c3 29.8 -> 29.2 us, 16 x 8192 verify 100 -> 92, 16 decode blocks 78.5 -> 76.5 against the schedule in which P overwrote
+//               S and the next S waited for PV.)  Long tensor-bound runs are at the board's power cap either way.
 //   warps 4-7   softmax of tile A, warps 8-11 softmax of tile B: one thread per query row (TMEM lane).
 //               The whole 128-column score row is held in registers (the two softmax warpgroups take
 //               registers from warps 0-3 with setmaxnreg), so S is read from TMEM once: row maximum,
-//               exponentials with packed f32x2 arithmetic, P written back over S as packed bf16 (the A
+//               exponentials with packed f32x2 arithmetic, P written to TMEM as packed bf16 (the A
 //               operand of the P V MMA comes from TMEM), O rescaled in TMEM only when the row maximum
 //               grew by more than 2^8.
 // The Q tiles arrive by cp.async from warps 2-11 while warp 0 already streams K/V; results leave through
 // a per-warp shared-memory staging area so that global stores are whole rows.
-// TMEM columns: S_A [0,128) S_B [128,256) O_A [256,384) O_B [384,512).
+// TMEM columns: S [0,128) P_A [128,192) P_B [192,256) O_A [256,384) O_B [384,512).
 // Every mbarrier wait is bounded: on time-out the CTA records AGX_DEV_WAIT_TIMEOUT and tears down.
 #include <cuda.h>
 #include <math.h>
@@ -37,7 +44,6 @@ namespace {
 
 constexpr int kD = 128;
 constexpr int kBN = 128;                    // KV tokens per tile
-constexpr int kStagesK = 3;                 // K is wanted right after the previous tile's softmax: one more stage
 // Two schedules share the kernel (template parameter kStreams):
 //   false  two 128-row Q tiles A and B per CTA (256 rows), both meet every KV tile;
 //   true   ONE 128-row Q tile per CTA (verify blocks and short suffixes: q * G <= 128 rows, most of them
@@ -47,7 +53,8 @@ constexpr int kStagesK = 3;                 // K is wanted right after the previ
 //          and the softmax of one tile hides behind the MMAs and copies of the next.
 template <bool kStreams> struct Sched {
     static constexpr int kRows = kStreams ? 128 : 256;     // query rows per CTA
-    static constexpr int kStagesV = kStreams ? 3 : 2;      // the second Q tile's shared memory becomes a V stage
+    static constexpr int kStagesK = kStreams ? 3 : 2;      // K is freed early (QK of a tile runs a unit ahead), V late
+    static constexpr int kStagesV = 3;
 };
 constexpr int kThreads = 384;
 constexpr uint32_t kTileBytes = 128 * 256;  // one operand tile: [2 halves of 64 dims][128 rows][128 B]
@@ -55,13 +62,15 @@ constexpr uint32_t kHalfBytes = 128 * 128;  // (Q tiles: [2 halves][128 rows][12
 constexpr uint32_t kPageBytes = kPage * 256; // K/V tiles: 8 pages of [2 row groups][2 halves of 64 dims][8 rows][128 B], as TMA writes them
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffK = 2 * kTileBytes;
-constexpr uint32_t kOffV = kOffK + kStagesK * kTileBytes;
+constexpr uint32_t kOffV = kOffK + 3 * kTileBytes;
 constexpr uint32_t kOffBar = kOffV + 2 * kTileBytes;
-// V stage s: the first two behind the K ring, the third (kStreams only) in the unused second Q tile
-__host__ __device__ constexpr uint32_t v_stage_off(int s) { return s < 2 ? kOffV + s * kTileBytes : kOffQ + kTileBytes; }
+// V stage s: the first two at kOffV, the third behind two K stages, or (kStreams: three K stages) in the unused second Q tile
+template <bool kStreams>
+__host__ __device__ constexpr uint32_t v_stage_off(int s) { return s < 2 ? kOffV + s * kTileBytes : kStreams ? kOffQ + kTileBytes : kOffK + 2 * kTileBytes; }
 constexpr uint32_t kOffPark = kOffK + 2 * kTileBytes;   // kStreams epilogue: stream 1's O rows (64 KB), then its (m, l)
 constexpr uint32_t kOffCtx = kOffBar + 256;            // what the epilogue needs to know, parked at kernel start
-constexpr uint32_t kSmemBytes = kOffBar + 512 + 1024;  // + barriers + epilogue context + alignment slack
+constexpr uint32_t kOffPages = kOffBar + 512;          // row-group coordinates of the pages of up to 16 tiles
+constexpr uint32_t kSmemBytes = kOffPages + 512 + 1024;   // + alignment slack
 constexpr float kRescaleThreshold = 8.0f;              // log2 units
 // Of every 8 column pairs, this many take the polynomial 2^x instead of the special-function unit (16 exponentials per clock
 // and SM: the two Q tiles' 2 x 128 x 128 take as long as their MMAs).  0 / 1 / 2: c3 30.2 / 29.5 / 30.6 us, 3584 uncached
@@ -70,7 +79,7 @@ constexpr int kPolyPairsOf8 = 1;
 
 // barrier slots (8 bytes each)
 enum { BAR_K_FULL = 0, BAR_K_EMPTY = 3, BAR_V_FULL = 6, BAR_V_EMPTY = 9, BAR_S_FULL = 12, BAR_P_READY = 14,
-       BAR_O_FULL = 16, BAR_Q_FULL = 17, BAR_P_TAIL = 18, BAR_CTX = 20, BAR_COUNT = 21 };
+       BAR_O_FULL = 16, BAR_Q_FULL = 17, BAR_P_TAIL = 18, BAR_CTX = 20, BAR_P_FREE = 21, BAR_S_FREE = 23, BAR_COUNT = 24 };
 // P is handed to the MMA warp in two parts: the first kPvHeadSteps k-steps (16 tokens each) as soon as they are
 // stored, so that their PV MMAs run while the softmax warpgroup still works on the last columns
 constexpr int kPvHeadSteps = 6;
@@ -78,7 +87,7 @@ constexpr int kQLoadThreads = kThreads - 64;  // warps 2..11 bring the Q tiles i
 constexpr int kRegsLow = 96, kRegsHigh = 200; // 128 * 96 + 256 * 200 <= 384 * 168
 
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColS = 0, kColO = 256;  // + 128 * tile
+constexpr uint32_t kColS = 0, kColP = 128, kColO = 256;  // one S for both; P + 64 * tile, O + 128 * tile
 
 // tcgen05 instruction descriptor, kind::f16: D = f32, A = B = bf16, M = 128, N = 128
 constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
@@ -401,14 +410,14 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
 // other warps 7 % on a long prefill that never takes it (instruction fetch).
 __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* pool_map, const CUtensorMap* rows8, const CUtensorMap* rows128,
                                         const unsigned char* pool, const unsigned char* rows, bool is_v, int g, int P, int L, int q_row0,
-                                        unsigned char* dst, uint32_t full_bar, int tok0, int npg, int id) {
+                                        unsigned char* dst, uint32_t full_bar, int tok0, int npg, int group) {
     const int lane = threadIdx.x & 31, hkv = p.hkv;
     const int pool_end = rows ? P : L, pool_full = pool_end & ~(kPage - 1);
-    const int pool_pg = min(npg, max(0, (pool_full - tok0) >> 4));        // pages of the tile that come from the pool; lane l holds page l's id
+    const int pool_pg = min(npg, max(0, (pool_full - tok0) >> 4));        // pages of the tile that come from the pool; lane l holds the first row group of page l
     const int own0 = tok0 + pool_pg * kPage, own1 = tok0 + npg * kPage;   // tokens of the pages that do not
     const int rows0 = min(own1, max(own0, (pool_end + 7) & ~7));          // row groups by TMA: [rows0, rows1)
     const int rows1 = rows ? max(rows0, min(own1, is_v ? (L & ~7) : ((L + 7) & ~7))) : rows0;
-    const int own_id = __shfl_sync(0xFFFFFFFFu, id, pool_pg & 31);
+    const int own_group = __shfl_sync(0xFFFFFFFFu, group, pool_pg & 31);
     // (the whole-tile copy may bring in rows of the next sequence: for V none of them may be met by the MMAs, 16 tokens at a time)
     const int row0_new = q_row0 + tok0 - P;
     const bool big = rows && tok0 >= P && row0_new + kBN <= p.total_rows && (!is_v || own1 <= L);
@@ -422,7 +431,7 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
         for (int j = 0; j < 4; ++j) {
             const int tok = base + (lane >> 4) + 2 * j;
             u[j] = make_uint4(0, 0, 0, 0);
-            if (tok < pool_end) u[j] = __ldcg((const uint4*)(pool + (((long long)own_id * hkv + g) * kPage + (tok & 15)) * 256 + (lane & 15) * 16));
+            if (tok < pool_end) u[j] = __ldcg((const uint4*)(pool + ((long long)own_group * 8 + (tok & 15)) * 256 + (lane & 15) * 16));
             else if (tok < L) u[j] = __ldg((const uint4*)(rows + ((long long)(q_row0 + tok - P) * hkv + g) * 256 + (lane & 15) * 16));
         }
 #pragma unroll
@@ -440,7 +449,7 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
     }
     __syncwarp();
     if (!big) {
-        if (lane < pool_pg) tma_load_page(d + lane * kPageBytes, pool_map, (id * hkv + g) * (kPage / 8), full_bar);
+        if (lane < pool_pg) tma_load_page(d + lane * kPageBytes, pool_map, group, full_bar);
         const int base = rows0 + lane * 8;
         if (base < rows1) tma_load_rows8(d + (base - tok0) * 256, rows8, q_row0 + base - P, g, full_bar);
     }
@@ -463,7 +472,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     constexpr int kRowsPerCta = Sched<kStreams>::kRows;
-    constexpr int kStagesV = Sched<kStreams>::kStagesV;
+    constexpr int kStagesK = Sched<kStreams>::kStagesK, kStagesV = Sched<kStreams>::kStagesV;
     // ---- work item
     const TileItem it = locate_item<kStreams>(p, blockIdx.x);
     const SeqPlan& sp = p.seq[find_seq(p, blockIdx.x)];
@@ -486,7 +495,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // ---- setup: barriers, TMEM, Q tiles
     if (tid == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1) ? 4u : (i == BAR_Q_FULL) ? (uint32_t)kQLoadThreads : 1u);
+            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : (i == BAR_Q_FULL) ? (uint32_t)kQLoadThreads : 1u);
         *abort_flag = 0;
         *(long long*)(smem + kOffBar + BAR_COUNT * 8 + 16) = p.wait_limit_cycles;   // for the out-of-line epilogue
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -544,68 +553,78 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
         const int page0 = kv_begin / kPage;
         const int n_pages_total = (kv_end - kv_begin + kPage - 1) / kPage;
-        int ids = 0;  // page ids of the current group of 4 tiles: lane l holds page (group * 32 + l)
+        // Page ids are read 32 (four tiles) at a time and two groups ahead of the copies that need them; their row-group coordinates wait in
+        // shared memory, so that the thread that issues the copies of a tile has them with two loads.
+        int* const page_ring = (int*)(smem + kOffPages);   // [4 groups][32]
+        auto fetch_ids = [&](int group) {   // (by the whole warp; -1: no such page)
+            const int pi = group * 32 + lane;
+            long long id = -1;
+            if (pi < n_pages_total) {
+                id = __ldg(pt_row + page0 + pi);
+                if (id < 0 || id >= p.num_pages) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
+            }
+            return (int)id;
+        };
+        auto put_ids = [&](int group, int id) { page_ring[(group & 3) * 32 + lane] = (id * p.hkv + g) * (kPage / 8); __syncwarp(); };
         bool ok = true;
         bool waited = !p.early_prefix;       // has this warp passed the dependency wait?
         const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
         // tokens [0, pool_end) come from the pool; a tile wholly inside the pool's full pages is eight page copies, see load_mixed for others
         const int pool_full = (p.k_new ? P : L) & ~(kPage - 1);
         int last_k = -1, last_v = -1;   // last tiles whose copies were armed (for the drain below)
-        for (int t = 0; t < n_tiles && ok; ++t) {
-            const int tok0 = kv_begin + t * kBN;
-            const bool stable = tok0 + kBN <= stable_end;
-            // K/V tiles wholly inside the cached prefix, as far as free stages go, may be requested before the wait
-            if (!waited && !(stable && t < kStagesK)) { pdl_wait(); waited = true; }
-            if ((t & 3) == 0) {
-                const int pi = t * 8 + lane;
-                long long id = 0;
-                if (pi < n_pages_total) {
-                    id = __ldg(pt_row + page0 + pi);
-                    if (id < 0 || id >= p.num_pages) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
+        const int n_groups = (n_tiles + 3) >> 2;
+        if (!waited && kv_begin + kBN > stable_end) { pdl_wait(); waited = true; }
+        put_ids(0, fetch_ids(0));
+        int ids_ahead = 0, ahead = -1;       // group `ahead` has been read (its ids are in ids_ahead), groups below it are in page_ring
+        int ks = 0, vs = 0;
+        uint32_t kph = 1, vph = 1;
+        // in the order of need: K(0), K(1), V(0), K(2), V(1), ..., V(n - 1)
+        for (int i = 0; i <= n_tiles; ++i) {
+#pragma unroll
+            for (int is_v = 0; is_v < 2; ++is_v) {
+                const int t = is_v ? i - 1 : i;
+                if (t < 0 || t >= n_tiles || !ok) continue;
+                const int tok0 = kv_begin + t * kBN;
+                // tiles wholly inside the cached prefix, as far as free stages go, may be requested before the wait
+                if (!waited && !(tok0 + kBN <= stable_end && t < (is_v ? kStagesV : kStagesK))) { pdl_wait(); waited = true; }
+                if (!is_v && (t & 3) == 0) {
+                    const int group = t >> 2;
+                    if (group > 0) put_ids(group, ahead == group ? ids_ahead : fetch_ids(group));
+                    if (waited && group + 1 < n_groups) { ids_ahead = fetch_ids(group + 1); ahead = group + 1; }
                 }
-                ids = (int)id;
+                if (t == p.drop_stage) {   // test hook: this tile never arrives, its consumers' waits run out
+                    if (is_v) { if (++vs == kStagesV) { vs = 0; vph ^= 1; } } else if (++ks == kStagesK) { ks = 0; kph ^= 1; }
+                    continue;
+                }
+                const int s = is_v ? vs : ks;
+                const uint32_t full = bar((is_v ? BAR_V_FULL : BAR_K_FULL) + s), empty = bar((is_v ? BAR_V_EMPTY : BAR_K_EMPTY) + s);
+                const uint32_t off = is_v ? v_stage_off<kStreams>(s) : kOffK + s * kTileBytes;
+                ok = mbar_wait(empty, is_v ? vph : kph, abort_flag, p.status, p.wait_limit_cycles);
+                if (!ok) continue;
+                if (is_v) last_v = t; else last_k = t;
+                if (tok0 + kBN <= pool_full && tok0 + kBN <= kv_end) {
+                    if (elect_one()) {
+                        const int4 c0 = *(const int4*)(page_ring + ((t * 8) & 127)), c1 = *(const int4*)(page_ring + ((t * 8) & 127) + 4);
+                        const CUtensorMap* map = is_v ? &map_v : &map_k;
+                        const uint32_t dst = smem_base + off;
+                        mbar_arrive_expect_tx(full, kTileBytes);
+                        tma_load_page(dst, map, c0.x, full);
+                        tma_load_page(dst + kPageBytes, map, c0.y, full);
+                        tma_load_page(dst + 2 * kPageBytes, map, c0.z, full);
+                        tma_load_page(dst + 3 * kPageBytes, map, c0.w, full);
+                        tma_load_page(dst + 4 * kPageBytes, map, c1.x, full);
+                        tma_load_page(dst + 5 * kPageBytes, map, c1.y, full);
+                        tma_load_page(dst + 6 * kPageBytes, map, c1.z, full);
+                        tma_load_page(dst + 7 * kPageBytes, map, c1.w, full);
+                    }
+                } else {
+                    load_mixed(p, is_v ? &map_v : &map_k, is_v ? &maps_new.v8 : &maps_new.k8, is_v ? &maps_new.v128 : &maps_new.k128,
+                               (const unsigned char*)(is_v ? p.v_pool : p.k_pool), (const unsigned char*)(is_v ? p.v_new : p.k_new), is_v, g, P, L,
+                               sp.q_row0, smem + off, full, tok0, pages_in_tile(t), page_ring[(t * 8 + (lane & 7)) & 127]);
+                }
+                __syncwarp();
+                if (is_v) { if (++vs == kStagesV) { vs = 0; vph ^= 1; } } else if (++ks == kStagesK) { ks = 0; kph ^= 1; }
             }
-            if (t == p.drop_stage) continue;   // test hook: this tile never arrives, its consumers' waits run out
-            const int ks = t % kStagesK, kph = (t / kStagesK) & 1;
-            const int vs = t % kStagesV, vph = (t / kStagesV) & 1;
-            const int npg = pages_in_tile(t);
-            const bool pure = tok0 + npg * kPage <= pool_full;
-            int group[8];                                   // first row group of each page of the tile
-            if (pure) {
-#pragma unroll
-                for (int pg = 0; pg < 8; ++pg) group[pg] = (__shfl_sync(0xFFFFFFFFu, ids, (t & 3) * 8 + pg) * p.hkv + g) * (kPage / 8);
-            }
-            // ---- K
-            ok = mbar_wait(bar(BAR_K_EMPTY + ks), kph ^ 1, abort_flag, p.status, p.wait_limit_cycles);
-            if (!ok) break;
-            last_k = t;
-            if (!pure)
-                load_mixed(p, &map_k, &maps_new.k8, &maps_new.k128, (const unsigned char*)p.k_pool, (const unsigned char*)p.k_new, false, g, P, L,
-                           sp.q_row0, smem + kOffK + ks * kTileBytes, bar(BAR_K_FULL + ks), tok0, npg, __shfl_sync(0xFFFFFFFFu, ids, ((t & 3) * 8 + lane) & 31));
-            else if (elect_one()) {
-                mbar_arrive_expect_tx(bar(BAR_K_FULL + ks), npg * kPageBytes);
-                const uint32_t dst = smem_base + kOffK + ks * kTileBytes;
-#pragma unroll
-                for (int pg = 0; pg < 8; ++pg)
-                    if (pg < npg) tma_load_page(dst + pg * kPageBytes, &map_k, group[pg], bar(BAR_K_FULL + ks));
-            }
-            __syncwarp();
-            // ---- V
-            if (!waited && !(stable && t < kStagesV)) { pdl_wait(); waited = true; }
-            ok = mbar_wait(bar(BAR_V_EMPTY + vs), vph ^ 1, abort_flag, p.status, p.wait_limit_cycles);
-            if (!ok) break;
-            last_v = t;
-            if (!pure)
-                load_mixed(p, &map_v, &maps_new.v8, &maps_new.v128, (const unsigned char*)p.v_pool, (const unsigned char*)p.v_new, true, g, P, L,
-                           sp.q_row0, smem + v_stage_off(vs), bar(BAR_V_FULL + vs), tok0, npg, __shfl_sync(0xFFFFFFFFu, ids, ((t & 3) * 8 + lane) & 31));
-            else if (elect_one()) {
-                mbar_arrive_expect_tx(bar(BAR_V_FULL + vs), npg * kPageBytes);
-                const uint32_t dst = smem_base + v_stage_off(vs);
-#pragma unroll
-                for (int pg = 0; pg < 8; ++pg)
-                    if (pg < npg) tma_load_page(dst + pg * kPageBytes, &map_v, group[pg], bar(BAR_V_FULL + vs));
-            }
-            __syncwarp();
         }
         // drain: the copies this warp started must land before the CTA's shared memory goes away.  Bounded by the
         // clock alone: after a time-out elsewhere in the CTA the abort flag is up, and the copies still have to land.
@@ -615,123 +634,82 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             for (int t = max(0, last_v - kStagesV + 1); t <= last_v; ++t)
                 if (t != p.drop_stage) mbar_drain(bar(BAR_V_FULL + t % kStagesV), (t / kStagesV) & 1, p.wait_limit_cycles);
         }
-    } else if (warp == 1) {
-        // ================= MMA issuer =================
-        if (elect_one()) {
-            const uint32_t tS[2] = {tmem_base + kColS, tmem_base + kColS + 128};
-            const uint32_t tO[2] = {tmem_base + kColO, tmem_base + kColO + 128};
+    } else if (warp == 1 || warp == 2) {
+        // ================= MMA issuers: one thread of warp 1 for S = Q K^T, one of warp 2 for O += P V =================
+        // Units of work u = 0, 1, ...: a KV tile against tile A or B (x = u & 1); with kStreams one KV tile each.  S holds one unit's scores: it
+        // is free again as soon as the softmax warps have them in registers, so QK of unit u + 1 runs under the softmax of unit u and
+        // beside PV of unit u - 1.  Two issuing threads, because one was busy all the time: every wait of a warp that shares its scheduler
+        // with two softmax warps costs it 90 cycles and more, also when there is nothing to wait for.
+        const int n_units = kStreams ? n_tiles : 2 * n_tiles;
+        if (warp == 1 && elect_one()) {
+            const uint32_t tS = tmem_base + kColS;
             // descriptors differ only in the start address: add (byte offset >> 4) to a base descriptor
-            const uint64_t q_desc[2] = {make_desc(smem_base + kOffQ, 16, 1024), make_desc(smem_base + kOffQ + kTileBytes, 16, 1024)};
+            const uint64_t q_desc0 = make_desc(smem_base + kOffQ, 16, 1024);
             const uint64_t k_desc0 = make_desc(smem_base + kOffK, 16, 2048);
-            auto issue_qk = [&](int qt, int stage, int x) {   // S_x = Q_qt K^T : 8 k-steps of 16 dims
-                const uint64_t kd = k_desc0 + (uint64_t)((stage * kTileBytes) >> 4);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t q_off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-                    const uint64_t k_off = (uint64_t)(((ks >> 2) * 1024 + (ks & 3) * 32) >> 4);
-                    umma_ss(tS[x], q_desc[qt] + q_off, kd + k_off, kIdescQK, ks > 0);
-                }
-            };
-            // O_x += P_x V, one k-step per page: the head part (pages 0 .. kPvHeadSteps-1) once P_READY says those columns
-            // of P are stored, the tail part after P_TAIL
-            auto issue_pv = [&](int x, int stage, int npg, bool first, bool tail) {
-                const uint64_t vd = make_desc(smem_base + v_stage_off(stage), 1024, 2048);
-                if (npg == 8) {
-                    if (!tail) {
-#pragma unroll
-                        for (int ks = 0; ks < kPvHeadSteps; ++ks)
-                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, !(first && ks == 0));
-                    } else {
-#pragma unroll
-                        for (int ks = kPvHeadSteps; ks < 8; ++ks)
-                            umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, true);
-                    }
-                } else {
-                    for (int ks = tail ? kPvHeadSteps : 0; ks < (tail ? npg : min(npg, kPvHeadSteps)); ++ks)
-                        umma_ts(tO[x], tS[x] + ks * 8, vd + (uint64_t)((ks * kPageBytes) >> 4), kIdescPV, !(first && ks == 0));
-                }
-            };
             bool ok = mbar_wait(bar(BAR_Q_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
-            if (kStreams) {
-                // stream x = t & 1 owns KV tile t:  S_0(0) S_1(1) | O_x += P_x V(t), S_x(t + 2) | ...
-                for (int t = 0; t < 2 && t < n_tiles && ok; ++t) {
-                    ok = mbar_wait(bar(BAR_K_FULL + t), 0, abort_flag, p.status, p.wait_limit_cycles);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_qk(0, t, t); umma_commit(bar(BAR_S_FULL + t));
-                    umma_commit(bar(BAR_K_EMPTY + t));
+            int ks = 0;
+            uint32_t kph = 0;
+            for (int u = 0; u < n_units && ok; ++u) {
+                const int x = u & 1;
+                if (kStreams || x == 0) ok = mbar_wait(bar(BAR_K_FULL + ks), kph, abort_flag, p.status, p.wait_limit_cycles);
+                if (ok && u > 0) ok = mbar_wait(bar(BAR_S_FREE), x ^ 1, abort_flag, p.status, p.wait_limit_cycles);   // unit u - 1 is in registers
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t qd = q_desc0 + (uint64_t)((kStreams ? 0 : x * kTileBytes) >> 4);
+                const uint64_t kd = k_desc0 + (uint64_t)((ks * kTileBytes) >> 4);
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {   // 8 k-steps of 16 dims
+                    const uint64_t q_off = (uint64_t)(((s >> 2) * kHalfBytes + (s & 3) * 32) >> 4);
+                    const uint64_t k_off = (uint64_t)(((s >> 2) * 1024 + (s & 3) * 32) >> 4);
+                    umma_ss(tS, qd + q_off, kd + k_off, kIdescQK, s > 0);
                 }
-                for (int t = 0; t < n_tiles && ok; ++t) {
-                    const int x = t & 1, vs = t % kStagesV, vph = (t / kStagesV) & 1, npg = pages_in_tile(t);
-                    ok = mbar_wait(bar(BAR_V_FULL + vs), vph, abort_flag, p.status, p.wait_limit_cycles);
-                    if (!ok) break;
-                    ok = mbar_wait(bar(BAR_P_READY + x), (t >> 1) & 1, abort_flag, p.status, p.wait_limit_cycles);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv(x, vs, npg, t < 2, false);
-                    ok = mbar_wait(bar(BAR_P_TAIL + x), (t >> 1) & 1, abort_flag, p.status, p.wait_limit_cycles);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv(x, vs, npg, t < 2, true);
+                umma_commit(bar(BAR_S_FULL + x));
+                if (kStreams || x) {
+                    umma_commit(bar(BAR_K_EMPTY + ks));
+                    if (++ks == kStagesK) { ks = 0; kph ^= 1; }
+                }
+            }
+        } else if (warp == 2 && elect_one()) {
+            bool ok = true;
+            int vs = 0;
+            uint32_t vph = 0;
+            for (int u = 0; u < n_units && ok; ++u) {
+                const int x = u & 1, t = kStreams ? u : u >> 1, npg = pages_in_tile(t);
+                const uint32_t ph = (u >> 1) & 1;
+                const uint32_t tP = tmem_base + kColP + x * 64, tO = tmem_base + kColO + x * 128;
+                const uint64_t vd = make_desc(smem_base + v_stage_off<kStreams>(vs), 1024, 2048);
+                if (kStreams || x == 0) ok = mbar_wait(bar(BAR_V_FULL + vs), vph, abort_flag, p.status, p.wait_limit_cycles);
+                // one k-step per page: the first kPvHeadSteps once P_READY says those columns of P are stored, the rest after P_TAIL
+                if (ok) ok = mbar_wait(bar(BAR_P_READY + x), ph, abort_flag, p.status, p.wait_limit_cycles);
+                if (!ok) break;
+                tc_fence_after();
+                if (npg == 8) {
+#pragma unroll
+                    for (int s = 0; s < kPvHeadSteps; ++s) umma_ts(tO, tP + s * 8, vd + (uint64_t)((s * kPageBytes) >> 4), kIdescPV, u >= 2 || s > 0);
+                } else {
+                    for (int s = 0; s < min(npg, kPvHeadSteps); ++s) umma_ts(tO, tP + s * 8, vd + (uint64_t)((s * kPageBytes) >> 4), kIdescPV, u >= 2 || s > 0);
+                }
+                ok = mbar_wait(bar(BAR_P_TAIL + x), ph, abort_flag, p.status, p.wait_limit_cycles);
+                if (!ok) break;
+                tc_fence_after();
+                if (npg == 8) {
+#pragma unroll
+                    for (int s = kPvHeadSteps; s < 8; ++s) umma_ts(tO, tP + s * 8, vd + (uint64_t)((s * kPageBytes) >> 4), kIdescPV, true);
+                } else {
+                    for (int s = kPvHeadSteps; s < npg; ++s) umma_ts(tO, tP + s * 8, vd + (uint64_t)((s * kPageBytes) >> 4), kIdescPV, true);
+                }
+                umma_commit(bar(BAR_P_FREE + x));
+                if (kStreams || x) {
                     umma_commit(bar(BAR_V_EMPTY + vs));
-                    if (t + 2 < n_tiles) {
-                        const int nks = (t + 2) % kStagesK, nkph = ((t + 2) / kStagesK) & 1;
-                        ok = mbar_wait(bar(BAR_K_FULL + nks), nkph, abort_flag, p.status, p.wait_limit_cycles);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_qk(0, nks, x); umma_commit(bar(BAR_S_FULL + x));
-                        umma_commit(bar(BAR_K_EMPTY + nks));
-                    }
+                    if (++vs == kStagesV) { vs = 0; vph ^= 1; }
                 }
-            } else {
-            if (ok) ok = mbar_wait(bar(BAR_K_FULL + 0), 0, abort_flag, p.status, p.wait_limit_cycles);
-            if (ok) {
-                tc_fence_after();
-                issue_qk(0, 0, 0); umma_commit(bar(BAR_S_FULL + 0));
-                issue_qk(1, 0, 1); umma_commit(bar(BAR_S_FULL + 1));
-                umma_commit(bar(BAR_K_EMPTY + 0));
-            }
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                const int vs = t % kStagesV, vph = (t / kStagesV) & 1, npg = pages_in_tile(t);
-                const bool more = t + 1 < n_tiles;
-                const int nks = (t + 1) % kStagesK, nkph = ((t + 1) / kStagesK) & 1;
-                ok = mbar_wait(bar(BAR_V_FULL + vs), vph, abort_flag, p.status, p.wait_limit_cycles);
-                if (!ok) break;
-                ok = mbar_wait(bar(BAR_P_READY + 0), t & 1, abort_flag, p.status, p.wait_limit_cycles);
-                if (!ok) break;
-                tc_fence_after();
-                issue_pv(0, vs, npg, t == 0, false);
-                ok = mbar_wait(bar(BAR_P_TAIL + 0), t & 1, abort_flag, p.status, p.wait_limit_cycles);
-                if (!ok) break;
-                tc_fence_after();
-                issue_pv(0, vs, npg, t == 0, true);
-                if (more) {
-                    ok = mbar_wait(bar(BAR_K_FULL + nks), nkph, abort_flag, p.status, p.wait_limit_cycles);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_qk(0, nks, 0); umma_commit(bar(BAR_S_FULL + 0));
-                }
-                ok = mbar_wait(bar(BAR_P_READY + 1), t & 1, abort_flag, p.status, p.wait_limit_cycles);
-                if (!ok) break;
-                tc_fence_after();
-                issue_pv(1, vs, npg, t == 0, false);
-                ok = mbar_wait(bar(BAR_P_TAIL + 1), t & 1, abort_flag, p.status, p.wait_limit_cycles);
-                if (!ok) break;
-                tc_fence_after();
-                issue_pv(1, vs, npg, t == 0, true);
-                umma_commit(bar(BAR_V_EMPTY + vs));
-                if (more) {
-                    issue_qk(1, nks, 1); umma_commit(bar(BAR_S_FULL + 1));
-                    umma_commit(bar(BAR_K_EMPTY + nks));
-                }
-            }
             }
             umma_commit(bar(BAR_O_FULL));  // arrives when every MMA issued above has completed
             mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
         }
         __syncwarp();
-    } else {   // warps 2 and 3, otherwise idle
-        if (tid == 32 * 3) {   // park the epilogue's context
+    } else {   // warp 3, otherwise idle
+        if (lane == 0) {   // park the epilogue's context
             EpiCtx* cx = (EpiCtx*)(smem + kOffCtx);
             cx->it = locate_item<kStreams>(p, blockIdx.x);
             cx->part_base = sp.part_base; cx->hq = p.hq;
@@ -747,7 +725,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const int x = (warp - 4) >> 2;                       // tile A / B
         const int rt = ((warp & 3) << 5) + lane;             // row in tile == TMEM lane
         const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-        const uint32_t tS = tmem_base + lane_addr + kColS + x * 128;
+        const uint32_t tS = tmem_base + lane_addr + kColS;
+        const uint32_t tP = tmem_base + lane_addr + kColP + x * 64;
         const uint32_t tO = tmem_base + lane_addr + kColO + x * 128;
         const int q_tile_row0 = row0 + (kStreams ? 0 : x * 128);   // kStreams: both warpgroups hold the same rows
         const int r = q_tile_row0 + rt;
@@ -761,11 +740,13 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         bool ok = true;
         constexpr int kStep = kStreams ? 2 : 1;
         const int t_first = kStreams ? x : 0;
-        if (!warp_has_rows) {   // keep S_FULL / P_READY in step, nothing else
+        if (!warp_has_rows) {   // keep the barriers in step, nothing else
             for (int t = t_first; t < n_tiles && ok; t += kStep) {
-                ok = mbar_wait(bar(BAR_S_FULL + x), ((t - t_first) / kStep) & 1, abort_flag, p.status, p.wait_limit_cycles);
+                const int j = (t - t_first) / kStep;
+                ok = mbar_wait(bar(BAR_S_FULL + x), j & 1, abort_flag, p.status, p.wait_limit_cycles);
+                if (ok && j > 0) ok = mbar_wait(bar(BAR_P_FREE + x), (j - 1) & 1, abort_flag, p.status, p.wait_limit_cycles);
                 __syncwarp();
-                if (ok && lane == 0) { mbar_arrive(bar(BAR_P_READY + x)); mbar_arrive(bar(BAR_P_TAIL + x)); }
+                if (ok && lane == 0) { mbar_arrive(bar(BAR_S_FREE)); mbar_arrive(bar(BAR_P_READY + x)); mbar_arrive(bar(BAR_P_TAIL + x)); }
             }
         } else
         for (int t = t_first; t < n_tiles; t += kStep) {
@@ -777,6 +758,9 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
 #pragma unroll
             for (int c4 = 0; c4 < 4; ++c4) tmem_ld_x32(tS + c4 * 32, sreg + c4 * 32);
             tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_S_FREE));   // (one arrival per warp: 32 on one barrier take turns)
             const int tok0 = kv_begin + t * kBN;
             const bool masked = (tok0 + kBN - 1 > P + tile_i_min) || (tok0 + kBN > kv_end);  // uniform per tile
             float lt0 = 0.f, lt1 = 0.f, lt2 = 0.f, lt3 = 0.f;   // this tile's row sum, four partial sums
@@ -798,7 +782,14 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             }
             const float m_tile = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sc;
             const bool need = m_tile > m_ref + kRescaleThreshold;
+            // P and O of this tile belong to the MMAs of its previous unit until these are done (long since, normally)
+            auto wait_p_free = [&]() {
+                if (j > 0) ok = mbar_wait(bar(BAR_P_FREE + x), (j - 1) & 1, abort_flag, p.status, p.wait_limit_cycles);
+                tc_fence_after();
+                return ok;
+            };
             if (__any_sync(0xFFFFFFFFu, need)) {
+                if (!wait_p_free()) break;
                 const float m_new = need ? m_tile : m_ref;
                 const float factor = need ? ex2(m_ref - m_new) : 1.f;   // m_ref = -inf gives 0
                 if (j > 0) {
@@ -838,15 +829,16 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             };
             constexpr int kHeadCols = kPvHeadSteps * 16;   // 96 score columns = 48 packed registers
             sweep(0, kHeadCols);
-            tmem_st_x32(tS, sreg);
-            tmem_st_x16(tS + 32, sreg + 32);
+            if (!wait_p_free()) break;
+            tmem_st_x32(tP, sreg);
+            tmem_st_x16(tP + 32, sreg + 32);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BAR_P_READY + x));   // (one arrival per warp: 32 on one barrier take turns)
+            if (lane == 0) mbar_arrive(bar(BAR_P_READY + x));
             sweep(kHeadCols, 128);
             l_run += (lt0 + lt1) + (lt2 + lt3);
-            tmem_st_x16(tS + 48, sreg + 48);
+            tmem_st_x16(tP + 48, sreg + 48);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
