@@ -158,8 +158,8 @@ AGX_API agx_status agx_attn_prefixed(agx_handle* handle, const void* q_block, co
  * agx_attn_prefixed_append - agx_kv_append and agx_attn_prefixed of the same block as one call.
  * Sec. 2.3: the block's K/V rows join the cache (after the cached prefix) and the block then attends to
  * prefix plus block.  Results, in the pools and in `out`, are those of the two calls made one after the
- * other.  bf16 handles with head_dim 128 need no append launch: the attention kernels read the block's rows from
- * k_new / v_new and store them into the pages on the side.  Other handles get an append launch in front.
+ * other, without an append launch: the attention kernels read the block's rows from k_new / v_new and store them into the
+ * pages on the side.
  *   k_new, v_new : device, [total_q][num_kv_heads][head_dim], 16-byte aligned (rows in the order of q_block)
  *   k_pool, v_pool : device pools (written, then read); the other arguments as for agx_attn_prefixed
  * Errors: those of agx_attn_prefixed; a page id outside [0, num_pages) sets AGX_DEV_BAD_PAGE and the row is not written.

@@ -162,16 +162,14 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         int unit, min_split, target;
         long long base_items = 0;  // items per split, summed over sequences
         std::vector<long long> per_seq_items(seqs.size());
-        if (k == KIND_SIMT) { unit = 64; min_split = 256; target = h->sm_count * 16; }
+        if (k == KIND_SIMT) { unit = 64; min_split = 64; target = h->sm_count * 2; }
         else if (k == KIND_TILE || k == KIND_STREAM) { unit = 128; min_split = k == KIND_TILE ? 128 : 256; target = h->sm_count; }
         else { unit = 16; min_split = h->small_min_split; target = h->sm_count * ((k == KIND_SMALL4 || small_kw == 8) ? 1 : 2); }
-        const int rows_per_chunk = (k == KIND_SMALL1) ? 16 : (k == KIND_SMALL2) ? 32 : (k == KIND_SMALL4) ? 64 : (k == KIND_STREAM) ? 128 : 256;
+        const int rows_per_chunk = (k == KIND_SIMT) ? 8 : (k == KIND_SMALL1) ? 16 : (k == KIND_SMALL2) ? 32 : (k == KIND_SMALL4) ? 64 : (k == KIND_STREAM) ? 128 : 256;
         long long work = 0;
         for (size_t n = 0; n < seqs.size(); ++n) {
             const int s = seqs[n];
-            long long items;
-            if (k == KIND_SIMT) items = (long long)Q[s] * c.num_q_heads;
-            else items = (long long)c.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk);
+            const long long items = (long long)c.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk);
             per_seq_items[n] = items;
             base_items += items;
             work += items * (P[s] + Q[s]);
@@ -240,6 +238,17 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
                 if (h->debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
             }
         }
+        // ---- scalar kernel: the splits of every item form a cluster, as many for all sequences, unless the longest context would take
+        //      more than 16 splits of 512 tokens (8 tiles, ~10 us) on an otherwise empty device
+        if (k == KIND_SIMT && h->cluster_merge) {
+            int max_len = 0;
+            for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
+            const int ns = std::min((max_len + C - 1) / C, 16);
+            if ((max_len + C - 1) / C <= 16 || max_len <= 16 * 512) {
+                cluster = ns;
+                C = round_up((max_len + ns - 1) / ns, kPage);
+            }
+        }
         // ---- small-q kernel, one wave of one CTA per SM, splits merged by the merge kernel: leave that kernel SMs of its own.
         //      An attention CTA takes a whole SM, so merge CTAs that find no free SM sit on SMs the next call's attention CTAs
         //      need, and those CTAs then start (and fetch their K/V) only after the merge instead of under it.  With a few SMs
@@ -286,7 +295,7 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
                 sp.split_tokens = round_up((L + sp.nsplit - 1) / sp.nsplit, unit);
                 sp.nsplit = (L + sp.split_tokens - 1) / sp.split_tokens;
                 if (cluster) { sp.nsplit = cluster; sp.split_tokens = round_up((L + cluster - 1) / cluster, kPage); }
-                sp.row_chunks = (k == KIND_SIMT) ? 1 : (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
+                sp.row_chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
                 // Row chunks of one KV head side by side share its K/V tiles through L2 (a whole long-context sequence does not fit
                 // there); where the sequence's K/V fits with room to spare, all heads' longest chunks go first instead, so that the
                 // short chunks of a causal block fill the last wave (3584 uncached tokens 114.7 -> 89.5 us, 2 x 1200 50.0 -> 43.0).
@@ -466,8 +475,8 @@ int64_t agx_attn_workspace_bytes(agx_handle* h, int32_t B, const int32_t* P, con
 }
 
 // Attention, optionally with the append of the block's own K/V rows (k_new != NULL): the attention kernels take the block's rows from
-// k_new / v_new and store them into the pages on the side.  Launches of the scalar kernel (and of the warp-MMA kernel with more than
-// one row chunk, which only AGX_FORCE_MMA_SYNC makes) get a separate append launch in front.
+// k_new / v_new and store them into the pages on the side.  Launches of the warp-MMA kernel with more than one row chunk, which only
+// AGX_FORCE_MMA_SYNC makes, get a separate append launch in front.
 static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_new, const void* v_new, const void* k_pool,
                             const void* v_pool, int64_t num_pages, const int32_t* page_table, int32_t pt_stride,
                             const int32_t* P, const int32_t* Q, int32_t B, void* out, float* lse, void* workspace,
@@ -535,7 +544,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         p.k_new = p.v_new = nullptr;
         if (k_new) {
             p.k_new = k_new; p.v_new = v_new;
-            if (ln.kind == KIND_SIMT || (!one_chunk && ln.kind != KIND_TILE && ln.kind != KIND_STREAM)) {
+            if (!one_chunk && ln.kind != KIND_TILE && ln.kind != KIND_STREAM && ln.kind != KIND_SIMT) {
                 e = launch_kv_append_plan(p, h->cfg.dtype, ln.total_rows, stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "append launch");
                 h->last_launches++;

@@ -1,0 +1,280 @@
+// Attention for fp32 pools (any q, head_dim 64 or 128) and for bf16 pools with head_dim 64: fp32 arithmetic on the FMA pipes.
+//
+// Work item = (sequence, KV head, chunk of 8 query rows, KV split); CTA = 8 warps.  Per tile of 64 tokens all threads bring K and V into
+// shared memory (one trip, every load in flight), score 8 x 64 pairs (a thread: one token, two rows), warp r does the softmax of
+// row r, and warp w adds up the tokens [8 w, 8 w + 8) of the tile for all rows, so that V is read from shared memory once; the
+// warps' sums meet at the end.  The KV splits of an item form a thread-block cluster and are merged through distributed
+// shared memory; only contexts that need more than 16 splits leave partials for the merge kernel.  With a fused append the block's
+// rows come from k_new / v_new, and the item of a head's last row chunk stores them into the pages.
+//
+// Bounded by latency at the sizes it is meant for.  256 cached tokens, q = 4, 4/2 heads, fp32: 6.2 us in one launch; append, attention and
+// merge were three launches of 29 us together, of which a kernel whose warps took one token at a time was 25 (whole step with
+// the accept launch 32.5 -> 9.9 us).
+#include <math.h>
+
+#include "agx_internal.cuh"
+#include "agx_sm100.cuh"
+
+namespace agx {
+
+namespace {
+
+constexpr int kR = 8;          // query rows per CTA
+constexpr int kT = 64;         // tokens per tile
+constexpr int kWarps = 8;
+constexpr int kThreads = 32 * kWarps;
+
+template <int D>
+struct SimtSmem {
+    float q[kR][D];
+    float k[kT][D + 4];        // (a row's 16-byte units start four banks after the row's before it: conflict-free)
+    float v[kT][D];
+    float s[kR][kT];
+    float corr[kR];
+    float2 ml[kR];
+    float o[kR][D];            // the split's rows, read by the cluster's other CTAs
+};
+
+// Four elements of a row at element offset `at` as floats.
+template <bool kBf16>
+__device__ __forceinline__ float4 load4(const void* base, long long at) {
+    if (kBf16) {
+        const uint2 r = __ldcg((const uint2*)((const __nv_bfloat16*)base + at));
+        return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xFFFF0000u));
+    }
+    return __ldcg((const float4*)((const float*)base + at));
+}
+template <bool kBf16>
+__device__ __forceinline__ void store4(void* base, long long at, float4 v) {
+    if (kBf16) *(uint2*)((__nv_bfloat16*)base + at) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    else *(float4*)((float*)base + at) = v;
+}
+
+__device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
+    int s = 0;
+#pragma unroll 1
+    for (int i = 1; i < p.num_seqs; ++i)
+        if (p.seq[i].item0 <= item) s = i;
+    return s;
+}
+
+}  // namespace
+
+template <int D, bool kBf16>
+__global__ void __launch_bounds__(kThreads)
+attn_simt_kernel(const __grid_constant__ AttnParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SimtSmem<D>& sm = *(SimtSmem<D>*)smem_raw;
+    constexpr int kUnits = D / 4;                              // groups of four elements per row
+    constexpr int kPer = kT * kUnits / kThreads;               // per thread and operand
+    constexpr int kCols = D / 32;                              // output columns per lane
+    pdl_launch_dependents();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const SeqPlan& sp = p.seq[find_seq(p, blockIdx.x)];
+    int local = blockIdx.x - sp.item0;                         // ((g * row_chunks) + rc) * nsplit + split
+    const int nsplit = sp.nsplit, split = local % nsplit;
+    local /= nsplit;
+    const int rc = local % sp.row_chunks, g = local / sp.row_chunks;
+    const int G = p.hq / p.hkv, P = sp.prefix_len, q = sp.q_len, L = P + q, rows = q * G, row0 = rc * kR;
+    const int vis_end = P + min(q - 1, (row0 + kR - 1) / G) + 1;
+    const int tok_begin = split * sp.split_tokens, tok_end = min(vis_end, tok_begin + sp.split_tokens);
+    const int pool_end = p.k_new ? P : L;
+    const bool writer = p.k_new && rc == sp.row_chunks - 1;
+    const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
+    pdl_wait();
+
+    for (int i = tid; i < kR * kUnits; i += kThreads) {        // Q, scaled so that the scores are in log2 units; rows past q * G are zeros
+        const int r = row0 + i / kUnits, c = (i % kUnits) * 4;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) x = load4<kBf16>(p.q, ((long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G) * D + c);
+        *(float4*)&sm.q[i / kUnits][c] = make_float4(x.x * p.scale_log2, x.y * p.scale_log2, x.z * p.scale_log2, x.w * p.scale_log2);
+    }
+    float acc[kR][kCols];
+#pragma unroll
+    for (int r = 0; r < kR; ++r)
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) acc[r][c] = 0.f;
+    float m_run = -INFINITY, l_run = 0.f;                      // of row `warp`
+    const int st = tid & (kT - 1), sr = (tid / kT) * 2;        // this thread's token and first row in the scoring step
+    const int lim0 = P + min((row0 + sr) / G, q - 1), lim1 = P + min((row0 + sr + 1) / G, q - 1);
+
+    for (int t0 = tok_begin; t0 < tok_end; t0 += kT) {
+        float4 kv[2][kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int u = tid + j * kThreads, tok = t0 + u / kUnits, c = (u % kUnits) * 4;
+            kv[0][j] = kv[1][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (tok >= tok_end) continue;
+            long long page = 0;
+            bool ok = true;
+            if (tok < pool_end || writer) {
+                page = (tok >> 4) < p.pt_stride ? __ldg(pt_row + (tok >> 4)) : -1;
+                ok = page >= 0 && page < p.num_pages;
+                if (!ok) atomicOr(p.status, AGX_DEV_BAD_PAGE);
+            }
+            const long long slot = ((page * p.hkv + g) * kPage + (tok & 15)) * (long long)D + c;
+            if (tok < pool_end) {
+                if (ok) { kv[0][j] = load4<kBf16>(p.k_pool, slot); kv[1][j] = load4<kBf16>(p.v_pool, slot); }
+            } else {
+                const long long at = ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * D + c;
+                kv[0][j] = load4<kBf16>(p.k_new, at); kv[1][j] = load4<kBf16>(p.v_new, at);
+                if (writer && ok) { store4<kBf16>((void*)p.k_pool, slot, kv[0][j]); store4<kBf16>((void*)p.v_pool, slot, kv[1][j]); }
+            }
+        }
+        __syncthreads();                                       // the tile before this one has been used
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int u = tid + j * kThreads;
+            *(float4*)&sm.k[u / kUnits][(u % kUnits) * 4] = kv[0][j];
+            *(float4*)&sm.v[u / kUnits][(u % kUnits) * 4] = kv[1][j];
+        }
+        __syncthreads();
+        {
+            float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+            for (int c = 0; c < D; c += 4) {
+                const float4 k = *(const float4*)&sm.k[st][c], a = *(const float4*)&sm.q[sr][c], b = *(const float4*)&sm.q[sr + 1][c];
+                s0[0] += a.x * k.x; s0[1] += a.y * k.y; s0[2] += a.z * k.z; s0[3] += a.w * k.w;
+                s1[0] += b.x * k.x; s1[1] += b.y * k.y; s1[2] += b.z * k.z; s1[3] += b.w * k.w;
+            }
+            const int tok = t0 + st;
+            sm.s[sr][st] = (tok <= lim0 && tok < tok_end) ? (s0[0] + s0[1]) + (s0[2] + s0[3]) : -INFINITY;
+            sm.s[sr + 1][st] = (tok <= lim1 && tok < tok_end) ? (s1[0] + s1[1]) + (s1[2] + s1[3]) : -INFINITY;
+        }
+        __syncthreads();
+        {   // warp r: softmax of row r
+            const float2 x = *(const float2*)&sm.s[warp][2 * lane];
+            float mx = fmaxf(x.x, x.y);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, d));
+            const float m_new = fmaxf(m_run, mx), m_ref = m_new == -INFINITY ? 0.f : m_new;
+            const float corr = exp2f(m_run - m_ref);
+            const float2 w = make_float2(exp2f(x.x - m_ref), exp2f(x.y - m_ref));
+            float sum = w.x + w.y;
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+            l_run = l_run * corr + sum;
+            m_run = m_new;
+            *(float2*)&sm.s[warp][2 * lane] = w;
+            if (lane == 0) sm.corr[warp] = corr;
+        }
+        __syncthreads();
+        float4 w0[kR], w1[kR];
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            const float corr = sm.corr[r];
+            w0[r] = *(const float4*)&sm.s[r][warp * 8];
+            w1[r] = *(const float4*)&sm.s[r][warp * 8 + 4];
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) acc[r][c] *= corr;
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            float v[kCols];
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) v[c] = sm.v[warp * 8 + t][c * 32 + lane];
+#pragma unroll
+            for (int r = 0; r < kR; ++r) {
+                const float4& w = t < 4 ? w0[r] : w1[r];
+                const float x = (t & 3) == 0 ? w.x : (t & 3) == 1 ? w.y : (t & 3) == 2 ? w.z : w.w;
+#pragma unroll
+                for (int c = 0; c < kCols; ++c) acc[r][c] += x * v[c];
+            }
+        }
+    }
+    // ---- the warps' sums, in warp order: [warp][row][D] in the K / V area
+    __syncthreads();
+    float* part = &sm.k[0][0];
+    static_assert(sizeof(sm.k) + sizeof(sm.v) >= sizeof(float) * kWarps * kR * D, "the partial sums of the warps fit the K / V tiles");
+#pragma unroll
+    for (int r = 0; r < kR; ++r)
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) part[(warp * kR + r) * D + c * 32 + lane] = acc[r][c];
+    if (lane == 0) sm.ml[warp] = make_float2(m_run, l_run);
+    __syncthreads();
+    const bool in_cluster = p.cluster_size > 1;
+    for (int i = tid; i < kR * kUnits; i += kThreads) {
+        const int rl = i / kUnits, c = (i % kUnits) * 4, r = row0 + rl;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const float4 x = *(const float4*)&part[(w * kR + rl) * D + c];
+            o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
+        }
+        const float2 ml = sm.ml[rl];
+        if (in_cluster) {
+            *(float4*)&sm.o[rl][c] = o;
+        } else if (r < rows) {
+            const long long at = (long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G;
+            if (nsplit == 1) {
+                store4<kBf16>(p.out, at * D + c, make_float4(o.x / ml.y, o.y / ml.y, o.z / ml.y, o.w / ml.y));
+                if (p.lse && c == 0) p.lse[at] = (ml.x + log2f(ml.y)) * 0.6931471805599453f;
+            } else {
+                const long long e = (long long)sp.part_base + ((long long)(r / G) * p.hq + g * G + r % G) * nsplit + split;
+                *(float4*)(p.part_o + e * D + c) = o;
+                if (c == 0) p.part_ml[e] = ml;
+            }
+        }
+    }
+    if (in_cluster) {
+        cluster_sync();
+        // groups of four columns are dealt round-robin to the cluster's CTAs
+        for (int i = split + nsplit * tid; i < kR * kUnits; i += nsplit * kThreads) {
+            const int rl = i / kUnits, c = (i % kUnits) * 4, r = row0 + rl;
+            if (r >= rows) continue;
+            const uint32_t ml_addr = smem_u32(&sm.ml[rl]), o_addr = smem_u32(&sm.o[rl][c]);
+            float2 ml[16];
+            float4 x[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (k < nsplit) { ml[k] = ld_cluster_f2(cluster_map(ml_addr, k)); x[k] = ld_cluster_f4(cluster_map(o_addr, k)); }
+            float m = -INFINITY, l = 0.f;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) if (k < nsplit) m = fmaxf(m, ml[k].x);
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (k < nsplit && ml[k].x != -INFINITY) {
+                    const float w = exp2f(ml[k].x - m);
+                    l += ml[k].y * w;
+                    o.x += x[k].x * w; o.y += x[k].y * w; o.z += x[k].z * w; o.w += x[k].w * w;
+                }
+            const long long at = (long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G;
+            store4<kBf16>(p.out, at * D + c, make_float4(o.x / l, o.y / l, o.z / l, o.w / l));
+            if (p.lse && c == 0) p.lse[at] = (m + log2f(l)) * 0.6931471805599453f;
+        }
+        cluster_sync();   // no CTA leaves while its rows may still be read
+    }
+}
+
+namespace {
+template <int D, bool kBf16>
+cudaError_t configure() {
+    static bool done[64] = {false};   // the attributes are per device
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    if (done[device]) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<D, kBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SimtSmem<D>));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_simt_kernel<D, kBf16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+    done[device] = e == cudaSuccess;
+    return e;
+}
+template <int D, bool kBf16>
+cudaError_t launch(const AttnParams& p, cudaStream_t stream) {
+    cudaError_t e = configure<D, kBf16>();
+    if (e != cudaSuccess) return e;
+    if (p.cluster_size > 1)
+        return launch_chained_cluster(attn_simt_kernel<D, kBf16>, dim3(p.num_items), dim3(kThreads), sizeof(SimtSmem<D>), (unsigned)p.cluster_size, stream, p);
+    return launch_chained(attn_simt_kernel<D, kBf16>, dim3(p.num_items), dim3(kThreads), sizeof(SimtSmem<D>), stream, p);
+}
+}  // namespace
+
+cudaError_t launch_attn_simt(const AttnParams& p, int dtype, cudaStream_t stream) {
+    if (p.num_items == 0) return cudaSuccess;
+    if (dtype == AGX_F32 && p.head_dim == 64) return launch<64, false>(p, stream);
+    if (dtype == AGX_F32 && p.head_dim == 128) return launch<128, false>(p, stream);
+    if (dtype == AGX_BF16 && p.head_dim == 64) return launch<64, true>(p, stream);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace agx

@@ -606,90 +606,6 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 }
 
 // --------------------------------------------------------------------------------------------
-// Scalar kernel for fp32 pools (any q; d = 64 or 128) and for bf16 pools with d = 64 (a correctness path: fp32 arithmetic
-// on the FMA pipes).  CTA = 4 warps on one (sequence, row, head, split); a warp takes every 4th token, lanes split the head
-// dim, dot products reduce by shuffle.
-template <bool kBf16>
-__device__ __forceinline__ float load_elem(const void* base, long long idx) {
-    if (kBf16) return __bfloat162float(((const __nv_bfloat16*)base)[idx]);
-    return ((const float*)base)[idx];
-}
-template <int D, bool kBf16>
-__global__ void __launch_bounds__(128)
-attn_simt_kernel(const __grid_constant__ AttnParams p) {
-    constexpr int kPer = D / 32;
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int si = find_seq(p, blockIdx.x);
-    const SeqPlan sp = p.seq[si];
-    int local = blockIdx.x - sp.item0;  // ((i * Hq) + h) * nsplit + split
-    const int split = local % sp.nsplit;
-    local /= sp.nsplit;
-    const int h = local % p.hq;
-    const int i = local / p.hq;
-    const int G = p.hq / p.hkv;
-    const int g = h / G;
-    const int tok_begin = split * sp.split_tokens;
-    const int tok_end = min(sp.prefix_len + i + 1, tok_begin + sp.split_tokens);  // causal limit for row i
-    const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
-
-    float qv[kPer], acc[kPer];
-    const long long q0 = ((long long)(sp.q_row0 + i) * p.hq + h) * D;
-#pragma unroll
-    for (int c = 0; c < kPer; ++c) { qv[c] = load_elem<kBf16>(p.q, q0 + lane + 32 * c) * p.scale_log2; acc[c] = 0.f; }
-    float m = -INFINITY, l = 0.f;
-    for (int tok = tok_begin + warp; tok < tok_end; tok += 4) {
-        long long page = __ldg(pt_row + (tok >> 4));
-        if (page < 0 || page >= p.num_pages) {
-            if (lane == 0) atomicOr(p.status, AGX_DEV_BAD_PAGE);
-            continue;
-        }
-        const long long base = ((page * p.hkv + g) * kPage + (tok & 15)) * (long long)D;
-        float dot = 0.f;
-#pragma unroll
-        for (int c = 0; c < kPer; ++c) dot += qv[c] * load_elem<kBf16>(p.k_pool, base + lane + 32 * c);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, off);
-        const float m_new = fmaxf(m, dot);
-        const float corr = exp2f(m - m_new);
-        const float w = exp2f(dot - m_new);
-        l = l * corr + w;
-#pragma unroll
-        for (int c = 0; c < kPer; ++c) acc[c] = acc[c] * corr + w * load_elem<kBf16>(p.v_pool, base + lane + 32 * c);
-        m = m_new;
-    }
-    __shared__ float sm_o[4][D];
-    __shared__ float2 sm_ml[4];
-#pragma unroll
-    for (int c = 0; c < kPer; ++c) sm_o[warp][lane + 32 * c] = acc[c];
-    if (lane == 0) sm_ml[warp] = make_float2(m, l);
-    __syncthreads();
-    for (int c = threadIdx.x; c < D; c += 128) {
-        float m_all = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) m_all = fmaxf(m_all, sm_ml[k].x);
-        float l_all = 0.f, a = 0.f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float w = (sm_ml[k].x == -INFINITY) ? 0.f : exp2f(sm_ml[k].x - m_all);
-            l_all += sm_ml[k].y * w;
-            a += sm_o[k][c] * w;
-        }
-        if (sp.nsplit == 1) {
-            const long long o = ((long long)(sp.q_row0 + i) * p.hq + h) * D + c;
-            if (kBf16) ((__nv_bfloat16*)p.out)[o] = __float2bfloat16_rn(a / l_all);
-            else ((float*)p.out)[o] = a / l_all;
-            if (p.lse && c == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
-        } else {
-            const long long e = (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + split;
-            p.part_o[e * D + c] = a;
-            if (c == 0) p.part_ml[e] = make_float2(m_all, l_all);
-        }
-    }
-}
-
-// --------------------------------------------------------------------------------------------
 // Combine: out[row, h] = sum_k O_k 2^(m_k - m) / sum_k l_k 2^(m_k - m), splits in index order.
 // One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
 // kMaxNs: no sequence of the launch has more splits than this (4, 16, or any number).  Four O rows per warp instead of 32
@@ -1054,14 +970,6 @@ cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CU
         case 4 * 16 + 4: return launch_small<4, 4, 5>(p, map_k, map_v, stream);
         default: return cudaErrorInvalidValue;
     }
-}
-
-cudaError_t launch_attn_simt(const AttnParams& p, int dtype, cudaStream_t stream) {
-    if (p.num_items == 0) return cudaSuccess;
-    if (dtype == AGX_F32 && p.head_dim == 64) return launch_chained(attn_simt_kernel<64, false>, dim3(p.num_items), dim3(128), 0, stream, p);
-    if (dtype == AGX_F32 && p.head_dim == 128) return launch_chained(attn_simt_kernel<128, false>, dim3(p.num_items), dim3(128), 0, stream, p);
-    if (dtype == AGX_BF16 && p.head_dim == 64) return launch_chained(attn_simt_kernel<64, true>, dim3(p.num_items), dim3(128), 0, stream, p);
-    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, cudaStream_t stream) {
