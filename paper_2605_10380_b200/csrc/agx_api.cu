@@ -96,6 +96,7 @@ struct Plan {
     std::vector<Launch> launches;
     long long part_entries = 0;  // (row, head, split) partial slots
     bool any_split = false;
+    bool tensor_core = false;    // a launch of the tensor-core kernel is among them
     long long total_rows = 0;    // block rows of the whole batch
 };
 
@@ -278,6 +279,7 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         for (size_t a = 0; a < seqs.size(); a += kMaxSeqs) {
             Launch ln;
             ln.kind = (Kind)k;
+            plan.tensor_core |= k == KIND_TILE || k == KIND_STREAM;
             ln.total_rows = 0;
             ln.num_items = 0;
             ln.cluster = cluster;
@@ -524,8 +526,8 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     if (h->cfg.dtype == AGX_BF16 && h->cfg.head_dim == 128) {
         if ((long long)num_pages * p.hkv * kPage > 0x7FFFFFFFll) return fail(h, AGX_E_RANGE, "pool too large for one tensor map");
         bool ok = make_pool_map(&map_k, k_pool, num_pages, p.hkv) && make_pool_map(&map_v, v_pool, num_pages, p.hkv);
-        if (ok && k_new) ok = make_rows_maps(&maps_new, k_new, v_new, plan.total_rows, p.hkv);
-        else memset(&maps_new, 0, sizeof maps_new);
+        if (ok && k_new && plan.tensor_core) ok = make_rows_maps(&maps_new, k_new, v_new, plan.total_rows, p.hkv);
+        else if (plan.tensor_core) memset(&maps_new, 0, sizeof maps_new);
         if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
     for (const Launch& ln : plan.launches) {
@@ -1014,7 +1016,7 @@ agx_status agx_ngram_build(agx_handle* h, const int32_t* stream_tokens, int32_t 
                     ngram_workspace_bytes(num_tokens));
     cudaError_t e = launch_ngram_build(stream_tokens, num_tokens, n, lut, workspace, h->d_status, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "n-gram build");
-    h->last_launches = num_tokens >= n ? 3 : 1;
+    h->last_launches = ngram_build_launches(num_tokens, n);
     return AGX_OK;
 }
 

@@ -155,7 +155,8 @@ cudaError_t launch_scatter_pages(int dtype, void* k_pool, void* v_pool, long lon
                                  const void* v_stage, const int* dst, int count, int hkv, int head_dim, int* status,
                                  cudaStream_t stream);
 
-// n-gram draft table (Sec. 4.3): sizes, build (three memsets + three small kernels) and chained lookups.
+// n-gram draft table (Sec. 4.3): sizes, build (one launch, or for long streams three memsets and three kernels) and chained lookups.
+int ngram_build_launches(int num_tokens, int n);
 long long ngram_lut_bytes(int max_stream_tokens);
 long long ngram_workspace_bytes(int stream_tokens);
 cudaError_t launch_ngram_build(const int* stream_tokens, int num_tokens, int n, void* lut, void* workspace, int* status,

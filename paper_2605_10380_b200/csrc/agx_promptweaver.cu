@@ -16,13 +16,15 @@
 
 namespace agx {
 
-// One CTA per (page pair, K or V): 16-byte loads and stores over the whole page (all KV heads).
+// Four CTAs per (page pair, K or V): 16-byte loads and stores over the whole page (all KV heads).  Bounded by the latency of two dependent
+// trips to memory (page ids, then the page: eight units per thread of a 32 KB page would go in two rounds with one CTA).
+constexpr int kCopyParts = 4;
 __global__ void __launch_bounds__(256)
 copy_pages_kernel(uint4* __restrict__ k_pool, uint4* __restrict__ v_pool, long long num_pages, const int* __restrict__ src,
                   const int* __restrict__ dst, long long vec_per_page, int* status) {
     pdl_launch_dependents();
     pdl_wait();
-    const int pair = blockIdx.x >> 1;
+    const int pair = blockIdx.x / (2 * kCopyParts), part = (blockIdx.x >> 1) % kCopyParts;
     uint4* pool = (blockIdx.x & 1) ? v_pool : k_pool;
     const long long s = src[pair], d = dst[pair];
     if (s < 0 || s >= num_pages || d < 0 || d >= num_pages) {
@@ -30,7 +32,16 @@ copy_pages_kernel(uint4* __restrict__ k_pool, uint4* __restrict__ v_pool, long l
         return;
     }
     if (s == d) return;
-    for (long long i = threadIdx.x; i < vec_per_page; i += blockDim.x) pool[d * vec_per_page + i] = pool[s * vec_per_page + i];
+    const uint4* from = pool + s * vec_per_page;
+    uint4* to = pool + d * vec_per_page;
+    const long long step = (long long)kCopyParts * 256;
+    long long i = (long long)part * 256 + threadIdx.x;
+    for (; i + step < vec_per_page; i += 2 * step) {
+        const uint4 a = __ldcg(from + i), b = __ldcg(from + i + step);
+        to[i] = a;
+        to[i + step] = b;
+    }
+    if (i < vec_per_page) to[i] = __ldcg(from + i);
 }
 
 // Scatter pages from a packed staging area (page i of the import) to pool pages dst[i]: one CTA per (page, K or V).
@@ -64,7 +75,7 @@ cudaError_t launch_copy_pages(int dtype, void* k_pool, void* v_pool, long long n
                               int count, int hkv, int head_dim, int* status, cudaStream_t stream) {
     if (count == 0) return cudaSuccess;
     const long long vec_per_page = (long long)hkv * kPage * head_dim * (dtype == AGX_BF16 ? 2 : 4) / 16;
-    return launch_chained(copy_pages_kernel, dim3(2 * count), dim3(256), 0, stream, (uint4*)k_pool, (uint4*)v_pool, num_pages,
+    return launch_chained(copy_pages_kernel, dim3(2 * kCopyParts * count), dim3(256), 0, stream, (uint4*)k_pool, (uint4*)v_pool, num_pages,
                           src, dst, vec_per_page, status);
 }
 

@@ -47,3 +47,30 @@ def test_arguments_that_are_none_or_of_the_wrong_type():
     h.close()
     with pytest.raises(agx.AgxError):
         h.attn_prefixed(q, pool, pool, table, [5], [1], q)
+
+
+@pytest.mark.parametrize("length", [32769, 32770, 32771, 16387, 2, 3])
+def test_ngram_build_on_both_sides_of_the_one_launch_limit(length):
+    """32768 windows is the largest stream built by one cluster; the table must not depend on which form built it."""
+    import torch
+
+    from oracle.toy_lm import build_ngram_table, ngram_drafts
+    from paper_2605_10380_b200 import agx
+    h = agx.Handle(32, 8, 128, "bf16")
+    rng = np.random.default_rng(length)
+    stream = rng.integers(0, 40, size=length).astype(np.int32)
+    st = torch.from_numpy(stream).cuda()
+    lut = torch.empty(agx.ngram_lut_bytes(length), dtype=torch.uint8, device="cuda")
+    ws = torch.empty(agx.ngram_workspace_bytes(length), dtype=torch.uint8, device="cuda")
+    h.ngram_build(st, 3, lut, ws)
+    assert h.last_launch_count() == (1 if length - 2 <= 32768 else 3)
+    table = build_ngram_table(stream.tolist(), 3)
+    keys = list(table)[:500] + [(39, 41)]
+    ctx = torch.tensor(keys, dtype=torch.int32, device="cuda")
+    drafts = torch.zeros(len(keys), 4, dtype=torch.int32, device="cuda")
+    has = torch.zeros(len(keys), dtype=torch.int32, device="cuda")
+    h.ngram_draft(lut, ctx, torch.zeros_like(drafts), 4, drafts, has)
+    torch.cuda.synchronize()
+    for i, key in enumerate(keys):
+        ref = ngram_drafts(table, list(key), 4, 3, fill=[0] * 4) if key in table else None
+        assert has[i].item() == (ref is not None) and (ref is None or drafts[i].tolist() == ref)
