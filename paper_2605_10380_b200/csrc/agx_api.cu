@@ -100,6 +100,110 @@ struct Plan {
     long long total_rows = 0;    // block rows of the whole batch
 };
 
+// KV tiles per split of a launch of the tensor-core kernel: the candidate with the smallest estimated time.
+//
+// Estimate (us, fitted to sweeps over split lengths of the shapes below; worst errors 2-3 us at 20-130): CTAs go to the SMs longest first.
+//   256-row schedule  1.9 per tile of the fullest SM, 3 tiles for the start and end of a CTA; merge 2.2 + 0.38 per MB of partials
+//                     up to 16 MB (they stay in L2), 0.3 beyond
+//   one-Q-tile        4.5 for the start and end of the first CTA, 3 tiles for those of others on its SM; a tile of 64 KB takes
+//                     0.1 + max(0.95, 0.0107 A) while A SMs are at work (HBM is busy at 6.1 TB/s with about 90 of them); merge 3 + 0.38 per MB,
+//                     1 + 0.2 per MB where all CTAs are resident at once and leave SMs to it
+// It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
+// 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, 16 decode blocks over 2k-14k tokens 76 -> 74.
+int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
+                       int rows_per_chunk, int min_tiles, long long base_items) {
+    const int sms = h->sm_count, hkv = h->cfg.num_kv_heads;
+    int max_tiles = 1;
+    for (int s : seqs) max_tiles = std::max(max_tiles, (P[s] + Q[s] + 127) / 128);
+    constexpr int kOverhead = 3;
+    struct Cand { int tiles; double bound, merge; };
+    std::vector<Cand> cands;
+    // items of a candidate, by tile count: (count, tiles)
+    std::vector<std::pair<int, long long>> items;
+    auto collect = [&](int split_tiles, long long& sum, long long& count, int& longest, double& part_mb) {
+        items.clear();
+        sum = count = 0; longest = 0; part_mb = 0;
+        for (int s : seqs) {
+            const int L = P[s] + Q[s], lt = (L + 127) / 128, ns = (lt + split_tiles - 1) / split_tiles, per = (lt + ns - 1) / ns;
+            const int chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
+            if (ns > 1) part_mb += (double)Q[s] * h->cfg.num_q_heads * ns * (streams ? 520 : 264) * 1e-6;
+            auto add = [&](int vis, long long n) {   // n (chunk, head) pairs that see `vis` tiles
+                const int full = vis / per, rest = vis - full * per;
+                if (full) items.push_back({per, n * full});
+                if (rest) items.push_back({rest, n});
+                sum += n * (vis + kOverhead * (full + (rest != 0)));
+                count += n * (full + (rest != 0));
+                longest = std::max(longest, full ? per : rest);
+            };
+            if (chunks <= 32) {
+                for (int rc = 0; rc < chunks; ++rc) add((P[s] + std::min(Q[s] - 1, ((rc + 1) * rows_per_chunk - 1) / G) + 128) / 128, hkv);
+            } else {   // in 32 groups of chunks with the tiles of the group's last one
+                for (int k = 0; k < 32; ++k) {
+                    const int rc0 = (int)((long long)chunks * k / 32), rc1 = (int)((long long)chunks * (k + 1) / 32);
+                    add((P[s] + std::min(Q[s] - 1, (rc1 * rows_per_chunk - 1) / G) + 128) / 128, (long long)hkv * (rc1 - rc0));
+                }
+            }
+        }
+    };
+    const int n_max = (int)std::min<long long>((max_tiles + min_tiles - 1) / min_tiles, std::max<long long>(32, 2 * sms / std::max<long long>(base_items, 1)));
+    for (int n = 1, last = 0; n <= n_max; ++n) {
+        const int t = std::max(min_tiles, (max_tiles + n - 1) / n);
+        if (t == last) continue;
+        last = t;
+        long long sum, count;
+        int longest;
+        double mb;
+        collect(t, sum, count, longest, mb);
+        const double load = std::max<double>((double)sum / sms, longest + kOverhead);
+        Cand cd;
+        cd.tiles = t;
+        cd.merge = mb == 0 ? 0 : streams && count <= sms * 15 / 16 ? 1.0 + 0.2 * mb
+                                         : (streams ? 3.0 : 2.2) + 0.38 * std::min(mb, 16.0) + 0.3 * std::max(mb - 16.0, 0.0);
+        cd.bound = (streams ? 4.5 + std::max((load - kOverhead) * 1.05, (sum - (double)kOverhead * std::min<long long>(count, sms)) * 0.0107) : load * 1.9) + cd.merge;
+        cands.push_back(cd);
+    }
+    std::stable_sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
+    double best = -1;
+    int best_tiles = max_tiles;
+    std::vector<int> load;
+    for (const Cand& cd : cands) {
+        if (best >= 0 && cd.bound >= best) break;   // (bounds ascend)
+        long long sum, count;
+        int longest;
+        double mb, t;
+        collect(cd.tiles, sum, count, longest, mb);
+        // load[x]: SMs with x tiles (and starts) so far; an item goes to an SM with the least
+        std::sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+        load.assign((size_t)(sum / sms) + longest + kOverhead + 2, 0);
+        load[0] = sms;
+        size_t lo = 0, hi = 0;
+        for (const auto& it : items)
+            for (long long left = it.second; left > 0;) {
+                while (load[lo] == 0) ++lo;
+                const int k = (int)std::min<long long>(load[lo], left);
+                load[lo] -= k;
+                load[lo + it.first + kOverhead] += k;
+                hi = std::max(hi, lo + it.first + kOverhead);
+                left -= k;
+            }
+        if (streams) {
+            t = 4.5;
+            size_t prev = kOverhead;
+            int busy = sms;
+            for (size_t x = 0; x <= hi; ++x) {
+                if (load[x] == 0) continue;
+                if (x > prev) { t += (x - prev) * (0.1 + std::max(0.95, 0.0107 * busy)); prev = x; }
+                busy -= load[x];
+            }
+        } else {
+            t = 1.9 * hi;
+        }
+        t += cd.merge;
+        if (best < 0 || t < best) { best = t; best_tiles = cd.tiles; }
+    }
+    return best_tiles;
+}
+
 // Decide kernel kind, KV splits and partial slots for every sequence (host lengths only).
 agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, int pt_stride, Plan& plan) {
     const agx_config& c = h->cfg;
@@ -190,26 +294,9 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             return items;
         };
         if (k == KIND_TILE || k == KIND_STREAM) {
-            // several waves are fine here: pick the split length with the smallest estimated makespan, in units of one KV
-            // tile's time (~1.6 us): waves * (tiles per item + fixed per-CTA cost of ~3 tiles), plus what the split costs
-            // afterwards: the merge launch (~2 units) and the partial rows written and read back (~0.3 units per MB beyond the
-            // first 16 MB, which stay in L2; measured on a ragged batch of eight suffix prefills: 95 MB of partials cost 60 us
-            // more than 22 MB, while 9 MB in one-tile splits of a 128-token suffix over 1000 tokens cost nothing)
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            const long long row_bytes = k == KIND_TILE ? 256 : 520;   // fp16 row | fp32 row + (m, l)
-            long long best_cost = -1;
-            for (int c_tokens = min_split; c_tokens < max_len + unit; c_tokens += unit) {
-                const long long waves = (count_items(c_tokens) + h->sm_count - 1) / h->sm_count;
-                long long part_bytes = 0;
-                for (int s : seqs) {
-                    const long long ns = (P[s] + Q[s] + c_tokens - 1) / c_tokens;
-                    if (ns > 1) part_bytes += (long long)Q[s] * c.num_q_heads * ns * row_bytes;
-                }
-                const long long cost = 16 * waves * (std::min(c_tokens, round_up(max_len, unit)) / unit + 3) +
-                                       (part_bytes ? 32 + 5 * std::max<long long>(0, (part_bytes >> 20) - 16) : 0);
-                if (best_cost < 0 || cost < best_cost) { best_cost = cost; C = c_tokens; }
-            }
+            C = unit * choose_split_tiles(h, k == KIND_STREAM, seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
             if (const char* force = getenv("AGX_TILE_SPLIT_TOKENS")) { if (atoi(force) >= unit) C = atoi(force) / unit * unit; }
             if (h->debug_plan)
                 fprintf(stderr, "agx plan: tile kernel, %lld row chunks, longest sequence %d tokens -> KV splits of %d tokens, %lld CTAs\n",
