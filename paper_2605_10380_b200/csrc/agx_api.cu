@@ -100,22 +100,42 @@ struct Plan {
     long long total_rows = 0;    // block rows of the whole batch
 };
 
-// KV tiles per split of a launch of the tensor-core kernel: the candidate with the smallest estimated time.
-//
-// Estimate (us, fitted to sweeps over split lengths of the shapes below; worst errors 2-3 us at 20-130): CTAs go to the SMs longest first.
-//   256-row schedule  1.9 per tile of the fullest SM, 3 tiles for the start and end of a CTA; merge 2.2 + 0.38 per MB of partials
-//                     up to 16 MB (they stay in L2), 0.3 beyond
-//   one-Q-tile        4.5 for the start and end of the first CTA, 3 tiles for those of others on its SM; a tile of 64 KB takes
-//                     0.1 + max(0.95, 0.0107 A) while A SMs are at work (HBM is busy at 6.1 TB/s with about 90 of them); merge 3 + 0.38 per MB,
-//                     1 + 0.2 per MB where all CTAs are resident at once and leave SMs to it
+// What a launch of one of the attention kernels costs (us), fitted to sweeps over split lengths and batches (GQA 32/8; worst errors 2-3 us at
+// 20-130): CTAs go to the SMs (or to their halves) longest first; a step of `unit` tokens takes per_add + max(per_min, per_busy * A) while
+// A CTAs are at work (per_busy: HBM, or the mma.sync rate, shared by all of them), the start and end of the first CTA `base`, those of
+// others behind it on an SM `overhead` steps.
+struct SplitModel {
+    int unit, slots, overhead;
+    double base, per_add, per_min, per_busy;
+    double merge, merge_mb, merge_mb_beyond_16;   // merge launch, per MB of partials up to 16 (they stay in L2) and beyond
+    int part_row_bytes;
+    bool lean;              // one-wave launches with few (row, head) pairs leave SMs to their merge kernel: 1 + 0.2 per MB
+};
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
-// 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, 16 decode blocks over 2k-14k tokens 76 -> 74.
-int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
-                       int rows_per_chunk, int min_tiles, long long base_items) {
-    const int sms = h->sm_count, hkv = h->cfg.num_kv_heads;
+// 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
+SplitModel tile_model(const agx_handle* h) { return {128, h->sm_count, 3, 5.7, 0, 1.9, 0, 2.2, 0.38, 0.3, 264, false}; }
+// (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them)
+SplitModel stream_model(const agx_handle* h, bool wide) {
+    return {128, h->sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, true};
+}
+// warp-MMA kernel with 4-page stages, two CTAs per SM: HBM-bound with one 16-row tile, bounded by its own chain with two (mma.sync)
+SplitModel small4_model(const agx_handle* h, int mt) {
+    return {64, 2 * h->sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, false};
+}
+
+// Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time.
+int choose_split(const agx_handle* h, const SplitModel& md, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
+                 int rows_per_chunk, int min_tiles, long long base_items, double* estimate = nullptr) {
+    const int sms = md.slots, hkv = h->cfg.num_kv_heads, kOverhead = md.overhead;
     int max_tiles = 1;
-    for (int s : seqs) max_tiles = std::max(max_tiles, (P[s] + Q[s] + 127) / 128);
-    constexpr int kOverhead = 3;
+    long long pairs = 0;      // (row, query head)
+    bool equal = true;
+    for (int s : seqs) {
+        const int lt = (P[s] + Q[s] + md.unit - 1) / md.unit;
+        equal &= s == seqs[0] || lt == max_tiles;
+        pairs += (long long)Q[s] * h->cfg.num_q_heads;
+        max_tiles = std::max(max_tiles, lt);
+    }
     struct Cand { int tiles; double bound, merge; };
     std::vector<Cand> cands;
     // items of a candidate, by tile count: (count, tiles)
@@ -124,9 +144,9 @@ int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>
         items.clear();
         sum = count = 0; longest = 0; part_mb = 0;
         for (int s : seqs) {
-            const int L = P[s] + Q[s], lt = (L + 127) / 128, ns = (lt + split_tiles - 1) / split_tiles, per = (lt + ns - 1) / ns;
+            const int L = P[s] + Q[s], lt = (L + md.unit - 1) / md.unit, ns = (lt + split_tiles - 1) / split_tiles, per = (lt + ns - 1) / ns;
             const int chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
-            if (ns > 1) part_mb += (double)Q[s] * h->cfg.num_q_heads * ns * (streams ? 520 : 264) * 1e-6;
+            if (ns > 1) part_mb += (double)Q[s] * h->cfg.num_q_heads * ns * md.part_row_bytes * 1e-6;
             auto add = [&](int vis, long long n) {   // n (chunk, head) pairs that see `vis` tiles
                 const int full = vis / per, rest = vis - full * per;
                 if (full) items.push_back({per, n * full});
@@ -136,11 +156,11 @@ int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>
                 longest = std::max(longest, full ? per : rest);
             };
             if (chunks <= 32) {
-                for (int rc = 0; rc < chunks; ++rc) add((P[s] + std::min(Q[s] - 1, ((rc + 1) * rows_per_chunk - 1) / G) + 128) / 128, hkv);
+                for (int rc = 0; rc < chunks; ++rc) add((P[s] + std::min(Q[s] - 1, ((rc + 1) * rows_per_chunk - 1) / G) + md.unit) / md.unit, hkv);
             } else {   // in 32 groups of chunks with the tiles of the group's last one
                 for (int k = 0; k < 32; ++k) {
                     const int rc0 = (int)((long long)chunks * k / 32), rc1 = (int)((long long)chunks * (k + 1) / 32);
-                    add((P[s] + std::min(Q[s] - 1, (rc1 * rows_per_chunk - 1) / G) + 128) / 128, (long long)hkv * (rc1 - rc0));
+                    add((P[s] + std::min(Q[s] - 1, (rc1 * rows_per_chunk - 1) / G) + md.unit) / md.unit, (long long)hkv * (rc1 - rc0));
                 }
             }
         }
@@ -157,9 +177,11 @@ int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>
         const double load = std::max<double>((double)sum / sms, longest + kOverhead);
         Cand cd;
         cd.tiles = t;
-        cd.merge = mb == 0 ? 0 : streams && count <= sms * 15 / 16 ? 1.0 + 0.2 * mb
-                                         : (streams ? 3.0 : 2.2) + 0.38 * std::min(mb, 16.0) + 0.3 * std::max(mb - 16.0, 0.0);
-        cd.bound = (streams ? 4.5 + std::max((load - kOverhead) * 1.05, (sum - (double)kOverhead * std::min<long long>(count, sms)) * 0.0107) : load * 1.9) + cd.merge;
+        cd.merge = mb == 0 ? 0 : md.lean && count <= sms * 15 / 16 && pairs <= 3 * sms ? 1.0 + 0.2 * mb
+                   : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
+                   : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
+        cd.bound = md.base + cd.merge + std::max((load - kOverhead) * (md.per_add + md.per_min),
+                                                 (sum - (double)kOverhead * std::min<long long>(count, sms)) * md.per_busy);
         cands.push_back(cd);
     }
     std::stable_sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
@@ -186,21 +208,18 @@ int choose_split_tiles(const agx_handle* h, bool streams, const std::vector<int>
                 hi = std::max(hi, lo + it.first + kOverhead);
                 left -= k;
             }
-        if (streams) {
-            t = 4.5;
-            size_t prev = kOverhead;
-            int busy = sms;
-            for (size_t x = 0; x <= hi; ++x) {
-                if (load[x] == 0) continue;
-                if (x > prev) { t += (x - prev) * (0.1 + std::max(0.95, 0.0107 * busy)); prev = x; }
-                busy -= load[x];
-            }
-        } else {
-            t = 1.9 * hi;
+        t = md.base;
+        size_t prev = kOverhead;
+        int busy = sms;
+        for (size_t x = 0; x <= hi; ++x) {
+            if (load[x] == 0) continue;
+            if (x > prev) { t += (x - prev) * (md.per_add + std::max(md.per_min, md.per_busy * busy)); prev = x; }
+            busy -= load[x];
         }
         t += cd.merge;
         if (best < 0 || t < best) { best = t; best_tiles = cd.tiles; }
     }
+    if (estimate) *estimate = best;
     return best_tiles;
 }
 
@@ -218,19 +237,50 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         row0[s + 1] = row0[s] + Q[s];
     }
     plan.total_rows = row0[B];
-    // Blocks of at most 32 rows: measured on B200 (GQA 32/8, equal sequences), what decides is the batch's total
-    // context, not each sequence's: from ~24k tokens in all (two sequences or more) the tensor-core stream schedule
-    // wins whatever the single lengths; below that the warp-MMA kernel, with 4-page stages and two CTAs per SM from
-    // ~8k tokens in all, with 8-page stages (one 16-warp CTA per SM) for less.  A single sequence keeps its own
-    // cross-over (stream_min_tokens).
-    long long small_tokens = 0;
-    int small_seqs = 0;
+    // Blocks of at most 32 rows go to the warp-MMA kernel or to the one-Q-tile tensor-core schedule, all of a batch together: to the one whose
+    // estimate is lower (SplitModel; for the warp-MMA kernel with 8-page stages, one CTA per SM, k tokens at 8 KV heads take 4.1 + 0.69 k up
+    // to 16 rows, max(8.8, 5.8 + 1.06 k) above).  What it decides against the fixed thresholds it replaces (24576 tokens in all; 7168 / 10240
+    // for one sequence): 32 decode blocks over 1000 tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over
+    // 20000 20.5 -> 17.5, 32 verify blocks over 1500 53 -> 43; 8 verify blocks over 8000 stay at 50 (55 the other way).
+    double small_k = 0;
+    int small_rows = 0;
+    std::vector<int> small_seqs, wide_seqs;   // up to 32 rows | others that take the schedule in any case
     const bool scalar_path = c.dtype == AGX_F32 || c.head_dim != 128;   // fp32 pools, and bf16 with head_dim 64
     if (!scalar_path)
-        for (int s = 0; s < B; ++s)
-            if (Q[s] * G <= 32) { small_tokens += P[s] + Q[s]; ++small_seqs; }
-    small_tokens = small_tokens * c.num_kv_heads / 8;   // the thresholds were measured with 8 KV heads: scale to the same bytes
-    const bool batch_streams = small_seqs >= 2 && small_tokens >= h->batch_stream_tokens;
+        for (int s = 0; s < B; ++s) {
+            const int rows = Q[s] * G;
+            if (rows <= 32) { small_k += (P[s] + Q[s]) * 1e-3 * c.num_kv_heads / 8; small_rows = std::max(small_rows, rows); small_seqs.push_back(s); }
+            else if (rows <= h->stream_max_rows) wide_seqs.push_back(s);
+        }
+    bool batch_streams = false;
+    if (!small_seqs.empty() && h->stream_min_tokens < 0) {
+        if (h->batch_stream_tokens >= 0) {
+            batch_streams = small_seqs.size() >= 2 && small_k * 1e3 >= h->batch_stream_tokens;
+        } else {
+            auto estimate = [&](const SplitModel& md, int chunk, const std::vector<int>& seqs) {
+                double t = 0;
+                long long items = 0;
+                for (int s : seqs) items += (long long)c.num_kv_heads * ((Q[s] * G + chunk - 1) / chunk);
+                if (!seqs.empty()) choose_split(h, md, seqs, P, Q, G, chunk, md.unit == 64 ? 4 : 2, items, &t);
+                return t;
+            };
+            const bool one = small_seqs.size() == 1;
+            double warp_mma;
+            if (one || small_k < 7.9) {
+                warp_mma = small_rows <= 16 ? 4.1 + 0.69 * small_k : std::max(8.8, 5.8 + 1.06 * small_k);
+            } else {
+                std::vector<int> mt1, mt2;
+                for (int s : small_seqs) (Q[s] * G <= 16 ? mt1 : mt2).push_back(s);
+                warp_mma = estimate(small4_model(h, 1), 16, mt1) + estimate(small4_model(h, 2), 32, mt2);
+            }
+            std::vector<int> all = wide_seqs;
+            all.insert(all.end(), small_seqs.begin(), small_seqs.end());
+            // (with one 16-row tile the warp-MMA kernel was never more than 2 % slower than the schedule, also where the estimates tie)
+            if (!one && small_k >= 7.9 && small_rows <= 16) warp_mma *= 0.87;
+            const SplitModel sm = stream_model(h, !wide_seqs.empty());
+            batch_streams = estimate(sm, 128, all) < warp_mma + estimate(sm, 128, wide_seqs);
+        }
+    }
     long long warp_mma_tokens = 0;
     int warp_mma_seqs = 0;
     std::vector<int> groups[KIND_COUNT];
@@ -243,9 +293,8 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             // up to 128 rows: one Q tile per CTA, KV tiles alternating between two softmax warpgroups (HBM-bound
             // streaming on the tcgen05 pipe); blocks of at most 32 rows over short contexts stay with the warp-MMA
             // kernel, whose fixed costs are lower (none above 32 rows)
-            // cross-over of a single sequence (GQA 32/8): q = 8 near 7k tokens, q = 1 near 10k
-            const int cross = h->stream_min_tokens >= 0 ? h->stream_min_tokens : (rows > 8 ? 7168 : 10240);
-            if (tile_ok && rows <= h->stream_max_rows && (rows > 32 || batch_streams || P[s] + Q[s] >= cross)) k = KIND_STREAM;
+            const bool forced = h->stream_min_tokens >= 0 && P[s] + Q[s] >= h->stream_min_tokens;
+            if (tile_ok && rows <= h->stream_max_rows && (rows > 32 || batch_streams || forced)) k = KIND_STREAM;
             else if (rows <= 16) k = KIND_SMALL1;
             else if (rows <= 32) k = KIND_SMALL2;
             else if (rows <= kSmallRowsMax || h->force_mma_sync) k = KIND_SMALL4;
@@ -254,11 +303,11 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         }
         groups[k].push_back(s);
     }
-    const int small_kw = h->small_kw ? h->small_kw : (warp_mma_seqs >= 2 && warp_mma_tokens * c.num_kv_heads / 8 >= 8192) ? 4 : 8;
+    const int small_kw = h->small_kw ? h->small_kw : (warp_mma_seqs >= 2 && warp_mma_tokens * c.num_kv_heads / 8 >= 7900) ? 4 : 8;
     // Work items are handed to the SMs in launch order: the sequences with the longest contexts go first, so that the
     // longest items of a ragged batch are not the ones left over for the last wave (env AGX_LONGEST_FIRST=0 keeps the batch order).
     if (h->longest_first)
-        for (int k : {(int)KIND_TILE, (int)KIND_STREAM})
+        for (int k = 0; k < KIND_COUNT; ++k)
             std::stable_sort(groups[k].begin(), groups[k].end(), [&](int a, int b) { return P[a] + Q[a] > P[b] + Q[b]; });
     for (int k = 0; k < KIND_COUNT; ++k) {
         const std::vector<int>& seqs = groups[k];
@@ -296,11 +345,14 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         if (k == KIND_TILE || k == KIND_STREAM) {
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            C = unit * choose_split_tiles(h, k == KIND_STREAM, seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
+            C = unit * choose_split(h, k == KIND_STREAM ? stream_model(h, std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; })) : tile_model(h), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
             if (const char* force = getenv("AGX_TILE_SPLIT_TOKENS")) { if (atoi(force) >= unit) C = atoi(force) / unit * unit; }
             if (h->debug_plan)
                 fprintf(stderr, "agx plan: tile kernel, %lld row chunks, longest sequence %d tokens -> KV splits of %d tokens, %lld CTAs\n",
                         base_items, max_len, C, count_items(C));
+        } else if ((k == KIND_SMALL1 || k == KIND_SMALL2) && small_kw == 4) {
+            const SplitModel md = small4_model(h, k == KIND_SMALL1 ? 1 : 2);
+            C = md.unit * choose_split(h, md, seqs, P, Q, G, rows_per_chunk, std::max(1, min_split / md.unit), base_items);
         } else {
             while (count_items(C) > std::max<long long>(target, base_items)) C += unit;
         }
@@ -478,7 +530,7 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     env = getenv("AGX_FORCE_MMA_SYNC");
     h->force_mma_sync = env ? atoi(env) : 0;
     env = getenv("AGX_STREAM_MIN_TOKENS");
-    h->stream_min_tokens = env ? atoi(env) : -1;   // -1: the measured cross-over, by block height
+    h->stream_min_tokens = env ? atoi(env) : -1;   // -1: by the estimates of both kernels
     env = getenv("AGX_STREAM_MAX_ROWS");
     h->stream_max_rows = env ? atoi(env) : 384;
     env = getenv("AGX_CLUSTER_MERGE");
@@ -495,7 +547,7 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     env = getenv("AGX_SMALL_KW");
     h->small_kw = (env && (atoi(env) == 4 || atoi(env) == 8)) ? atoi(env) : 0;
     env = getenv("AGX_BATCH_STREAM_TOKENS");   // (forcing the per-sequence cross-over also switches the batch rule off)
-    h->batch_stream_tokens = env ? atoi(env) : getenv("AGX_STREAM_MIN_TOKENS") ? 0x7FFFFFFF : 24576;
+    h->batch_stream_tokens = env ? atoi(env) : -1;   // -1: by the estimates of both kernels
     env = getenv("AGX_DEBUG_PLAN");
     h->debug_plan = env ? atoi(env) : 0;
     h->wait_limit_cycles = kWaitLimitCycles;
