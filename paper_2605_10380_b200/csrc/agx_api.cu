@@ -378,13 +378,12 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
                 if (h->debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
             }
         }
-        // ---- scalar kernel: the splits of every item form a cluster, as many for all sequences, unless the longest context would take
-        //      more than 16 splits of 512 tokens (8 tiles, ~10 us) on an otherwise empty device
+        // ---- fp32-arithmetic kernel: up to 16 splits of an item form a cluster, as many for all sequences; more leave partials
         if (k == KIND_SIMT && h->cluster_merge) {
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            const int ns = std::min((max_len + C - 1) / C, 16);
-            if ((max_len + C - 1) / C <= 16 || max_len <= 16 * 512) {
+            const int ns = (max_len + C - 1) / C;
+            if (ns <= 16) {
                 cluster = ns;
                 C = round_up((max_len + ns - 1) / ns, kPage);
             }

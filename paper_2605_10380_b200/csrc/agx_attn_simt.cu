@@ -4,12 +4,13 @@
 // shared memory (one trip, every load in flight), score 8 x 64 pairs (a thread: one token, two rows), warp r does the softmax of
 // row r, and warp w adds up the tokens [8 w, 8 w + 8) of the tile for all rows, so that V is read from shared memory once; the
 // warps' sums meet at the end.  The KV splits of an item form a thread-block cluster and are merged through distributed
-// shared memory; only contexts that need more than 16 splits leave partials for the merge kernel.  With a fused append the block's
+// shared memory; contexts that take more than 16 splits leave partials for the merge kernel.  With a fused append the block's
 // rows come from k_new / v_new, and the item of a head's last row chunk stores them into the pages.
 //
-// Bounded by latency at the sizes it is meant for.  256 cached tokens, q = 4, 4/2 heads, fp32: 6.2 us in one launch; append, attention and
-// merge were three launches of 29 us together, of which a kernel whose warps took one token at a time was 25 (whole step with
-// the accept launch 32.5 -> 9.9 us).
+// Bounded by latency at the sizes it is meant for.  256 cached tokens, q = 4, 4/2 heads, fp32: 5.0 us in one launch; append, attention and
+// merge were three launches of 27 us together, of which a kernel whose warps took one token at a time was most.  A second tile in
+// a row costs a CTA 2.3-3.2 us (page ids, loads, four barriers), so that contexts of more than 16 tiles are better split further than a
+// cluster reaches, with partials and the merge launch: 1500 tokens, head_dim 128 11.5 us in clusters, 8.1 with partials.
 #include <math.h>
 
 #include "agx_internal.cuh"
@@ -61,7 +62,7 @@ __device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
 }  // namespace
 
 template <int D, bool kBf16>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 attn_simt_kernel(const __grid_constant__ AttnParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SimtSmem<D>& sm = *(SimtSmem<D>*)smem_raw;
@@ -81,13 +82,27 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
     const int pool_end = p.k_new ? P : L;
     const bool writer = p.k_new && rc == sp.row_chunks - 1;
     const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
+    // the first tile's page ids may be read before the dependency wait if the caller vouches for the page table
+    auto page_id = [&](int tok) {
+        const bool need = tok < tok_end && (tok < pool_end || writer);
+        return !need ? 0 : (tok >> 4) < p.pt_stride ? __ldg(pt_row + (tok >> 4)) : -1;
+    };
+    int id[kPer];
+    if (p.early_prefix) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) id[j] = page_id(tok_begin + (tid + j * kThreads) / kUnits);
+    }
     pdl_wait();
-
-    for (int i = tid; i < kR * kUnits; i += kThreads) {        // Q, scaled so that the scores are in log2 units; rows past q * G are zeros
-        const int r = row0 + i / kUnits, c = (i % kUnits) * 4;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < rows) x = load4<kBf16>(p.q, ((long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G) * D + c);
-        *(float4*)&sm.q[i / kUnits][c] = make_float4(x.x * p.scale_log2, x.y * p.scale_log2, x.z * p.scale_log2, x.w * p.scale_log2);
+    if (!p.early_prefix) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) id[j] = page_id(tok_begin + (tid + j * kThreads) / kUnits);
+    }
+    // Q (a unit per thread), scaled so that the scores are in log2 units; rows past q * G are zeros
+    static_assert(kR * kUnits <= kThreads, "one unit of Q per thread");
+    float4 qx = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < kR * kUnits && row0 + tid / kUnits < rows) {
+        const int r = row0 + tid / kUnits;
+        qx = load4<kBf16>(p.q, ((long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G) * D + (tid % kUnits) * 4);
     }
     float acc[kR][kCols];
 #pragma unroll
@@ -105,13 +120,9 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             const int u = tid + j * kThreads, tok = t0 + u / kUnits, c = (u % kUnits) * 4;
             kv[0][j] = kv[1][j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (tok >= tok_end) continue;
-            long long page = 0;
-            bool ok = true;
-            if (tok < pool_end || writer) {
-                page = (tok >> 4) < p.pt_stride ? __ldg(pt_row + (tok >> 4)) : -1;
-                ok = page >= 0 && page < p.num_pages;
-                if (!ok) atomicOr(p.status, AGX_DEV_BAD_PAGE);
-            }
+            const long long page = id[j];
+            const bool ok = page >= 0 && page < p.num_pages;
+            if (!ok) atomicOr(p.status, AGX_DEV_BAD_PAGE);
             const long long slot = ((page * p.hkv + g) * kPage + (tok & 15)) * (long long)D + c;
             if (tok < pool_end) {
                 if (ok) { kv[0][j] = load4<kBf16>(p.k_pool, slot); kv[1][j] = load4<kBf16>(p.v_pool, slot); }
@@ -122,6 +133,8 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             }
         }
         __syncthreads();                                       // the tile before this one has been used
+        if (t0 == tok_begin && tid < kR * kUnits)
+            *(float4*)&sm.q[tid / kUnits][(tid % kUnits) * 4] = make_float4(qx.x * p.scale_log2, qx.y * p.scale_log2, qx.z * p.scale_log2, qx.w * p.scale_log2);
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int u = tid + j * kThreads;
@@ -129,6 +142,10 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             *(float4*)&sm.v[u / kUnits][(u % kUnits) * 4] = kv[1][j];
         }
         __syncthreads();
+        if (t0 + kT < tok_end) {                               // page ids of the next tile
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) id[j] = page_id(t0 + kT + (tid + j * kThreads) / kUnits);
+        }
         {
             float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
