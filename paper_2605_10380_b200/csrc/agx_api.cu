@@ -655,6 +655,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.pt_stride = pt_stride;
     p.hq = h->cfg.num_q_heads; p.hkv = h->cfg.num_kv_heads; p.head_dim = h->cfg.head_dim;
     p.scale_log2 = h->scale * 1.4426950408889634f;
+    p.gqa = p.hq / p.hkv;
     p.row_div_magic = (0x100000000ull + (unsigned)(p.hq / p.hkv) - 1) / (unsigned)(p.hq / p.hkv);
     p.wait_limit_cycles = h->wait_limit_cycles;
     p.early_prefix = early_prefix;

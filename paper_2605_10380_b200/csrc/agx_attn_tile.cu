@@ -79,7 +79,7 @@ constexpr int kPolyPairsOf8 = 1;
 
 // barrier slots (8 bytes each)
 enum { BAR_K_FULL = 0, BAR_K_EMPTY = 3, BAR_V_FULL = 6, BAR_V_EMPTY = 9, BAR_S_FULL = 12, BAR_P_READY = 14,
-       BAR_O_FULL = 16, BAR_Q_FULL = 17, BAR_P_TAIL = 18, BAR_CTX = 20, BAR_P_FREE = 21, BAR_S_FREE = 23, BAR_COUNT = 24 };
+       BAR_O_FULL = 16, BAR_Q_FULL = 17, BAR_P_TAIL = 18, BAR_CTX = 20, BAR_P_FREE = 21, BAR_S_FREE = 23, BAR_Q_FULL_B = 24, BAR_COUNT = 25 };
 // P is handed to the MMA warp in two parts: the first kPvHeadSteps k-steps (16 tokens each) as soon as they are
 // stored, so that their PV MMAs run while the softmax warpgroup still works on the last columns
 constexpr int kPvHeadSteps = 6;
@@ -213,6 +213,7 @@ struct EpiCtx {
     float* part_o;
     float2* part_ml;
     float* lse;
+    int* status;
     unsigned long long magic;   // (row * magic) >> 32 == row / G exactly for rows < 2^22
 };
 template <bool kStreams>
@@ -223,19 +224,18 @@ __device__ __forceinline__ TileItem locate_item(const AttnParams& p, int block) 
     TileItem it;
     // work items reach the SMs in block order: the row chunks that see the most tokens (the last ones) go first.
     // block - item0 = ((g * row_chunks) + last - rc) * nsplit + split, or (((last - rc) * hkv) + g) * nsplit + split
-    int local = block - sp.item0;
+    const unsigned item = block - sp.item0, group = item / (unsigned)sp.nsplit;   // (signed divisions take twice as long)
     it.nsplit = sp.nsplit;
-    it.split = local % sp.nsplit;
-    local /= sp.nsplit;
+    it.split = (int)(item - group * sp.nsplit);
     const int inner = sp.chunk_major ? p.hkv : sp.row_chunks;
-    const int outer_idx = local / inner, inner_idx = local - outer_idx * inner;
+    const int outer_idx = (int)(group / (unsigned)inner), inner_idx = (int)group - outer_idx * inner;
     it.g = sp.chunk_major ? inner_idx : outer_idx;
     const int rc = sp.row_chunks - 1 - (sp.chunk_major ? outer_idx : inner_idx);
-    it.G = p.hq / p.hkv;
+    it.G = p.gqa;
     it.P = sp.prefix_len; it.q = sp.q_len;
     it.rows = it.q * it.G;
     it.row0 = rc * kRowsPerCta;
-    it.vis_end = it.P + min(it.q - 1, (it.row0 + kRowsPerCta - 1) / it.G) + 1;  // tokens the chunk's last row sees
+    it.vis_end = it.P + min(it.q - 1, (int)(((uint64_t)(uint32_t)(it.row0 + kRowsPerCta - 1) * p.row_div_magic) >> 32)) + 1;  // tokens the chunk's last row sees
     it.kv_begin = it.split * sp.split_tokens;
     it.kv_end = min(it.vis_end, it.kv_begin + sp.split_tokens);
     it.n_tiles = max(0, (it.kv_end - it.kv_begin + kBN - 1) / kBN);
@@ -311,6 +311,9 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             }
         }
     }
+    // (the scalars above cost 0.4 us: they go under the last PV; 2 x 1200 uncached tokens 44.0 -> 43.1 us, 1000 + 128 13.5 -> 13.3)
+    if (!kStreams && !mbar_wait(smem_u32(smem) + kOffBar + 8u * BAR_O_FULL, 0, (volatile int*)(smem + kOffBar + BAR_COUNT * 8), cx.status,
+                                *(const long long*)(smem + kOffBar + BAR_COUNT * 8 + 16))) return;
     tc_fence_after();
     {
         uint32_t oreg[64];   // two 32-column chunks per TMEM round trip
@@ -493,9 +496,17 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     }
 
     // ---- setup: barriers, TMEM, Q tiles
+    // Early loads: with p.early_prefix the caller vouches that the page table and the K/V pages below the cached-prefix
+    // length are not written by any launch still in flight, so the producer warp may fetch them while the launch in
+    // front of this one drains.  Its first page ids are on their way while it sets the barriers up.
+    const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
+    const bool early_ids = p.early_prefix && kv_begin + kBN <= stable_end;
+    int first_id = -1;
+    const int* const first_id_at = p.page_table + (long long)sp.seq_index * p.pt_stride + kv_begin / kPage + lane;
+    if (warp == 0 && early_ids && lane * kPage < kv_end - kv_begin) first_id = __ldg(first_id_at);
     if (tid == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : (i == BAR_Q_FULL) ? (uint32_t)kQLoadThreads : 1u);
+            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : (i == BAR_Q_FULL || i == BAR_Q_FULL_B) ? (uint32_t)(kQLoadThreads / 32) : 1u);
         *abort_flag = 0;
         *(long long*)(smem + kOffBar + BAR_COUNT * 8 + 16) = p.wait_limit_cycles;   // for the out-of-line epilogue
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -506,31 +517,46 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
-    // Early loads: with p.early_prefix the caller vouches that the page table and the K/V pages below the cached-prefix
-    // length are not written by any launch still in flight, so the producer warp may fetch them while the launch in
-    // front of this one drains.
-    if (!(warp == 0 && p.early_prefix)) pdl_wait();   // from here on global memory written by the launch before this one is read (Q, page table, K/V)
+    if (warp != 0 || !early_ids) pdl_wait();   // from here on global memory written by the launch before this one is read (Q, page table, K/V)
     // Q: 256 rows x 256 B by 16-byte cp.async (all of a thread's copies in flight at once), written in
-    // the 128-byte-swizzled K-major operand layout; rows past q * G are zero-filled.
+    // the 128-byte-swizzled K-major operand layout; rows past q * G are zero-filled.  Issuing them takes the CTA 1-1.8 us, so tile A is
+    // handed over by itself (2 x 1200 uncached tokens 45.1 -> 44.0 us a layer).  Loads into registers and stores instead: 45.6 us.
     if (warp >= 2) {
-        for (int c = tid - 64; c < kRowsPerCta * 16; c += kQLoadThreads) {   // kStreams: one tile
-            const int rl = c >> 4, ch = c & 15;     // row in chunk, 16-byte chunk of the 256-byte row
-            const int r = row0 + rl;
-            const bool valid = r < rows;
-            const int rr = valid ? r : 0;
-            const int i = (int)(((uint64_t)(uint32_t)rr * p.row_div_magic) >> 32), hg = rr - i * G;   // rr / G without the division
-            const unsigned char* src = (const unsigned char*)p.q + (((long long)(sp.q_row0 + i) * p.hq + g * G + hg) * 256 + ch * 16);
-            const int tile = rl >> 7, rt = rl & 127, half = ch >> 3, u = ch & 7;
-            cp_async_16(smem_base + kOffQ + tile * kTileBytes + half * kHalfBytes + rt * 128 + ((u ^ (rt & 7)) << 4), src, valid ? 16u : 0u);
+        // a thread copies the same 16 bytes of every kQLoadThreads / 16th row, tile A's rows as one group of copies, then tile B's
+        const int ch = tid & 15, half = ch >> 3, u = ch & 7;
+        const unsigned char* src0 = (const unsigned char*)p.q + ((long long)sp.q_row0 * p.hq + g * G) * 256 + ch * 16;
+        const int hq_minus_g = p.hq - G;
+        int rl = (tid - 64) >> 4;
+#pragma unroll
+        for (int tile = 0; tile < kRowsPerCta / 128; ++tile) {
+            const uint32_t dst0 = smem_base + kOffQ + tile * kTileBytes + half * kHalfBytes;
+#pragma unroll
+            for (int k = 0; k < (128 + kQLoadThreads / 16 - 1) / (kQLoadThreads / 16); ++k) {
+                const int r = row0 + tile * 128 + rl;
+                const bool valid = r < rows;
+                const int rr = valid ? r : 0;
+                const int i = (int)(((uint64_t)(uint32_t)rr * p.row_div_magic) >> 32);   // rr / G without the division
+                if (rl < 128) {   // (head g * G + r - i * G of row i)
+                    cp_async_16(dst0 + rl * 128 + ((u ^ (rl & 7)) << 4), src0 + (long long)(i * hq_minus_g + rr) * 256, valid ? 16u : 0u);
+                    rl += kQLoadThreads / 16;
+                }
+            }
+            rl -= 128;
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
         }
     }
-    // fused append: the CTAs of a row chunk store the block rows whose first query row lies in the chunk, each split its share, while the
-    // first K tile and Q are on their way
+    // fused append: the CTAs of a row chunk store the block rows whose first query row lies in the chunk, each split its share: loaded here,
+    // while Q is on its way, stored (and the rest of a large share loaded and stored) once Q is handed over
+    BlockRows own;
+    int own_lo = 0, own_hi = 0;
     if (p.k_new && warp >= 2) {
-        const int i_lo = (row0 + G - 1) / G, i_n = min(q, (row0 + kRowsPerCta + G - 1) / G) - i_lo;
-        const int parts = (it.vis_end + sp.split_tokens - 1) / sp.split_tokens;   // splits with work (the last ones may have none)
-        store_block_rows(p, sp, g, i_lo + i_n * split / parts, i_lo + i_n * (split + 1) / parts, tid - 64, kQLoadThreads);
+        const int i_lo = (int)(((uint64_t)(uint32_t)(row0 + G - 1) * p.row_div_magic) >> 32);
+        const int i_n = min(q, (int)(((uint64_t)(uint32_t)(row0 + kRowsPerCta + G - 1) * p.row_div_magic) >> 32)) - i_lo;
+        const unsigned parts = (unsigned)(it.vis_end + sp.split_tokens - 1) / (unsigned)sp.split_tokens;   // splits with work (the last ones may have none)
+        own_lo = i_lo + (unsigned)(i_n * split) / parts; own_hi = i_lo + (unsigned)(i_n * (split + 1)) / parts;
+        own.load(p, sp, g, own_lo, own_hi, tid - 64, kQLoadThreads);
     }
+    if (warp == 0 && !early_ids && lane * kPage < kv_end - kv_begin) first_id = __ldg(first_id_at);
     // Barriers initialised, TMEM address published.  Warp 0 (which set the barriers up and needs nothing
     // from the others) only signals and goes straight to the page table and its first K/V copies.
     tc_fence_before();
@@ -539,9 +565,23 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = (warp == 0) ? 0u : *tmem_slot;
     if (warp >= 2) {
+        if (!kStreams) {
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_Q_FULL));
+        }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        mbar_arrive(bar(BAR_Q_FULL));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kStreams ? BAR_Q_FULL : BAR_Q_FULL_B));
+        if (p.k_new) {
+            own.store(p, sp, g, own_lo, own_hi, tid - 64, kQLoadThreads);
+            for (int idx0 = tid - 64 + BlockRows::kBatch * kQLoadThreads; idx0 < (own_hi - own_lo) * 32; idx0 += BlockRows::kBatch * kQLoadThreads) {
+                own.load(p, sp, g, own_lo, own_hi, idx0, kQLoadThreads);
+                own.store(p, sp, g, own_lo, own_hi, idx0, kQLoadThreads);
+            }
+        }
     }
     auto pages_in_tile = [&](int t) { return min(8, (kv_end - (kv_begin + t * kBN) + kPage - 1) / kPage); };
 
@@ -556,25 +596,23 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // Page ids are read 32 (four tiles) at a time and two groups ahead of the copies that need them; their row-group coordinates wait in
         // shared memory, so that the thread that issues the copies of a tile has them with two loads.
         int* const page_ring = (int*)(smem + kOffPages);   // [4 groups][32]
-        auto fetch_ids = [&](int group) {   // (by the whole warp; -1: no such page)
+        auto load_ids = [&](int group) {   // (by the whole warp)
             const int pi = group * 32 + lane;
-            long long id = -1;
-            if (pi < n_pages_total) {
-                id = __ldg(pt_row + page0 + pi);
-                if (id < 0 || id >= p.num_pages) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
-            }
-            return (int)id;
+            return pi < n_pages_total ? __ldg(pt_row + page0 + pi) : -1;
         };
+        auto check_ids = [&](int group, int id) {
+            if (group * 32 + lane < n_pages_total && (id < 0 || id >= p.num_pages)) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
+            return id;
+        };
+        auto fetch_ids = [&](int group) { return check_ids(group, load_ids(group)); };
         auto put_ids = [&](int group, int id) { page_ring[(group & 3) * 32 + lane] = (id * p.hkv + g) * (kPage / 8); __syncwarp(); };
         bool ok = true;
-        bool waited = !p.early_prefix;       // has this warp passed the dependency wait?
-        const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
+        bool waited = !early_ids;            // has this warp passed the dependency wait?
         // tokens [0, pool_end) come from the pool; a tile wholly inside the pool's full pages is eight page copies, see load_mixed for others
         const int pool_full = (p.k_new ? P : L) & ~(kPage - 1);
         int last_k = -1, last_v = -1;   // last tiles whose copies were armed (for the drain below)
         const int n_groups = (n_tiles + 3) >> 2;
-        if (!waited && kv_begin + kBN > stable_end) { pdl_wait(); waited = true; }
-        put_ids(0, fetch_ids(0));
+        put_ids(0, check_ids(0, first_id));
         int ids_ahead = 0, ahead = -1;       // group `ahead` has been read (its ids are in ids_ahead), groups below it are in page_ring
         int ks = 0, vs = 0;
         uint32_t kph = 1, vph = 1;
@@ -652,6 +690,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             for (int u = 0; u < n_units && ok; ++u) {
                 const int x = u & 1;
                 if (kStreams || x == 0) ok = mbar_wait(bar(BAR_K_FULL + ks), kph, abort_flag, p.status, p.wait_limit_cycles);
+                if (!kStreams && ok && u == 1) ok = mbar_wait(bar(BAR_Q_FULL_B), 0, abort_flag, p.status, p.wait_limit_cycles);
                 if (ok && u > 0) ok = mbar_wait(bar(BAR_S_FREE), x ^ 1, abort_flag, p.status, p.wait_limit_cycles);   // unit u - 1 is in registers
                 if (!ok) break;
                 tc_fence_after();
@@ -714,7 +753,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cx->it = locate_item<kStreams>(p, blockIdx.x);
             cx->part_base = sp.part_base; cx->hq = p.hq;
             cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->lse = p.lse;
-            cx->magic = p.row_div_magic;
+            cx->magic = p.row_div_magic; cx->status = p.status;
             cx->part_half = p.part_half;
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }
@@ -844,7 +883,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BAR_P_TAIL + x));
         }
-        if (ok) ok = mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
+        if (kStreams && ok) ok = mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);   // (else waited for in the epilogue)
         if (ok || kStreams) tile_epilogue<kStreams>(smem, tO, m_ref, l_run, ok);
     }
     // ---- teardown

@@ -56,6 +56,7 @@ struct AttnParams {
     int total_rows;      // rows of k_new / v_new
     int pt_stride;
     int hq, hkv, head_dim;
+    int gqa;             // hq / hkv
     int num_seqs;
     int num_items;
     float scale_log2;  // scale * log2(e)

@@ -91,13 +91,13 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 // Fused KV append (bf16, d = 128): the block's rows [i_lo, i_hi) of KV head g go into the sequence's pages (Sec. 2.3: the block's KV
 // joins the cache).  Nothing in the same launch reads them there: the attention CTAs take the block's own rows from k_new / v_new,
 // so there is nothing to wait for.
-__device__ __forceinline__ void store_block_rows(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int tid, int nthreads) {
-    const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
-    const int units = (i_hi - i_lo) * 32;
-    constexpr int kBatch = 4;   // loads in flight per thread
-    for (int idx0 = tid; idx0 < units; idx0 += kBatch * nthreads) {
-        uint4 v[kBatch];
-        int id[kBatch];
+struct BlockRows {
+    static constexpr int kBatch = 4;   // 16-byte units in flight per thread: idx0, idx0 + nthreads, ...
+    uint4 v[kBatch];
+    int id[kBatch];
+    __device__ __forceinline__ void load(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int idx0, int nthreads) {
+        const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
+        const int units = (i_hi - i_lo) * 32;
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const int idx = idx0 + j * nthreads, i = i_lo + (idx >> 5), slot = (sp.prefix_len + i) >> 4;
@@ -107,6 +107,8 @@ __device__ __forceinline__ void store_block_rows(const AttnParams& p, const SeqP
                 v[j] = __ldg((const uint4*)((const unsigned char*)((idx & 16) ? p.v_new : p.k_new) + (((long long)(sp.q_row0 + i) * p.hkv + g) * 256 + (idx & 15) * 16)));
             }
         }
+    }
+    __device__ __forceinline__ void store(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int idx0, int nthreads) {
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const int idx = idx0 + j * nthreads, tok = sp.prefix_len + i_lo + (idx >> 5);
@@ -115,7 +117,7 @@ __device__ __forceinline__ void store_block_rows(const AttnParams& p, const SeqP
             else if (id[j] != -2) atomicOr(p.status, AGX_DEV_BAD_PAGE);
         }
     }
-}
+};
 
 // ---- thread-block clusters: barrier over all threads of all CTAs, and loads from a peer CTA's shared memory
 __device__ __forceinline__ void cluster_sync() {
