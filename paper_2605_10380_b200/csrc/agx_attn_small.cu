@@ -121,19 +121,23 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 
     const int si = find_seq(p, blockIdx.x);
     const SeqPlan sp = p.seq[si];
-    int local = blockIdx.x - sp.item0;  // ((g * row_chunks) + rc) * nsplit + split
-    const int split = local % sp.nsplit;
-    local /= sp.nsplit;
-    const int rc = local % sp.row_chunks;
-    const int g = local / sp.row_chunks;
-    const int G = p.hq / p.hkv;
+    const unsigned item = blockIdx.x - sp.item0;   // ((g * row_chunks) + rc) * nsplit + split
+    const unsigned chunk = item / (unsigned)sp.nsplit;
+    const int split = (int)(item - chunk * sp.nsplit);
+    const int g = sp.row_chunks == 1 ? (int)chunk : (int)(chunk / (unsigned)sp.row_chunks);
+    const int rc = (int)chunk - g * sp.row_chunks;
+    const int G = p.gqa;
+    // r / G without the division.  Signed divisions here, at the Q tile's addresses and in the epilogue cost a CTA 0.2-0.9 us in all (one
+    // layer: 8-row verify over 1024 / 4096 tokens 8.29 -> 7.78 / 9.34 -> 9.09 us, 4 x 4096 18.4 -> 17.5, one row over 300 / 4096 5.34 -> 5.07
+    // / 6.92 -> 6.74; one row over 16000 and more, bound by HBM, 15.3 -> 15.6).
+    auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div_magic) >> 32); };
     const int P = sp.prefix_len;
     const int q = sp.q_len;
     const int L = P + q;
     const int rows = q * G;          // query rows of this KV head, r = i * G + (h % G)
     const int row0 = rc * 16 * MT;   // first row of this CTA's chunk
     // the chunk's last row sees tokens 0 .. P + i_last
-    const int vis_end = P + min(q - 1, (row0 + 16 * MT - 1) / G) + 1;
+    const int vis_end = P + min(q - 1, div_g(row0 + 16 * MT - 1)) + 1;
     const int tok_begin = split * sp.split_tokens;
     const int tok_end = min(vis_end, tok_begin + sp.split_tokens);
     const int n_stages = max(0, (tok_end - tok_begin + kStageTokens - 1) / kStageTokens);
@@ -268,7 +272,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
             const int c = tid - 32 + j * kLoaders, r = c >> 4, ch = c & 15;
             v[j] = make_uint4(0, 0, 0, 0);
             if (c < kUnits && row0 + r < rows) {
-                const int i = (row0 + r) / G, hg = (row0 + r) - i * G;
+                const int i = div_g(row0 + r), hg = (row0 + r) - i * G;
                 const long long off = ((long long)(sp.q_row0 + i) * p.hq + g * G + hg) * kRowBytes + ch * 16;
                 v[j] = __ldg((const uint4*)((const unsigned char*)p.q + off));
             }
@@ -315,8 +319,8 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         m_run[w][0] = m_run[w][1] = -INFINITY;
         l_run[w][0] = l_run[w][1] = 0.f;
         const int rA = row0 + (mt0 + w) * 16 + (lane >> 2);
-        limit[w][0] = P + min(rA / G, q - 1);
-        limit[w][1] = P + min((rA + 8) / G, q - 1);
+        limit[w][0] = P + min(div_g(rA), q - 1);
+        limit[w][1] = P + min(div_g(rA + 8), q - 1);
     }
     // Per-lane ldmatrix offsets inside one page of the TMA layout [row group 2][half 2][8 rows][128 B], where the
     // 16-byte unit u of row r sits at ((u ^ (r & 7)) << 4).  K (x4): row = nt*8 + lane%8, unit = (kp&1)*4 + lane/8.
@@ -558,7 +562,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
             l_all += (v.x + v.y) + (v.z + v.w);
         }
         const float m_all = m_run[w][h];
-        const int i = (row0 + r) / G, hg = (row0 + r) - i * G;
+        const int i = div_g(row0 + r), hg = (row0 + r) - i * G;
         const int hd = g * G + hg;
         const bool first = kg == 0 && (lane & 3) == 0;       // one lane per row writes the row's (m, l)
         if (sp.nsplit == 1) {
@@ -635,7 +639,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 const float wk = __shfl_sync(0xFFFFFFFFu, w, k);
                 if (k < cs && wk != 0.f) { acc.x += v[k].x * wk; acc.y += v[k].y * wk; acc.z += v[k].z * wk; acc.w += v[k].w * wk; }
             }
-            const int i = (row0 + r) / G, hg = (row0 + r) - i * G;
+            const int i = div_g(row0 + r), hg = (row0 + r) - i * G;
             const int h = g * G + hg;
             const float inv = 1.f / l_all;
             uint2 packed;
