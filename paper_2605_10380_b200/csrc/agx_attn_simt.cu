@@ -51,14 +51,6 @@ __device__ __forceinline__ void store4(void* base, long long at, float4 v) {
     else *(float4*)((float*)base + at) = v;
 }
 
-__device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
-    int s = 0;
-#pragma unroll 1
-    for (int i = 1; i < p.num_seqs; ++i)
-        if (p.seq[i].item0 <= item) s = i;
-    return s;
-}
-
 }  // namespace
 
 template <int D, bool kBf16>

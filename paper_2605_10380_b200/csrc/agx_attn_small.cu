@@ -24,7 +24,7 @@
 
 #include "agx_internal.cuh"
 
-#include <type_traits>
+#include <algorithm>
 #include "agx_sm100.cuh"
 
 namespace agx {
@@ -72,24 +72,12 @@ __device__ __forceinline__ float2 ld_volatile_f2(const void* p) {
     return v;
 }
 
-// Locate the work item: sequence plan + (kv head, split).
-__device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
-    int s = 0;
-#pragma unroll 1
-    for (int i = 1; i < p.num_seqs; ++i)
-        if (p.seq[i].item0 <= item) s = i;
-    return s;
-}
-
 }  // namespace
 
 // MW = m-tiles per warp: with MW = 2 a warp scores its page against both 16-row tiles of a 32-row block and accumulates
 // both tiles' output columns, so every K and V fragment is read from shared memory once instead of twice.
-// SP stages per trip through the loop.  SP = 2 is for launches whose splits fit the ring (up to NS stages, 384 tokens with 8-page stages):
-// every stage is requested at the start, and a warp scores two pages between two meetings of its group, which halves the meetings and
-// doubles the independent work between them.  Longer splits take one stage at a time and keep the ring full.
-template <int MT, int KW, int NS, int MW, int SP>
-__global__ void __launch_bounds__(32 * (MT / MW) * KW, ((MT / MW) * KW <= 8 && MW == 1 && SP == 1) ? 2 : 1)
+template <int MT, int KW, int NS, int MW>
+__global__ void __launch_bounds__(32 * (MT / MW) * KW, ((MT / MW) * KW <= 8 && MW == 1) ? 2 : 1)
 attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k,
                        const __grid_constant__ CUtensorMap map_v) {
     extern __shared__ unsigned char smem_raw[];
@@ -109,7 +97,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     // exchange area of the KV groups: per-page row maxima, per-group row sums, P fragments of the stage's pages
     float* x_max = (float*)(q_smem + MT * 16 * kRowBytes + 2 * NS * 8 + 16);   // [MT][16][KW]
     float* x_l = x_max + MT * 16 * KW;                                          // [MT][16][KW]
-    uint4* x_p = (uint4*)(x_l + MT * 16 * KW);                                  // [MT][SP * KW][32]
+    uint4* x_p = (uint4*)(x_l + MT * 16 * KW);                                  // [MT][KW][32]
     auto full_bar = [&](int i) { return bar_base + 8u * i; };
     auto empty_bar = [&](int i) { return bar_base + 8u * (NS + i); };
 
@@ -255,7 +243,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         bool waited = !pre;
         const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
 #pragma unroll 1
-        for (int s = 0; s < (SP == 2 ? NS : NS - 1); ++s) {
+        for (int s = 0; s < NS - 1; ++s) {
             // (with a fused append only pages below stable_end come from the pool)
             if (!waited && !p.k_new && tok_begin + (n_stages - s) * kStageTokens > stable_end) { pdl_wait(); waited = true; }
             produce(s);
@@ -338,107 +326,89 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 
     const int rg = lane >> 2;                      // this lane's rows in an m-tile: rg and rg + 8
     float* my_max = x_max + (mt0 * 16 + rg) * KW;  // x_max[mt][row][kg]; m-tile mt0 + w: + w * 16 * KW
-    uint4* my_p = x_p + (mt0 * SP * KW) * 32 + lane;   // x_p[mt][sp * KW + kg][lane]: page kg's P as the lanes' MMA A fragments; + w * SP * KW * 32
+    uint4* my_p = x_p + (mt0 * KW) * 32 + lane;    // x_p[mt][kg][lane]: page kg's P as the lanes' MMA A fragments; + w * KW * 32
     auto group_sync = [&]() { asm volatile("bar.sync %0, %1;\n" ::"r"(1 + mt0 / MW), "n"(32 * KW) : "memory"); };
 
     bool live = true;   // a warp whose wait gave up keeps meeting the others at the group barriers
-    // CNT stages from `stage` on
-    auto trip = [&](auto count, int stage) {
-        constexpr int CNT = decltype(count)::value;
-        float s[CNT][MW][2][4];
+#pragma unroll 1
+    for (int stage = 0; stage < n_stages; ++stage) {
+        const int slot = stage % NS;
+        if (warp == 0) produce(stage + NS - 1);
+        if (live) live = mbar_wait(full_bar(slot), (stage / NS) & 1, abort_flag, p.status, p.wait_limit_cycles);
+
+        const int stage_tok0 = tok_begin + (n_stages - 1 - stage) * kStageTokens;
+        const int npg = live ? min(kKW, (tok_end - stage_tok0 + kPage - 1) / kPage) : 0;   // pages of this stage
+        const int tok0 = stage_tok0 + kg * kPage;
+        const bool has_page = kg < npg;
+        const uint32_t stage_base = smem_base + slot * kStageBytes;
+        float s[MW][2][4];
         float mx[MW][2];
-        int npg[CNT];          // pages of the trip's stages
-        uint32_t base[CNT];    // the stages in shared memory
-        bool has_page[CNT];    // this warp's page of each
 #pragma unroll
         for (int w = 0; w < MW; ++w) mx[w][0] = mx[w][1] = -INFINITY;
-        if (SP == 1 && warp == 0) produce(stage + NS - 1);
+        if (has_page) {
+            const uint32_t k_base = stage_base + kg * 4096;
+            // S = Q K^T for 16 tokens: two n-tiles of 8 tokens, as four accumulation chains of four MMAs each per m-tile
+            // (even and odd k-steps of both n-tiles): a dependent mma.sync is slow to issue.  A K fragment serves every m-tile.
+            float s_odd[MW][2][4];
 #pragma unroll
-        for (int sp_i = 0; sp_i < CNT; ++sp_i) {
-            const int slot = (stage + sp_i) % NS;
-            if (live) live = mbar_wait(full_bar(slot), ((stage + sp_i) / NS) & 1, abort_flag, p.status, p.wait_limit_cycles);
-            const int stage_tok0 = tok_begin + (n_stages - 1 - stage - sp_i) * kStageTokens;
-            base[sp_i] = smem_base + slot * kStageBytes;
-            npg[sp_i] = live ? min(kKW, (tok_end - stage_tok0 + kPage - 1) / kPage) : 0;
-            const int tok0 = stage_tok0 + kg * kPage;
-            has_page[sp_i] = kg < npg[sp_i];
-            if (has_page[sp_i]) {
-                const uint32_t k_base = base[sp_i] + kg * 4096;
-                // S = Q K^T for 16 tokens: two n-tiles of 8 tokens, as four accumulation chains of four MMAs each per m-tile
-                // (even and odd k-steps of both n-tiles): a dependent mma.sync is slow to issue.  A K fragment serves every m-tile.
-                float s_odd[MW][2][4];
+            for (int w = 0; w < MW; ++w) {
 #pragma unroll
-                for (int w = 0; w < MW; ++w) {
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) s[sp_i][w][nt][e] = s_odd[w][nt][e] = 0.f;
-                    }
+                for (int nt = 0; nt < 2; ++nt) {
+                    s[w][nt][0] = s[w][nt][1] = s[w][nt][2] = s[w][nt][3] = 0.f;
+                    s_odd[w][nt][0] = s_odd[w][nt][1] = s_odd[w][nt][2] = s_odd[w][nt][3] = 0.f;
                 }
+            }
 #pragma unroll
-                for (int kp = 0; kp < 4; ++kp) {
+            for (int kp = 0; kp < 4; ++kp) {
 #pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        uint32_t b0, b1, b2, b3;
-                        ldmatrix_x4(b0, b1, b2, b3, k_base + (kp >> 1) * 1024 + nt * 2048 + k_off[kp & 1]);
+                for (int nt = 0; nt < 2; ++nt) {
+                    uint32_t b0, b1, b2, b3;
+                    ldmatrix_x4(b0, b1, b2, b3, k_base + (kp >> 1) * 1024 + nt * 2048 + k_off[kp & 1]);
 #pragma unroll
-                        for (int w = 0; w < MW; ++w) {
-                            mma_bf16(s[sp_i][w][nt], qa[w][2 * kp], b0, b1);
-                            mma_bf16(s_odd[w][nt], qa[w][2 * kp + 1], b2, b3);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int w = 0; w < MW; ++w) {
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) s[sp_i][w][nt][e] += s_odd[w][nt][e];
-                    }
-                    // mask the causal edge / the end of the split (raw scores; the scale is folded into the exp)
-                    if ((tok0 + kPage - 1 > P) || (tok0 + kPage > tok_end)) {
-#pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int tok = tok0 + nt * 8 + 2 * (lane & 3) + (e & 1);
-                                if (tok > limit[w][e >> 1] || tok >= tok_end) s[sp_i][w][nt][e] = -INFINITY;
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float v = fmaxf(fmaxf(s[sp_i][w][0][2 * h], s[sp_i][w][0][2 * h + 1]), fmaxf(s[sp_i][w][1][2 * h], s[sp_i][w][1][2 * h + 1]));
-                        if (CNT == 1) {   // (here, inside the branch: behind it, one row over 20000 tokens took 17.95 us instead of 17.45)
-                            v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1));
-                            v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, 2));
-                            mx[w][h] = v * p.scale_log2;
-                        } else {
-                            mx[w][h] = fmaxf(mx[w][h], v);
-                        }
+                    for (int w = 0; w < MW; ++w) {
+                        mma_bf16(s[w][nt], qa[w][2 * kp], b0, b1);
+                        mma_bf16(s_odd[w][nt], qa[w][2 * kp + 1], b2, b3);
                     }
                 }
             }
-        }
 #pragma unroll
-        for (int w = 0; w < MW; ++w) {
+            for (int w = 0; w < MW; ++w) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (CNT > 1) {
-                    float v = mx[w][h];
+                for (int nt = 0; nt < 2; ++nt) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) s[w][nt][e] += s_odd[w][nt][e];
+                }
+                // mask the causal edge / the end of the split (raw scores; the scale is folded into the exp)
+                if ((tok0 + kPage - 1 > P) || (tok0 + kPage > tok_end)) {
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int tok = tok0 + nt * 8 + 2 * (lane & 3) + (e & 1);
+                            if (tok > limit[w][e >> 1] || tok >= tok_end) s[w][nt][e] = -INFINITY;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float v = fmaxf(fmaxf(s[w][0][2 * h], s[w][0][2 * h + 1]), fmaxf(s[w][1][2 * h], s[w][1][2 * h + 1]));
                     v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1));
                     v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, 2));
                     mx[w][h] = v * p.scale_log2;
                 }
             }
-            if ((lane & 3) == 0) { my_max[w * 16 * KW + kg] = mx[w][0]; my_max[w * 16 * KW + 8 * KW + kg] = mx[w][1]; }
         }
-        group_sync();   // the trip's page maxima of this warp's m-tiles are in place
+        if ((lane & 3) == 0) {
+#pragma unroll
+            for (int w = 0; w < MW; ++w) { my_max[w * 16 * KW + kg] = mx[w][0]; my_max[w * 16 * KW + 8 * KW + kg] = mx[w][1]; }
+        }
+        group_sync();   // the stage's page maxima of this warp's m-tiles are in place
 
-        // one running maximum per row for a whole m-tile; P of this warp's pages against it
+        // one running maximum per row for a whole m-tile; P of this warp's page against it
 #pragma unroll
         for (int w = 0; w < MW; ++w) {
-            float corr[2], m_ref[2];
+            float corr[2];
+            uint32_t pa[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float m_new = m_run[w][h];
@@ -447,35 +417,27 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                     const float4 v = *(const float4*)(my_max + w * 16 * KW + h * 8 * KW + k4);
                     m_new = fmaxf(fmaxf(m_new, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
                 }
-                m_ref[h] = (m_new == -INFINITY) ? 0.f : m_new;
-                corr[h] = ex2(m_run[w][h] - m_ref[h]);
+                const float m_ref = (m_new == -INFINITY) ? 0.f : m_new;
+                corr[h] = ex2(m_run[w][h] - m_ref);
                 m_run[w][h] = m_new;
-            }
-            float sum[2] = {0.f, 0.f};
+                float sum = 0.f;
+                if (has_page) {
 #pragma unroll
-            for (int sp_i = 0; sp_i < CNT; ++sp_i) {
-                uint32_t pa[4] = {0u, 0u, 0u, 0u};
-                if (has_page[sp_i]) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) {
-                            s[sp_i][w][nt][2 * h] = ex2(fmaf(s[sp_i][w][nt][2 * h], p.scale_log2, -m_ref[h]));
-                            s[sp_i][w][nt][2 * h + 1] = ex2(fmaf(s[sp_i][w][nt][2 * h + 1], p.scale_log2, -m_ref[h]));
-                            sum[h] += s[sp_i][w][nt][2 * h] + s[sp_i][w][nt][2 * h + 1];
-                        }
+                    for (int nt = 0; nt < 2; ++nt) {
+                        s[w][nt][2 * h] = ex2(fmaf(s[w][nt][2 * h], p.scale_log2, -m_ref));
+                        s[w][nt][2 * h + 1] = ex2(fmaf(s[w][nt][2 * h + 1], p.scale_log2, -m_ref));
+                        sum += s[w][nt][2 * h] + s[w][nt][2 * h + 1];
                     }
                 }
-                if (has_page[sp_i]) {
-                    pa[0] = pack_bf16(s[sp_i][w][0][0], s[sp_i][w][0][1]);
-                    pa[1] = pack_bf16(s[sp_i][w][0][2], s[sp_i][w][0][3]);
-                    pa[2] = pack_bf16(s[sp_i][w][1][0], s[sp_i][w][1][1]);
-                    pa[3] = pack_bf16(s[sp_i][w][1][2], s[sp_i][w][1][3]);
-                }
-                my_p[(w * SP * KW + sp_i * KW + kg) * 32] = make_uint4(pa[0], pa[1], pa[2], pa[3]);
+                l_run[w][h] = l_run[w][h] * corr[h] + sum;
             }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) l_run[w][h] = l_run[w][h] * corr[h] + sum[h];
+            if (has_page) {
+                pa[0] = pack_bf16(s[w][0][0], s[w][0][1]);
+                pa[1] = pack_bf16(s[w][0][2], s[w][0][3]);
+                pa[2] = pack_bf16(s[w][1][0], s[w][1][1]);
+                pa[3] = pack_bf16(s[w][1][2], s[w][1][3]);
+            }
+            my_p[(w * KW + kg) * 32] = make_uint4(pa[0], pa[1], pa[2], pa[3]);
             if (__any_sync(0xFFFFFFFFu, corr[0] != 1.f || corr[1] != 1.f)) {
 #pragma unroll
                 for (int n = 0; n < 2 * kCG; ++n) {
@@ -486,41 +448,29 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         }
         group_sync();   // every page's P fragments are in place
 
-        // O[:, this warp's columns] += P V over the trip's pages (a V fragment serves every m-tile)
+        // O[:, this warp's columns] += P V over the stage's pages (a V fragment serves every m-tile)
 #pragma unroll
-        for (int sp_i = 0; sp_i < CNT; ++sp_i) {
+        for (int k = 0; k < kKW; ++k) {
+            if (k < npg) {
+                uint4 pk[MW];
 #pragma unroll
-            for (int k = 0; k < kKW; ++k) {
-                if (k < npg[sp_i]) {
-                    uint4 pk[MW];
+                for (int w = 0; w < MW; ++w) pk[w] = my_p[(w * KW + k) * 32];
+                const uint32_t v_base = stage_base + kStageTokens * kRowBytes + k * 4096;
 #pragma unroll
-                    for (int w = 0; w < MW; ++w) pk[w] = my_p[(w * SP * KW + sp_i * KW + k) * 32];
-                    const uint32_t v_base = base[sp_i] + kStageTokens * kRowBytes + k * 4096;
+                for (int c = 0; c < kCG; ++c) {
+                    uint32_t b0, b1, b2, b3;
+                    ldmatrix_x4_trans(b0, b1, b2, b3, v_base + v_off[c]);
 #pragma unroll
-                    for (int c = 0; c < kCG; ++c) {
-                        uint32_t b0, b1, b2, b3;
-                        ldmatrix_x4_trans(b0, b1, b2, b3, v_base + v_off[c]);
-#pragma unroll
-                        for (int w = 0; w < MW; ++w) {
-                            const uint32_t a[4] = {pk[w].x, pk[w].y, pk[w].z, pk[w].w};
-                            mma_bf16(o[w][2 * c], a, b0, b1);
-                            mma_bf16(o[w][2 * c + 1], a, b2, b3);
-                        }
+                    for (int w = 0; w < MW; ++w) {
+                        const uint32_t a[4] = {pk[w].x, pk[w].y, pk[w].z, pk[w].w};
+                        mma_bf16(o[w][2 * c], a, b0, b1);
+                        mma_bf16(o[w][2 * c + 1], a, b2, b3);
                     }
                 }
             }
-            __syncwarp();
-            if (live && lane == 0) mbar_arrive(empty_bar((stage + sp_i) % NS));
         }
-    };
-    int stage = 0;
-    if constexpr (SP == 2) {
-#pragma unroll 1
-        for (; stage + 1 < n_stages; stage += 2) trip(std::integral_constant<int, 2>{}, stage);
-    }
-#pragma unroll 1
-    for (; stage < n_stages; ++stage) {
-        trip(std::integral_constant<int, 1>{}, stage);
+        __syncwarp();
+        if (live && lane == 0) mbar_arrive(empty_bar(slot));
     }
 
     // ---- row sums of the m-tile: each KV group's share through shared memory
@@ -612,44 +562,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
             }
         }
     }
-    if (in_cluster && sp.nsplit > 1) {   // (uniform over the cluster: all its CTAs belong to one sequence)
-        cluster_sync();   // every split's rows are in place
-        const int cs = sp.nsplit;
-        const int n_rows = min(rows - row0, MT * 16);
-        // rows are dealt round-robin to the cluster's CTAs; one warp merges one row, lane k < cs holding split k's
-        // (m, l), every lane four columns of each split's O row (all loads in flight at once)
-        for (int r = split + warp * cs; r < n_rows; r += kWarps * cs) {
-            float2 ml = make_float2(-INFINITY, 0.f);
-            if (lane < cs) ml = ld_cluster_f2(cluster_map(smem_u32(cl_ml + r), lane));
-            float m_all = ml.x;
-#pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, d));
-            const float w = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
-            float l_all = ml.y * w;
-#pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, d);
-            const uint32_t row_addr = smem_u32(cl_o + r * kD + lane * 4);
-            float4 v[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if (k < cs) v[k] = ld_cluster_f4(cluster_map(row_addr, k));
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float wk = __shfl_sync(0xFFFFFFFFu, w, k);
-                if (k < cs && wk != 0.f) { acc.x += v[k].x * wk; acc.y += v[k].y * wk; acc.z += v[k].z * wk; acc.w += v[k].w * wk; }
-            }
-            const int i = div_g(row0 + r), hg = (row0 + r) - i * G;
-            const int h = g * G + hg;
-            const float inv = 1.f / l_all;
-            uint2 packed;
-            packed.x = pack_bf16(acc.x * inv, acc.y * inv);
-            packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-            *(uint2*)((__nv_bfloat16*)p.out + ((long long)(sp.q_row0 + i) * p.hq + h) * kD + lane * 4) = packed;
-            if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
-        }
-        cluster_sync();   // no CTA leaves while its rows may still be read
-    }
+    if (in_cluster && sp.nsplit > 1) merge_cluster_rows<kWarps>(p, sp, cl_o, cl_ml, g, split, row0, min(rows - row0, MT * 16));
 }
 
 // --------------------------------------------------------------------------------------------
@@ -931,53 +844,53 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
 
 // --------------------------------------------------------------------------------------------
 namespace {
-template <int MT, int KW, int NS, int MW, int SP>
+template <int MT, int KW, int NS>
 constexpr int small_smem_bytes() {
     constexpr int kClusterBytes = MT * 16 * (kD * 4 + 8);
     constexpr int kRing = NS * 2 * KW * kPage * kRowBytes;
-    constexpr int kExchange = 2 * MT * 16 * KW * 4 + MT * SP * KW * 32 * 16;
+    constexpr int kExchange = 2 * MT * 16 * KW * 4 + MT * KW * 32 * 16;
     // [ring | cluster rows][Q tile][2 * NS barriers + abort flag][exchange area] + slack for the 1024-byte alignment
     return (kRing > kClusterBytes ? kRing : kClusterBytes) + MT * 16 * kRowBytes + 2 * NS * 8 + 16 + kExchange + 1024;
 }
 
-template <int MT, int KW, int NS, int MW = 1, int SP = 1>
+template <int MT, int KW, int NS, int MW = 1>
 cudaError_t launch_small(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    constexpr int kSmem = small_smem_bytes<MT, KW, NS, MW, SP>();
+    constexpr int kSmem = small_smem_bytes<MT, KW, NS>();
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
     static bool configured_on[64] = {false};
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
     bool& configured = configured_on[device];
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        cudaError_t e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+        e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
         if (e != cudaSuccess) return e;
         configured = true;
     }
     if (p.cluster_size > 1)
-        return launch_chained_cluster(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem,
+        return launch_chained_cluster(attn_small_bf16_kernel<MT, KW, NS, MW>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem,
                                       (unsigned)p.cluster_size, stream, p, map_k, map_v);
-    return launch_chained(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem, stream, p, map_k, map_v);
+    return launch_chained(attn_small_bf16_kernel<MT, KW, NS, MW>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem, stream, p, map_k, map_v);
 }
 
-template <int MT, int KW, int NS, int MW = 1, int SP = 1>
+template <int MT, int KW, int NS, int MW = 1>
 int max_clusters(int cluster) {
     static int cached[64][17];   // 0 = not asked yet, else 1 + answer
     int device = 0;
     if (cluster < 2 || cluster > 16 || cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return 0;
     if (cached[device][cluster]) return cached[device][cluster] - 1;
-    constexpr int kSmem = small_smem_bytes<MT, KW, NS, MW, SP>();
+    constexpr int kSmem = small_smem_bytes<MT, KW, NS>();
     int n = 0;
-    if (cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess &&
-        cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, SP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    if (cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(cluster * 64); cfg.blockDim = dim3(32 * (MT / MW) * KW); cfg.dynamicSmemBytes = kSmem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n, attn_small_bf16_kernel<MT, KW, NS, MW, SP>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+        if (cudaOccupancyMaxActiveClusters(&n, attn_small_bf16_kernel<MT, KW, NS, MW>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
     } else {
         (void)cudaGetLastError();
     }
@@ -1008,15 +921,14 @@ int attn_small_max_clusters(int mt, int kw, int cluster) {
 cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                    cudaStream_t stream) {
     if (p.num_items == 0) return cudaSuccess;
-    // 8-page stages: two stages per trip where every split of the launch fits the ring (one layer, one sequence: 8-row verify over 4096 /
-    // 1024 tokens 9.76 -> 9.45 / 8.78 -> 8.40 us, one row over 300 tokens 5.58 -> 5.35); a kernel with both loops was slower on long
-    // splits (one row over 20000 tokens 17.45 -> 18.43).
-    int longest = 0;
-    for (int i = 0; i < p.num_seqs; ++i) longest = p.seq[i].split_tokens > longest ? p.seq[i].split_tokens : longest;
-    const bool pairs = kw == 8 && longest <= 3 * 8 * kPage;
-    if (mt == 2 && kw == 8 && two_tiles_per_warp())
-        return pairs ? launch_small<2, 8, 3, 2, 2>(p, map_k, map_v, stream) : launch_small<2, 8, 3, 2>(p, map_k, map_v, stream);
-    if (mt == 1 && pairs) return launch_small<1, 8, 3, 1, 2>(p, map_k, map_v, stream);
+    int longest = 0, rows = 0;
+    for (int i = 0; i < p.num_seqs; ++i) {
+        longest = std::max(longest, p.seq[i].split_tokens);
+        rows = std::max(rows, std::min(p.seq[i].q_len * p.gqa, 16 * mt));
+    }
+    // splits that fit one CTA whole (figures there)
+    if (kw == 8 && mt <= 2 && longest <= kSwapMaxTokens) return launch_attn_swap(p, rows, longest, map_k, map_v, stream);
+    if (mt == 2 && kw == 8 && two_tiles_per_warp()) return launch_small<2, 8, 3, 2>(p, map_k, map_v, stream);
     switch (mt * 16 + kw) {
         case 1 * 16 + 4: return launch_small<1, 4, 3>(p, map_k, map_v, stream);
         case 2 * 16 + 4: return launch_small<2, 4, 3>(p, map_k, map_v, stream);

@@ -1,0 +1,426 @@
+// Small-q attention over short KV splits on tcgen05 with the operands swapped (bf16, d = 128): decode and verify blocks of at most 32
+// query rows per KV head whose splits hold at most NT * 128 tokens.
+//
+// Such a launch is bound by latency: a CTA brings in its split (at most 96 pages' worth of K and V) while the launch before it
+// drains, and then everything between the arrival of Q and the last store is a chain.  With query rows as the M side of the MMAs
+// (mma.sync over 16-row tiles, or tcgen05 over 128 mostly empty rows) that chain is the matrix instructions.  Here the tokens take the M
+// side, S^T = K Q^T, and the head dimension in the second product, O^T = V^T P^T: the query rows are the N side, 16 or 32 columns, so
+// that both products of a split are some 25 to 50 instructions of one thread.  TMEM then holds a token per lane and a query row per
+// column: every thread owns one token's scores, row maxima and row sums are butterflies over lanes that leave row r in lane r, and P goes
+// back through shared memory (dead K) as the B operand.  All of a split's K, V and scores are on the SM at once: one softmax, no rescaling.
+// A CTA of one verify layer over 4096 tokens, from Q's arrival: scores 0.6 us behind it, P 1.6, O 2.6, stored 3.2 (mma.sync kernel: 4.3).
+// What is left is the chain itself: three barriers, two MMA round trips (a 128 x 16 operand tile takes the MMA unit about 64 clocks to
+// read whatever N is), and around it the launch, the dependency waits and the merge of the splits.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "agx_internal.cuh"
+#include "agx_sm100.cuh"
+
+namespace agx {
+namespace {
+
+constexpr int kTileTok = 128;
+constexpr uint32_t kTile = 128 * 256;   // 8 pages of K or V
+constexpr uint32_t kCols = 128;         // TMEM: O^T at column 0, S^T of tile t at 32 + 32 t
+
+// NR query rows that a CTA works on (4, 8, 16 or 32), NC columns of the MMAs (the rows behind NR are zeros nobody reads)
+template <int NR, int NT>
+struct Lay {
+    static constexpr int NC = NR < 16 ? 16 : NR;
+    static constexpr uint32_t kK = 0, kV = NT * kTile, kQ = 2 * NT * kTile, kBar = kQ + NC * 256;
+    static constexpr uint32_t kMax = kBar + 128;                       // [warp][NR] row maxima, then row sums
+    static constexpr uint32_t kRef = kMax + NT * 4 * NR * 4;           // [warp][NR] the row references, a copy per warp
+    static constexpr uint32_t kSum = kRef + NT * 4 * NR * 4;           // [warp][NR]
+    static constexpr uint32_t kDst = kSum + NT * 4 * NR * 4;           // [warp][NR] where the rows go
+    static constexpr uint32_t kBytes = kDst + NT * 4 * NR * 8 + 1024;  // + alignment slack
+    static constexpr uint32_t kP = kK;                                 // P: [64-token block][NC rows][128 B], 128-byte swizzle
+    static constexpr uint32_t kO = kV;                                 // cluster merge: [NR][128] floats, then [NR] (m, l)
+    static_assert(kBytes <= 232448, "one CTA's shared memory");
+};
+
+// v[r] of every lane -> lane l holds the combination over all lanes of row l % NR.  The lanes meet in the same order for every NR.
+template <int NR, class Op>
+__device__ __forceinline__ float across_lanes(float (&v)[NR], Op op) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = 16; d >= NR; d >>= 1) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) v[i] = op(v[i], __shfl_xor_sync(0xFFFFFFFFu, v[i], d));
+    }
+#pragma unroll
+    for (int d = NR / 2; d >= 1; d >>= 1) {
+        const bool up = lane & d;
+#pragma unroll
+        for (int i = 0; i < d; ++i) {
+            const float keep = up ? v[i + d] : v[i], send = up ? v[i] : v[i + d];
+            v[i] = op(keep, __shfl_xor_sync(0xFFFFFFFFu, send, d));
+        }
+    }
+    return v[0];
+}
+
+}  // namespace
+
+template <int NR, int NT>
+__global__ void __launch_bounds__(NT * 128 + 32, 1)
+attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+    using S = Lay<NR, NT>;
+    constexpr int NC = S::NC;
+    constexpr int kThreads = NT * 128, kWarps = NT * 4;   // of the softmax warps; one more warp issues the copies and the MMAs
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
+    auto k_bar = [&](int t) { return base + S::kBar + 8u * t; };
+    auto v_bar = [&](int t) { return base + S::kBar + 8u * (NT + t); };
+    auto s_bar = [&](int t) { return base + S::kBar + 8u * (2 * NT + t); };
+    const uint32_t o_bar = base + S::kBar + 8u * (3 * NT);
+    volatile int* abort_flag = (volatile int*)(smem + S::kBar + 8 * (3 * NT + 1));
+    uint32_t* tmem_slot = (uint32_t*)(smem + S::kBar + 8 * (3 * NT + 2));
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tile = warp >> 2;
+    const bool issuer = warp == kWarps;
+    const SeqPlan& sp = p.seq[find_seq(p, blockIdx.x)];
+    const unsigned item = blockIdx.x - sp.item0;   // ((g * row_chunks) + rc) * nsplit + split
+    const unsigned chunk = item / (unsigned)sp.nsplit;
+    const int split = (int)(item - chunk * sp.nsplit);
+    const int g = sp.row_chunks == 1 ? (int)chunk : (int)(chunk / (unsigned)sp.row_chunks);
+    const int rc = (int)chunk - g * sp.row_chunks;
+    const int G = p.gqa, P = sp.prefix_len, q = sp.q_len, L = P + q;
+    const int rows = q * G, row0 = rc * NC, n_rows = min(NR, rows - row0);   // query rows of this KV head, r = i * G + (h % G)
+    auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div_magic) >> 32); };   // r / G without the division
+    const int vis_end = P + min(q - 1, div_g(row0 + NC - 1)) + 1;   // tokens the chunk's last row sees
+    const int tok_begin = split * sp.split_tokens, tok_end = min(vis_end, tok_begin + sp.split_tokens);
+    const int n_pages = max(0, (tok_end - tok_begin + kPage - 1) / kPage), n_tiles = (n_pages + 7) >> 3;
+
+    // ---- setup.  With p.early_prefix (the caller vouches that the page table and the pages below the cached-prefix length are not written by a
+    // launch still in flight) page ids and pool pages are fetched before the dependency wait; with a fused append only pages below the block
+    // come from the pool.  Pages from own_pg on are put together by hand beside Q: block rows come from k_new / v_new and go into the pool on
+    // the way, and a last page that is only partly valid gets zeros behind the last token (V must not hold a NaN there).
+    const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
+    const int page0 = tok_begin / kPage;
+    const bool pre = p.early_prefix;
+    const int pool_end = p.k_new ? P : L;
+    const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
+    const int own_units = (n_pages - own_pg) * 512;   // 16-byte units, [page][K, V][16 rows][16 units]
+    constexpr int kOwn = (512 + kThreads - 1) / kThreads;   // a thread's units of the first own page
+    auto own_id = [&](int u) { const int slot = page0 + own_pg + (u >> 9); return slot < p.pt_stride ? __ldg(pt_row + slot) : -1; };
+    auto own_load = [&](int u, int id) {
+        const int tok = tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15), is_v = (u >> 8) & 1, ch = u & 15;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (tok < pool_end) {
+            const long long page = (id < 0 || id >= p.num_pages) ? 0 : id;   // (reported below)
+            v = __ldcg((const uint4*)((const unsigned char*)(is_v ? p.v_pool : p.k_pool) + ((page * p.hkv + g) * kPage + (tok & 15)) * 256 + ch * 16));
+        } else if (tok < L) {
+            v = __ldg((const uint4*)((const unsigned char*)(is_v ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * 256 + ch * 16));
+        }
+        return v;
+    };
+    auto own_store = [&](int u, int id, const uint4 v) {
+        const int pg = own_pg + (u >> 9), r = (u >> 4) & 15, is_v = (u >> 8) & 1, ch = u & 15, tok = tok_begin + pg * kPage + r;
+        *(uint4*)(smem + (is_v ? S::kV : S::kK) + pg * 4096 + (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v;
+        if (tok >= pool_end && tok < L && id >= 0 && id < p.num_pages)
+            *(uint4*)((unsigned char*)(is_v ? p.v_pool : p.k_pool) + (((long long)id * p.hkv + g) * kPage + (tok & 15)) * 256 + ch * 16) = v;
+    };
+    int first_id[kOwn];   // issuer: the id of page `lane`
+    auto fetch_ids = [&]() {
+        if (issuer) first_id[0] = lane < n_pages ? __ldg(pt_row + page0 + lane) : 0;
+        else
+#pragma unroll
+            for (int j = 0; j < kOwn; ++j)
+                if (tid + j * kThreads < own_units) first_id[j] = own_id(tid + j * kThreads);
+    };
+    if (pre) fetch_ids();
+    if (issuer && lane == 0) {
+        for (int i = 0; i < 3 * NT + 1; ++i) mbar_init(base + S::kBar + 8u * i, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(&map_k) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(&map_v) : "memory");
+    }
+    pdl_launch_dependents();
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (!(issuer && pre)) pdl_wait();   // from here on global memory written by the launch before this one is read
+    if (!pre) fetch_ids();
+    if (issuer) {
+        __syncwarp();
+        int id = first_id[0];
+        if (lane < n_pages && (id < 0 || id >= p.num_pages)) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
+        bool waited = !pre;
+        if (!waited && !p.k_new && tok_end > (P & ~(kPage - 1))) { pdl_wait(); waited = true; }
+        if (lane < n_tiles && lane != p.drop_stage) {   // (drop_stage, a test hook: this tile never arrives, its consumers' waits run out)
+            const uint32_t bytes = 4096u * min(8, max(0, own_pg - lane * 8));
+            mbar_arrive_expect_tx(k_bar(lane), bytes);
+            mbar_arrive_expect_tx(v_bar(lane), bytes);
+        }
+        __syncwarp();   // the barriers are armed before any copy can complete on them
+        const bool copies = lane < own_pg && (lane >> 3) != p.drop_stage;   // lane l copies page l, all of K first
+        const int group = (id * p.hkv + g) * (kPage / 8);
+        if (copies) tma_load_page(base + S::kK + lane * 4096, &map_k, group, k_bar(lane >> 3));
+        __syncwarp();
+        if (copies) tma_load_page(base + S::kV + lane * 4096, &map_v, group, v_bar(lane >> 3));
+        __syncwarp();
+        if (!waited) pdl_wait();
+    } else {
+        // Q: [half of 64 dims][NC rows][128 B], 128-byte swizzle; rows past q * G are zeros.  (All loads are issued before the first store.)
+        constexpr int kUnits = NC * 16, kPer = (kUnits + kThreads - 1) / kThreads;
+        uint4 v[kPer], w[kOwn];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int c = tid + j * kThreads, r = c >> 4;
+            v[j] = make_uint4(0, 0, 0, 0);
+            if (c < kUnits && r < n_rows) {
+                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
+                v[j] = __ldg((const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j)
+            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, first_id[j]);
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int c = tid + j * kThreads, r = c >> 4, ch = c & 15;
+            if (c < kUnits) *(uint4*)(smem + S::kQ + (ch >> 3) * (NC * 128) + r * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v[j];
+        }
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j)
+            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, first_id[j], w[j]);
+        for (int u = tid + kOwn * kThreads; u < own_units; u += kThreads) { const int id = own_id(u); own_store(u, id, own_load(u, id)); }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();   // barriers, TMEM address, Q and the own pages are in place
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    // ---- S^T = K Q^T: tokens x rows, a tile at a time
+    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NC >> 3) << 17) | ((128u >> 4) << 24);   // f32 += bf16 x bf16, M = 128, N = NC
+    if (issuer) {
+        if (elect_one()) {
+            bool ok = true;
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                ok = mbar_wait(k_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t kd = make_desc(base + S::kK + t * kTile, 16, 2048), qd = make_desc(base + S::kQ, 16, 1024);
+#pragma unroll
+                for (int s = 0; s < 8; ++s)   // 8 k-steps of 16 dims
+                    umma_ss(tmem + 32 + 32 * t, kd + (uint64_t)(((s >> 2) * 1024 + (s & 3) * 32) >> 4),
+                            qd + (uint64_t)(((s >> 2) * (NC * 128) + (s & 3) * 32) >> 4), kIdesc, s > 0);
+                umma_commit(s_bar(t));
+            }
+        }
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;\n" ::"n"(kThreads + 32) : "memory");   // P is in place
+        tc_fence_after();
+        // ---- O^T = V^T P^T: head dims x rows, one k-step per page
+        if (elect_one()) {
+            bool ok = !*abort_flag;
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                ok = mbar_wait(v_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t vd = make_desc(base + S::kV + t * kTile, 1024, 2048), pd = make_desc(base + S::kP + t * (2 * NC * 128), 16, 1024);
+                auto step = [&](int pg) {
+                    umma_ss(tmem, vd + (uint64_t)((pg * 4096) >> 4), pd + (uint64_t)(((pg >> 2) * (NC * 128) + (pg & 3) * 32) >> 4),
+                            kIdesc | (1u << 15), t > 0 || pg > 0);   // (bit 15: A = V is MN-major)
+                };
+                const int npg = n_pages - t * 8;
+                if (npg >= 8) {
+#pragma unroll
+                    for (int pg = 0; pg < 8; ++pg) step(pg);
+                } else {
+                    for (int pg = 0; pg < npg; ++pg) step(pg);
+                }
+            }
+            umma_commit(o_bar);   // (arrives at once where nothing was issued)
+        }
+        __syncwarp();
+    }
+
+    const bool merged_here = p.cluster_size > 1 && sp.nsplit > 1;
+    float* cl_o = (float*)(smem + S::kO);
+    float2* cl_ml = (float2*)(smem + S::kO + NR * 512);
+    if (!issuer) {
+    // ---- one token per thread: mask, row maxima, P = 2^(S * scale - m)
+    const uint32_t lanes = (uint32_t)((warp & 3) << 5) << 16;
+    const int t_warp = tile * kTileTok + (warp & 3) * 32, tok = tok_begin + t_warp + lane;   // (t_warp: first token of the warp, from tok_begin)
+    bool live = tile < n_tiles && __all_sync(0xFFFFFFFFu, mbar_wait(s_bar(min(tile, NT - 1)), 0, abort_flag, p.status, p.wait_limit_cycles));
+    float s[NR], x[NR];
+    if (live) {
+        tc_fence_after();
+        tmem_ld<NR>(tmem + lanes + 32 + 32 * tile, (uint32_t*)s);
+        tmem_wait_ld();
+        if (tok_begin + t_warp + 31 > P || tok_begin + t_warp + 32 > tok_end) {   // rows below `lo` do not see this token
+            const int lo = tok >= tok_end ? NR : (tok - P) * G - row0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) if (r < lo) s[r] = -INFINITY;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) s[r] = -INFINITY;
+    }
+    float* x_max = (float*)(smem + S::kMax);
+    float* x_sum = (float*)(smem + S::kSum);
+    const int my_row = lane & (NR - 1);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) x[r] = s[r];
+    const float w_max = across_lanes<NR>(x, [](float a, float b) { return fmaxf(a, b); });
+    x_max[warp * NR + my_row] = w_max * p.scale_log2;   // (NR < 32: several lanes write the same)
+    tc_fence_before();
+    asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");   // every warp's maxima; all scores are in registers, so K is dead
+    tc_fence_after();
+    float m_row = -INFINITY;   // of row my_row
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) m_row = fmaxf(m_row, x_max[w * NR + my_row]);
+    float* ref = (float*)(smem + S::kRef) + warp * NR;
+    ref[my_row] = (m_row == -INFINITY) ? 0.f : -m_row;
+    __syncwarp();
+    if (tile < n_tiles) {
+        const int t = t_warp + lane, c = (t & 63) >> 3;
+        unsigned char* pt = smem + S::kP + (t >> 6) * (NC * 128) + (t & 7) * 2;
+#pragma unroll
+        for (int r4 = 0; r4 < NR; r4 += 4) {
+            if (r4 >= n_rows) {   // (padding: the columns of O^T that come of it are not stored, whatever P holds)
+                x[r4] = x[r4 + 1] = x[r4 + 2] = x[r4 + 3] = 0.f;
+                continue;
+            }
+            const float4 nm = *(const float4*)(ref + r4);
+            const float n[4] = {nm.x, nm.y, nm.z, nm.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = r4 + k;
+                x[r] = ex2(fmaf(s[r], p.scale_log2, n[k]));
+                *(__nv_bfloat16*)(pt + r * 128 + ((c ^ (r & 7)) << 4)) = __float2bfloat16_rn(x[r]);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    } else {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) x[r] = 0.f;
+    }
+    tc_fence_before();
+    asm volatile("bar.arrive 1, %0;\n" ::"n"(kThreads + 32) : "memory");   // P is in place
+
+    // ---- row sums, while O^T is under way
+    const float w_sum = across_lanes<NR>(x, [](float a, float b) { return a + b; });
+    x_sum[warp * NR + my_row] = w_sum;
+    asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");   // every warp's sums
+    float l_row = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) l_row += x_sum[w * NR + my_row];
+
+    // ---- epilogue: lane = head dim, column = row; the first two warpgroups take half of the rows each
+    constexpr int kHalf = NR / 2;
+    // weight and destination of row my_row, for all lanes of the warp through shared memory (its copy of the row references is dead)
+    unsigned long long* row_dst = (unsigned long long*)(smem + S::kDst) + warp * NR;
+    if (tile < 2) {
+        unsigned long long dst = 0;
+        if (my_row < n_rows && !merged_here) {
+            const int i = div_g(row0 + my_row), hd = g * G + (row0 + my_row) - i * G;
+            if (sp.nsplit == 1) {
+                const long long at = (long long)(sp.q_row0 + i) * p.hq + hd;
+                dst = (unsigned long long)((unsigned char*)p.out + at * 256);
+                if (p.lse && warp == 0 && lane < NR) p.lse[at] = (m_row + log2f(l_row)) * 0.6931471805599453f;
+            } else {
+                const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
+                dst = (unsigned long long)(p.part_o + e * 128);
+                if (warp == 0 && lane < NR) p.part_ml[e] = make_float2(m_row, l_row);
+            }
+        }
+        row_dst[my_row] = dst;
+        ref[my_row] = (l_row > 0.f) ? 1.f / l_row : 0.f;
+        __syncwarp();
+    }
+    const bool done = __all_sync(0xFFFFFFFFu, mbar_wait(o_bar, 0, abort_flag, p.status, p.wait_limit_cycles));
+    if (tile < 2) {
+        float o[kHalf];
+        if (done && n_tiles > 0) {
+            tc_fence_after();
+            tmem_ld<kHalf>(tmem + lanes + tile * kHalf, (uint32_t*)o);
+            tmem_wait_ld();
+        } else {
+#pragma unroll
+            for (int j = 0; j < kHalf; ++j) o[j] = 0.f;
+        }
+        const int d = (warp & 3) * 32 + lane;
+        if (merged_here) {
+            if (warp == 0 && lane < NR) cl_ml[lane] = make_float2(m_row, l_row);
+#pragma unroll
+            for (int j = 0; j < kHalf; ++j) cl_o[(tile * kHalf + j) * 128 + d] = o[j];
+        } else if (sp.nsplit > 1 && !p.part_half) {   // the un-normalised fp32 rows
+#pragma unroll
+            for (int j = 0; j < kHalf; ++j) {
+                const unsigned long long at = row_dst[tile * kHalf + j];
+                if (at) __stcg((float*)at + d, o[j]);
+            }
+        } else {
+            // 16-bit rows (bf16 results, normalised fp16 partials): lane pairs swap so that the even lane stores two columns of the first
+            // row of a pair, the odd lane two of the second
+            const bool odd = lane & 1;
+#pragma unroll
+            for (int j = 0; j < kHalf; j += 2) {
+                const float a = o[j] * ref[tile * kHalf + j], b = o[j + 1] * ref[tile * kHalf + j + 1];
+                const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1);
+                const float lo = odd ? got : a, hi = odd ? b : got;
+                unsigned char* const at = (unsigned char*)row_dst[tile * kHalf + j + odd];
+                if (sp.nsplit == 1) { if (at) *(uint32_t*)(at + (d & ~1) * 2) = pack_bf16(lo, hi); }
+                else if (at) __stcg((uint32_t*)(at + (d & ~1) * 2), pack_f16(lo, hi));
+            }
+        }
+    }
+    }
+    // After a wait gave up, copies armed above may still be on their way into shared memory: they land (bounded by the clock alone)
+    // before the CTA reuses or releases it.
+    if (issuer && lane == 0 && *abort_flag)
+        for (int t = 0; t < n_tiles; ++t)
+            if (t != p.drop_stage) { mbar_drain(k_bar(t), 0, p.wait_limit_cycles); mbar_drain(v_bar(t), 0, p.wait_limit_cycles); }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+    }
+    if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
+}
+
+namespace {
+template <int NR, int NT>
+cudaError_t launch_swap(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
+    constexpr int kSmem = (int)Lay<NR, NT>::kBytes;
+    // the attribute is per device: remember which devices have it (a process normally drives one GPU)
+    static bool configured_on[64] = {false};
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    if (!configured_on[device]) {
+        cudaError_t e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+        if (e != cudaSuccess) return e;
+        configured_on[device] = true;
+    }
+    if (p.cluster_size > 1)
+        return launch_chained_cluster(attn_swap_bf16_kernel<NR, NT>, dim3(p.num_items), dim3(NT * 128 + 32), kSmem, (unsigned)p.cluster_size, stream, p, map_k, map_v);
+    return launch_chained(attn_swap_bf16_kernel<NR, NT>, dim3(p.num_items), dim3(NT * 128 + 32), kSmem, stream, p, map_k, map_v);
+}
+
+template <int NT>
+cudaError_t launch_rows(const AttnParams& p, int rows, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
+    if (rows <= 4) return launch_swap<4, NT>(p, map_k, map_v, stream);
+    if (rows <= 8) return launch_swap<8, NT>(p, map_k, map_v, stream);
+    return rows <= 16 ? launch_swap<16, NT>(p, map_k, map_v, stream) : launch_swap<32, NT>(p, map_k, map_v, stream);
+}
+}  // namespace
+
+// One layer of one sequence, GQA 32/8, mma.sync kernel with the same splits -> this one: 8-row verify over 4096 / 1024 tokens 9.07 -> 8.08 / 7.77 ->
+// 7.12 us, one row over 300 / 1500 / 4096 / 7000 tokens 5.08 -> 4.93 / 6.28 -> 6.01 / 6.78 -> 6.49 / 9.40 -> 9.37.  Only the rows that exist are
+// worked on (one row with the softmax of 16: 7.01 us over 4096 tokens instead of 6.49).
+cudaError_t launch_attn_swap(const AttnParams& p, int rows, int longest, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
+    return longest <= 2 * kTileTok ? launch_rows<2>(p, rows, map_k, map_v, stream) : launch_rows<3>(p, rows, map_k, map_v, stream);
+}
+
+}  // namespace agx

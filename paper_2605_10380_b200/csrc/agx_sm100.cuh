@@ -119,6 +119,66 @@ struct BlockRows {
     }
 };
 
+// The sequence plan of a work item.
+__device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
+    int s = 0;
+#pragma unroll 1
+    for (int i = 1; i < p.num_seqs; ++i)
+        if (p.seq[i].item0 <= item) s = i;
+    return s;
+}
+
+// ---- tcgen05: descriptors, MMA, TMEM
+// shared-memory matrix descriptor, SWIZZLE_128B, descriptor version 1
+__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
+}
+
+__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void umma_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+
+__device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr));
+}
+// N = 2, 4, 8, 16 or 32 columns from taddr on
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
+    if constexpr (N == 2) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+    } else if constexpr (N == 4) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+    } else if constexpr (N == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
+    } else if constexpr (N == 16) {
+        tmem_ld<8>(taddr, r);
+        tmem_ld<8>(taddr + 8, r + 8);
+    } else {
+        tmem_ld_x32(taddr, r);
+    }
+}
+__device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;\n" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
 // ---- thread-block clusters: barrier over all threads of all CTAs, and loads from a peer CTA's shared memory
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
@@ -148,6 +208,47 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// Merge of the KV splits of one (sequence, KV head) = the CTAs of a cluster (rank = split), each holding n_rows un-normalised fp32 rows of O
+// ([row][128]) and their (m, l) in shared memory.  Rows are dealt round-robin to the CTAs; one warp merges one row, lane k < splits
+// holding split k's (m, l), every lane four columns of each split's O row (all loads in flight at once).
+template <int kWarps>
+__device__ __forceinline__ void merge_cluster_rows(const AttnParams& p, const SeqPlan& sp, const float* cl_o, const float2* cl_ml, int g, int split,
+                                                   int row0, int n_rows) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = p.gqa;
+    cluster_sync();   // every split's rows are in place
+    const int cs = sp.nsplit;
+    for (int r = split + warp * cs; r < n_rows; r += kWarps * cs) {
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (lane < cs) ml = ld_cluster_f2(cluster_map(smem_u32(cl_ml + r), lane));
+        float m_all = ml.x;
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, d));
+        const float w = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
+        float l_all = ml.y * w;
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, d);
+        const uint32_t row_addr = smem_u32(cl_o + r * 128 + lane * 4);
+        float4 v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (k < cs) v[k] = ld_cluster_f4(cluster_map(row_addr, k));
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const float wk = __shfl_sync(0xFFFFFFFFu, w, k);
+            if (k < cs && wk != 0.f) { acc.x += v[k].x * wk; acc.y += v[k].y * wk; acc.z += v[k].z * wk; acc.w += v[k].w * wk; }
+        }
+        const int i = (int)(((uint64_t)(uint32_t)(row0 + r) * p.row_div_magic) >> 32), h = g * G + (row0 + r) - i * G;
+        const float inv = 1.f / l_all;
+        uint2 packed;
+        packed.x = pack_bf16(acc.x * inv, acc.y * inv);
+        packed.y = pack_bf16(acc.z * inv, acc.w * inv);
+        *(uint2*)((__nv_bfloat16*)p.out + ((long long)(sp.q_row0 + i) * p.hq + h) * 128 + lane * 4) = packed;
+        if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+    }
+    cluster_sync();   // no CTA leaves while its rows may still be read
 }
 
 }  // namespace
