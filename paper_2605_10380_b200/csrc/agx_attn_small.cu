@@ -568,8 +568,8 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 // --------------------------------------------------------------------------------------------
 // Combine: out[row, h] = sum_k O_k 2^(m_k - m) / sum_k l_k 2^(m_k - m), splits in index order.
 // One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
-// kMaxNs: no sequence of the launch has more splits than this (4, 16, or any number).  Four O rows per warp instead of 32
-// keep the register count low enough for ten CTAs per SM, which is what the partials of a split prefill need.
+// kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel takes more).  Four O rows per
+// warp instead of 32 keep the register count low enough for ten CTAs per SM, which is what the partials of a split prefill need.
 // kHalfPart: the partial rows are fp16 and already divided by their own sums l_k (the 256-row tensor-core schedule), so
 // split k weighs l_k 2^(m_k - m) instead of 2^(m_k - m).
 template <bool kHalfPart>
@@ -610,79 +610,41 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m_all, l_all;
     pdl_wait();   // the partials are complete
-    if (kMaxNs <= 32 || ns <= 32) {
-        // One round trip to memory: lane k fetches (m, l) of split k while every lane already fetches its
-        // columns of every split's O row; the weights then travel by shuffle, splits in index order.
-        // (volatile loads: the compiler leaves them in this order, ahead of the first use of any of them)
-        float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < ns) ml = ld_volatile_f2(p.part_ml + e0 + lane);
-        float4 v[kInFlight], v2[kFew ? 1 : 16];
+    // One round trip to memory: lane k fetches (m, l) of split k while every lane already fetches its
+    // columns of every split's O row; the weights then travel by shuffle, splits in index order.
+    // (volatile loads: the compiler leaves them in this order, ahead of the first use of any of them)
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (lane < ns) ml = ld_volatile_f2(p.part_ml + e0 + lane);
+    float4 v[kInFlight], v2[kFew ? 1 : 16];
 #pragma unroll
-        for (int j = 0; j < kInFlight; ++j)
-            if (j < ns && c4 < D) v[j] = load_part4<kHalfPart>(p, e0 + j, c4);
-        if (!kFew && ns > 16) {
+    for (int j = 0; j < kInFlight; ++j)
+        if (j < ns && c4 < D) v[j] = load_part4<kHalfPart>(p, e0 + j, c4);
+    if (!kFew && ns > 16) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (16 + j < ns && c4 < D) v2[j] = load_part4<kHalfPart>(p, e0 + 16 + j, c4);
+        for (int j = 0; j < 16; ++j)
+            if (16 + j < ns && c4 < D) v2[j] = load_part4<kHalfPart>(p, e0 + 16 + j, c4);
+    }
+    m_all = ml.x;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
+    const float e_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
+    l_all = ml.y * e_mine;
+    const float w_mine = kHalfPart ? l_all : e_mine;   // weight of this lane's split's O row
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);
+#pragma unroll
+    for (int j = 0; j < kInFlight; ++j) {
+        const float w = __shfl_sync(0xFFFFFFFFu, w_mine, j);
+        if (j < ns && w != 0.f && c4 < D) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0)
+            acc.x += v[j].x * w; acc.y += v[j].y * w; acc.z += v[j].z * w; acc.w += v[j].w * w;
         }
-        m_all = ml.x;
+    }
+    if (!kFew && ns > 16) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
-        const float e_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
-        l_all = ml.y * e_mine;
-        const float w_mine = kHalfPart ? l_all : e_mine;   // weight of this lane's split's O row
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);
-#pragma unroll
-        for (int j = 0; j < kInFlight; ++j) {
-            const float w = __shfl_sync(0xFFFFFFFFu, w_mine, j);
-            if (j < ns && w != 0.f && c4 < D) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0)
-                acc.x += v[j].x * w; acc.y += v[j].y * w; acc.z += v[j].z * w; acc.w += v[j].w * w;
-            }
-        }
-        if (!kFew && ns > 16) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float w = __shfl_sync(0xFFFFFFFFu, w_mine, 16 + j);
-                if (16 + j < ns && w != 0.f && c4 < D) {
-                    acc.x += v2[j].x * w; acc.y += v2[j].y * w; acc.z += v2[j].z * w; acc.w += v2[j].w * w;
-                }
-            }
-        }
-    } else {
-        // many splits: lanes take splits side by side for (m, l), then 4 O rows in flight at a time
-        m_all = -INFINITY;
-        for (int k = lane; k < ns; k += 32) m_all = fmaxf(m_all, p.part_ml[e0 + k].x);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
-        l_all = 0.f;
-        for (int k = lane; k < ns; k += 32) {
-            const float2 ml = p.part_ml[e0 + k];
-            l_all += (ml.x == -INFINITY) ? 0.f : ml.y * exp2f(ml.x - m_all);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);
-        if (c4 < D) {
-            int k = 0;
-            for (; k + 4 <= ns; k += 4) {
-                float w[4];
-                float4 v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 mlk = p.part_ml[e0 + k + j];
-                    w[j] = (mlk.x == -INFINITY) ? 0.f : exp2f(mlk.x - m_all) * (kHalfPart ? mlk.y : 1.f);
-                    v[j] = load_part4<kHalfPart>(p, e0 + k + j, c4);
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (w[j] != 0.f) { acc.x += v[j].x * w[j]; acc.y += v[j].y * w[j]; acc.z += v[j].z * w[j]; acc.w += v[j].w * w[j]; }
-                }
-            }
-            for (; k < ns; ++k) {
-                const float2 mlk = p.part_ml[e0 + k];
-                const float w = (mlk.x == -INFINITY) ? 0.f : exp2f(mlk.x - m_all) * (kHalfPart ? mlk.y : 1.f);
-                const float4 v = load_part4<kHalfPart>(p, e0 + k, c4);
-                if (w != 0.f) { acc.x += v.x * w; acc.y += v.y * w; acc.z += v.z * w; acc.w += v.w * w; }
+        for (int j = 0; j < 16; ++j) {
+            const float w = __shfl_sync(0xFFFFFFFFu, w_mine, 16 + j);
+            if (16 + j < ns && w != 0.f && c4 < D) {
+                acc.x += v2[j].x * w; acc.y += v2[j].y * w; acc.z += v2[j].z * w; acc.w += v2[j].w * w;
             }
         }
     }
@@ -697,6 +659,87 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         } else {
             *(float4*)((float*)p.out + off) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
         }
+    }
+    if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+}
+
+// The same merge where a sequence has more than 32 splits (long contexts over few KV heads): one CTA per (row, head), whose warps take
+// kManyBatch splits each with all their loads in flight, and the first warp adds the warps' sums in order.  Bound by one trip to memory
+// as the kernels for fewer splits are; one warp per pair went through the splits four at a time, a trip each (one layer, 16/2 heads, one row
+// over 12000 / 20000 / 55000 tokens, 47 to 74 splits: 12.0 / 17.9 / 22.4 -> 6.8 / 9.2 / 14.5 us; 8 rows over 34000 24.0 -> 15.8).
+constexpr int kManyBatch = 16, kManyWarps = 16;   // (256 splits in one trip; more go round)
+template <bool kBf16Out, bool kHalfPart>
+__global__ void __launch_bounds__(kManyWarps * 32)
+attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
+    __shared__ float4 s_acc[kManyWarps][32];
+    __shared__ float2 s_ml[kManyWarps];
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int lrow = blockIdx.x / p.hq, h = blockIdx.x - lrow * p.hq;
+    int si = 0, acc_rows = 0;
+#pragma unroll 1
+    for (int s = 0; s < p.num_seqs; ++s) {
+        if (lrow >= acc_rows && lrow < acc_rows + p.seq[s].q_len) { si = s; break; }
+        acc_rows += p.seq[s].q_len;
+    }
+    const SeqPlan& sp = p.seq[si];
+    const int ns = sp.nsplit, D = p.head_dim, c4 = lane * 4, i = lrow - acc_rows;
+    if (ns == 1) return;   // written directly by the attention kernel
+    const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float m = -INFINITY, l = 0.f;
+    pdl_wait();   // the partials are complete
+    for (int k0 = warp * kManyBatch; k0 < ns; k0 += warps * kManyBatch) {
+        const int n = min(kManyBatch, ns - k0);
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (lane < n) ml = ld_volatile_f2(p.part_ml + e0 + k0 + lane);
+        float4 v[kManyBatch];
+#pragma unroll
+        for (int j = 0; j < kManyBatch; ++j)
+            if (j < n && c4 < D) v[j] = load_part4<kHalfPart>(p, e0 + k0 + j, c4);
+        float m_new = ml.x;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xFFFFFFFFu, m_new, off));
+        m_new = fmaxf(m, m_new);
+        const float e = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_new), keep = (m == -INFINITY) ? 0.f : exp2f(m - m_new);
+        float sum = ml.y * e;
+        const float w_mine = kHalfPart ? sum : e;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+        l = l * keep + sum;
+        acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+#pragma unroll
+        for (int j = 0; j < kManyBatch; ++j) {
+            const float w = __shfl_sync(0xFFFFFFFFu, w_mine, j);
+            if (j < n && w != 0.f && c4 < D) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0)
+                acc.x += v[j].x * w; acc.y += v[j].y * w; acc.z += v[j].z * w; acc.w += v[j].w * w;
+            }
+        }
+        m = m_new;
+    }
+    s_acc[warp][lane] = acc;
+    if (lane == 0) s_ml[warp] = make_float2(m, l);
+    __syncthreads();
+    if (warp != 0 || c4 >= D) return;
+    float m_all = -INFINITY, l_all = 0.f;
+    for (int w = 0; w < warps; ++w) m_all = fmaxf(m_all, s_ml[w].x);
+    acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int w = 0; w < warps; ++w) {
+        const float2 ml = s_ml[w];
+        const float e = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
+        const float4 a = s_acc[w][lane];
+        l_all += ml.y * e;
+        acc.x += a.x * e; acc.y += a.y * e; acc.z += a.z * e; acc.w += a.w * e;
+    }
+    const float inv = 1.f / l_all;
+    const long long off = ((long long)(sp.q_row0 + i) * p.hq + h) * D + c4;
+    if (kBf16Out) {
+        uint2 packed;
+        packed.x = pack_bf16(acc.x * inv, acc.y * inv);
+        packed.y = pack_bf16(acc.z * inv, acc.w * inv);
+        *(uint2*)((__nv_bfloat16*)p.out + off) = packed;
+    } else {
+        *(float4*)((float*)p.out + off) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     }
     if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
@@ -945,6 +988,7 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
     const int blocks = (int)((n + 3) / 4);
     int ns_max = 1;
     for (int i = 0; i < p.num_seqs; ++i) ns_max = p.seq[i].nsplit > ns_max ? p.seq[i].nsplit : ns_max;
+    const int many_threads = 32 * std::min(kManyWarps, (ns_max + kManyBatch - 1) / kManyBatch);
     if (dtype == AGX_BF16 && p.part_half) {
         if (ns_max <= 4) {
             // CTAs whose warps take kCombineRows pairs each
@@ -957,16 +1001,18 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
             if (ns_max <= 20) return launch_chained(attn_combine_half32_kernel<20>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             return launch_chained(attn_combine_half32_kernel<32>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
         }
-        return launch_chained(attn_combine_kernel<true, 1 << 30, true>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        return launch_chained(attn_combine_many_kernel<true, true>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
     }
     if (dtype == AGX_BF16) {
         if (ns_max <= 4) return launch_chained(attn_combine_kernel<true, 4, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
         if (ns_max <= 16) return launch_chained(attn_combine_kernel<true, 16, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-        return launch_chained(attn_combine_kernel<true, 1 << 30, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        if (ns_max <= 32) return launch_chained(attn_combine_kernel<true, 32, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        return launch_chained(attn_combine_many_kernel<true, false>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
     }
     if (ns_max <= 4) return launch_chained(attn_combine_kernel<false, 4, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
     if (ns_max <= 16) return launch_chained(attn_combine_kernel<false, 16, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-    return launch_chained(attn_combine_kernel<false, 1 << 30, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+    if (ns_max <= 32) return launch_chained(attn_combine_kernel<false, 32, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+    return launch_chained(attn_combine_many_kernel<false, false>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
 }
 
 }  // namespace agx
