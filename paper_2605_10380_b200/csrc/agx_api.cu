@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <climits>
 #include <new>
 #include <vector>
 
@@ -38,7 +39,8 @@ struct agx_handle {
     int batch_stream_tokens; // total tokens of a batch's small blocks from which they all take the stream schedule (env AGX_BATCH_STREAM_TOKENS)
     bool longest_first;     // sequences of a launch ordered by decreasing context length (env AGX_LONGEST_FIRST=0: batch order)
     bool merge_sms;         // one-wave small-q launches leave SMs free for their merge kernel (env AGX_MERGE_SMS=0 turns it off)
-    bool cluster_merge;     // KV splits of the small-q kernel merged inside thread-block clusters where the batch allows (env AGX_CLUSTER_MERGE=0 turns it off)
+    int cluster_merge;      // KV splits of the small-q kernel merged inside thread-block clusters: 1 = where the batch allows and it is the faster merge,
+                            // 2 = wherever the batch allows (env AGX_CLUSTER_MERGE=1), 0 = never (AGX_CLUSTER_MERGE=0)
     int zero_copy;          // host steps: bit 0 = kernels read small pinned inputs, bit 1 = kernels write `out` into a pinned buffer (env AGX_ZERO_COPY, default 3)
     int stream_max_rows;    // blocks of up to this many rows per KV head may take the one-Q-tile schedule in 128-row chunks (env AGX_STREAM_MAX_ROWS)
     int stream_min_tokens;  // context length from which blocks of <= 32 rows take the tensor-core stream schedule (env AGX_STREAM_MIN_TOKENS; -1 = by block height)
@@ -223,6 +225,22 @@ int choose_split(const agx_handle* h, const SplitModel& md, const std::vector<in
     return best_tiles;
 }
 
+// Tokens per KV split (a multiple of `unit`) with which the sequences' items are one wave of `target` CTAs, at least about min_split.
+int one_wave_split(const agx_handle* h, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G, int rows_per_chunk, int unit, int min_split,
+                   int target, bool shrink) {
+    long long work = 0, base = 0;
+    auto items_of = [&](int s) { return (long long)h->cfg.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk); };
+    for (int s : seqs) { base += items_of(s); work += items_of(s) * (P[s] + Q[s]); }
+    const int even = round_up((work + target - 1) / target, unit);
+    // (splits only a little shorter than the minimum are taken where they are one wave: they fill more SMs)
+    int C = shrink && even < min_split && even * 20 >= min_split * 17 ? even : std::max(min_split, even);
+    for (;; C += unit) {
+        long long n = 0;
+        for (int s : seqs) n += items_of(s) * ((P[s] + Q[s] + C - 1) / C);
+        if (n <= std::max<long long>(target, base)) return C;
+    }
+}
+
 // Decide kernel kind, KV splits and partial slots for every sequence (host lengths only).
 agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, int pt_stride, Plan& plan) {
     const agx_config& c = h->cfg;
@@ -239,8 +257,8 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
     plan.total_rows = row0[B];
     // Blocks of at most 32 rows go to the warp-MMA kernel or to the one-Q-tile tensor-core schedule, all of a batch together: to the one whose
     // estimate is lower (SplitModel; for the warp-MMA kernel with 8-page stages, one CTA per SM, k tokens at 8 KV heads take 4.1 + 0.69 k up
-    // to 16 rows, max(8.8, 5.8 + 1.06 k) above).  What it decides against the fixed thresholds it replaces (24576 tokens in all; 7168 / 10240
-    // for one sequence): 32 decode blocks over 1000 tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over
+    // to 16 rows, 5.6 + 0.8 k above in splits that an SM holds whole, max(8.8, 5.8 + 1.06 k) otherwise).  What it decides against the fixed
+    // thresholds it replaces (24576 tokens in all; 7168 / 10240 for one sequence): 32 decode blocks over 1000 tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over
     // 20000 20.5 -> 17.5, 32 verify blocks over 1500 53 -> 43; 8 verify blocks over 8000 stay at 50 (55 the other way).
     double small_k = 0;
     int small_rows = 0;
@@ -266,11 +284,12 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             };
             const bool one = small_seqs.size() == 1;
             double warp_mma;
+            std::vector<int> mt1, mt2;
+            for (int s : small_seqs) (Q[s] * G <= 16 ? mt1 : mt2).push_back(s);
             if (one || small_k < 7.9) {
-                warp_mma = small_rows <= 16 ? 4.1 + 0.69 * small_k : std::max(8.8, 5.8 + 1.06 * small_k);
+                const bool whole = mt2.empty() || one_wave_split(h, mt2, P, Q, G, 32, 16, h->small_min_split, h->sm_count, true) <= kSwapMaxTokens;
+                warp_mma = small_rows <= 16 ? 4.1 + 0.69 * small_k : whole ? 5.6 + 0.8 * small_k : std::max(8.8, 5.8 + 1.06 * small_k);
             } else {
-                std::vector<int> mt1, mt2;
-                for (int s : small_seqs) (Q[s] * G <= 16 ? mt1 : mt2).push_back(s);
                 warp_mma = estimate(small4_model(h, 1), 16, mt1) + estimate(small4_model(h, 2), 32, mt2);
             }
             std::vector<int> all = wide_seqs;
@@ -318,22 +337,27 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         std::vector<long long> per_seq_items(seqs.size());
         if (k == KIND_SIMT) { unit = 64; min_split = 64; target = h->sm_count * 2; }
         else if (k == KIND_TILE || k == KIND_STREAM) { unit = 128; min_split = k == KIND_TILE ? 128 : 256; target = h->sm_count; }
-        else { unit = 16; min_split = h->small_min_split; target = h->sm_count * ((k == KIND_SMALL4 || small_kw == 8) ? 1 : 2); }
+        else { unit = 16; min_split = h->small_min_split; target = h->sm_count; }
         const int rows_per_chunk = (k == KIND_SIMT) ? 8 : (k == KIND_SMALL1) ? 16 : (k == KIND_SMALL2) ? 32 : (k == KIND_SMALL4) ? 64 : (k == KIND_STREAM) ? 128 : 256;
-        long long work = 0;
         for (size_t n = 0; n < seqs.size(); ++n) {
             const int s = seqs[n];
             const long long items = (long long)c.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk);
             per_seq_items[n] = items;
             base_items += items;
-            work += items * (P[s] + Q[s]);
         }
-        int C = std::max(min_split, round_up((work + target - 1) / target, unit));
-        // small-q kernel: when one wave of CTAs needs splits only a little shorter than the minimum, take them (the
-        // headline decode-verify shape then fills 144 SMs with 18 splits of 240 tokens instead of 136 with 17 of 256)
-        if (k != KIND_SIMT && k != KIND_TILE && k != KIND_STREAM && C == min_split &&
-            round_up((work + target - 1) / target, unit) * 20 >= min_split * 17)
-            C = round_up((work + target - 1) / target, unit);
+        const bool small_kind = k == KIND_SMALL1 || k == KIND_SMALL2;
+        int C = min_split, kw = k == KIND_SMALL4 ? 4 : small_kw;
+        if (k != KIND_TILE && k != KIND_STREAM && !(small_kind && kw == 4)) {
+            C = one_wave_split(h, seqs, P, Q, G, rows_per_chunk, unit, min_split, target, k != KIND_SIMT);
+            // several verify blocks whose splits no SM holds whole: two CTAs per SM with 4-page stages where the lengths are alike (7 x 1000
+            // tokens 14.3 -> 12.3 us, 8 x 900 14.3 -> 11.8, 2 x 3500 12.5 -> 11.4, 3700 + 3900 12.7 -> 12.3; but 1500 + 2500 + 3500 12.9 -> 13.4.
+            // Up to 16 rows: 7 x 1000 10.7 / 11.4, 8 x 900 10.8 / 10.2)
+            int longest = 0, shortest = INT_MAX;
+            for (int s : seqs) { longest = std::max(longest, P[s] + Q[s]); shortest = std::min(shortest, P[s] + Q[s]); }
+            if (k == KIND_SMALL2 && seqs.size() >= 2 && C > kSwapMaxTokens && longest < 2 * shortest && !h->small_kw) kw = 4;
+        }
+        // one CTA per SM that holds its split whole (agx_attn_swap.cu)
+        const bool whole = small_kind && kw == 8 && C <= kSwapMaxTokens;
         auto count_items = [&](int c_tokens) {
             long long items = 0;
             for (size_t n = 0; n < seqs.size(); ++n) {
@@ -350,17 +374,19 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             if (h->debug_plan)
                 fprintf(stderr, "agx plan: tile kernel, %lld row chunks, longest sequence %d tokens -> KV splits of %d tokens, %lld CTAs\n",
                         base_items, max_len, C, count_items(C));
-        } else if ((k == KIND_SMALL1 || k == KIND_SMALL2) && small_kw == 4) {
+        } else if (small_kind && kw == 4) {
             const SplitModel md = small4_model(h, k == KIND_SMALL1 ? 1 : 2);
             C = md.unit * choose_split(h, md, seqs, P, Q, G, rows_per_chunk, std::max(1, min_split / md.unit), base_items);
-        } else {
-            while (count_items(C) > std::max<long long>(target, base_items)) C += unit;
         }
         // ---- small-q kernel: when every sequence has one row chunk and the same number of KV splits (2..16), the
         //      splits of a (sequence, KV head) form a thread-block cluster and are merged through distributed shared
         //      memory: no partials in global memory, no combine launch.  17..20 splits are squeezed into 16.
+        //      Not where a CTA holds its split whole: a CTA that waits for its cluster keeps an SM from the next call, whose K/V then come late
+        //      (8 rows over 300 / 700 / 2000 tokens 8.3 / 8.7 / 7.2 us, through memory 6.9 / 7.1 / 6.3; 4 x 500 7.8 / 6.4; one row over 3 x 700
+        //      5.9 / 5.0).  One block of one row or two keeps the clusters: as fast, and a launch fewer for the host (6.0 / 6.2 us a call).
         int cluster = 0;
-        if ((k == KIND_SMALL1 || k == KIND_SMALL2 || k == KIND_SMALL4) && h->cluster_merge && seqs.size() <= (size_t)kMaxSeqs) {
+        bool memory_merge = false;   // (fp32 partials, as the clusters' are)
+        if ((small_kind || k == KIND_SMALL4) && h->cluster_merge && seqs.size() <= (size_t)kMaxSeqs) {
             int common = -1;
             bool ok = true;
             for (size_t n = 0; n < seqs.size() && ok; ++n) {
@@ -373,8 +399,11 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             }
             if (ok && common >= 2 && common <= 16) {
                 const int mt = k == KIND_SMALL1 ? 1 : k == KIND_SMALL2 ? 2 : 4;
-                const int fit = attn_small_max_clusters(mt, mt == 4 ? 4 : small_kw, common);
-                if (fit >= base_items) cluster = common;
+                const int fit = attn_small_max_clusters(mt, kw, common);
+                if (fit >= base_items) {
+                    memory_merge = whole && !(seqs.size() == 1 && Q[seqs[0]] <= 2) && h->cluster_merge != 2;
+                    if (!memory_merge) cluster = common;
+                }
                 if (h->debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
             }
         }
@@ -396,9 +425,9 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
         //      of them fit an SM.
         bool lean_merge = false;   // fp16 partials and the two-warp merge kernel (slower than fp32 partials and the four-warp
                                    // one where the attention grid fills every SM twice over, e.g. four verify blocks of 4096)
-        const bool small_one_per_sm = (k == KIND_SMALL1 || k == KIND_SMALL2 || k == KIND_SMALL4) && (k == KIND_SMALL4 || small_kw == 8);
+        const bool small_one_per_sm = k == KIND_SMALL4 || (small_kind && kw == 8);
         // (the one-Q-tile tensor-core schedule as well: a single long sequence is one wave of whole-SM CTAs too)
-        if (!cluster && (small_one_per_sm || k == KIND_STREAM) && seqs.size() <= (size_t)kMaxSeqs && h->merge_sms) {
+        if (!cluster && !memory_merge && (small_one_per_sm || k == KIND_STREAM) && seqs.size() <= (size_t)kMaxSeqs && h->merge_sms) {
             long long pairs = 0;
             for (int s : seqs) pairs += (long long)Q[s] * c.num_q_heads;
             for (;;) {
@@ -410,6 +439,7 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
                 if (reserve > h->sm_count / 8) break;   // a merge that large needs the whole device anyway
                 lean_merge = true;
                 if (items <= h->sm_count - reserve || items <= base_items) break;
+                if (whole && C + unit > kSwapMaxTokens) break;   // (6 x 1000 tokens, one row, 10.1 -> 8.1 us; 8 rows over 6700 12.7 -> 11.5)
                 C += unit;
             }
         }
@@ -422,7 +452,7 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
             ln.num_items = 0;
             ln.cluster = cluster;
             ln.lean_merge = lean_merge;
-            ln.kw = (k == KIND_SMALL4) ? 4 : small_kw;
+            ln.kw = kw;
             for (size_t n = a; n < std::min(seqs.size(), a + kMaxSeqs); ++n) {
                 const int s = seqs[n];
                 const int L = P[s] + Q[s];
@@ -533,7 +563,7 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     env = getenv("AGX_STREAM_MAX_ROWS");
     h->stream_max_rows = env ? atoi(env) : 384;
     env = getenv("AGX_CLUSTER_MERGE");
-    h->cluster_merge = !(env && atoi(env) == 0);
+    h->cluster_merge = !env ? 1 : atoi(env) ? 2 : 0;
     env = getenv("AGX_HOST_PIPELINE_ROWS");
     h->pipe_rows = env ? std::max(0, atoi(env)) : 384;   // measured on the long-context step: 256 / 384 / 512 / 768 / 1024 rows -> 1.54 / 1.43 / 1.57 / 1.56 / 1.72 ms
     h->pipe_in = h->pipe_out = nullptr;

@@ -35,3 +35,19 @@ def test_several_row_chunks():
     kp, vp = oracle_pools_after_append(w)
     ref, _ = oracle.attn_paged_batch(w.q_block, kp, vp, w.page_table, w.dtype, w.prefix_len, w.q_len, w.cu_q)
     check_attention(out, ref, "chunks")
+
+
+@pytest.mark.parametrize("q,lengths", [
+    (8, [6518]), (8, [6522]), (8, [6902]), (8, [6906]), (8, [7000]),   # 17 and 18 splits of 384 tokens, and the first that need longer ones
+    (1, [1000] * 6), (8, [1000] * 6), (8, [1000] * 7), (8, [3700, 3900]), (8, [1500, 2500, 3500]),   # one wave of 384 tokens or not, alike or ragged
+])
+def test_edge_of_whole_splits(q, lengths):
+    import oracle
+    from tests.gpu_util import DeviceBatch, check_attention, oracle_pools_after_append
+    w = W.make_attn_workload("edge", sum(lengths) + q, "bf16", 32, 8, 128, lengths, [q] * len(lengths), spare_pages=1)
+    b = DeviceBatch(w)
+    out, _ = b.attend_append()
+    assert b.status() == 0
+    kp, vp = oracle_pools_after_append(w)
+    ref, _ = oracle.attn_paged_batch(w.q_block, kp, vp, w.page_table, w.dtype, w.prefix_len, w.q_len, w.cu_q)
+    check_attention(out, ref, "edge")
