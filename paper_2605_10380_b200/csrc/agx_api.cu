@@ -407,6 +407,13 @@ agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, 
                 if (h->debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
             }
         }
+        // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, with fp32 partials, are faster than 17 to 24 with SMs left to
+        // the merge of fp16 rows (32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
+        // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).
+        if (whole && !cluster && !memory_merge && seqs.size() == 1 && h->merge_sms && (k == KIND_SMALL2 || count_items(C) * 2 > h->sm_count)) {
+            const int L = P[seqs[0]] + Q[seqs[0]], longer = std::max(320, round_up((L + 15) / 16, unit));
+            if ((L + C - 1) / C > 16 && longer <= kSwapMaxTokens) { C = std::max(C, longer); memory_merge = true; }
+        }
         // ---- fp32-arithmetic kernel: up to 16 splits of an item form a cluster, as many for all sequences; more leave partials
         if (k == KIND_SIMT && h->cluster_merge) {
             int max_len = 0;
