@@ -123,14 +123,25 @@ __device__ __forceinline__ uint64_t add2p(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ uint64_t mul2p(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 // 2^x for a packed pair on the FMA pipes instead of the special-function unit: n = round(x) by the
 // 1.5 * 2^23 trick, f = x - n in [-0.5, 0.5], 2^f by a polynomial of degree 5 fitted (Lawson's
 // iteration) to minimise the maximum relative error on that interval (2.1e-7 evaluated in fp32, no more than the
-// special-function unit's), then n is added into the exponent field.  x is clamped at -126 so the exponent cannot wrap.
+// special-function unit's), times 2^n.  As with that unit a NaN stays a NaN and -inf, a masked score, gives exactly 0: x is clamped at -127
+// by a maximum that passes NaN on, and the exponent field of 2^-127 is 0.
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
 __device__ __forceinline__ void ex2_poly2(uint64_t x, float& p0, float& p1) {
     float x0, x1;
     upk2(x, x0, x1);
-    x = pk2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    x = pk2(max_nan(x0, -127.f), max_nan(x1, -127.f));
     const uint64_t magic = pk2(12582912.f, 12582912.f), neg_magic = pk2(-12582912.f, -12582912.f);
     const uint64_t t = add2p(x, magic);
     const uint64_t n = add2p(t, neg_magic);
@@ -141,11 +152,9 @@ __device__ __forceinline__ void ex2_poly2(uint64_t x, float& p0, float& p1) {
     q = fma2p(q, f, c2(2.40221202e-1f));
     q = fma2p(q, f, c2(6.93146944e-1f));
     q = fma2p(q, f, c2(1.00000012f));
-    float q0, q1, t0, t1;
-    upk2(q, q0, q1);
-    upk2(t, t0, t1);
-    p0 = __int_as_float(__float_as_int(t0) * 8388608 + __float_as_int(q0));
-    p1 = __int_as_float(__float_as_int(t1) * 8388608 + __float_as_int(q1));
+    float t0, t1;
+    upk2(t, t0, t1);   // (the low bits of t are n: shifted into the exponent field, on top of that of 1.0)
+    upk2(mul2p(q, pk2(__int_as_float(__float_as_int(t0) * 8388608 + 0x3F800000), __int_as_float(__float_as_int(t1) * 8388608 + 0x3F800000))), p0, p1);
 }
 __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1) {
     upk2(add2p(pk2(d0, d1), pk2(a0, a1)), d0, d1);
