@@ -31,9 +31,10 @@ struct SimtSmem {
     float k[kT][D + 4];        // (a row's 16-byte units start four banks after the row's before it: conflict-free)
     float v[kT][D];
     float s[kR][kT];
+    float o[kR][D];            // the split's rows, read by the cluster's other CTAs
     float corr[kR];
     float2 ml[kR];
-    float o[kR][D];            // the split's rows, read by the cluster's other CTAs
+    int odd;                   // != 0: V of the block holds a value that is not finite
 };
 
 // Four elements of a row at element offset `at` as floats.
@@ -49,6 +50,17 @@ template <bool kBf16>
 __device__ __forceinline__ void store4(void* base, long long at, float4 v) {
     if (kBf16) *(uint2*)((__nv_bfloat16*)base + at) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
     else *(float4*)((float*)base + at) = v;
+}
+
+// The tile's products where V holds values that are not finite: a row stops at its last visible token.  Out of line, so that the kernel's
+// instructions stay in one piece (inline it cost every launch 0.25 us).
+template <int D>
+__device__ __noinline__ void add_visible(const SimtSmem<D>& sm, float (&acc)[kR][D / 32], int t0, int P, int q, int row0, int G) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int t = warp * 8; t < warp * 8 + 8; ++t)
+        for (int r = 0; r < kR; ++r)
+            if (t0 + t <= P + min((row0 + r) / G, q - 1))
+                for (int c = 0; c < D / 32; ++c) acc[r][c] += sm.s[r][t] * sm.v[t][c * 32 + lane];
 }
 
 }  // namespace
@@ -105,6 +117,8 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
     const int st = tid & (kT - 1), sr = (tid / kT) * 2;        // this thread's token and first row in the scoring step
     const int lim0 = P + min((row0 + sr) / G, q - 1), lim1 = P + min((row0 + sr + 1) / G, q - 1);
 
+    const int hidden = P + row0 / G + 1;                       // the first token that not every row sees
+    if (tid == 0) sm.odd = 0;
     for (int t0 = tok_begin; t0 < tok_end; t0 += kT) {
         float4 kv[2][kPer];
 #pragma unroll
@@ -132,6 +146,13 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             const int u = tid + j * kThreads;
             *(float4*)&sm.k[u / kUnits][(u % kUnits) * 4] = kv[0][j];
             *(float4*)&sm.v[u / kUnits][(u % kUnits) * 4] = kv[1][j];
+        }
+        if (t0 + kT > hidden) {   // (a weight of 0 does not hide a value that is not finite from a row that must not see it)
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const float4 v = kv[1][j];
+                if (v.x * 0.f + v.y * 0.f + v.z * 0.f + v.w * 0.f != 0.f) sm.odd = 1;
+            }
         }
         __syncthreads();
         if (t0 + kT < tok_end) {                               // page ids of the next tile
@@ -176,6 +197,19 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             w1[r] = *(const float4*)&sm.s[r][warp * 8 + 4];
 #pragma unroll
             for (int c = 0; c < kCols; ++c) acc[r][c] *= corr;
+        }
+        if (__builtin_expect(sm.odd, 0)) {
+            float a[kR][kCols];
+#pragma unroll
+            for (int r = 0; r < kR; ++r)
+#pragma unroll
+                for (int c = 0; c < kCols; ++c) a[r][c] = acc[r][c];
+            add_visible(sm, a, t0, P, q, row0, G);
+#pragma unroll
+            for (int r = 0; r < kR; ++r)
+#pragma unroll
+                for (int c = 0; c < kCols; ++c) acc[r][c] = a[r][c];
+            continue;
         }
 #pragma unroll
         for (int t = 0; t < 8; ++t) {

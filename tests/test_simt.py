@@ -34,3 +34,23 @@ def test_simt_kernel_against_the_oracle(dtype, d, hq, hkv, merge, monkeypatch):
         assert np.max(np.abs(lse - ref_lse)) < 1e-4
         if dtype == "f32":
             assert np.max(np.abs(out - ref)) < 2e-4, (P, q)   # (2 x 5e-5 x max |v|)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("dtype,d", [("f32", 64), ("f32", 128), ("bf16", 64)])
+def test_what_a_row_does_not_see_does_not_reach_it(dtype, d, value):
+    """V of the block's last token: earlier rows keep every bit, whichever tile and split the token sits in."""
+    import torch
+
+    from tests.gpu_util import DeviceBatch
+    for P, q in ((0, 9), (60, 5), (64, 3), (1000, 12), (2500, 2)):
+        outs = []
+        for x in (1.0, value):
+            b = DeviceBatch(W.make_attn_workload("hidden", P + q, dtype, 8, 2, d, [P], [q], spare_pages=1))
+            b.v_new[q - 1] = x
+            b.attend_append()
+            assert b.status() == 0
+            outs.append((b.out, b.lse))
+        assert bool(torch.isfinite(outs[1][0][:q - 1]).all()), (P, q)
+        assert torch.equal(outs[0][0][:q - 1], outs[1][0][:q - 1]) and torch.equal(outs[0][1], outs[1][1])
+        assert not bool(torch.isfinite(outs[1][0][q - 1]).any())
