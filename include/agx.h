@@ -162,7 +162,9 @@ AGX_API agx_status agx_attn_prefixed(agx_handle* handle, const void* q_block, co
  * pages on the side.
  *   k_new, v_new : device, [total_q][num_kv_heads][head_dim], 16-byte aligned (rows in the order of q_block)
  *   k_pool, v_pool : device pools (written, then read); the other arguments as for agx_attn_prefixed
- * Errors: those of agx_attn_prefixed; a page id outside [0, num_pages) sets AGX_DEV_BAD_PAGE and the row is not written.
+ * Errors: those of agx_attn_prefixed; a page id outside [0, num_pages) sets AGX_DEV_BAD_PAGE and the row is not
+ * written.  The block of that call attends to the row all the same, since it takes it from k_new / v_new; only calls whose page ids are
+ * valid have the results of the two calls.
  */
 AGX_API agx_status agx_attn_prefixed_append(agx_handle* handle, const void* q_block, const void* k_new,
                                             const void* v_new, void* k_pool, void* v_pool, int64_t num_pages,
