@@ -35,7 +35,7 @@ struct PyFailed : std::exception {};   // a Python error is set
 // Address of a torch tensor's or a numpy array's first element; NULL for None.
 void* address(PyObject* o) {
     if (o == Py_None) return nullptr;
-    if (THPVariable_Check(o)) return const_cast<void*>(THPVariable_Unpack(o).const_data_ptr());
+    if (THPVariable_Check(o)) return THPVariable_Unpack(o).mutable_data_ptr();   // (as Tensor.data_ptr(): a copy-on-write tensor gets its own memory first)
     Py_buffer view;
     if (PyObject_GetBuffer(o, &view, PyBUF_STRIDED_RO) != 0) throw PyFailed();
     void* p = view.buf;
