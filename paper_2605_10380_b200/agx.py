@@ -175,7 +175,7 @@ def _binding():
         spec = importlib.util.spec_from_file_location("agx_torch", path)
         native = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(native)
-        native.bind(_h_i32, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in (
+        native.bind(_h_i32, np.ndarray, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in (
             "agx_kv_append", "agx_attn_prefixed", "agx_attn_prefixed_append", "agx_accept_greedy", "agx_verify_step_host",
             "agx_verify_step_host_enqueue", "agx_ngram_build", "agx_ngram_draft", "agx_kv_copy_pages")))
         _native = native
@@ -276,9 +276,7 @@ class Handle:
     # -- agx_attn_prefixed_append
     def attn_prefixed_append(self, q_block, k_new, v_new, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse=None,
                              workspace=None, stream=None):
-        if k_new is None:   # (None there would select the call without an append)
-            raise AgxError(-1, "agx_attn_prefixed_append", "null pointer")
-        st = self._n.attn(self._p, q_block, k_new, v_new, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse, workspace, stream)
+        st = self._n.attn_append(self._p, q_block, k_new, v_new, k_pool, v_pool, page_table, h_prefix_len, h_q_len, out, lse, workspace, stream)
         if st:
             self._check(st, "agx_attn_prefixed_append")
 
