@@ -167,7 +167,7 @@ def _binding():
     the functions of ``load()``'s library; raises if it was not built."""
     global _native
     if _native is None:
-        import torch  # noqa: F401  (its libraries have to be in the process first)
+        import torch  # (its libraries have to be in the process first)
         lib = load()
         path = Path(__file__).resolve().parent / "lib" / "agx_torch.so"
         if not path.exists():
@@ -175,6 +175,9 @@ def _binding():
         spec = importlib.util.spec_from_file_location("agx_torch", path)
         native = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(native)
+        if native.torch_version != torch.__version__.split("+")[0]:   # (it uses torch's C++ classes)
+            raise RuntimeError(f"{path} was built with torch {native.torch_version}, this is {torch.__version__}: build the library again "
+                               "(python -m paper_2605_10380_b200.build)")
         native.bind(_h_i32, np.ndarray, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in (
             "agx_kv_append", "agx_attn_prefixed", "agx_attn_prefixed_append", "agx_accept_greedy", "agx_verify_step_host",
             "agx_verify_step_host_enqueue", "agx_ngram_build", "agx_ngram_draft", "agx_kv_copy_pages")))

@@ -57,6 +57,18 @@ def _binding_command(out: Path):
             str(CSRC / "agx_torch.cpp"), "-o", str(out), f"-L{base / 'lib'}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
+def _binding_stamp() -> str:
+    """What the argument-marshalling module is tied to besides its sources."""
+    import torch
+    return "\n".join([torch.__version__, sys.version, *_binding_command(BINDING)])
+
+
+def _binding_stale() -> bool:
+    stamp = OBJ_DIR / "agx_torch.stamp"
+    return (_stale(BINDING, [CSRC / "agx_torch.cpp", ROOT / "include" / "agx.h"]) or not stamp.exists()
+            or stamp.read_text() != _binding_stamp())
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
     srcs = sources()
     headers = list(CSRC.glob("*.cuh")) + list((ROOT / "include").glob("*.h"))
@@ -74,7 +86,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
             jobs.append(cmd)
 
     binding_tmp = BINDING.with_suffix(f".tmp{os.getpid()}.so")
-    if force or _stale(BINDING, [CSRC / "agx_torch.cpp", ROOT / "include" / "agx.h"]):
+    if force or _binding_stale():
         jobs.append(_binding_command(binding_tmp))
 
     def run(cmd):
@@ -88,6 +100,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         list(ex.map(run, jobs))
     if binding_tmp.exists():
         os.replace(binding_tmp, BINDING)
+        (OBJ_DIR / "agx_torch.stamp").write_text(_binding_stamp())
     objs = [OBJ_DIR / (s.stem + ".o") for s in srcs]
     if force or jobs or _stale(OUT, objs):
         tmp = OUT.with_suffix(f".tmp{os.getpid()}.so")

@@ -8,6 +8,7 @@
 // No arithmetic and no state beyond the addresses of the C functions, which agx.py passes in once (bind), so that there
 // is one copy of the library in the process.  The GIL is released around every C call, as ctypes does.
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/version.h>
 
 #include <c10/cuda/CUDAStream.h>
 
@@ -263,4 +264,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "agx_torch", nullptr, -1, methods, 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_agx_torch() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit_agx_torch() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "torch_version", TORCH_VERSION) != 0) Py_CLEAR(m);   // (agx.py does not use it with another torch)
+    return m;
+}

@@ -120,3 +120,15 @@ def test_addresses_of_host_arrays(calls, array):
     t = _tensors()
     native.step(0, False, t["kp"], t["vp"], t["table"], [1], [1], array, t["k"], t["v"], None, 0, 9, 0, None, t["out"], None, None, None, t["ws"], 0)
     assert (seen[0][1][9] or 0) == array.ctypes.data
+
+
+def test_the_module_belongs_to_one_version_of_torch(monkeypatch):
+    """It uses torch's C++ classes: another torch makes it stale for the build, and unusable until it is built again."""
+    from paper_2605_10380_b200 import build
+    agx._binding()
+    assert not build._binding_stale()
+    monkeypatch.setattr(torch, "__version__", "1.2.3+cu99")
+    assert build._binding_stale()
+    monkeypatch.setattr(agx, "_native", None)
+    with pytest.raises(RuntimeError, match="1.2.3"):
+        agx._binding()
