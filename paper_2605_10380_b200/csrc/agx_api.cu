@@ -1,4 +1,4 @@
-// C ABI of the agx library: argument checks, launch planning, dispatch.  No kernel lives here.
+// C ABI of the agx library: argument checks, dispatch.  No kernel lives here; what is launched is planned in agx_plan.cu.
 #include <stdarg.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -12,6 +12,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "agx_internal.cuh"
+#include "agx_plan.cuh"
 
 namespace {
 // An NVTX range around every call that enqueues work: a timeline tool shows the library's calls by name; with no tool
@@ -20,7 +21,6 @@ struct CallRange {
     explicit CallRange(const char* name) { nvtxRangePushA(name); }
     ~CallRange() { nvtxRangePop(); }
 };
-struct Plan;
 }  // namespace
 
 struct agx_handle {
@@ -32,18 +32,8 @@ struct agx_handle {
     unsigned int* d_ticket; // ticket counter of the accept kernel (self-resetting)
     unsigned long long* d_row_keys;   // one argmax key per logits row of the accept kernel (all zero between launches)
     int last_launches;
-    int small_min_split;    // tokens; tuning knob (env AGX_SMALL_MIN_SPLIT)
-    int force_mma_sync;     // route large q through the mma.sync kernel (env AGX_FORCE_MMA_SYNC)
-    int debug_plan;         // print launch plans to stderr (env AGX_DEBUG_PLAN)
-    int small_kw;           // pages per pipeline stage of the warp-MMA kernel: 4, 8, or 0 = chosen per batch (env AGX_SMALL_KW)
-    int batch_stream_tokens; // total tokens of a batch's small blocks from which they all take the stream schedule (env AGX_BATCH_STREAM_TOKENS)
-    bool longest_first;     // sequences of a launch ordered by decreasing context length (env AGX_LONGEST_FIRST=0: batch order)
-    bool merge_sms;         // one-wave small-q launches leave SMs free for their merge kernel (env AGX_MERGE_SMS=0 turns it off)
-    int cluster_merge;      // KV splits of the small-q kernel merged inside thread-block clusters: 1 = where the batch allows and it is the faster merge,
-                            // 2 = wherever the batch allows (env AGX_CLUSTER_MERGE=1), 0 = never (AGX_CLUSTER_MERGE=0)
     int zero_copy;          // host steps: bit 0 = kernels read small pinned inputs, bit 1 = kernels write `out` into a pinned buffer (env AGX_ZERO_COPY, default 3)
-    int stream_max_rows;    // blocks of up to this many rows per KV head may take the one-Q-tile schedule in 128-row chunks (env AGX_STREAM_MAX_ROWS)
-    int stream_min_tokens;  // context length from which blocks of <= 32 rows take the tensor-core stream schedule (env AGX_STREAM_MIN_TOKENS; -1 = by block height)
+    agx::PlanConfig plan;   // what the planner needs to know, and its knobs
     long long wait_limit_cycles;   // AGX_OPT_WAIT_LIMIT_CYCLES
     int early_prefix;       // AGX_OPT_EARLY_PREFIX_LOADS
     int drop_stage;         // AGX_OPT_TEST_DROP_STAGE (-1 = none)
@@ -54,7 +44,7 @@ struct agx_handle {
     cudaStream_t pipe_in, pipe_out;
     std::vector<cudaEvent_t> pipe_events;
     // the launch plan of the last batch seen: the layers of a model step all ask for the same one
-    Plan* plan_cache;
+    agx::Plan* plan_cache;
     std::vector<int32_t> plan_P, plan_Q;
     char err[512];
 };
@@ -79,428 +69,7 @@ agx_status cuda_fail(agx_handle* h, cudaError_t e, const char* what) {
 
 inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
-inline int round_up(long long v, int m) { return (int)((v + m - 1) / m * m); }
 inline int elem_size(int dtype) { return dtype == AGX_BF16 ? 2 : 4; }
-
-enum Kind { KIND_SMALL1 = 0, KIND_SMALL2, KIND_SMALL4, KIND_STREAM, KIND_TILE, KIND_SIMT, KIND_COUNT };
-
-struct Launch {
-    Kind kind;
-    int total_rows;  // sum of q_len over the launch's sequences
-    int num_items;
-    int kw;          // small-q kernel: pages per pipeline stage (KV groups), 4 or 8
-    int cluster;     // > 1: CTAs per cluster = KV splits of every sequence of the launch, merged in-kernel (no partials)
-    bool lean_merge; // small-q kernel or one-Q-tile schedule: fp16 partials, merged by the two-warp merge kernel on SMs left out of the attention grid
-    std::vector<SeqPlan> seqs;
-};
-
-struct Plan {
-    std::vector<Launch> launches;
-    long long part_entries = 0;  // (row, head, split) partial slots
-    bool any_split = false;
-    bool tensor_core = false;    // a launch of the tensor-core kernel is among them
-    long long total_rows = 0;    // block rows of the whole batch
-};
-
-// What a launch of one of the attention kernels costs (us), fitted to sweeps over split lengths and batches (GQA 32/8; worst errors 2-3 us at
-// 20-130): CTAs go to the SMs (or to their halves) longest first; a step of `unit` tokens takes per_add + max(per_min, per_busy * A) while
-// A CTAs are at work (per_busy: HBM, or the mma.sync rate, shared by all of them), the start and end of the first CTA `base`, those of
-// others behind it on an SM `overhead` steps.
-struct SplitModel {
-    int unit, slots, overhead;
-    double base, per_add, per_min, per_busy;
-    double merge, merge_mb, merge_mb_beyond_16;   // merge launch, per MB of partials up to 16 (they stay in L2) and beyond
-    int part_row_bytes;
-    bool lean;              // one-wave launches with few (row, head) pairs leave SMs to their merge kernel: 1 + 0.2 per MB
-};
-// It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
-// 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
-SplitModel tile_model(const agx_handle* h) { return {128, h->sm_count, 3, 5.7, 0, 1.9, 0, 2.2, 0.38, 0.3, 264, false}; }
-// (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them)
-SplitModel stream_model(const agx_handle* h, bool wide) {
-    return {128, h->sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, true};
-}
-// warp-MMA kernel with 4-page stages, two CTAs per SM: HBM-bound with one 16-row tile, bounded by its own chain with two (mma.sync)
-SplitModel small4_model(const agx_handle* h, int mt) {
-    return {64, 2 * h->sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, false};
-}
-
-// Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time.
-int choose_split(const agx_handle* h, const SplitModel& md, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
-                 int rows_per_chunk, int min_tiles, long long base_items, double* estimate = nullptr) {
-    const int sms = md.slots, hkv = h->cfg.num_kv_heads, kOverhead = md.overhead;
-    int max_tiles = 1;
-    long long pairs = 0;      // (row, query head)
-    bool equal = true;
-    for (int s : seqs) {
-        const int lt = (P[s] + Q[s] + md.unit - 1) / md.unit;
-        equal &= s == seqs[0] || lt == max_tiles;
-        pairs += (long long)Q[s] * h->cfg.num_q_heads;
-        max_tiles = std::max(max_tiles, lt);
-    }
-    struct Cand { int tiles; double bound, merge; };
-    std::vector<Cand> cands;
-    // items of a candidate, by tile count: (count, tiles)
-    std::vector<std::pair<int, long long>> items;
-    auto collect = [&](int split_tiles, long long& sum, long long& count, int& longest, double& part_mb) {
-        items.clear();
-        sum = count = 0; longest = 0; part_mb = 0;
-        for (int s : seqs) {
-            const int L = P[s] + Q[s], lt = (L + md.unit - 1) / md.unit, ns = (lt + split_tiles - 1) / split_tiles, per = (lt + ns - 1) / ns;
-            const int chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
-            if (ns > 1) part_mb += (double)Q[s] * h->cfg.num_q_heads * ns * md.part_row_bytes * 1e-6;
-            auto add = [&](int vis, long long n) {   // n (chunk, head) pairs that see `vis` tiles
-                const int full = vis / per, rest = vis - full * per;
-                if (full) items.push_back({per, n * full});
-                if (rest) items.push_back({rest, n});
-                sum += n * (vis + kOverhead * (full + (rest != 0)));
-                count += n * (full + (rest != 0));
-                longest = std::max(longest, full ? per : rest);
-            };
-            if (chunks <= 32) {
-                for (int rc = 0; rc < chunks; ++rc) add((P[s] + std::min(Q[s] - 1, ((rc + 1) * rows_per_chunk - 1) / G) + md.unit) / md.unit, hkv);
-            } else {   // in 32 groups of chunks with the tiles of the group's last one
-                for (int k = 0; k < 32; ++k) {
-                    const int rc0 = (int)((long long)chunks * k / 32), rc1 = (int)((long long)chunks * (k + 1) / 32);
-                    add((P[s] + std::min(Q[s] - 1, (rc1 * rows_per_chunk - 1) / G) + md.unit) / md.unit, (long long)hkv * (rc1 - rc0));
-                }
-            }
-        }
-    };
-    const int n_max = (int)std::min<long long>((max_tiles + min_tiles - 1) / min_tiles, std::max<long long>(32, 2 * sms / std::max<long long>(base_items, 1)));
-    for (int n = 1, last = 0; n <= n_max; ++n) {
-        const int t = std::max(min_tiles, (max_tiles + n - 1) / n);
-        if (t == last) continue;
-        last = t;
-        long long sum, count;
-        int longest;
-        double mb;
-        collect(t, sum, count, longest, mb);
-        const double load = std::max<double>((double)sum / sms, longest + kOverhead);
-        Cand cd;
-        cd.tiles = t;
-        cd.merge = mb == 0 ? 0 : md.lean && count <= sms * 15 / 16 && pairs <= 3 * sms ? 1.0 + 0.2 * mb
-                   : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
-                   : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
-        cd.bound = md.base + cd.merge + std::max((load - kOverhead) * (md.per_add + md.per_min),
-                                                 (sum - (double)kOverhead * std::min<long long>(count, sms)) * md.per_busy);
-        cands.push_back(cd);
-    }
-    std::stable_sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
-    double best = -1;
-    int best_tiles = max_tiles;
-    std::vector<int> load;
-    for (const Cand& cd : cands) {
-        if (best >= 0 && cd.bound >= best) break;   // (bounds ascend)
-        long long sum, count;
-        int longest;
-        double mb, t;
-        collect(cd.tiles, sum, count, longest, mb);
-        // load[x]: SMs with x tiles (and starts) so far; an item goes to an SM with the least
-        std::sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-        load.assign((size_t)(sum / sms) + longest + kOverhead + 2, 0);
-        load[0] = sms;
-        size_t lo = 0, hi = 0;
-        for (const auto& it : items)
-            for (long long left = it.second; left > 0;) {
-                while (load[lo] == 0) ++lo;
-                const int k = (int)std::min<long long>(load[lo], left);
-                load[lo] -= k;
-                load[lo + it.first + kOverhead] += k;
-                hi = std::max(hi, lo + it.first + kOverhead);
-                left -= k;
-            }
-        t = md.base;
-        size_t prev = kOverhead;
-        int busy = sms;
-        for (size_t x = 0; x <= hi; ++x) {
-            if (load[x] == 0) continue;
-            if (x > prev) { t += (x - prev) * (md.per_add + std::max(md.per_min, md.per_busy * busy)); prev = x; }
-            busy -= load[x];
-        }
-        t += cd.merge;
-        if (best < 0 || t < best) { best = t; best_tiles = cd.tiles; }
-    }
-    if (estimate) *estimate = best;
-    return best_tiles;
-}
-
-// Tokens per KV split (a multiple of `unit`) with which the sequences' items are one wave of `target` CTAs, at least about min_split.
-int one_wave_split(const agx_handle* h, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G, int rows_per_chunk, int unit, int min_split,
-                   int target, bool shrink) {
-    long long work = 0, base = 0;
-    auto items_of = [&](int s) { return (long long)h->cfg.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk); };
-    for (int s : seqs) { base += items_of(s); work += items_of(s) * (P[s] + Q[s]); }
-    const int even = round_up((work + target - 1) / target, unit);
-    // (splits only a little shorter than the minimum are taken where they are one wave: they fill more SMs)
-    int C = shrink && even < min_split && even * 20 >= min_split * 17 ? even : std::max(min_split, even);
-    for (;; C += unit) {
-        long long n = 0;
-        for (int s : seqs) n += items_of(s) * ((P[s] + Q[s] + C - 1) / C);
-        if (n <= std::max<long long>(target, base)) return C;
-    }
-}
-
-// Decide kernel kind, KV splits and partial slots for every sequence (host lengths only).
-agx_status build_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, int pt_stride, Plan& plan) {
-    const agx_config& c = h->cfg;
-    const int G = c.num_q_heads / c.num_kv_heads;
-    std::vector<int> row0(B + 1, 0);
-    for (int s = 0; s < B; ++s) {
-        if (Q[s] < 1) return fail(h, AGX_E_INVAL, "q_len[%d] = %d < 1", s, Q[s]);
-        if (P[s] < 0) return fail(h, AGX_E_INVAL, "prefix_len[%d] = %d < 0", s, P[s]);
-        if (pt_stride >= 0 && (long long)P[s] + Q[s] > (long long)pt_stride * kPage)
-            return fail(h, AGX_E_RANGE, "sequence %d: %d + %d tokens exceed the page table (%d pages)", s, P[s], Q[s], pt_stride);
-        if ((long long)row0[s] + Q[s] > (1 << 30)) return fail(h, AGX_E_RANGE, "too many rows");
-        row0[s + 1] = row0[s] + Q[s];
-    }
-    plan.total_rows = row0[B];
-    // Blocks of at most 32 rows go to the warp-MMA kernel or to the one-Q-tile tensor-core schedule, all of a batch together: to the one whose
-    // estimate is lower (SplitModel; for the warp-MMA kernel with 8-page stages, one CTA per SM, k tokens at 8 KV heads take 4.1 + 0.69 k up
-    // to 16 rows, 5.6 + 0.8 k above in splits that an SM holds whole, max(8.8, 5.8 + 1.06 k) otherwise).  What it decides against the fixed
-    // thresholds it replaces (24576 tokens in all; 7168 / 10240 for one sequence): 32 decode blocks over 1000 tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over
-    // 20000 20.5 -> 17.5, 32 verify blocks over 1500 53 -> 43; 8 verify blocks over 8000 stay at 50 (55 the other way).
-    double small_k = 0;
-    int small_rows = 0;
-    std::vector<int> small_seqs, wide_seqs;   // up to 32 rows | others that take the schedule in any case
-    const bool scalar_path = c.dtype == AGX_F32 || c.head_dim != 128;   // fp32 pools, and bf16 with head_dim 64
-    if (!scalar_path)
-        for (int s = 0; s < B; ++s) {
-            const int rows = Q[s] * G;
-            if (rows <= 32) { small_k += (P[s] + Q[s]) * 1e-3 * c.num_kv_heads / 8; small_rows = std::max(small_rows, rows); small_seqs.push_back(s); }
-            else if (rows <= h->stream_max_rows) wide_seqs.push_back(s);
-        }
-    bool batch_streams = false;
-    if (!small_seqs.empty() && h->stream_min_tokens < 0) {
-        if (h->batch_stream_tokens >= 0) {
-            batch_streams = small_seqs.size() >= 2 && small_k * 1e3 >= h->batch_stream_tokens;
-        } else {
-            auto estimate = [&](const SplitModel& md, int chunk, const std::vector<int>& seqs) {
-                double t = 0;
-                long long items = 0;
-                for (int s : seqs) items += (long long)c.num_kv_heads * ((Q[s] * G + chunk - 1) / chunk);
-                if (!seqs.empty()) choose_split(h, md, seqs, P, Q, G, chunk, md.unit == 64 ? 4 : 2, items, &t);
-                return t;
-            };
-            const bool one = small_seqs.size() == 1;
-            double warp_mma;
-            std::vector<int> mt1, mt2;
-            for (int s : small_seqs) (Q[s] * G <= 16 ? mt1 : mt2).push_back(s);
-            if (one || small_k < 7.9) {
-                const bool whole = mt2.empty() || one_wave_split(h, mt2, P, Q, G, 32, 16, h->small_min_split, h->sm_count, true) <= kSwapMaxTokens;
-                warp_mma = small_rows <= 16 ? 4.1 + 0.69 * small_k : whole ? 5.6 + 0.8 * small_k : std::max(8.8, 5.8 + 1.06 * small_k);
-            } else {
-                warp_mma = estimate(small4_model(h, 1), 16, mt1) + estimate(small4_model(h, 2), 32, mt2);
-            }
-            std::vector<int> all = wide_seqs;
-            all.insert(all.end(), small_seqs.begin(), small_seqs.end());
-            // (with one 16-row tile the warp-MMA kernel was never more than 2 % slower than the schedule, also where the estimates tie)
-            if (!one && small_k >= 7.9 && small_rows <= 16) warp_mma *= 0.87;
-            const SplitModel sm = stream_model(h, !wide_seqs.empty());
-            batch_streams = estimate(sm, 128, all) < warp_mma + estimate(sm, 128, wide_seqs);
-        }
-    }
-    long long warp_mma_tokens = 0;
-    int warp_mma_seqs = 0;
-    std::vector<int> groups[KIND_COUNT];
-    for (int s = 0; s < B; ++s) {
-        Kind k;
-        if (scalar_path) k = KIND_SIMT;
-        else {
-            const int rows = Q[s] * G;
-            const bool tile_ok = !h->force_mma_sync;
-            // up to 128 rows: one Q tile per CTA, KV tiles alternating between two softmax warpgroups (HBM-bound
-            // streaming on the tcgen05 pipe); blocks of at most 32 rows over short contexts stay with the warp-MMA
-            // kernel, whose fixed costs are lower (none above 32 rows)
-            const bool forced = h->stream_min_tokens >= 0 && P[s] + Q[s] >= h->stream_min_tokens;
-            if (tile_ok && rows <= h->stream_max_rows && (rows > 32 || batch_streams || forced)) k = KIND_STREAM;
-            else if (rows <= 16) k = KIND_SMALL1;
-            else if (rows <= 32) k = KIND_SMALL2;
-            else if (rows <= kSmallRowsMax || h->force_mma_sync) k = KIND_SMALL4;
-            else k = KIND_TILE;
-            if (k == KIND_SMALL1 || k == KIND_SMALL2) { warp_mma_tokens += P[s] + Q[s]; ++warp_mma_seqs; }
-        }
-        groups[k].push_back(s);
-    }
-    const int small_kw = h->small_kw ? h->small_kw : (warp_mma_seqs >= 2 && warp_mma_tokens * c.num_kv_heads / 8 >= 7900) ? 4 : 8;
-    // Work items are handed to the SMs in launch order: the sequences with the longest contexts go first, so that the
-    // longest items of a ragged batch are not the ones left over for the last wave (env AGX_LONGEST_FIRST=0 keeps the batch order).
-    if (h->longest_first)
-        for (int k = 0; k < KIND_COUNT; ++k)
-            std::stable_sort(groups[k].begin(), groups[k].end(), [&](int a, int b) { return P[a] + Q[a] > P[b] + Q[b]; });
-    for (int k = 0; k < KIND_COUNT; ++k) {
-        const std::vector<int>& seqs = groups[k];
-        if (seqs.empty()) continue;
-        // ---- choose the split length C (tokens) so that one wave of CTAs covers the group
-        int unit, min_split, target;
-        long long base_items = 0;  // items per split, summed over sequences
-        std::vector<long long> per_seq_items(seqs.size());
-        if (k == KIND_SIMT) { unit = 64; min_split = 64; target = h->sm_count * 2; }
-        else if (k == KIND_TILE || k == KIND_STREAM) { unit = 128; min_split = k == KIND_TILE ? 128 : 256; target = h->sm_count; }
-        else { unit = 16; min_split = h->small_min_split; target = h->sm_count; }
-        const int rows_per_chunk = (k == KIND_SIMT) ? 8 : (k == KIND_SMALL1) ? 16 : (k == KIND_SMALL2) ? 32 : (k == KIND_SMALL4) ? 64 : (k == KIND_STREAM) ? 128 : 256;
-        for (size_t n = 0; n < seqs.size(); ++n) {
-            const int s = seqs[n];
-            const long long items = (long long)c.num_kv_heads * ((Q[s] * G + rows_per_chunk - 1) / rows_per_chunk);
-            per_seq_items[n] = items;
-            base_items += items;
-        }
-        const bool small_kind = k == KIND_SMALL1 || k == KIND_SMALL2;
-        int C = min_split, kw = k == KIND_SMALL4 ? 4 : small_kw;
-        if (k != KIND_TILE && k != KIND_STREAM && !(small_kind && kw == 4)) {
-            C = one_wave_split(h, seqs, P, Q, G, rows_per_chunk, unit, min_split, target, k != KIND_SIMT);
-            // several verify blocks whose splits no SM holds whole: two CTAs per SM with 4-page stages where the lengths are alike (7 x 1000
-            // tokens 14.3 -> 12.3 us, 8 x 900 14.3 -> 11.8, 2 x 3500 12.5 -> 11.4, 3700 + 3900 12.7 -> 12.3; but 1500 + 2500 + 3500 12.9 -> 13.4.
-            // Up to 16 rows: 7 x 1000 10.7 / 11.4, 8 x 900 10.8 / 10.2)
-            int longest = 0, shortest = INT_MAX;
-            for (int s : seqs) { longest = std::max(longest, P[s] + Q[s]); shortest = std::min(shortest, P[s] + Q[s]); }
-            if (k == KIND_SMALL2 && seqs.size() >= 2 && C > kSwapMaxTokens && longest < 2 * shortest && !h->small_kw) kw = 4;
-        }
-        // one CTA per SM that holds its split whole (agx_attn_swap.cu)
-        const bool whole = small_kind && kw == 8 && C <= kSwapMaxTokens;
-        auto count_items = [&](int c_tokens) {
-            long long items = 0;
-            for (size_t n = 0; n < seqs.size(); ++n) {
-                const int L = P[seqs[n]] + Q[seqs[n]];
-                items += per_seq_items[n] * ((L + c_tokens - 1) / c_tokens);
-            }
-            return items;
-        };
-        if (k == KIND_TILE || k == KIND_STREAM) {
-            int max_len = 0;
-            for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            C = unit * choose_split(h, k == KIND_STREAM ? stream_model(h, std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; })) : tile_model(h), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
-            if (const char* force = getenv("AGX_TILE_SPLIT_TOKENS")) { if (atoi(force) >= unit) C = atoi(force) / unit * unit; }
-            if (h->debug_plan)
-                fprintf(stderr, "agx plan: tile kernel, %lld row chunks, longest sequence %d tokens -> KV splits of %d tokens, %lld CTAs\n",
-                        base_items, max_len, C, count_items(C));
-        } else if (small_kind && kw == 4) {
-            const SplitModel md = small4_model(h, k == KIND_SMALL1 ? 1 : 2);
-            C = md.unit * choose_split(h, md, seqs, P, Q, G, rows_per_chunk, std::max(1, min_split / md.unit), base_items);
-        }
-        // ---- small-q kernel: when every sequence has one row chunk and the same number of KV splits (2..16), the
-        //      splits of a (sequence, KV head) form a thread-block cluster and are merged through distributed shared
-        //      memory: no partials in global memory, no combine launch.  17..20 splits are squeezed into 16.
-        //      Not where a CTA holds its split whole: a CTA that waits for its cluster keeps an SM from the next call, whose K/V then come late
-        //      (8 rows over 300 / 700 / 2000 tokens 8.3 / 8.7 / 7.2 us, through memory 6.9 / 7.1 / 6.3; 4 x 500 7.8 / 6.4; one row over 3 x 700
-        //      5.9 / 5.0).  One block of one row or two keeps the clusters: as fast, and a launch fewer for the host (6.0 / 6.2 us a call).
-        int cluster = 0;
-        bool memory_merge = false;   // (fp32 partials, as the clusters' are)
-        if ((small_kind || k == KIND_SMALL4) && h->cluster_merge && seqs.size() <= (size_t)kMaxSeqs) {
-            int common = -1;
-            bool ok = true;
-            for (size_t n = 0; n < seqs.size() && ok; ++n) {
-                const int L = P[seqs[n]] + Q[seqs[n]];
-                int ns = (L + C - 1) / C;
-                ns = (L + round_up((L + ns - 1) / ns, unit) - 1) / round_up((L + ns - 1) / ns, unit);
-                if (ns > 16 && ns <= 20) ns = 16;
-                ok = per_seq_items[n] == c.num_kv_heads && (common < 0 || ns == common);
-                common = ns;
-            }
-            if (ok && common >= 2 && common <= 16) {
-                const int mt = k == KIND_SMALL1 ? 1 : k == KIND_SMALL2 ? 2 : 4;
-                const int fit = attn_small_max_clusters(mt, kw, common);
-                if (fit >= base_items) {
-                    memory_merge = whole && !(seqs.size() == 1 && Q[seqs[0]] <= 2) && h->cluster_merge != 2;
-                    if (!memory_merge) cluster = common;
-                }
-                if (h->debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
-            }
-        }
-        // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, with fp32 partials, are faster than 17 to 24 with SMs left to
-        // the merge of fp16 rows (32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
-        // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).
-        if (whole && !cluster && !memory_merge && seqs.size() == 1 && h->merge_sms && (k == KIND_SMALL2 || count_items(C) * 2 > h->sm_count)) {
-            const int L = P[seqs[0]] + Q[seqs[0]], longer = std::max(320, round_up((L + 15) / 16, unit));
-            if ((L + C - 1) / C > 16 && longer <= kSwapMaxTokens) { C = std::max(C, longer); memory_merge = true; }
-        }
-        // ---- fp32-arithmetic kernel: up to 16 splits of an item form a cluster, as many for all sequences; more leave partials
-        if (k == KIND_SIMT && h->cluster_merge) {
-            int max_len = 0;
-            for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            const int ns = (max_len + C - 1) / C;
-            if (ns <= 16) {
-                cluster = ns;
-                C = round_up((max_len + ns - 1) / ns, kPage);
-            }
-        }
-        // ---- small-q kernel, one wave of one CTA per SM, splits merged by the merge kernel: leave that kernel SMs of its own.
-        //      An attention CTA takes a whole SM, so merge CTAs that find no free SM sit on SMs the next call's attention CTAs
-        //      need, and those CTAs then start (and fetch their K/V) only after the merge instead of under it.  With a few SMs
-        //      left out of the attention grid the merge CTAs are resident there from the start and the next call's grid
-        //      follows this one without a gap.  A two-warp merge CTA handles two (row, head) pairs; 12 (up to 20 splits) or 8
-        //      of them fit an SM.
-        bool lean_merge = false;   // fp16 partials and the two-warp merge kernel (slower than fp32 partials and the four-warp
-                                   // one where the attention grid fills every SM twice over, e.g. four verify blocks of 4096)
-        const bool small_one_per_sm = k == KIND_SMALL4 || (small_kind && kw == 8);
-        // (the one-Q-tile tensor-core schedule as well: a single long sequence is one wave of whole-SM CTAs too)
-        if (!cluster && !memory_merge && (small_one_per_sm || k == KIND_STREAM) && seqs.size() <= (size_t)kMaxSeqs && h->merge_sms) {
-            long long pairs = 0;
-            for (int s : seqs) pairs += (long long)Q[s] * c.num_q_heads;
-            for (;;) {
-                const long long items = count_items(C);
-                int ns_max = 1;
-                for (int s : seqs) ns_max = std::max(ns_max, (P[s] + Q[s] + C - 1) / C);
-                if (ns_max == 1 || items > h->sm_count) break;   // no merge, or more than one wave anyway
-                const long long reserve = (pairs + (ns_max <= 20 ? 24 : 16) - 1) / (ns_max <= 20 ? 24 : 16);
-                if (reserve > h->sm_count / 8) break;   // a merge that large needs the whole device anyway
-                lean_merge = true;
-                if (items <= h->sm_count - reserve || items <= base_items) break;
-                if (whole && C + unit > kSwapMaxTokens) break;   // (6 x 1000 tokens, one row, 10.1 -> 8.1 us; 8 rows over 6700 12.7 -> 11.5)
-                C += unit;
-            }
-        }
-        // ---- emit launches of at most kMaxSeqs sequences
-        for (size_t a = 0; a < seqs.size(); a += kMaxSeqs) {
-            Launch ln;
-            ln.kind = (Kind)k;
-            plan.tensor_core |= k == KIND_TILE || k == KIND_STREAM;
-            ln.total_rows = 0;
-            ln.num_items = 0;
-            ln.cluster = cluster;
-            ln.lean_merge = lean_merge;
-            ln.kw = kw;
-            for (size_t n = a; n < std::min(seqs.size(), a + kMaxSeqs); ++n) {
-                const int s = seqs[n];
-                const int L = P[s] + Q[s];
-                SeqPlan sp;
-                sp.prefix_len = P[s];
-                sp.q_len = Q[s];
-                sp.q_row0 = row0[s];
-                sp.seq_index = s;
-                sp.nsplit = (L + C - 1) / C;
-                sp.split_tokens = round_up((L + sp.nsplit - 1) / sp.nsplit, unit);
-                sp.nsplit = (L + sp.split_tokens - 1) / sp.split_tokens;
-                if (cluster) { sp.nsplit = cluster; sp.split_tokens = round_up((L + cluster - 1) / cluster, kPage); }
-                sp.row_chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
-                // Row chunks of one KV head side by side share its K/V tiles through L2 (a whole long-context sequence does not fit
-                // there); where the sequence's K/V fits with room to spare, all heads' longest chunks go first instead, so that the
-                // short chunks of a causal block fill the last wave (3584 uncached tokens 114.7 -> 89.5 us, 2 x 1200 50.0 -> 43.0).
-                sp.chunk_major = (long long)L * c.num_kv_heads * c.head_dim * 4 <= (48ll << 20);
-                sp.item0 = ln.num_items;
-                sp.part_base = 0;
-                if (sp.nsplit > 1 && !cluster) {
-                    if (plan.part_entries + (long long)Q[s] * c.num_q_heads * sp.nsplit > 0x7FFFFFFFll)
-                        return fail(h, AGX_E_RANGE, "split partials exceed 2^31 entries");
-                    sp.part_base = (int)plan.part_entries;
-                    plan.part_entries += (long long)Q[s] * c.num_q_heads * sp.nsplit;
-                    plan.any_split = true;
-                }
-                const long long items = per_seq_items[n] * sp.nsplit;
-                if (ln.num_items + items > 0x7FFFFFFFll) return fail(h, AGX_E_RANGE, "too many work items");
-                ln.num_items += (int)items;
-                ln.total_rows += Q[s];
-                ln.seqs.push_back(sp);
-            }
-            if (h->debug_plan && k != KIND_TILE && k != KIND_STREAM)
-                fprintf(stderr, "agx plan: kind %d (stages of %d pages), %zu sequences, %d CTAs, first sequence %d splits of %d tokens%s\n", k,
-                        ln.kw, ln.seqs.size(), ln.num_items, ln.seqs[0].nsplit, ln.seqs[0].split_tokens,
-                        cluster ? ", merged in clusters" : "");
-            plan.launches.push_back(std::move(ln));
-        }
-    }
-    return AGX_OK;
-}
 
 // The plan for this batch: the cached one when the lengths are those of the last call on the handle.
 agx_status make_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, int pt_stride, const Plan*& out) {
@@ -517,7 +86,7 @@ agx_status make_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, i
     if (!h->plan_cache) return fail(h, AGX_E_NOMEM, "out of host memory");
     h->plan_P.clear();   // (invalid while it is rebuilt)
     *h->plan_cache = Plan();
-    agx_status st = build_plan(h, B, P, Q, pt_stride, *h->plan_cache);
+    agx_status st = build_plan(h->plan, B, P, Q, pt_stride, *h->plan_cache, h->err, sizeof h->err);
     if (st != AGX_OK) return st;
     h->plan_P.assign(P, P + B);
     h->plan_Q.assign(Q, Q + B);
@@ -561,31 +130,12 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     h->scale = cfg->scale > 0.f ? cfg->scale : 1.0f / sqrtf((float)cfg->head_dim);
     h->err[0] = 0;
     h->last_launches = 0;
-    const char* env = getenv("AGX_SMALL_MIN_SPLIT");
-    h->small_min_split = env ? std::max(64, atoi(env) / 64 * 64) : 256;
-    env = getenv("AGX_FORCE_MMA_SYNC");
-    h->force_mma_sync = env ? atoi(env) : 0;
-    env = getenv("AGX_STREAM_MIN_TOKENS");
-    h->stream_min_tokens = env ? atoi(env) : -1;   // -1: by the estimates of both kernels
-    env = getenv("AGX_STREAM_MAX_ROWS");
-    h->stream_max_rows = env ? atoi(env) : 384;
-    env = getenv("AGX_CLUSTER_MERGE");
-    h->cluster_merge = !env ? 1 : atoi(env) ? 2 : 0;
+    const char* env;
     env = getenv("AGX_HOST_PIPELINE_ROWS");
     h->pipe_rows = env ? std::max(0, atoi(env)) : 384;   // measured on the long-context step: 256 / 384 / 512 / 768 / 1024 rows -> 1.54 / 1.43 / 1.57 / 1.56 / 1.72 ms
     h->pipe_in = h->pipe_out = nullptr;
-    env = getenv("AGX_LONGEST_FIRST");
-    h->longest_first = !(env && atoi(env) == 0);
-    env = getenv("AGX_MERGE_SMS");
-    h->merge_sms = !(env && atoi(env) == 0);
     env = getenv("AGX_ZERO_COPY");
     h->zero_copy = env ? atoi(env) : 3;
-    env = getenv("AGX_SMALL_KW");
-    h->small_kw = (env && (atoi(env) == 4 || atoi(env) == 8)) ? atoi(env) : 0;
-    env = getenv("AGX_BATCH_STREAM_TOKENS");   // (forcing the per-sequence cross-over also switches the batch rule off)
-    h->batch_stream_tokens = env ? atoi(env) : -1;   // -1: by the estimates of both kernels
-    env = getenv("AGX_DEBUG_PLAN");
-    h->debug_plan = env ? atoi(env) : 0;
     h->wait_limit_cycles = kWaitLimitCycles;
     env = getenv("AGX_EARLY_PREFIX");
     h->early_prefix = env ? atoi(env) : 0;
@@ -600,6 +150,7 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     if (e != cudaSuccess) { delete h; return e == cudaErrorMemoryAllocation ? AGX_E_NOMEM : AGX_E_CUDA; }
     e = cudaMemset(h->d_status, 0, kStateBytes);
     if (e != cudaSuccess) { cudaFree(h->d_status); delete h; return AGX_E_CUDA; }
+    h->plan = plan_config(h->cfg, h->sm_count, attn_small_max_clusters);
     h->d_ticket = (unsigned int*)(h->d_status + 16);
     h->d_row_keys = (unsigned long long*)(h->d_status + 64);
     *out = h;

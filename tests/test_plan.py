@@ -1,0 +1,64 @@
+"""The launch planner, without a GPU: what any plan has to hold, and which kernel takes which blocks."""
+import numpy as np
+import pytest
+
+from tests.plan_util import plan
+
+ROWS = {"small1": 16, "small2": 32, "small4": 64, "stream": 128, "tile": 256, "simt": 8}
+UNIT = {"small1": 16, "small2": 16, "small4": 16, "stream": 128, "tile": 128, "simt": 16}
+
+
+def check(P, Q, hq, hkv, d, dtype):
+    """Every sequence once, its splits cover its tokens, CTAs and partial slots are dealt without gap or overlap."""
+    pl = plan(P, Q, hq, hkv, d, dtype)
+    assert pl.status == 0, pl.error
+    G, seen, slots = hq // hkv, set(), []
+    for ln in pl.launches:
+        items = 0
+        assert 1 <= len(ln.seqs) <= 48 and ln.rows == sum(int(Q[s.index]) for s in ln.seqs)
+        for s in ln.seqs:
+            p, q = int(P[s.index]), int(Q[s.index])
+            assert s.index not in seen
+            seen.add(s.index)
+            assert s.row_chunks == -(-q * G // ROWS[ln.kind]) and s.split_tokens % UNIT[ln.kind] == 0
+            assert s.nsplit * s.split_tokens >= p + q
+            if ln.cluster:
+                assert s.nsplit == ln.cluster <= 16
+            else:
+                assert (s.nsplit - 1) * s.split_tokens < p + q   # (no split without tokens)
+                if s.nsplit > 1:
+                    slots.append((s.part_base, q * hq * s.nsplit))
+            assert s.item0 == items
+            items += hkv * s.row_chunks * s.nsplit
+        assert ln.items == items
+        if ln.kind in ("small1", "small2"):
+            assert all(s.row_chunks == 1 for s in ln.seqs)
+    assert seen == set(range(len(P)))
+    at = 0
+    for base, n in sorted(slots):
+        assert base == at
+        at += n
+    assert at == pl.part_entries
+    return pl
+
+
+@pytest.mark.parametrize("hq,hkv,d,dtype", [(32, 8, 128, "bf16"), (24, 8, 128, "bf16"), (40, 8, 128, "bf16"), (16, 2, 128, "bf16"), (8, 8, 128, "bf16"),
+                                            (4, 1, 128, "bf16"), (8, 2, 64, "bf16"), (4, 2, 64, "f32"), (32, 8, 128, "f32")])
+def test_any_plan_is_sound(hq, hkv, d, dtype):
+    rng = np.random.default_rng(hq * 100 + hkv)
+    lengths = lambda lo, hi, n: np.exp(rng.uniform(np.log(lo), np.log(hi), n)).astype(np.int64)  # noqa: E731
+    for i in range(150):
+        B = int(lengths(1, 130, 1)[0])
+        P = lengths(1, 40000, B) - 1
+        Q = lengths(1, 2500, B) if i % 3 == 0 else np.where(rng.random(B) < 0.7, rng.integers(1, 17, B), lengths(16, 1500, B)) if i % 3 == 1 else np.full(B, i % 9 + 1)
+        if i % 2:
+            P[:] = P[0]
+        check(P, Q, hq, hkv, d, dtype)
+
+
+def test_which_kernel_takes_which_rows():
+    """(rows per KV head: q * hq / hkv)"""
+    for rows, kind in ((16, "small1"), (17, "small2"), (32, "small2"), (33, "stream"), (384, "stream"), (385, "tile")):
+        assert plan([300], [rows], 8, 8).kind_of(0) == kind
+    assert plan([300], [1], 40, 1).kind_of(0) == "stream"   # 40 rows of one token
+    assert plan([300], [8], d=64).kind_of(0) == "simt" and plan([300], [8], dtype="f32").kind_of(0) == "simt"
