@@ -5,7 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
-#include <climits>
+#include <exception>
 #include <new>
 #include <vector>
 
@@ -82,14 +82,18 @@ agx_status make_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, i
         out = h->plan_cache;
         return AGX_OK;
     }
-    if (!h->plan_cache) h->plan_cache = new (std::nothrow) Plan;
-    if (!h->plan_cache) return fail(h, AGX_E_NOMEM, "out of host memory");
     h->plan_P.clear();   // (invalid while it is rebuilt)
-    *h->plan_cache = Plan();
-    agx_status st = build_plan(h->plan, B, P, Q, pt_stride, *h->plan_cache, h->err, sizeof h->err);
-    if (st != AGX_OK) return st;
-    h->plan_P.assign(P, P + B);
-    h->plan_Q.assign(Q, Q + B);
+    try {
+        if (!h->plan_cache) h->plan_cache = new Plan;
+        *h->plan_cache = Plan();
+        agx_status st = build_plan(h->plan, B, P, Q, pt_stride, *h->plan_cache, h->err, sizeof h->err);
+        if (st != AGX_OK) return st;
+        h->plan_Q.assign(Q, Q + B);
+        h->plan_P.assign(P, P + B);
+    } catch (const std::exception&) {   // (no exception leaves a C entry)
+        h->plan_P.clear();
+        return fail(h, AGX_E_NOMEM, "out of host memory for the plan of %d sequences", B);
+    }
     out = h->plan_cache;
     return AGX_OK;
 }

@@ -10,6 +10,9 @@ namespace agx {
 
 namespace {
 
+constexpr long long kMaxTokens = 0x7FFFFFFFll - 4096;   // of one sequence: rounded up to tiles they still fit an int
+
+inline int ceil_div(int a, int b) { return (int)(((unsigned)a + (unsigned)b - 1u) / (unsigned)b); }   // (of two positive numbers)
 inline int round_up(long long v, int m) { return (int)((v + m - 1) / m * m); }
 
 // What a launch of one of the attention kernels costs (us), fitted to sweeps over split lengths and batches (GQA 32/8; worst errors 2-3 us at
@@ -146,7 +149,7 @@ int one_wave_split(const PlanConfig& c, const std::vector<int>& seqs, const int3
     int C = shrink && even < min_split && even * 20 >= min_split * 17 ? even : std::max(min_split, even);
     for (;; C += unit) {
         long long n = 0;
-        for (int s : seqs) n += items_of(s) * ((P[s] + Q[s] + C - 1) / C);
+        for (int s : seqs) n += items_of(s) * ceil_div(P[s] + Q[s], C);
         if (n <= std::max<long long>(target, base)) return C;
     }
 }
@@ -182,6 +185,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         if (P[s] < 0) return fail(AGX_E_INVAL, "prefix_len[%d] = %d < 0", s, P[s]);
         if (pt_stride >= 0 && (long long)P[s] + Q[s] > (long long)pt_stride * kPage)
             return fail(AGX_E_RANGE, "sequence %d: %d + %d tokens exceed the page table (%d pages)", s, P[s], Q[s], pt_stride);
+        if ((long long)P[s] + Q[s] > kMaxTokens) return fail(AGX_E_RANGE, "sequence %d: %d + %d tokens", s, P[s], Q[s]);
         if ((long long)row0[s] + Q[s] > (1 << 30)) return fail(AGX_E_RANGE, "too many rows");
         row0[s + 1] = row0[s] + Q[s];
     }
@@ -293,7 +297,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             long long items = 0;
             for (size_t n = 0; n < seqs.size(); ++n) {
                 const int L = P[seqs[n]] + Q[seqs[n]];
-                items += per_seq_items[n] * ((L + c_tokens - 1) / c_tokens);
+                items += per_seq_items[n] * ceil_div(L, c_tokens);
             }
             return items;
         };
@@ -322,8 +326,8 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             bool ok = true;
             for (size_t n = 0; n < seqs.size() && ok; ++n) {
                 const int L = P[seqs[n]] + Q[seqs[n]];
-                int ns = (L + C - 1) / C;
-                ns = (L + round_up((L + ns - 1) / ns, unit) - 1) / round_up((L + ns - 1) / ns, unit);
+                int ns = ceil_div(L, C);
+                ns = ceil_div(L, round_up(ceil_div(L, ns), unit));
                 if (ns > 16 && ns <= 20) ns = 16;
                 ok = per_seq_items[n] == c.num_kv_heads && (common < 0 || ns == common);
                 common = ns;
@@ -343,16 +347,16 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).
         if (whole && !cluster && !memory_merge && seqs.size() == 1 && c.merge_sms && (k == KIND_SMALL2 || count_items(C) * 2 > c.sm_count)) {
             const int L = P[seqs[0]] + Q[seqs[0]], longer = std::max(320, round_up((L + 15) / 16, unit));
-            if ((L + C - 1) / C > 16 && longer <= kSwapMaxTokens) { C = std::max(C, longer); memory_merge = true; }
+            if (ceil_div(L, C) > 16 && longer <= kSwapMaxTokens) { C = std::max(C, longer); memory_merge = true; }
         }
         // ---- fp32-arithmetic kernel: up to 16 splits of an item form a cluster, as many for all sequences; more leave partials
         if (k == KIND_SIMT && c.cluster_merge) {
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            const int ns = (max_len + C - 1) / C;
+            const int ns = ceil_div(max_len, C);
             if (ns <= 16) {
                 cluster = ns;
-                C = round_up((max_len + ns - 1) / ns, kPage);
+                C = round_up(ceil_div(max_len, ns), kPage);
             }
         }
         // ---- small-q kernel, one wave of one CTA per SM, splits merged by the merge kernel: leave that kernel SMs of its own.
@@ -371,7 +375,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             for (;;) {
                 const long long items = count_items(C);
                 int ns_max = 1;
-                for (int s : seqs) ns_max = std::max(ns_max, (P[s] + Q[s] + C - 1) / C);
+                for (int s : seqs) ns_max = std::max(ns_max, ceil_div(P[s] + Q[s], C));
                 if (ns_max == 1 || items > c.sm_count) break;   // no merge, or more than one wave anyway
                 const long long reserve = (pairs + (ns_max <= 20 ? 24 : 16) - 1) / (ns_max <= 20 ? 24 : 16);
                 if (reserve > c.sm_count / 8) break;   // a merge that large needs the whole device anyway
@@ -399,10 +403,10 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 sp.q_len = Q[s];
                 sp.q_row0 = row0[s];
                 sp.seq_index = s;
-                sp.nsplit = (L + C - 1) / C;
-                sp.split_tokens = round_up((L + sp.nsplit - 1) / sp.nsplit, unit);
-                sp.nsplit = (L + sp.split_tokens - 1) / sp.split_tokens;
-                if (cluster) { sp.nsplit = cluster; sp.split_tokens = round_up((L + cluster - 1) / cluster, kPage); }
+                sp.nsplit = ceil_div(L, C);
+                sp.split_tokens = round_up(ceil_div(L, sp.nsplit), unit);
+                sp.nsplit = ceil_div(L, sp.split_tokens);
+                if (cluster) { sp.nsplit = cluster; sp.split_tokens = round_up(ceil_div(L, cluster), kPage); }
                 sp.row_chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
                 // Row chunks of one KV head side by side share its K/V tiles through L2 (a whole long-context sequence does not fit
                 // there); where the sequence's K/V fits with room to spare, all heads' longest chunks go first instead, so that the

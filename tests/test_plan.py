@@ -62,3 +62,12 @@ def test_which_kernel_takes_which_rows():
         assert plan([300], [rows], 8, 8).kind_of(0) == kind
     assert plan([300], [1], 40, 1).kind_of(0) == "stream"   # 40 rows of one token
     assert plan([300], [8], d=64).kind_of(0) == "simt" and plan([300], [8], dtype="f32").kind_of(0) == "simt"
+
+
+@pytest.mark.parametrize("hq,hkv,d,dtype", [(32, 8, 128, "bf16"), (4, 1, 128, "bf16"), (4, 1, 64, "f32")])
+def test_lengths_beyond_what_the_planner_counts_are_refused(hq, hkv, d, dtype):
+    for P, Q in ((2**31 - 8, 7), (2**31 - 48, 8), (2**31 - 1, 1), (2**31 - 1, 2**30), (2**31 - 4000, 8)):
+        assert plan([100, P], [1, Q], hq, hkv, d, dtype).status == -2   # AGX_E_RANGE, no exception
+    for P in (2**31 - 5000, 1500000000, 2**30):
+        check([P, 100], [1, 8], hq, hkv, d, dtype)
+        check([P], [8], hq, hkv, d, dtype)
