@@ -38,60 +38,82 @@ SplitModel small4_model(const PlanConfig& c, int mt) {
     return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, false};
 }
 
-// Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time.
-int choose_split(const PlanConfig& c, const SplitModel& md, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
-                 int rows_per_chunk, int min_tiles, long long base_items, double* estimate = nullptr) {
+// Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time, and that time.  A server's lengths change with every
+// step, so this is host time of every step; what all candidates share is worked out once, and the CTAs of one that cannot win are not dealt out.
+struct SplitChoice {
+    int tiles = 0;        // 0: not asked for
+    double time = 0;
+};
+SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::vector<int>& seqs, const int32_t* P, const int32_t* Q, int G,
+                         int rows_per_chunk, int min_tiles, long long base_items) {
     const int sms = md.slots, hkv = c.num_kv_heads, kOverhead = md.overhead;
     int max_tiles = 1;
     long long pairs = 0;      // (row, query head)
     bool equal = true;
+    struct Seq { int tiles, seen_end; double rows_heads; };
+    struct Seen { int tiles; long long n; };   // n (row chunk, KV head) pairs that see this many tiles
+    std::vector<Seq> work;
+    std::vector<Seen> seen;
+    work.reserve(seqs.size());
+    seen.reserve(seqs.size());
     for (int s : seqs) {
         const int lt = (P[s] + Q[s] + md.unit - 1) / md.unit;
         equal &= s == seqs[0] || lt == max_tiles;
         pairs += (long long)Q[s] * c.num_q_heads;
         max_tiles = std::max(max_tiles, lt);
+        const int chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk, first = (int)seen.size();
+        auto add = [&](int last_row, long long n) {
+            const int tiles = (P[s] + std::min(Q[s] - 1, last_row / G) + md.unit) / md.unit;
+            if ((int)seen.size() > first && seen.back().tiles == tiles) seen.back().n += n;
+            else seen.push_back({tiles, n});
+        };
+        if (chunks <= 32) {
+            for (int rc = 0; rc < chunks; ++rc) add((rc + 1) * rows_per_chunk - 1, hkv);
+        } else {   // in 32 groups of chunks with the tiles of the group's last one
+            for (int k = 0; k < 32; ++k) {
+                const int rc0 = (int)((long long)chunks * k / 32), rc1 = (int)((long long)chunks * (k + 1) / 32);
+                add(rc1 * rows_per_chunk - 1, (long long)hkv * (rc1 - rc0));
+            }
+        }
+        work.push_back({lt, (int)seen.size(), (double)Q[s] * c.num_q_heads});
     }
-    struct Cand { int tiles; double bound, merge; };
-    std::vector<Cand> cands;
-    // items of a candidate, by tile count: (count, tiles)
-    std::vector<std::pair<int, long long>> items;
-    auto collect = [&](int split_tiles, long long& sum, long long& count, int& longest, double& part_mb) {
-        items.clear();
-        sum = count = 0; longest = 0; part_mb = 0;
-        for (int s : seqs) {
-            const int L = P[s] + Q[s], lt = (L + md.unit - 1) / md.unit, ns = (lt + split_tiles - 1) / split_tiles, per = (lt + ns - 1) / ns;
-            const int chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;
-            if (ns > 1) part_mb += (double)Q[s] * c.num_q_heads * ns * md.part_row_bytes * 1e-6;
-            auto add = [&](int vis, long long n) {   // n (chunk, head) pairs that see `vis` tiles
-                const int full = vis / per, rest = vis - full * per;
-                if (full) items.push_back({per, n * full});
-                if (rest) items.push_back({rest, n});
-                sum += n * (vis + kOverhead * (full + (rest != 0)));
-                count += n * (full + (rest != 0));
-                longest = std::max(longest, full ? per : rest);
-            };
-            if (chunks <= 32) {
-                for (int rc = 0; rc < chunks; ++rc) add((P[s] + std::min(Q[s] - 1, ((rc + 1) * rows_per_chunk - 1) / G) + md.unit) / md.unit, hkv);
-            } else {   // in 32 groups of chunks with the tiles of the group's last one
-                for (int k = 0; k < 32; ++k) {
-                    const int rc0 = (int)((long long)chunks * k / 32), rc1 = (int)((long long)chunks * (k + 1) / 32);
-                    add((P[s] + std::min(Q[s] - 1, (rc1 * rows_per_chunk - 1) / G) + md.unit) / md.unit, (long long)hkv * (rc1 - rc0));
-                }
+    // calls item(tiles, n) for the CTAs of a candidate
+    auto deal = [&](int split_tiles, auto item) {
+        int i = 0;
+        for (const Seq& w : work) {
+            const unsigned ns = ((unsigned)w.tiles + split_tiles - 1) / (unsigned)split_tiles, per = ((unsigned)w.tiles + ns - 1) / ns;
+            for (; i < w.seen_end; ++i) {
+                const unsigned full = (unsigned)seen[i].tiles / per;
+                item(seen[i], (int)per, (int)full, (int)((unsigned)seen[i].tiles - full * per));
             }
         }
     };
+    struct Cand { int tiles, longest; double bound, merge; long long sum; };
+    std::vector<Cand> cands;
     const int n_max = (int)std::min<long long>((max_tiles + min_tiles - 1) / min_tiles, std::max<long long>(32, 2 * sms / std::max<long long>(base_items, 1)));
+    cands.reserve(n_max);
     for (int n = 1, last = 0; n <= n_max; ++n) {
         const int t = std::max(min_tiles, (max_tiles + n - 1) / n);
         if (t == last) continue;
         last = t;
-        long long sum, count;
-        int longest;
-        double mb;
-        collect(t, sum, count, longest, mb);
+        long long sum = 0, count = 0;
+        int longest = 0;
+        double mb = 0;
+        for (const Seq& w : work) {
+            const int ns = (w.tiles + t - 1) / t;
+            if (ns > 1) mb += w.rows_heads * ns * md.part_row_bytes * 1e-6;
+        }
+        deal(t, [&](const Seen& v, int per, int full, int rest) {
+            const int starts = full + (rest != 0);
+            sum += v.n * (v.tiles + kOverhead * starts);
+            count += v.n * starts;
+            longest = std::max(longest, full ? per : rest);
+        });
         const double load = std::max<double>((double)sum / sms, longest + kOverhead);
         Cand cd;
         cd.tiles = t;
+        cd.longest = longest;
+        cd.sum = sum;
         cd.merge = mb == 0 ? 0 : md.lean && count <= sms * 15 / 16 && pairs <= 3 * sms ? 1.0 + 0.2 * mb
                    : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
                    : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
@@ -100,30 +122,30 @@ int choose_split(const PlanConfig& c, const SplitModel& md, const std::vector<in
         cands.push_back(cd);
     }
     std::stable_sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
-    double best = -1;
-    int best_tiles = max_tiles;
+    SplitChoice best;
     std::vector<int> load;
+    std::vector<long long> of_size;   // CTAs with that many tiles
     for (const Cand& cd : cands) {
-        if (best >= 0 && cd.bound >= best) break;   // (bounds ascend)
-        long long sum, count;
-        int longest;
-        double mb, t;
-        collect(cd.tiles, sum, count, longest, mb);
-        // load[x]: SMs with x tiles (and starts) so far; an item goes to an SM with the least
-        std::sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-        load.assign((size_t)(sum / sms) + longest + kOverhead + 2, 0);
+        if (best.tiles && cd.bound >= best.time) break;   // (bounds ascend)
+        of_size.assign(cd.longest + 1, 0);
+        deal(cd.tiles, [&](const Seen& v, int per, int full, int rest) {
+            if (full) of_size[per] += v.n * full;
+            of_size[rest] += v.n;   // (of_size[0] is not looked at)
+        });
+        // load[x]: SMs with x tiles (and starts) so far; a CTA goes to an SM with the least
+        load.assign((size_t)(cd.sum / sms) + cd.longest + kOverhead + 2, 0);
         load[0] = sms;
         size_t lo = 0, hi = 0;
-        for (const auto& it : items)
-            for (long long left = it.second; left > 0;) {
+        for (int size = cd.longest; size > 0; --size)
+            for (long long left = of_size[size]; left > 0;) {
                 while (load[lo] == 0) ++lo;
                 const int k = (int)std::min<long long>(load[lo], left);
                 load[lo] -= k;
-                load[lo + it.first + kOverhead] += k;
-                hi = std::max(hi, lo + it.first + kOverhead);
+                load[lo + size + kOverhead] += k;
+                hi = std::max(hi, lo + size + kOverhead);
                 left -= k;
             }
-        t = md.base;
+        double t = md.base;
         size_t prev = kOverhead;
         int busy = sms;
         for (size_t x = 0; x <= hi; ++x) {
@@ -132,10 +154,9 @@ int choose_split(const PlanConfig& c, const SplitModel& md, const std::vector<in
             busy -= load[x];
         }
         t += cd.merge;
-        if (best < 0 || t < best) { best = t; best_tiles = cd.tiles; }
+        if (!best.tiles || t < best.time) best = {cd.tiles, t};
     }
-    if (estimate) *estimate = best;
-    return best_tiles;
+    return best;
 }
 
 // Tokens per KV split (a multiple of `unit`) with which the sequences' items are one wave of `target` CTAs, at least about min_split.
@@ -206,16 +227,15 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             else if (rows <= c.stream_max_rows) wide_seqs.push_back(s);
         }
     bool batch_streams = false;
+    SplitChoice stream_choice, small_choice[2];   // splits that the estimates below were made with, where they were
     if (!small_seqs.empty() && c.stream_min_tokens < 0) {
         if (c.batch_stream_tokens >= 0) {
             batch_streams = small_seqs.size() >= 2 && small_k * 1e3 >= c.batch_stream_tokens;
         } else {
             auto estimate = [&](const SplitModel& md, int chunk, const std::vector<int>& seqs) {
-                double t = 0;
                 long long items = 0;
                 for (int s : seqs) items += (long long)c.num_kv_heads * ((Q[s] * G + chunk - 1) / chunk);
-                if (!seqs.empty()) choose_split(c, md, seqs, P, Q, G, chunk, md.unit == 64 ? 4 : 2, items, &t);
-                return t;
+                return seqs.empty() ? SplitChoice() : choose_split(c, md, seqs, P, Q, G, chunk, md.unit == 64 ? 4 : 2, items);
             };
             const bool one = small_seqs.size() == 1;
             double warp_mma;
@@ -225,14 +245,20 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 const bool whole = mt2.empty() || one_wave_split(c, mt2, P, Q, G, 32, 16, c.small_min_split, c.sm_count, true) <= kSwapMaxTokens;
                 warp_mma = small_rows <= 16 ? 4.1 + 0.69 * small_k : whole ? 5.6 + 0.8 * small_k : std::max(8.8, 5.8 + 1.06 * small_k);
             } else {
-                warp_mma = estimate(small4_model(c, 1), 16, mt1) + estimate(small4_model(c, 2), 32, mt2);
+                small_choice[0] = estimate(small4_model(c, 1), 16, mt1);
+                small_choice[1] = estimate(small4_model(c, 2), 32, mt2);
+                warp_mma = small_choice[0].time + small_choice[1].time;
             }
             std::vector<int> all = wide_seqs;
             all.insert(all.end(), small_seqs.begin(), small_seqs.end());
             // (with one 16-row tile the warp-MMA kernel was never more than 2 % slower than the schedule, also where the estimates tie)
             if (!one && small_k >= 7.9 && small_rows <= 16) warp_mma *= 0.87;
             const SplitModel sm = stream_model(c, !wide_seqs.empty());
-            batch_streams = estimate(sm, 128, all) < warp_mma + estimate(sm, 128, wide_seqs);
+            if (!wide_seqs.empty() || warp_mma > sm.base) {   // (no launch of the schedule is estimated below its base)
+                const SplitChoice together = estimate(sm, 128, all), wide = estimate(sm, 128, wide_seqs);
+                batch_streams = together.time < warp_mma + wide.time;
+                stream_choice = batch_streams ? together : wide;
+            }
         }
     }
     long long warp_mma_tokens = 0;
@@ -304,14 +330,21 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         if (k == KIND_TILE || k == KIND_STREAM) {
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            C = unit * choose_split(c, k == KIND_STREAM ? stream_model(c, std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; })) : tile_model(c), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
+            SplitChoice choice = k == KIND_STREAM ? stream_choice : SplitChoice();
+            if (!choice.tiles) {
+                const bool wide = std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; });
+                choice = choose_split(c, k == KIND_STREAM ? stream_model(c, wide) : tile_model(c), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
+            }
+            C = unit * choice.tiles;
             if (const char* force = getenv("AGX_TILE_SPLIT_TOKENS")) { if (atoi(force) >= unit) C = atoi(force) / unit * unit; }
             if (c.debug_plan)
                 fprintf(stderr, "agx plan: tile kernel, %lld row chunks, longest sequence %d tokens -> KV splits of %d tokens, %lld CTAs\n",
                         base_items, max_len, C, count_items(C));
         } else if (small_kind && kw == 4) {
             const SplitModel md = small4_model(c, k == KIND_SMALL1 ? 1 : 2);
-            C = md.unit * choose_split(c, md, seqs, P, Q, G, rows_per_chunk, std::max(1, min_split / md.unit), base_items);
+            const int least = std::max(1, min_split / md.unit);
+            const SplitChoice& known = small_choice[k == KIND_SMALL1 ? 0 : 1];
+            C = md.unit * (known.tiles && least == 4 ? known : choose_split(c, md, seqs, P, Q, G, rows_per_chunk, least, base_items)).tiles;
         }
         // ---- small-q kernel: when every sequence has one row chunk and the same number of KV splits (2..16), the
         //      splits of a (sequence, KV head) form a thread-block cluster and are merged through distributed shared
