@@ -19,7 +19,7 @@
  *     The library never frees or retains caller memory.
  *   - A handle must be used from one stream at a time: calls on the same handle that overlap on
  *     the GPU share that state and race.  Host threads: a handle is not thread-safe (it caches the last
- *     launch plan, the pools' tensor maps and the last error text); use it from one host thread at a
+ *     launch plans and the last error text); use it from one host thread at a
  *     time, or one handle per thread.  Different handles may be used concurrently: the only
  *     process-wide state is a per-device note that a kernel's launch attributes have been set, which
  *     every thread writes with the same value.

@@ -43,9 +43,13 @@ struct agx_handle {
     int pipe_rows;
     cudaStream_t pipe_in, pipe_out;
     std::vector<cudaEvent_t> pipe_events;
-    // the launch plan of the last batch seen: the layers of a model step all ask for the same one
-    agx::Plan* plan_cache;
-    std::vector<int32_t> plan_P, plan_Q;
+    // The launch plans of the last batches seen: the layers of a model step all ask for the same one, those of a pipelined host step for one per chunk.
+    static constexpr int kPlans = 16;
+    struct CachedPlan {
+        agx::Plan plan;
+        std::vector<int32_t> P, Q;   // empty: no plan
+    } plans[kPlans];
+    int plan_last;                   // the one used last
     char err[512];
 };
 
@@ -71,30 +75,35 @@ inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
 inline int elem_size(int dtype) { return dtype == AGX_BF16 ? 2 : 4; }
 
-// The plan for this batch: the cached one when the lengths are those of the last call on the handle.
+// The plan for this batch: a cached one when the lengths are those of one of the last calls on the handle.
 agx_status make_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, int pt_stride, const Plan*& out) {
-    if (h->plan_cache && (int)h->plan_P.size() == B && memcmp(h->plan_P.data(), P, sizeof(int32_t) * B) == 0 &&
-        memcmp(h->plan_Q.data(), Q, sizeof(int32_t) * B) == 0) {
+    for (int i = 0; i < agx_handle::kPlans; ++i) {
+        const int at = (h->plan_last + agx_handle::kPlans - i) % agx_handle::kPlans;
+        const agx_handle::CachedPlan& e = h->plans[at];
+        if ((int)e.P.size() != B || memcmp(e.P.data(), P, sizeof(int32_t) * B) != 0 || memcmp(e.Q.data(), Q, sizeof(int32_t) * B) != 0) continue;
         if (pt_stride >= 0)
             for (int s = 0; s < B; ++s)
                 if ((long long)P[s] + Q[s] > (long long)pt_stride * kPage)
                     return fail(h, AGX_E_RANGE, "sequence %d: %d + %d tokens exceed the page table (%d pages)", s, P[s], Q[s], pt_stride);
-        out = h->plan_cache;
+        h->plan_last = at;
+        out = &e.plan;
         return AGX_OK;
     }
-    h->plan_P.clear();   // (invalid while it is rebuilt)
+    const int at = (h->plan_last + 1) % agx_handle::kPlans;   // (round robin)
+    agx_handle::CachedPlan& e = h->plans[at];
+    e.P.clear();   // (invalid while it is rebuilt)
     try {
-        if (!h->plan_cache) h->plan_cache = new Plan;
-        *h->plan_cache = Plan();
-        agx_status st = build_plan(h->plan, B, P, Q, pt_stride, *h->plan_cache, h->err, sizeof h->err);
+        e.plan = Plan();
+        agx_status st = build_plan(h->plan, B, P, Q, pt_stride, e.plan, h->err, sizeof h->err);
         if (st != AGX_OK) return st;
-        h->plan_Q.assign(Q, Q + B);
-        h->plan_P.assign(P, P + B);
+        e.Q.assign(Q, Q + B);
+        e.P.assign(P, P + B);
     } catch (const std::exception&) {   // (no exception leaves a C entry)
-        h->plan_P.clear();
+        e.P.clear();
         return fail(h, AGX_E_NOMEM, "out of host memory for the plan of %d sequences", B);
     }
-    out = h->plan_cache;
+    h->plan_last = at;
+    out = &e.plan;
     return AGX_OK;
 }
 
@@ -167,7 +176,6 @@ agx_status agx_destroy(agx_handle* h) {
     if (h->pipe_in) cudaStreamDestroy(h->pipe_in);
     if (h->pipe_out) cudaStreamDestroy(h->pipe_out);
     for (cudaEvent_t ev : h->pipe_events) cudaEventDestroy(ev);
-    delete h->plan_cache;
     delete h;
     return AGX_OK;
 }
