@@ -228,10 +228,10 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         }
     bool batch_streams = false;
     SplitChoice stream_choice, small_choice[2];   // splits that the estimates below were made with, where they were
-    if (!small_seqs.empty() && c.stream_min_tokens < 0) {
+    if (!small_seqs.empty()) {
         if (c.batch_stream_tokens >= 0) {
             batch_streams = small_seqs.size() >= 2 && small_k * 1e3 >= c.batch_stream_tokens;
-        } else {
+        } else if (c.stream_min_tokens < 0) {
             auto estimate = [&](const SplitModel& md, int chunk, const std::vector<int>& seqs) {
                 long long items = 0;
                 for (int s : seqs) items += (long long)c.num_kv_heads * ((Q[s] * G + chunk - 1) / chunk);
@@ -273,7 +273,9 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             // up to 128 rows: one Q tile per CTA, KV tiles alternating between two softmax warpgroups (HBM-bound
             // streaming on the tcgen05 pipe); blocks of at most 32 rows over short contexts stay with the warp-MMA
             // kernel, whose fixed costs are lower (none above 32 rows)
-            const bool forced = c.stream_min_tokens >= 0 && P[s] + Q[s] >= c.stream_min_tokens;
+            // (with the batch rule forced the estimates are not asked, and a sequence of its own keeps the cross-over between the two kernels)
+            const int cross = c.stream_min_tokens >= 0 ? c.stream_min_tokens : c.batch_stream_tokens < 0 ? INT_MAX : rows > 8 ? 7168 : 10240;
+            const bool forced = P[s] + Q[s] >= cross;
             if (tile_ok && rows <= c.stream_max_rows && (rows > 32 || batch_streams || forced)) k = KIND_STREAM;
             else if (rows <= 16) k = KIND_SMALL1;
             else if (rows <= 32) k = KIND_SMALL2;

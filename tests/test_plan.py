@@ -71,3 +71,18 @@ def test_lengths_beyond_what_the_planner_counts_are_refused(hq, hkv, d, dtype):
     for P in (2**31 - 5000, 1500000000, 2**30):
         check([P, 100], [1, 8], hq, hkv, d, dtype)
         check([P], [8], hq, hkv, d, dtype)
+
+
+def test_forced_cross_overs(monkeypatch):
+    """AGX_BATCH_STREAM_TOKENS replaces the rule for batches only, AGX_STREAM_MIN_TOKENS that for one sequence only; they can be given together."""
+    def kinds(P, Q):
+        return [plan(P, Q).kind_of(s) for s in range(len(P))]
+    monkeypatch.setenv("AGX_BATCH_STREAM_TOKENS", "20000")
+    assert kinds([60000], [8]) == ["stream"] and kinds([10230], [2]) == ["small1"] == kinds([10230], [1]) and kinds([10240], [2]) == ["stream"]
+    assert kinds([7100], [8]) == ["small2"] and kinds([7168], [8]) == ["stream"] and kinds([7168], [3]) == ["stream"]
+    assert kinds([9000, 12000], [1, 1]) == ["stream"] * 2 and kinds([9000, 9000], [1, 1]) == ["small1"] * 2
+    assert kinds([900, 12000], [1, 1]) == ["small1", "stream"]
+    monkeypatch.setenv("AGX_STREAM_MIN_TOKENS", "500")
+    assert kinds([400, 600], [1, 1]) == ["small1", "stream"] and kinds([400] * 51, [1] * 51) == ["stream"] * 51
+    monkeypatch.delenv("AGX_BATCH_STREAM_TOKENS")
+    assert kinds([400] * 51, [1] * 51) == ["small1"] * 51 and kinds([600], [1]) == ["stream"]
