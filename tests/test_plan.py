@@ -86,3 +86,11 @@ def test_forced_cross_overs(monkeypatch):
     assert kinds([400, 600], [1, 1]) == ["small1", "stream"] and kinds([400] * 51, [1] * 51) == ["stream"] * 51
     monkeypatch.delenv("AGX_BATCH_STREAM_TOKENS")
     assert kinds([400] * 51, [1] * 51) == ["small1"] * 51 and kinds([600], [1]) == ["stream"]
+
+
+@pytest.mark.parametrize("P,q,items", [([2500] * 4, 1, 288), ([2500] * 6, 4, 288), ([2500] * 4, 8, 288), ([4650] * 2, 4, 288), ([6000] * 4, 4, 288),
+                                       ([5102, 1819, 1520], 4, 296), ([1500] * 12, 1, 288), ([2500] * 8, 1, 256), ([300] * 32, 1, 256)])
+def test_one_wave_of_small_blocks_fills_the_half_sms(P, q, items):
+    """Two CTAs per SM: as many splits as are one wave, in steps of a page."""
+    ln, = plan(P, [q] * len(P)).launches
+    assert ln.kw == 4 and ln.items == items <= 296
