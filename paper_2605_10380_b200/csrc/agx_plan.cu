@@ -24,18 +24,19 @@ struct SplitModel {
     double base, per_add, per_min, per_busy;
     double merge, merge_mb, merge_mb_beyond_16;   // merge launch, per MB of partials up to 16 (they stay in L2) and beyond
     int part_row_bytes;
-    bool lean;              // one-wave launches with few (row, head) pairs leave SMs to their merge kernel: 1 + 0.2 per MB
+    double lean;            // > 0: one-wave launches with few (row, head) pairs leave SMs to their merge kernel, which costs this and 0.2 per MB
 };
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
-SplitModel tile_model(const PlanConfig& c) { return {128, c.sm_count, 3, 5.7, 0, 1.9, 0, 2.2, 0.38, 0.3, 264, false}; }
-// (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them)
+SplitModel tile_model(const PlanConfig& c) { return {128, c.sm_count, 3, 5.7, 0, 1.9, 0, 2.2, 0.38, 0.3, 264, 0}; }
+// (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them.  40 rows over 300 / 450 / 600
+// tokens, 40/8 heads, take 9.0 / 9.8 / 10.5 us whole and 10.5 / 10.1 / 9.9 in splits of 256 tokens: the merge behind two tiles costs as much as two)
 SplitModel stream_model(const PlanConfig& c, bool wide) {
-    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, true};
+    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, wide ? 2.2 : 1.0};
 }
 // warp-MMA kernel with 4-page stages, two CTAs per SM: HBM-bound with one 16-row tile, bounded by its own chain with two (mma.sync)
 SplitModel small4_model(const PlanConfig& c, int mt) {
-    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, false};
+    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, 0};
 }
 
 // Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time, and that time.  A server's lengths change with every
@@ -114,7 +115,7 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         cd.tiles = t;
         cd.longest = longest;
         cd.sum = sum;
-        cd.merge = mb == 0 ? 0 : md.lean && count <= sms * 15 / 16 && pairs <= 3 * sms ? 1.0 + 0.2 * mb
+        cd.merge = mb == 0 ? 0 : md.lean > 0 && count <= sms * 15 / 16 && pairs <= 3 * sms ? md.lean + 0.2 * mb
                    : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
                    : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
         cd.bound = md.base + cd.merge + std::max((load - kOverhead) * (md.per_add + md.per_min),

@@ -94,3 +94,9 @@ def test_one_wave_of_small_blocks_fills_the_half_sms(P, q, items):
     """Two CTAs per SM: as many splits as are one wave, in steps of a page."""
     ln, = plan(P, [q] * len(P)).launches
     assert ln.kw == 4 and ln.items == items <= 296
+
+
+def test_three_tiles_of_a_wide_block_are_not_split():
+    for q, hq, hkv in ((5, 16, 2), (8, 16, 2), (8, 40, 8)):
+        assert plan([300], [q], hq, hkv).launches[0].seqs[0].nsplit == 1
+        assert plan([1000], [q], hq, hkv).launches[0].seqs[0].nsplit == 4
