@@ -313,6 +313,10 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         int C = min_split, kw = k == KIND_SMALL4 ? 4 : small_kw;
         if (k != KIND_TILE && k != KIND_STREAM && !(small_kind && kw == 4)) {
             C = one_wave_split(c, seqs, P, Q, G, rows_per_chunk, unit, min_split, target, k != KIND_SIMT);
+            // fp32-arithmetic kernel: a CTA's tiles are a chain of 2.5-8 us each, so that where one wave would take chains of more than eight, several
+            // waves of four are faster (32/8 heads, fp32, d 128 / 64: one row over 20000 + 30 x 40 tokens 364 -> 107 / 200 -> 62 us, 6 x 8000
+            // 330 -> 201 / 185 -> 113; in chains of eight 16 x 1000 74 / 41 us, of four 79 / 45)
+            if (k == KIND_SIMT && C > 512) C = std::min(C, one_wave_split(c, seqs, P, Q, G, rows_per_chunk, unit, 256, 16 * c.sm_count, false));
             // several verify blocks whose splits no SM holds whole: two CTAs per SM with 4-page stages where the lengths are alike (7 x 1000
             // tokens 14.3 -> 12.3 us, 8 x 900 14.3 -> 11.8, 2 x 3500 12.5 -> 11.4, 3700 + 3900 12.7 -> 12.3; but 1500 + 2500 + 3500 12.9 -> 13.4.
             // Up to 16 rows: 7 x 1000 10.7 / 11.4, 8 x 900 10.8 / 10.2)

@@ -100,3 +100,11 @@ def test_three_tiles_of_a_wide_block_are_not_split():
     for q, hq, hkv in ((5, 16, 2), (8, 16, 2), (8, 40, 8)):
         assert plan([300], [q], hq, hkv).launches[0].seqs[0].nsplit == 1
         assert plan([1000], [q], hq, hkv).launches[0].seqs[0].nsplit == 4
+
+
+def test_chains_of_the_fp32_kernel_are_bounded():
+    """Tiles of 64 tokens per CTA where a launch is a few waves; what fills the GPU unsplit stays so."""
+    def longest(P, Q):
+        return max(s.split_tokens for l in plan(P, Q, dtype="f32", hq=32, hkv=8).launches for s in l.seqs)
+    assert longest([20000] + [40] * 30, [1] * 31) <= 256 and longest([8000] * 6, [1] * 6) <= 256 and longest([1000] * 16, [1] * 16) == 512
+    assert plan([0], [4000], dtype="f32", hq=32, hkv=8).launches[0].seqs[0].nsplit == 1
