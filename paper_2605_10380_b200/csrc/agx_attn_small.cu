@@ -988,12 +988,14 @@ cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CU
                                    cudaStream_t stream) {
     if (p.num_items == 0) return cudaSuccess;
     int longest = 0, rows = 0;
+    bool one_chunk = true;
     for (int i = 0; i < p.num_seqs; ++i) {
         longest = std::max(longest, p.seq[i].split_tokens);
         rows = std::max(rows, std::min(p.seq[i].q_len * p.gqa, 16 * mt));
+        one_chunk &= p.seq[i].row_chunks == 1;
     }
     // splits that fit one CTA whole (figures there)
-    if (kw == 8 && mt <= 2 && longest <= kSwapMaxTokens) return launch_attn_swap(p, rows, longest, map_k, map_v, stream);
+    if (kw == 8 && mt <= 2 && one_chunk && longest <= kSwapMaxTokens) return launch_attn_swap(p, rows, longest, map_k, map_v, stream);
     if (mt == 2 && kw == 8 && two_tiles_per_warp()) return launch_small<2, 8, 3, 2>(p, map_k, map_v, stream);
     switch (mt * 16 + kw) {
         case 1 * 16 + 4: return launch_small<1, 4, 3>(p, map_k, map_v, stream);

@@ -131,7 +131,7 @@ cudaError_t launch_kv_append(int dtype, void* k_pool, void* v_pool, long long nu
 int attn_small_max_clusters(int mt, int kw, int cluster);
 cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                    cudaStream_t stream);
-// The same blocks (at most `rows` = 16 or 32 query rows per KV head and CTA) where no split is longer than kSwapMaxTokens.
+// The same blocks (at most `rows` = 16 or 32 query rows per KV head and CTA) of one row chunk, where no split is longer than kSwapMaxTokens.
 constexpr int kSwapMaxTokens = 384;
 cudaError_t launch_attn_swap(const AttnParams& p, int rows, int longest, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream);
 // fp32-math kernel (agx_attn_simt.cu) for AGX_F32 pools (any q, d in {64, 128}) and for AGX_BF16 pools with d = 64.
