@@ -87,8 +87,9 @@ static __device__ __noinline__ void zero_v_tail(unsigned char* v_page, int from,
 
 // MW = m-tiles per warp: with MW = 2 a warp scores its page against both 16-row tiles of a 32-row block and accumulates
 // both tiles' output columns, so every K and V fragment is read from shared memory once instead of twice.
-// kAppend = the block's rows come from k_new / v_new; two kernels, because what only one form needs costs the other 2-4 % wherever it stands.
-template <int MT, int KW, int NS, int MW, bool kAppend>
+// kByHand: pages that cannot come by TMA as they are, see own_pg below; two kernels, because what only one form needs costs the other 2-4 %
+// wherever it stands.
+template <int MT, int KW, int NS, int MW, bool kByHand>
 __global__ void __launch_bounds__(32 * (MT / MW) * KW, ((MT / MW) * KW <= 8 && MW == 1) ? 2 : 1)
 attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k,
                        const __grid_constant__ CUtensorMap map_v) {
@@ -157,14 +158,14 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     // launch still in flight) the producer warp fetches page ids and K/V stages that lie wholly inside the cached prefix before
     // the dependency wait, i.e. while the launch in front drains.
     const bool pre = p.early_prefix;
-    // With a fused append the pages from own_pg on (counted from the split's first page), which hold block rows, are put together by hand, beside
-    // the Q tile: the rows come from k_new / v_new and go into the pool on the way.  They are at the end of the sequence, and a split's stages are
-    // worked off from its end, so they are always among the first in the ring.  Without an append every page comes from the pool by TMA, the last
-    // one too, although what lies behind the last token may be anything and V has to be zero there: a page of a cold pool fetched by hand holds
-    // the whole CTA up (one layer, 48 x (300, 1) 18.2 us by TMA, 23.1 by hand; 12 x (1000, 4) 12.0 / 14.9).
-    const int pool_end = kAppend ? P : (L + kPage - 1) & ~(kPage - 1);
+    // kByHand: the pages from own_pg on (counted from the split's first page) are put together by hand, beside the Q tile: with a fused append
+    // those that hold block rows, which come from k_new / v_new and go into the pool on the way; otherwise a last page that is only partly valid
+    // (what lies behind the last token may be anything, and V has to be zero there).  They are at the end of the sequence, and a split's stages are
+    // worked off from its end, so they are always among the first in the ring.  A page of a cold pool fetched by hand holds the whole CTA up, so
+    // that without an append short splits take the other form: every page by TMA, the last one's tail zeroed when it has arrived.
+    const int pool_end = !kByHand ? (L + kPage - 1) & ~(kPage - 1) : p.k_new ? P : L;
     const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
-    const int own_units = kAppend ? (n_pages - own_pg) * 512 : 0;   // 16-byte units, [page][K, V][16 rows][16 units]
+    const int own_units = kByHand ? (n_pages - own_pg) * 512 : 0;   // 16-byte units, [page][K, V][16 rows][16 units]
     constexpr int kLoaders = kThreads - 32;           // all warps but the producer's
     constexpr int kOwn = (512 + kLoaders - 1) / kLoaders;   // a thread's units of the first own page
     auto own_id = [&](int u) { const int slot = page0 + own_pg + (u >> 9); return slot < p.pt_stride ? __ldg(pt_row + slot) : -1; };
@@ -193,9 +194,9 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         for (int j = 0; j < kOwn; ++j)
             if (tid >= 32 && tid - 32 + j * kLoaders < own_units) first_id[j] = own_id(tid - 32 + j * kLoaders);
     };
-    if (kAppend && pre) fetch_own_ids();         // (the caller vouches for the page table too)
+    if (kByHand && pre) fetch_own_ids();         // (the caller vouches for the page table too)
     if (!(warp == 0 && pre)) pdl_wait();   // from here on global memory written by the launch before this one is read
-    if (kAppend && !pre) fetch_own_ids();
+    if (kByHand && !pre) fetch_own_ids();
     // ---- producer state (warp 0; lane 0 issues the TMA copies).  Page ids are fetched 32 at a time,
     //      one group ahead, so the page-table latency never sits in front of a copy.
     int ids_cur = 0, ids_next = 0, group_cur = max(0, (n_stages - 1) * kKW) >> 5;
@@ -258,7 +259,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 #pragma unroll 1
         for (int s = 0; s < NS - 1; ++s) {
             // (with a fused append only pages below stable_end come from the pool)
-            if (!waited && !kAppend && tok_begin + (n_stages - s) * kStageTokens > stable_end) { pdl_wait(); waited = true; }
+            if (!waited && !p.k_new && tok_begin + (n_stages - s) * kStageTokens > stable_end) { pdl_wait(); waited = true; }
             produce(s);
         }
         if (!waited) pdl_wait();
@@ -280,7 +281,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         }
         // own pages: their loads go out behind Q's, before anything is stored
         uint4 w[kOwn];
-        if constexpr (kAppend) {
+        if constexpr (kByHand) {
 #pragma unroll
         for (int j = 0; j < kOwn; ++j)
             if (tid - 32 + j * kLoaders < own_units) w[j] = own_load(tid - 32 + j * kLoaders, first_id[j]);
@@ -297,7 +298,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     }
     __syncthreads();  // barriers initialised, Q tile visible
     // The last page of the sequence is in the first stage to be worked off; the warps that score it zero what lies behind the last token.
-    if (!kAppend && pool_end > L && n_pages > 0 && kg == n_pages - 1 - (n_stages - 1) * kKW && tok_begin + n_pages * kPage > L)
+    if (!kByHand && pool_end > L && n_pages > 0 && kg == n_pages - 1 - (n_stages - 1) * kKW && tok_begin + n_pages * kPage > L)
         zero_v_tail(ring + kStageTokens * kRowBytes + kg * 4096, L & (kPage - 1), full_bar(0), abort_flag, p.status, p.wait_limit_cycles);
 
     uint32_t qa[MW][8][4];
@@ -914,7 +915,7 @@ constexpr int small_smem_bytes() {
     return (kRing > kClusterBytes ? kRing : kClusterBytes) + MT * 16 * kRowBytes + 2 * NS * 8 + 16 + kExchange + 1024;
 }
 
-template <int MT, int KW, int NS, int MW, bool kAppend>
+template <int MT, int KW, int NS, int MW, bool kByHand>
 cudaError_t launch_form(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
     constexpr int kSmem = small_smem_bytes<MT, KW, NS>();
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
@@ -923,21 +924,29 @@ cudaError_t launch_form(const AttnParams& p, const CUtensorMap& map_k, const CUt
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
     bool& configured = configured_on[device];
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, kAppend>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        cudaError_t e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, kByHand>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, kAppend>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+        e = cudaFuncSetAttribute(attn_small_bf16_kernel<MT, KW, NS, MW, kByHand>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
         if (e != cudaSuccess) return e;
         configured = true;
     }
     if (p.cluster_size > 1)
-        return launch_chained_cluster(attn_small_bf16_kernel<MT, KW, NS, MW, kAppend>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem,
+        return launch_chained_cluster(attn_small_bf16_kernel<MT, KW, NS, MW, kByHand>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem,
                                       (unsigned)p.cluster_size, stream, p, map_k, map_v);
-    return launch_chained(attn_small_bf16_kernel<MT, KW, NS, MW, kAppend>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem, stream, p, map_k, map_v);
+    return launch_chained(attn_small_bf16_kernel<MT, KW, NS, MW, kByHand>, dim3(p.num_items), dim3(32 * (MT / MW) * KW), kSmem, stream, p, map_k, map_v);
 }
 
 template <int MT, int KW, int NS, int MW = 1>
 cudaError_t launch_small(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    return p.k_new ? launch_form<MT, KW, NS, MW, true>(p, map_k, map_v, stream) : launch_form<MT, KW, NS, MW, false>(p, map_k, map_v, stream);
+    // Without an append, splits of up to 512 tokens on two CTAs per SM by TMA alone: one layer, 48 x (300, 1) 23.0 -> 18.2 us, 12 x (1000, 4)
+    // 14.9 -> 12.0, 24 x (1000, 1) 24.6 -> 23.1; a longer chain hides the trip (24 x (6000, 1) 121 by hand, 125 the other way), and so does the one
+    // CTA of an SM with 8-page stages (one row over 8000 10.1 / 10.6, over 12000 12.4 / 12.9).
+    if constexpr (KW == 4) {
+        int longest = 0;
+        for (int i = 0; i < p.num_seqs; ++i) longest = std::max(longest, p.seq[i].split_tokens);
+        if (!p.k_new && longest <= 512) return launch_form<MT, KW, NS, MW, false>(p, map_k, map_v, stream);
+    }
+    return launch_form<MT, KW, NS, MW, true>(p, map_k, map_v, stream);
 }
 
 template <int MT, int KW, int NS, int MW = 1>
