@@ -137,13 +137,11 @@ AGX_API int64_t agx_attn_workspace_bytes(agx_handle* handle, int32_t B, const in
  *                  scaled scores
  *   workspace    : device, >= agx_attn_workspace_bytes(...) bytes, 256-byte aligned (may be NULL
  *                  when that figure is 0)
- * Dispatch (G = num_q_heads / num_kv_heads; bf16 handles with head_dim 128 - other handles run the scalar kernel): up to 32 query rows per KV head (q_len * G) over a context
- * shorter than about 7k tokens (10k for q_len * G <= 8) run the split-KV warp-MMA kernel (latency-bound); up to 32 rows over a
- * longer context, or 33..128 rows over any context, run the tensor-core kernel with one padded Q tile
- * whose KV tiles alternate between two softmax warpgroups (HBM-bound); longer blocks run the
- * tensor-core kernel with 256-row tiles (tensor-bound).  Sequences of all kinds may share a batch; two or
- * more blocks of at most 32 rows whose contexts add up to 24576 tokens or more (at 8 KV heads) all take the
- * padded-tile kernel, whatever their single lengths.
+ * Dispatch (G = num_q_heads / num_kv_heads; bf16 handles with head_dim 128 - other handles run the fp32-arithmetic kernel): up to 32 query rows
+ * per KV head (q_len * G) run a split-KV kernel (latency-bound; tcgen05 with swapped operands where one wave of KV splits of at most 384 tokens
+ * covers the launch, warp MMAs otherwise) or, all of a batch together, the tensor-core kernel with one padded Q tile whose KV tiles alternate
+ * between two softmax warpgroups (HBM-bound), whichever an estimate of the launch gives the shorter time; 33..384 rows run the latter in
+ * chunks of 128 rows, longer blocks the tensor-core kernel with 256-row tiles (tensor-bound).  Sequences of all kinds may share a batch.
  * Errors: AGX_E_INVAL (null/misaligned, q_len < 1, prefix_len < 0, workspace too small),
  * AGX_E_RANGE ((P + q) exceeds 16 * page_table_stride), AGX_E_CUDA.  Page ids outside
  * [0, num_pages) set AGX_DEV_BAD_PAGE and read as zeros.

@@ -82,12 +82,19 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tile = warp >> 2;
     const bool issuer = warp == kWarps;
     const SeqPlan& sp = p.seq[find_seq(p, blockIdx.x)];
-    const unsigned item = blockIdx.x - sp.item0;   // g * nsplit + split (blocks of one row chunk only)
-    const int g = (int)(item / (unsigned)sp.nsplit), split = (int)(item - (unsigned)g * sp.nsplit);
+    // Items are ((g * row_chunks) + rc) * nsplit + split.  The planner sends blocks of one row chunk only, but the kernel keeps the general form:
+    // with the chunk's first row a constant 0 the compiler's schedule costs a verify layer over 4096 tokens 0.16 us (9.1 -> 9.3 us with its append,
+    // three forms of it tried) and gives a decode layer 0.04 us.
+    const unsigned item = blockIdx.x - sp.item0;
+    const unsigned chunk = item / (unsigned)sp.nsplit;
+    const int split = (int)(item - chunk * sp.nsplit);
+    const int g = sp.row_chunks == 1 ? (int)chunk : (int)(chunk / (unsigned)sp.row_chunks);
+    const int rc = (int)chunk - g * sp.row_chunks;
     const int G = p.gqa, P = sp.prefix_len, q = sp.q_len, L = P + q;
-    const int n_rows = q * G;   // query rows of this KV head, r = i * G + (h % G); at most NR
+    const int rows = q * G, row0 = rc * NC, n_rows = min(NR, rows - row0);   // query rows of this KV head, r = i * G + (h % G)
     auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div_magic) >> 32); };   // r / G without the division
-    const int tok_begin = split * sp.split_tokens, tok_end = min(L, tok_begin + sp.split_tokens);
+    const int vis_end = P + min(q - 1, div_g(row0 + NC - 1)) + 1;   // tokens the chunk's last row sees
+    const int tok_begin = split * sp.split_tokens, tok_end = min(vis_end, tok_begin + sp.split_tokens);
     const int n_pages = max(0, (tok_end - tok_begin + kPage - 1) / kPage), n_tiles = (n_pages + 7) >> 3;
 
     // ---- setup.  With p.early_prefix (the caller vouches that the page table and the pages below the cached-prefix length are not written by a
@@ -170,7 +177,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             const int c = tid + j * kThreads, r = c >> 4;
             v[j] = make_uint4(0, 0, 0, 0);
             if (c < kUnits && r < n_rows) {
-                const int i = div_g(r), hd = g * G + r - i * G;
+                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
                 v[j] = __ldg((const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16));
             }
         }
@@ -252,7 +259,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         tmem_ld<NR>(tmem + lanes + 32 + 32 * tile, (uint32_t*)s);
         tmem_wait_ld();
         if (tok_begin + t_warp + 31 > P || tok_begin + t_warp + 32 > tok_end) {   // rows below `lo` do not see this token
-            const int lo = tok >= tok_end ? NR : (tok - P) * G;
+            const int lo = tok >= tok_end ? NR : (tok - P) * G - row0;
 #pragma unroll
             for (int r = 0; r < NR; ++r) if (r < lo) s[r] = -INFINITY;
         }
@@ -317,7 +324,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (tile < 2) {
         unsigned long long dst = 0;
         if (my_row < n_rows && !merged_here) {
-            const int i = div_g(my_row), hd = g * G + my_row - i * G;
+            const int i = div_g(row0 + my_row), hd = g * G + (row0 + my_row) - i * G;
             if (sp.nsplit == 1) {
                 const long long at = (long long)(sp.q_row0 + i) * p.hq + hd;
                 dst = (unsigned long long)((unsigned char*)p.out + at * 256);
@@ -381,7 +388,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
     }
-    if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, 0, n_rows);   // (uniform over the cluster)
+    if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
 }
 
 namespace {
