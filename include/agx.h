@@ -79,7 +79,7 @@ enum {
 typedef struct agx_config {
     int32_t num_q_heads;  /* Hq */
     int32_t num_kv_heads; /* Hkv, divides Hq */
-    int32_t head_dim;     /* d: 64 or 128 (AGX_BF16 with 64 and AGX_F32 run a scalar fp32 kernel: a correctness path) */
+    int32_t head_dim;     /* d: 64 or 128 (AGX_BF16 with 64 and AGX_F32 run a kernel of fp32 arithmetic, without tensor cores) */
     int32_t page_size;    /* must be 16 */
     int32_t dtype;        /* AGX_BF16 or AGX_F32 */
     float scale;          /* softmax scale; 0 selects 1/sqrt(head_dim) */

@@ -31,7 +31,7 @@ __device__ __forceinline__ float bf16_bits_to_float(unsigned int lo16) { return 
 // Running maximum of one thread over 16-byte vectors met in ascending order.  A vector costs a packed maximum of its elements and one
 // comparison (NaN operands lose, and a NaN result compares false); only a vector that beats the maximum is kept, and which of its
 // elements it was is worked out once at the end.  Ordering every element by an integer key instead took eight instructions each and
-// bounded the scan of many rows (8 / 32 / 256 rows of 128256 bf16: 6.2 / 7.7 / 26.3 us before, 5.9 / 6.2 / 18.6 now).
+// bounded the scan of many rows (32 / 256 rows of 128256 bf16: 7.2 / 27.2 us before, 6.1 / 19.5 now; 8 rows 5.2).
 template <bool kBf16>
 struct VecMax {
     float best = -INFINITY;

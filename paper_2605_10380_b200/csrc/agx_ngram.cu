@@ -87,7 +87,8 @@ __global__ void ngram_select_kernel(const unsigned long long* __restrict__ win_k
 
 constexpr int kClusterCtas = 16, kClusterThreads = 1024, kPerThread = 2;
 // GPU time of one launch against the chain of launches in a graph, streams of recurring phrases: 300 tokens 4.2 / 13.2 us, 4096 6.8 / 11.2,
-// 16384 10.2 / 12.9, 40000 22 / 12.3; host time 2.7 against 17.7 us.
+// 16384 10.2 / 12.9, 40000 22 / 12.3; host time 2.7 against 17.7 us.  (Windows that nearly all differ claim a slot each: over 4096 uniformly
+// random tokens one launch takes 17.8 us.)
 constexpr int kClusterWindows = kClusterCtas * kClusterThreads * kPerThread;
 
 __global__ void __launch_bounds__(kClusterThreads)

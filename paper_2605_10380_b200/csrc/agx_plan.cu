@@ -213,10 +213,13 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
     }
     plan.total_rows = row0[B];
     // Blocks of at most 32 rows go to the warp-MMA kernel or to the one-Q-tile tensor-core schedule, all of a batch together: to the one whose
-    // estimate is lower (SplitModel; for the warp-MMA kernel with 8-page stages, one CTA per SM, k tokens at 8 KV heads take 4.1 + 0.69 k up
-    // to 16 rows, 5.6 + 0.8 k above in splits that an SM holds whole, max(8.8, 5.8 + 1.06 k) otherwise).  What it decides against the fixed
-    // thresholds it replaces (24576 tokens in all; 7168 / 10240 for one sequence): 32 decode blocks over 1000 tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over
-    // 20000 20.5 -> 17.5, 32 verify blocks over 1500 53 -> 43; 8 verify blocks over 8000 stay at 50 (55 the other way).
+    // estimate is lower (SplitModel; for the small-q kernels with 8-page stages, one CTA per SM, k thousand tokens at 8 KV heads take
+    // 4.1 + 0.69 k us up to 16 rows, 5.6 + 0.8 k above in splits that an SM holds whole, max(8.8, 5.8 + 1.06 k) otherwise.  The ground of these
+    // lines is narrow: one to eight blocks with 32/8 heads, where one block over 1000-12000 tokens takes up to 0.9 us less or more than they say;
+    // other KV head counts only scale k.  7.9: on 148 SMs, from about there two CTAs per SM with 4-page stages are the faster form for several blocks).
+    // What it decides against the fixed thresholds it replaces (24576 tokens in all; 7168 / 10240 for one sequence): 32 decode blocks over 1000
+    // tokens 38.3 -> 25.3 us, 24 over 2000 54 -> 43, 16 over 4000 48.3 -> 46, one over 20000 20.5 -> 17.5, 32 verify blocks over 1500 53 -> 43;
+    // 8 verify blocks over 8000 stay at 50 (55 the other way).
     double small_k = 0;
     int small_rows = 0;
     std::vector<int> small_seqs, wide_seqs;   // up to 32 rows | others that take the schedule in any case
@@ -252,7 +255,8 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             }
             std::vector<int> all = wide_seqs;
             all.insert(all.end(), small_seqs.begin(), small_seqs.end());
-            // (with one 16-row tile the warp-MMA kernel was never more than 2 % slower than the schedule, also where the estimates tie)
+            // (with one 16-row tile the warp-MMA kernel was never more than 2 % slower than the schedule in the sweeps of equal and ragged decode
+            // batches behind the models, though its estimate is up to 15 % higher there: 0.87 takes that out)
             if (!one && small_k >= 7.9 && small_rows <= 16) warp_mma *= 0.87;
             const SplitModel sm = stream_model(c, !wide_seqs.empty());
             if (!wide_seqs.empty() || warp_mma > sm.base) {   // (no launch of the schedule is estimated below its base)
@@ -389,7 +393,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         }
         // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, with fp32 partials, are faster than 17 to 24 with SMs left to
         // the merge of fp16 rows (32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
-        // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).
+        // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).  (All of it from 14 shapes.)
         if (whole && !cluster && !memory_merge && seqs.size() == 1 && c.merge_sms && (k == KIND_SMALL2 || count_items(C) * 2 > c.sm_count)) {
             const int L = P[seqs[0]] + Q[seqs[0]], longer = std::max(320, round_up((L + 15) / 16, unit));
             if (ceil_div(L, C) > 16 && longer <= kSwapMaxTokens) { C = std::max(C, longer); memory_merge = true; }
