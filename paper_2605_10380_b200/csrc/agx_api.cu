@@ -265,7 +265,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     if (h->cfg.dtype == AGX_BF16 && h->cfg.head_dim == 128) {
         if ((long long)num_pages * p.hkv * kPage > 0x7FFFFFFFll) return fail(h, AGX_E_RANGE, "pool too large for one tensor map");
         bool ok = make_pool_map(&map_k, k_pool, num_pages, p.hkv) && make_pool_map(&map_v, v_pool, num_pages, p.hkv);
-        if (ok && k_new && plan.tensor_core) ok = make_rows_maps(&maps_new, k_new, v_new, plan.total_rows, p.hkv);
+        if (ok && k_new && plan.tensor_core) ok = make_rows_maps(&maps_new, k_new, v_new, plan.total_rows, k_pool, v_pool, num_pages, p.hkv);
         else if (plan.tensor_core) memset(&maps_new, 0, sizeof maps_new);
         if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
@@ -281,7 +281,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         }
         cudaError_t e;
         p.cluster_size = ln.cluster;
-        p.part_half = ln.kind == KIND_TILE || ln.lean_merge;
+        p.part_half = ln.kind == KIND_TILE ? PART_HALF_TILES : ln.lean_merge ? PART_HALF_SLOTS : PART_F32;
         p.k_new = p.v_new = nullptr;
         if (k_new) {
             p.k_new = k_new; p.v_new = v_new;
@@ -297,8 +297,17 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
             case KIND_SMALL2: e = launch_attn_small_bf16(p, 2, ln.kw, map_k, map_v, stream); break;
             case KIND_SMALL4: e = launch_attn_small_bf16(p, 4, 4, map_k, map_v, stream); break;
             case KIND_SIMT: e = launch_attn_simt(p, h->cfg.dtype, stream); break;
-            case KIND_TILE: e = launch_attn_tile_bf16(p, false, map_k, map_v, maps_new, stream); break;
-            case KIND_STREAM: e = launch_attn_tile_bf16(p, true, map_k, map_v, maps_new, stream); break;
+            case KIND_TILE:
+            case KIND_STREAM: {
+                // Q boxes: as many tokens as a 128-row tile holds from any row on, and no more than a block of the launch has
+                int longest = 1;
+                for (const SeqPlan& sp : ln.seqs) longest = std::max(longest, sp.q_len);
+                const int fit = p.gqa > 128 ? 0 : 128 % p.gqa == 0 ? 128 / p.gqa : (129 - p.gqa) / p.gqa;
+                if (!make_q_maps(&maps_new, p.q, plan.total_rows, p.hq, p.hkv, std::min(fit, longest)))
+                    return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
+                e = launch_attn_tile_bf16(p, ln.kind == KIND_STREAM, map_k, map_v, maps_new, stream);
+                break;
+            }
             default: return fail(h, AGX_E_UNSUPPORTED, "unknown kernel kind");
         }
         if (e != cudaSuccess) return cuda_fail(h, e, "attention launch");

@@ -589,19 +589,24 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 // One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
 // kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel takes more).  Four O rows per
 // warp instead of 32 keep the register count low enough for ten CTAs per SM, which is what the partials of a split prefill need.
-// kHalfPart: the partial rows are fp16 and already divided by their own sums l_k (the 256-row tensor-core schedule), so
-// split k weighs l_k 2^(m_k - m) instead of 2^(m_k - m).
-template <bool kHalfPart>
-__device__ __forceinline__ float4 load_part4(const AttnParams& p, long long entry, int c4) {
-    if (kHalfPart) {
-        const uint2 raw = ld_volatile_u2((const unsigned char*)p.part_o + entry * 512 + c4 * 2);   // written by other SMs just before: past the L1
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-        return make_float4(a.x, a.y, b.x, b.y);
+// Where the fp16 partials of row i, head h lie: split 0's, at this lane's four columns, and the bytes from split to split.
+struct HalfRows {
+    const unsigned char* at;
+    int stride;
+    __device__ __forceinline__ HalfRows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane) {
+        if (p.part_half == PART_HALF_TILES) {
+            const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rl = r & 255;
+            at = (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 +
+                 rl * 256 + (((lane >> 1) ^ (rl & 15)) << 4) + (lane & 1) * 8;
+            stride = 65536;
+        } else {
+            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + lane * 8;
+            stride = 512;
+        }
     }
-    return ld_volatile_f4(p.part_o + entry * p.head_dim + c4);
-}
-template <bool kBf16Out, int kMaxNs, bool kHalfPart>
+    __device__ __forceinline__ uint2 load(int split) const { return ld_volatile_u2(at + (long long)split * stride); }   // (written by other SMs just before: past the L1)
+};
+template <bool kBf16Out, int kMaxNs>
 __global__ void __launch_bounds__(128, kMaxNs <= 4 ? 10 : kMaxNs <= 16 ? 5 : 3)
 attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     constexpr bool kFew = kMaxNs <= 16;          // no second batch of 16 rows
@@ -637,18 +642,18 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     float4 v[kInFlight], v2[kFew ? 1 : 16];
 #pragma unroll
     for (int j = 0; j < kInFlight; ++j)
-        if (j < ns && c4 < D) v[j] = load_part4<kHalfPart>(p, e0 + j, c4);
+        if (j < ns && c4 < D) v[j] = ld_volatile_f4(p.part_o + (e0 + j) * D + c4);
     if (!kFew && ns > 16) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-            if (16 + j < ns && c4 < D) v2[j] = load_part4<kHalfPart>(p, e0 + 16 + j, c4);
+            if (16 + j < ns && c4 < D) v2[j] = ld_volatile_f4(p.part_o + (e0 + 16 + j) * D + c4);
     }
     m_all = ml.x;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
     const float e_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
     l_all = ml.y * e_mine;
-    const float w_mine = kHalfPart ? l_all : e_mine;   // weight of this lane's split's O row
+    const float w_mine = e_mine;   // weight of this lane's split's O row
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);
 #pragma unroll
@@ -705,6 +710,7 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     const int ns = sp.nsplit, D = p.head_dim, c4 = lane * 4, i = lrow - acc_rows;
     if (ns == 1) return;   // written directly by the attention kernel
     const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
+    const HalfRows rows(p, sp, i, h, lane);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m = -INFINITY, l = 0.f;
     pdl_wait();   // the partials are complete
@@ -715,7 +721,15 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         float4 v[kManyBatch];
 #pragma unroll
         for (int j = 0; j < kManyBatch; ++j)
-            if (j < n && c4 < D) v[j] = load_part4<kHalfPart>(p, e0 + k0 + j, c4);
+            if (j < n && c4 < D) {
+                if (kHalfPart) {
+                    const uint2 raw = rows.load(k0 + j);
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
+                    v[j] = make_float4(a.x, a.y, b.x, b.y);
+                } else {
+                    v[j] = ld_volatile_f4(p.part_o + (e0 + k0 + j) * D + c4);
+                }
+            }
         float m_new = ml.x;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xFFFFFFFFu, m_new, off));
@@ -778,11 +792,12 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
     const int stride = gridDim.x * 4;
     const int rh0 = blockIdx.x * 4 + (threadIdx.x >> 5);
     long long e0[kCombineRows], out_off[kCombineRows];
-    int ns[kCombineRows];
+    const unsigned char* rows[kCombineRows];
+    int ns[kCombineRows], stride_bytes[kCombineRows];
 #pragma unroll
     for (int j = 0; j < kCombineRows; ++j) {
         const int rh = rh0 + j * stride;
-        ns[j] = 0; e0[j] = 0; out_off[j] = 0;
+        ns[j] = 0; e0[j] = 0; out_off[j] = 0; rows[j] = nullptr; stride_bytes[j] = 0;
         if (rh < n_pairs) {
             const int lrow = rh / p.hq, h = rh - lrow * p.hq;
             int si = 0, acc_rows = 0;
@@ -797,6 +812,8 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
                 ns[j] = sp.nsplit;
                 e0[j] = (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit;
                 out_off[j] = (long long)(sp.q_row0 + i) * p.hq + h;
+                const HalfRows hr(p, sp, i, h, lane);
+                rows[j] = hr.at; stride_bytes[j] = hr.stride;
             }
         }
     }
@@ -809,7 +826,7 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
         if (lane < ns[j]) ml[j] = ld_volatile_f2(p.part_ml + e0[j] + lane);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (k < ns[j]) v[j][k] = ld_volatile_u2((const unsigned char*)p.part_o + (e0[j] + k) * 512 + lane * 8);
+            if (k < ns[j]) v[j][k] = ld_volatile_u2(rows[j] + k * stride_bytes[j]);
     }
 #pragma unroll
     for (int j = 0; j < kCombineRows; ++j) {
@@ -867,7 +884,7 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
         const int i = lrow - acc_rows;
         const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
         const long long out_off = (long long)(sp.q_row0 + i) * p.hq + h;
-        const unsigned char* rows = (const unsigned char*)p.part_o + e0 * 512 + lane * 8;
+        const HalfRows rows(p, sp, i, h, lane);
         pdl_wait();   // the partials are complete
         // Every load is issued before the first use of any of them: volatile loads keep their place in the instruction stream
         // (left to itself the compiler moved the row loads behind the reduction of the maxima, i.e. behind a first trip to
@@ -875,7 +892,7 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
         // nothing below.
         uint2 v[kNsMax];
 #pragma unroll
-        for (int k = 0; k < kNsMax; ++k) v[k] = ld_volatile_u2(rows + min(k, ns - 1) * 512);
+        for (int k = 0; k < kNsMax; ++k) v[k] = rows.load(min(k, ns - 1));
         float2 ml = make_float2(-INFINITY, 0.f);
         if (lane < ns) ml = ld_volatile_f2(p.part_ml + e0 + lane);
         float m_all = ml.x;
@@ -1038,14 +1055,14 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
         return launch_chained(attn_combine_many_kernel<true, true>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
     }
     if (dtype == AGX_BF16) {
-        if (ns_max <= 4) return launch_chained(attn_combine_kernel<true, 4, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-        if (ns_max <= 16) return launch_chained(attn_combine_kernel<true, 16, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-        if (ns_max <= 32) return launch_chained(attn_combine_kernel<true, 32, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        if (ns_max <= 4) return launch_chained(attn_combine_kernel<true, 4>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        if (ns_max <= 16) return launch_chained(attn_combine_kernel<true, 16>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+        if (ns_max <= 32) return launch_chained(attn_combine_kernel<true, 32>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
         return launch_chained(attn_combine_many_kernel<true, false>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
     }
-    if (ns_max <= 4) return launch_chained(attn_combine_kernel<false, 4, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-    if (ns_max <= 16) return launch_chained(attn_combine_kernel<false, 16, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
-    if (ns_max <= 32) return launch_chained(attn_combine_kernel<false, 32, false>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+    if (ns_max <= 4) return launch_chained(attn_combine_kernel<false, 4>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+    if (ns_max <= 16) return launch_chained(attn_combine_kernel<false, 16>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
+    if (ns_max <= 32) return launch_chained(attn_combine_kernel<false, 32>, dim3(blocks), dim3(128), 0, stream, p, total_rows);
     return launch_chained(attn_combine_many_kernel<false, false>, dim3((unsigned)n), dim3(many_threads), 0, stream, p, total_rows);
 }
 

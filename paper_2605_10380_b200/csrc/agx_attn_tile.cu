@@ -28,12 +28,15 @@
 //               exponentials with packed f32x2 arithmetic, P written to TMEM as packed bf16 (the A
 //               operand of the P V MMA comes from TMEM), O rescaled in TMEM only when the row maximum
 //               grew by more than 2^8.
-// The Q tiles arrive by cp.async from warps 2-11 while warp 0 already streams K/V; results leave through
-// a per-warp shared-memory staging area so that global stores are whole rows.
+// The Q tiles arrive by TMA (warps 3 and 2) while warp 0 already streams K/V; results leave through a per-warp shared-memory staging area (the
+// Q tiles, dead by then): split partials as they lie there, one bulk copy a warp, finished rows as whole-row stores.  The block's own K/V rows go
+// from the tiles into the pool by TMA.  What a CTA does once runs at five clocks and more an instruction and counts as much as its tiles where these
+// are few (from the dependency wait to the first scores 3.1 -> 2.3 us, c3 29.2 -> 27.2 us, 3584 uncached tokens, 24/8 heads, 85.7 -> 79.9).
 // TMEM columns: S [0,128) P_A [128,192) P_B [192,256) O_A [256,384) O_B [384,512).
 // Every mbarrier wait is bounded: on time-out the CTA records AGX_DEV_WAIT_TIMEOUT and tears down.
 #include <cuda.h>
 #include <math.h>
+#include <string.h>
 
 #include "agx_internal.cuh"
 #include "agx_sm100.cuh"
@@ -83,7 +86,6 @@ enum { BAR_K_FULL = 0, BAR_K_EMPTY = 3, BAR_V_FULL = 6, BAR_V_EMPTY = 9, BAR_S_F
 // P is handed to the MMA warp in two parts: the first kPvHeadSteps k-steps (16 tokens each) as soon as they are
 // stored, so that their PV MMAs run while the softmax warpgroup still works on the last columns
 constexpr int kPvHeadSteps = 6;
-constexpr int kQLoadThreads = kThreads - 64;  // warps 2..11 bring the Q tiles in
 constexpr int kRegsLow = 96, kRegsHigh = 200; // 128 * 96 + 256 * 200 <= 384 * 168
 
 constexpr uint32_t kTmemCols = 512;
@@ -164,10 +166,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-
 // What one CTA works on, derived from its block index alone.
 struct TileItem {
     int g, G, P, q, rows, row0, split, nsplit, n_tiles, kv_begin, kv_end, vis_end, q_row0, seq_index;
@@ -177,7 +175,8 @@ struct TileItem {
 struct EpiCtx {
     TileItem it;
     int part_base, hq;
-    int part_half;   // split partials leave as fp16 rows divided by their own sums (always so on the 256-row schedule)
+    int part_half;   // a PartHalf
+    unsigned char* part_tile;   // 256-row schedule: this CTA's tile of fp16 partials
     void* out;
     float* part_o;
     float2* part_ml;
@@ -212,9 +211,8 @@ __device__ __forceinline__ TileItem locate_item(const AttnParams& p, int block) 
     return it;
 }
 
-// Epilogue of a softmax thread: the un-normalised fp32 O row leaves TMEM through this warp's 16 KB of
-// the (now idle) K/V rings, so that global stores are whole rows written by whole warps.  With a single
-// KV split the rows are normalised and written as bf16; otherwise fp32 partials and (m, l) go to the
+// Epilogue of a softmax thread: the O row leaves TMEM through this warp's 8 KB of the (now idle) Q tiles (256-row schedule).
+// With a single KV split the rows are normalised and written as bf16; otherwise partials and (m, l) go to the
 // workspace for the combine kernel.  Kept out of line, and re-deriving its indices from the block index,
 // so that nothing but its few arguments has to stay alive across the register-hungry main loop.
 template <bool kStreams>
@@ -258,7 +256,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
         m_ref = m_new;
     }
     if (!warp_has_rows) return;
-    unsigned char* stage = smem + kOffK + (warp - 4) * 16384;    // [32 rows][512 B], 16-byte units XOR-swizzled by row
+    unsigned char* stage = smem + kOffQ + (warp - 4) * 8192;     // [32 rows][256 B], 16-byte units XOR-swizzled by row (Q is dead)
     const int r_warp0 = it.row0 + (warp - 4) * 32;               // first row of this warp
     const uint64_t magic = cx.magic;                             // (row * magic) >> 32 == row / G exactly for rows < 2^22
     const bool single = it.nsplit == 1;
@@ -276,7 +274,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             } else {
                 const long long e = (long long)cx.part_base + ((long long)i * cx.hq + h) * it.nsplit + it.split;
                 cx.part_ml[e] = make_float2(m_ref, l_run);
-                row_dst = (unsigned long long)(cx.part_o + e * kD);
+                if (kStreams) row_dst = (unsigned long long)(cx.part_o + e * kD);
             }
         }
     }
@@ -286,8 +284,8 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     tc_fence_after();
     {
         uint32_t oreg[64];   // two 32-column chunks per TMEM round trip
-#pragma unroll
-        for (int c8 = 0; c8 < 4; c8 += 2) {
+#pragma unroll 1
+        for (int c8 = 0; c8 < 4; c8 += 2) {   // (code that runs once a CTA is fetched as it runs: not unrolled)
             tmem_ld_x32(tO + c8 * 32, oreg);
             tmem_ld_x32(tO + c8 * 32 + 32, oreg + 32);
             tmem_wait_ld();
@@ -302,7 +300,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                     oreg[4 * v + 3] = __float_as_uint(__uint_as_float(oreg[4 * v + 3]) * w_own + (w_other != 0.f ? o1.w * w_other : 0.f));
                 }
             }
-            const bool half_part = kStreams && !single && cx.part_half;
+            const bool half_part = kStreams && !single && cx.part_half != PART_F32;
             if (single || !kStreams || half_part) {   // (the 256-row schedule normalises its split partials too: they leave as fp16)
 #pragma unroll
                 for (int c = 0; c < 64; ++c) oreg[c] = __float_as_uint(__uint_as_float(oreg[c]) * inv);
@@ -352,10 +350,22 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
         }
     }
     if (kStreams) return;
+    const int n_valid = min(32, it.rows - r_warp0);
+    if (!single) {
+        // Split partials leave as they lie in the staging area, one bulk copy a warp: they are in a layout of their own, that of the staging
+        // area.  Row by row through the LSU to a slot per (row, head, split) took 1.4 us instead of 0.1.
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(cx.part_tile + (warp - 4) * 8192), "r"(smem_u32(stage)), "r"(n_valid * 256) : "memory");
+            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
+        }
+        return;
+    }
     __syncwarp();
     // a half-warp writes one 256-byte row per instruction (lane j moves 16-byte unit j % 16 of row 2 u + j / 16); eight
     // row pairs' loads are in flight before the first store
-    const int n_valid = min(32, it.rows - r_warp0);
     for (int rl0 = 0; rl0 < n_valid; rl0 += 16) {
         uint4 v[8];
 #pragma unroll
@@ -367,10 +377,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
         for (int u = 0; u < 8; ++u) {
             const int rl = rl0 + 2 * u + (lane >> 4);
             const unsigned long long dst = __shfl_sync(0xFFFFFFFFu, row_dst, rl & 31);
-            if (rl < n_valid) {
-                if (single) *(uint4*)((unsigned char*)dst + (lane & 15) * 16) = v[u];
-                else __stcg((uint4*)((unsigned char*)dst + (lane & 15) * 16), v[u]);   // split partial: read next by other SMs
-            }
+            if (rl < n_valid) *(uint4*)((unsigned char*)dst + (lane & 15) * 16) = v[u];
         }
     }
 }
@@ -378,11 +385,12 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
 // K or V of a tile that holds block rows or ends inside a page, by the whole producer warp.  Tokens [0, pool_end) come from the pool,
 // with a fused append the block's own from k_new / v_new: pages from the pool; a tile of nothing but block rows as one copy where
 // 128 rows are there; else row groups of 8 tokens from k_new / v_new; and by hand the groups that mix prefix and block or, for V,
-// reach beyond the last token (zeros: P is 0 there, but 0 * NaN is not).  Out of line: inlined twice into the producer's loop it cost the
-// other warps 7 % on a long prefill that never takes it (instruction fetch).
+// reach beyond the last token (zeros: P is 0 there, but 0 * NaN is not).  The copies are on their way before the loads by hand are waited for, and
+// with `waited` false (a fused append whose cached-prefix pages may be fetched early) those of the pool's pages before the dependency wait.
+// Out of line: inlined twice into the producer's loop it cost the other warps 7 % on a long prefill that never takes it (instruction fetch).
 __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* pool_map, const CUtensorMap* rows8, const CUtensorMap* rows128,
                                         const unsigned char* pool, const unsigned char* rows, bool is_v, int g, int P, int L, int q_row0,
-                                        unsigned char* dst, uint32_t full_bar, int tok0, int npg, int group) {
+                                        unsigned char* dst, uint32_t full_bar, int tok0, int npg, int group, bool waited) {
     const int lane = threadIdx.x & 31, hkv = p.hkv;
     const int pool_end = rows ? P : L, pool_full = pool_end & ~(kPage - 1);
     const int pool_pg = min(npg, max(0, (pool_full - tok0) >> 4));        // pages of the tile that come from the pool; lane l holds the first row group of page l
@@ -393,6 +401,19 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
     // (the whole-tile copy may bring in rows of the next sequence: for V none of them may be met by the MMAs, 16 tokens at a time)
     const int row0_new = q_row0 + tok0 - P;
     const bool big = rows && tok0 >= P && row0_new + kBN <= p.total_rows && (!is_v || own1 <= L);
+    const uint32_t d = smem_u32(dst);
+    if (lane == 0) mbar_expect_tx(full_bar, big ? kTileBytes : pool_pg * kPageBytes + (rows1 - rows0) * 256);
+    __syncwarp();
+    if (!big && lane < pool_pg) tma_load_page(d + lane * kPageBytes, pool_map, group, full_bar);
+    __syncwarp();
+    if (!waited) pdl_wait();
+    if (big) {
+        if (lane == 0) tma_load_rows128(d, rows128, row0_new, g, full_bar);
+    } else {
+        const int base = rows0 + lane * 8;
+        if (base < rows1) tma_load_rows8(d + (base - tok0) * 256, rows8, q_row0 + base - P, g, full_bar);
+    }
+    __syncwarp();
     bool by_hand = false;
     for (int base = own0; base < own1 && !big; base += 8) {
         if (base == rows0) base = rows1;
@@ -414,19 +435,40 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
     }
     if (by_hand) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncwarp();
-    const uint32_t d = smem_u32(dst);
-    if (lane == 0) {
-        mbar_arrive_expect_tx(full_bar, big ? kTileBytes : pool_pg * kPageBytes + (rows1 - rows0) * 256);
-        if (big) tma_load_rows128(d, rows128, row0_new, g, full_bar);
-    }
-    __syncwarp();
-    if (!big) {
-        if (lane < pool_pg) tma_load_page(d + lane * kPageBytes, pool_map, group, full_bar);
-        const int base = rows0 + lane * 8;
-        if (base < rows1) tma_load_rows8(d + (base - tok0) * 256, rows8, q_row0 + base - P, g, full_bar);
-    }
+    if (lane == 0) mbar_arrive(full_bar);
     __syncwarp();
 }
+
+// A Q tile's rows [row0, row0 + n) of KV head g, n <= 128, by one thread: single rows up to the next whole token, boxes of q_tokens tokens
+// while they fit the tile (the last one may bring rows nobody looks at), single rows again.  Where G divides 128 that is one box per half.
+struct QTile {
+    int n, i0, hh0, front, boxed;   // rows; token and head of the first; rows [front, boxed) come in boxes
+    __device__ __forceinline__ QTile(int row0, int rows, int G, int box, unsigned long long magic) {
+        n = max(0, min(128, rows - row0));
+        i0 = (int)(((uint64_t)(uint32_t)row0 * magic) >> 32);
+        hh0 = row0 - i0 * G;
+        front = boxed = hh0 ? min(n, G - hh0) : 0;
+        while (box > 0 && boxed < n && boxed + box <= 128) boxed += box;
+    }
+    __device__ __forceinline__ void load(const RowsMaps& maps, uint32_t tile, uint32_t bar, int G, int q_row0, int g) const {
+        mbar_arrive_expect_tx(bar, 256u * (uint32_t)max(n, boxed));
+        int token = q_row0 + i0, hh = hh0, r = 0;
+        auto copy = [&](const CUtensorMap* map) {
+            tma_load_q(tile + r * 128, map, hh, token, 0, g, bar);
+            tma_load_q(tile + r * 128 + kHalfBytes, map, hh, token, 1, g, bar);
+        };
+#pragma unroll 1
+        for (; r < front; ++r, ++hh) copy(&maps.q_row);
+        if (hh0) { hh = 0; ++token; }
+#pragma unroll 1
+        for (; r < boxed; r += maps.q_tokens * G, token += maps.q_tokens) copy(&maps.q_box);
+#pragma unroll 1
+        for (; r < n; ++r) {
+            copy(&maps.q_row);
+            if (++hh == G) { hh = 0; ++token; }
+        }
+    }
+};
 
 }  // namespace
 
@@ -469,89 +511,59 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // length are not written by any launch still in flight, so the producer warp may fetch them while the launch in
     // front of this one drains.  Its first page ids are on their way while it sets the barriers up.
     const int stable_end = P & ~(kPage - 1);   // tokens below this sit in pages no append of this block touches
-    const bool early_ids = p.early_prefix && kv_begin + kBN <= stable_end;
+    const bool early_ids = p.early_prefix;
+    const int n_pool_pages = max(0, (min(kv_end, p.k_new ? P : L) - kv_begin + kPage - 1) / kPage);   // pages of this CTA that the pool is read for
     int first_id = -1;
     const int* const first_id_at = p.page_table + (long long)sp.seq_index * p.pt_stride + kv_begin / kPage + lane;
-    if (warp == 0 && early_ids && lane * kPage < kv_end - kv_begin) first_id = __ldg(first_id_at);
+    if (warp == 0 && early_ids && lane < n_pool_pages) first_id = __ldg(first_id_at);
     if (tid == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : (i == BAR_Q_FULL || i == BAR_Q_FULL_B) ? (uint32_t)(kQLoadThreads / 32) : 1u);
+            if (i != BAR_Q_FULL && i != BAR_Q_FULL_B) mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : 1u);
         *abort_flag = 0;
         *(long long*)(smem + kOffBar + BAR_COUNT * 8 + 16) = p.wait_limit_cycles;   // for the out-of-line epilogue
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&map_k) : "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(&map_v) : "memory");
+        if (p.k_new && kv_end > stable_end) {
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps_new.k128) : "memory");
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps_new.k8) : "memory");
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps_new.v128) : "memory");
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps_new.v8) : "memory");
+        }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
-    if (warp != 0 || !early_ids) pdl_wait();   // from here on global memory written by the launch before this one is read (Q, page table, K/V)
-    // Q: 256 rows x 256 B by 16-byte cp.async (all of a thread's copies in flight at once), written in
-    // the 128-byte-swizzled K-major operand layout; rows past q * G are zero-filled.  Issuing them takes the CTA 1-1.8 us, so tile A is
-    // handed over by itself (2 x 1200 uncached tokens 45.1 -> 44.0 us a layer).  Loads into registers and stores instead: 45.6 us.
-    if (warp >= 2) {
-        // a thread copies the same 16 bytes of every kQLoadThreads / 16th row, tile A's rows as one group of copies, then tile B's
-        const int ch = tid & 15, half = ch >> 3, u = ch & 7;
-        const unsigned char* src0 = (const unsigned char*)p.q + ((long long)sp.q_row0 * p.hq + g * G) * 256 + ch * 16;
-        const int hq_minus_g = p.hq - G;
-        int rl = (tid - 64) >> 4;
-#pragma unroll
-        for (int tile = 0; tile < kRowsPerCta / 128; ++tile) {
-            const uint32_t dst0 = smem_base + kOffQ + tile * kTileBytes + half * kHalfBytes;
-#pragma unroll
-            for (int k = 0; k < (128 + kQLoadThreads / 16 - 1) / (kQLoadThreads / 16); ++k) {
-                const int r = row0 + tile * 128 + rl;
-                const bool valid = r < rows;
-                const int rr = valid ? r : 0;
-                const int i = (int)(((uint64_t)(uint32_t)rr * p.row_div_magic) >> 32);   // rr / G without the division
-                if (rl < 128) {   // (head g * G + r - i * G of row i)
-                    cp_async_16(dst0 + rl * 128 + ((u ^ (rl & 7)) << 4), src0 + (long long)(i * hq_minus_g + rr) * 256, valid ? 16u : 0u);
-                    rl += kQLoadThreads / 16;
-                }
-            }
-            rl -= 128;
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
+    if (warp == 3 && elect_one()) {
+        mbar_init(bar(BAR_Q_FULL), 1);
+        mbar_init(bar(BAR_Q_FULL_B), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"(maps_new.q_tokens ? &maps_new.q_box : &maps_new.q_row) : "memory");
+    }
+    // One Q tile: its rows of padding (most of them) are zeros, in Q here and in P below.  The MMAs work on them all the same, but zeros take less
+    // of the board's power than whatever lay there: 16 x 8192 verify, for seconds on end, 208 us with neither, 201 with Q, 197 with both.
+    if (kStreams && warp >= 4) {
+        const QTile qt(row0, rows, G, maps_new.q_tokens * G, p.row_div_magic);
+        for (int c = tid - 128 + max(qt.n, qt.boxed) * 8; c < 128 * 8; c += kThreads - 128) {
+            *(uint4*)(smem + kOffQ + c * 16) = make_uint4(0, 0, 0, 0);
+            *(uint4*)(smem + kOffQ + kHalfBytes + c * 16) = make_uint4(0, 0, 0, 0);
         }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    // fused append: the CTAs of a row chunk store the block rows whose first query row lies in the chunk, each split its share: loaded here,
-    // while Q is on its way, stored (and the rest of a large share loaded and stored) once Q is handed over
-    BlockRows own;
-    int own_lo = 0, own_hi = 0;
-    if (p.k_new && warp >= 2) {
-        const int i_lo = (int)(((uint64_t)(uint32_t)(row0 + G - 1) * p.row_div_magic) >> 32);
-        const int i_n = min(q, (int)(((uint64_t)(uint32_t)(row0 + kRowsPerCta + G - 1) * p.row_div_magic) >> 32)) - i_lo;
-        const unsigned parts = (unsigned)(it.vis_end + sp.split_tokens - 1) / (unsigned)sp.split_tokens;   // splits with work (the last ones may have none)
-        own_lo = i_lo + (unsigned)(i_n * split) / parts; own_hi = i_lo + (unsigned)(i_n * (split + 1)) / parts;
-        own.load(p, sp, g, own_lo, own_hi, tid - 64, kQLoadThreads);
-    }
-    if (warp == 0 && !early_ids && lane * kPage < kv_end - kv_begin) first_id = __ldg(first_id_at);
-    // Barriers initialised, TMEM address published.  Warp 0 (which set the barriers up and needs nothing
-    // from the others) only signals and goes straight to the page table and its first K/V copies.
+    // Barriers initialised, TMEM address published.  Warps 0 and 3, which set the barriers up and need nothing from the others, only signal and
+    // go straight to their first copies.  No warp has waited for the launch in front yet: what follows such a wait (warps 0, 2 and 3 have one
+    // each; whatever else the CTA reads or writes comes behind the Q tiles) is a chain of latencies with as little code as can be.
     tc_fence_before();
-    if (warp == 0) { __syncwarp(); asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory"); }
+    if (warp == 0 || warp == 3) { __syncwarp(); asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory"); }
     else asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
     tc_fence_after();
-    const uint32_t tmem_base = (warp == 0) ? 0u : *tmem_slot;
-    if (warp >= 2) {
-        if (!kStreams) {
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BAR_Q_FULL));
-        }
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(kStreams ? BAR_Q_FULL : BAR_Q_FULL_B));
-        if (p.k_new) {
-            own.store(p, sp, g, own_lo, own_hi, tid - 64, kQLoadThreads);
-            for (int idx0 = tid - 64 + BlockRows::kBatch * kQLoadThreads; idx0 < (own_hi - own_lo) * 32; idx0 += BlockRows::kBatch * kQLoadThreads) {
-                own.load(p, sp, g, own_lo, own_hi, idx0, kQLoadThreads);
-                own.store(p, sp, g, own_lo, own_hi, idx0, kQLoadThreads);
-            }
-        }
-    }
+    const uint32_t tmem_base = (warp == 0 || warp == 3) ? 0u : *tmem_slot;
+    // Fused append: a row group (eight tokens of half a page) is stored by the CTA whose row chunk's first query rows and whose split its first
+    // block token lies in.  That CTA has the group in its last K and V tiles, and a whole one leaves from there by TMA (by_tma).
+    const int own_lo = max(kv_begin, P + (int)(((uint64_t)(uint32_t)(row0 + G - 1) * p.row_div_magic) >> 32));
+    const int own_hi = p.k_new ? min(kv_end, kv_begin + sp.split_tokens) : 0;
+    auto by_tma = [&](int tok) { return !kStreams && tok >= P && tok + 8 <= L && tok >= kv_begin + (n_tiles - kStagesK) * kBN; };
     auto pages_in_tile = [&](int t) { return min(8, (kv_end - (kv_begin + t * kBN) + kPage - 1) / kPage); };
 
     // the softmax warpgroups keep a whole score row in registers: warps 0-3 hand registers over to them
@@ -559,18 +571,21 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsLow));
     if (warp == 0) {
         // ================= TMA producer =================
+        if (!early_ids) {
+            pdl_wait();
+            if (lane < n_pool_pages) first_id = __ldg(first_id_at);
+        }
         const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
         const int page0 = kv_begin / kPage;
-        const int n_pages_total = (kv_end - kv_begin + kPage - 1) / kPage;
         // Page ids are read 32 (four tiles) at a time and two groups ahead of the copies that need them; their row-group coordinates wait in
         // shared memory, so that the thread that issues the copies of a tile has them with two loads.
         int* const page_ring = (int*)(smem + kOffPages);   // [4 groups][32]
         auto load_ids = [&](int group) {   // (by the whole warp)
             const int pi = group * 32 + lane;
-            return pi < n_pages_total ? __ldg(pt_row + page0 + pi) : -1;
+            return pi < n_pool_pages ? __ldg(pt_row + page0 + pi) : -1;
         };
         auto check_ids = [&](int group, int id) {
-            if (group * 32 + lane < n_pages_total && (id < 0 || id >= p.num_pages)) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
+            if (group * 32 + lane < n_pool_pages && (id < 0 || id >= p.num_pages)) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
             return id;
         };
         auto fetch_ids = [&](int group) { return check_ids(group, load_ids(group)); };
@@ -580,8 +595,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // tokens [0, pool_end) come from the pool; a tile wholly inside the pool's full pages is eight page copies, see load_mixed for others
         const int pool_full = (p.k_new ? P : L) & ~(kPage - 1);
         int last_k = -1, last_v = -1;   // last tiles whose copies were armed (for the drain below)
-        const int n_groups = (n_tiles + 3) >> 2;
-        put_ids(0, check_ids(0, first_id));
+        const int n_groups = (n_pool_pages + 31) >> 5;
+        if (n_groups > 0) put_ids(0, check_ids(0, first_id));
         int ids_ahead = 0, ahead = -1;       // group `ahead` has been read (its ids are in ids_ahead), groups below it are in page_ring
         int ks = 0, vs = 0;
         uint32_t kph = 1, vph = 1;
@@ -592,11 +607,12 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 const int t = is_v ? i - 1 : i;
                 if (t < 0 || t >= n_tiles || !ok) continue;
                 const int tok0 = kv_begin + t * kBN;
-                // tiles wholly inside the cached prefix, as far as free stages go, may be requested before the wait
-                if (!waited && !(tok0 + kBN <= stable_end && t < (is_v ? kStagesV : kStagesK))) { pdl_wait(); waited = true; }
+                const bool whole = tok0 + kBN <= pool_full && tok0 + kBN <= kv_end;
+                // tiles inside the cached prefix, as far as free stages go, may be requested before the wait, also part of a tile (load_mixed)
+                if (!waited && !((tok0 + kBN <= stable_end || (!whole && p.k_new)) && t < (is_v ? kStagesV : kStagesK))) { pdl_wait(); waited = true; }
                 if (!is_v && (t & 3) == 0) {
                     const int group = t >> 2;
-                    if (group > 0) put_ids(group, ahead == group ? ids_ahead : fetch_ids(group));
+                    if (group > 0 && group < n_groups) put_ids(group, ahead == group ? ids_ahead : fetch_ids(group));
                     if (waited && group + 1 < n_groups) { ids_ahead = fetch_ids(group + 1); ahead = group + 1; }
                 }
                 if (t == p.drop_stage) {   // test hook: this tile never arrives, its consumers' waits run out
@@ -609,7 +625,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 ok = mbar_wait(empty, is_v ? vph : kph, abort_flag, p.status, p.wait_limit_cycles);
                 if (!ok) continue;
                 if (is_v) last_v = t; else last_k = t;
-                if (tok0 + kBN <= pool_full && tok0 + kBN <= kv_end) {
+                if (whole) {
                     if (elect_one()) {
                         const int4 c0 = *(const int4*)(page_ring + ((t * 8) & 127)), c1 = *(const int4*)(page_ring + ((t * 8) & 127) + 4);
                         const CUtensorMap* map = is_v ? &map_v : &map_k;
@@ -627,7 +643,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 } else {
                     load_mixed(p, is_v ? &map_v : &map_k, is_v ? &maps_new.v8 : &maps_new.k8, is_v ? &maps_new.v128 : &maps_new.k128,
                                (const unsigned char*)(is_v ? p.v_pool : p.k_pool), (const unsigned char*)(is_v ? p.v_new : p.k_new), is_v, g, P, L,
-                               sp.q_row0, smem + off, full, tok0, pages_in_tile(t), page_ring[(t * 8 + (lane & 7)) & 127]);
+                               sp.q_row0, smem + off, full, tok0, pages_in_tile(t), page_ring[(t * 8 + (lane & 7)) & 127], waited);
+                    waited = true;
                 }
                 __syncwarp();
                 if (is_v) { if (++vs == kStagesV) { vs = 0; vph ^= 1; } } else if (++ks == kStagesK) { ks = 0; kph ^= 1; }
@@ -641,6 +658,24 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             for (int t = max(0, last_v - kStagesV + 1); t <= last_v; ++t)
                 if (t != p.drop_stage) mbar_drain(bar(BAR_V_FULL + t % kStagesV), (t / kStagesV) & 1, p.wait_limit_cycles);
         }
+        __syncwarp();
+        // The block's own row groups go from the tiles into the pool, a lane per group.  Through registers it was 85 tokens' worth of loads
+        // and stores a CTA (3584 uncached tokens, 24/8 heads): in front of the softmax warps' loop 3 us of their way to the first scores; on warp 3
+        // beside the loop its instructions slowed the softmax warps of its scheduler, and with them the CTA, by a quarter.
+        if (!kStreams && ok && p.drop_stage < 0)
+            for (int tok = ((max(own_lo, P) + 7) & ~7) + lane * 8; tok < own_hi; tok += 256) {
+                if (!by_tma(tok)) continue;
+                const int id = tok / kPage < p.pt_stride ? __ldg(pt_row + tok / kPage) : -1, t = (tok - kv_begin) / kBN;
+                if (id < 0 || id >= p.num_pages) { atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
+                const int group = (id * p.hkv + g) * (kPage / 8) + ((tok >> 3) & 1), at = ((tok - kv_begin) & (kBN - 1)) * 256;
+                tma_store_group(&maps_new.k_pool8, group, smem_base + kOffK + (t % kStagesK) * kTileBytes + at);
+                tma_store_group(&maps_new.v_pool8, group, smem_base + v_stage_off<kStreams>(t % kStagesV) + at);
+            }
+        if (!kStreams) {   // (they are read before the CTA's shared memory goes away)
+            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+        }
+        __syncwarp();
     } else if (warp == 1 || warp == 2) {
         // ================= MMA issuers: one thread of warp 1 for S = Q K^T, one of warp 2 for O += P V =================
         // Units of work u = 0, 1, ...: a KV tile against tile A or B (x = u & 1); with kStreams one KV tile each.  S holds one unit's scores: it
@@ -648,6 +683,15 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // beside PV of unit u - 1.  Two issuing threads, because one was busy all the time: every wait of a warp that shares its scheduler
         // with two softmax warps costs it 90 cycles and more, also when there is nothing to wait for.
         const int n_units = kStreams ? n_tiles : 2 * n_tiles;
+        if (!kStreams && warp == 2) {
+            const QTile b(row0 + 128, rows, G, maps_new.q_tokens * G, p.row_div_magic);
+            if (elect_one()) {
+                pdl_wait();
+                if (b.n > 0) b.load(maps_new, smem_base + kOffQ + kTileBytes, bar(BAR_Q_FULL_B), G, sp.q_row0, g);
+                else mbar_arrive(bar(BAR_Q_FULL_B));   // (a tile of padding only: whatever is there)
+            }
+            __syncwarp();
+        }
         if (warp == 1 && elect_one()) {
             const uint32_t tS = tmem_base + kColS;
             // descriptors differ only in the start address: add (byte offset >> 4) to a base descriptor
@@ -714,9 +758,19 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             }
             umma_commit(bar(BAR_O_FULL));  // arrives when every MMA issued above has completed
             mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);
+            // (the copies must land before the CTA's shared memory goes away, also after a time-out elsewhere)
+            if (!kStreams) mbar_drain(bar(BAR_Q_FULL_B), 0, p.wait_limit_cycles);
         }
         __syncwarp();
-    } else {   // warp 3, otherwise idle
+    } else {   // warp 3
+        // Q by TMA, with everything worked out before the dependency wait (a single thread takes five clocks and more an instruction).  cp.async of
+        // one row by 16 threads took 2.1-2.7 us from the wait to the last byte, addresses and LSU; this 1.2.
+        const QTile a(row0, rows, G, maps_new.q_tokens * G, p.row_div_magic);
+        if (elect_one()) {
+            pdl_wait();
+            a.load(maps_new, smem_base + kOffQ, bar(BAR_Q_FULL), G, sp.q_row0, g);
+        }
+        __syncwarp();
         if (lane == 0) {   // park the epilogue's context
             EpiCtx* cx = (EpiCtx*)(smem + kOffCtx);
             cx->it = locate_item<kStreams>(p, blockIdx.x);
@@ -724,11 +778,27 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->lse = p.lse;
             cx->magic = p.row_div_magic; cx->status = p.status;
             cx->part_half = p.part_half;
+            const int rc = row0 / kRowsPerCta;
+            cx->part_tile = (unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536;
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }
+        // what of the fused append is no whole row group of a tile that stays in shared memory (see the end of warp 0)
+        if (p.k_new) {
+            pdl_wait();
+            for (int tok = own_lo & ~7; tok < own_hi; tok += 8) {
+                const int first = max(tok, P);
+                if (first < own_lo || by_tma(tok)) continue;
+                BlockRows<8> own;
+                own.load(p, sp, g, first - P, min(tok + 8, L) - P, lane, 32);
+                own.store(p, sp, g, first - P, min(tok + 8, L) - P, lane, 32);
+            }
+        }
+        // (the copies must land before the CTA's shared memory goes away, also after a time-out elsewhere)
+        if (lane == 0) mbar_drain(bar(BAR_Q_FULL), 0, p.wait_limit_cycles);
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kRegsHigh));
+        pdl_wait();
         // ================= softmax + epilogue: one thread per query row =================
         const int x = (warp - 4) >> 2;                       // tile A / B
         const int rt = ((warp & 3) << 5) + lane;             // row in tile == TMEM lane
@@ -740,7 +810,6 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const int r = q_tile_row0 + rt;
         const int limit = P + min(r / G, q - 1);             // last token this row sees
         const int tile_i_min = min(q_tile_row0 / G, q - 1);
-        // a warp whose 32 rows are all padding only keeps the barriers in step
         const bool warp_has_rows = q_tile_row0 + ((warp & 3) << 5) < rows;
         const float sc = p.scale_log2;
         float m_ref = -INFINITY;
@@ -748,7 +817,16 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         bool ok = true;
         constexpr int kStep = kStreams ? 2 : 1;
         const int t_first = kStreams ? x : 0;
-        if (!warp_has_rows) {   // keep the barriers in step, nothing else
+        if (!warp_has_rows) {   // a warp whose 32 rows are all padding keeps the barriers in step, nothing else
+            if (kStreams) {
+                uint32_t zero[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) zero[c] = 0;
+                tmem_st_x32(tP, zero);
+                tmem_st_x32(tP + 32, zero);
+                tmem_wait_st();
+                tc_fence_before();
+            }
             for (int t = t_first; t < n_tiles && ok; t += kStep) {
                 const int j = (t - t_first) / kStep;
                 ok = mbar_wait(bar(BAR_S_FULL + x), j & 1, abort_flag, p.status, p.wait_limit_cycles);
@@ -881,13 +959,13 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 // View of a pool [num_pages * Hkv * 16 rows][128 dims] bf16 as [row groups of 8][halves of 64 dims][8 rows][64 dims]; a box is two row
-// groups = the 4 KB of one page and KV head, 128-byte swizzle
-bool make_pool_map_impl(CUtensorMap* map, const void* pool, long long num_pages, int hkv) {
+// groups = the 4 KB of one page and KV head, or one of them, 128-byte swizzle
+bool make_pool_map_impl(CUtensorMap* map, const void* pool, long long num_pages, int hkv, int groups) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[4] = {64, 8, 2, (cuuint64_t)num_pages * hkv * (kPage / 8)};
     const cuuint64_t strides[3] = {(cuuint64_t)kD * 2, 128, (cuuint64_t)kD * 2 * 8};
-    const cuuint32_t box[4] = {64, 8, 2, (cuuint32_t)(kPage / 8)};
+    const cuuint32_t box[4] = {64, 8, 2, (cuuint32_t)groups};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(pool), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -896,7 +974,7 @@ bool make_pool_map_impl(CUtensorMap* map, const void* pool, long long num_pages,
 }  // namespace
 
 bool make_pool_map(CUtensorMap* map, const void* pool, long long num_pages, int hkv) {
-    return make_pool_map_impl(map, pool, num_pages, hkv);
+    return make_pool_map_impl(map, pool, num_pages, hkv, kPage / 8);
 }
 
 // [KV heads][row groups of 8][halves of 64 dims][rows][64 dims]; the row and the row-group dimension overlap (a box of 16 groups from any
@@ -913,9 +991,28 @@ static bool make_rows_map(CUtensorMap* map, const void* rows, long long total_q,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-bool make_rows_maps(RowsMaps* m, const void* k_new, const void* v_new, long long total_q, int hkv) {
-    return make_rows_map(&m->k8, k_new, total_q, hkv, 1) && make_rows_map(&m->v8, v_new, total_q, hkv, 1) &&
+bool make_rows_maps(RowsMaps* m, const void* k_new, const void* v_new, long long total_q, const void* k_pool, const void* v_pool, long long num_pages,
+                    int hkv) {
+    return make_pool_map_impl(&m->k_pool8, k_pool, num_pages, hkv, 1) && make_pool_map_impl(&m->v_pool8, v_pool, num_pages, hkv, 1) &&
+           make_rows_map(&m->k8, k_new, total_q, hkv, 1) && make_rows_map(&m->v8, v_new, total_q, hkv, 1) &&
            make_rows_map(&m->k128, k_new, total_q, hkv, 16) && make_rows_map(&m->v128, v_new, total_q, hkv, 16);
+}
+
+// [KV heads][halves of 64 dims][tokens][heads of the group][64 dims]; a box is all heads of q_tokens tokens, or one row
+bool make_q_maps(RowsMaps* m, const void* q, long long total_q, int hq, int hkv, int q_tokens) {
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return false;
+    const cuuint32_t G = (cuuint32_t)(hq / hkv);
+    const cuuint64_t dims[5] = {64, G, (cuuint64_t)total_q, 2, (cuuint64_t)hkv};
+    const cuuint64_t strides[4] = {(cuuint64_t)kD * 2, (cuuint64_t)hq * kD * 2, 128, (cuuint64_t)G * kD * 2};
+    const cuuint32_t one[5] = {64, 1, 1, 1, 1}, box[5] = {64, G, (cuuint32_t)q_tokens, 1, 1}, estr[5] = {1, 1, 1, 1, 1};
+    auto make = [&](CUtensorMap* map, const cuuint32_t* b) {
+        return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(q), dims, strides, b, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    m->q_tokens = q_tokens;
+    if (q_tokens == 0) memset(&m->q_box, 0, sizeof m->q_box);
+    return make(&m->q_row, one) && (q_tokens == 0 || make(&m->q_box, box));
 }
 
 namespace {

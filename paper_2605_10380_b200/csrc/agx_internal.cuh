@@ -16,11 +16,17 @@ constexpr long long kWaitLimitCycles = 4000000000ll;  // ~2 s at 1.9 GHz: defaul
 
 // TMA view of a KV pool (head_dim 128, bf16): one box is the 16 rows of one page and KV head, see tma_load_page.
 bool make_pool_map(CUtensorMap* map, const void* pool, long long num_pages, int hkv);
-// TMA views of a block's own K and V rows [total_q][hkv][128] bf16: one box is 8 or 128 rows of one KV head, see tma_load_rows8 / 128.
+// TMA views of a block's own K and V rows [total_q][hkv][128] bf16: one box is 8 or 128 rows of one KV head, see tma_load_rows8 / 128, and
+// of the pools they are appended to, one box being half a page (8 rows) of a KV head, see tma_store_group;
+// and of its Q [total_q][hq][128]: one box is one half of 64 dims of the rows of `q_tokens` tokens (0: none) or of one row of a KV head,
+// see tma_load_q.
 struct alignas(64) RowsMaps {
-    CUtensorMap k8, v8, k128, v128;
+    CUtensorMap k8, v8, k128, v128, k_pool8, v_pool8, q_box, q_row;
+    int q_tokens;
 };
-bool make_rows_maps(RowsMaps* maps, const void* k_new, const void* v_new, long long total_q, int hkv);
+bool make_rows_maps(RowsMaps* maps, const void* k_new, const void* v_new, long long total_q, const void* k_pool, const void* v_pool, long long num_pages,
+                    int hkv);
+bool make_q_maps(RowsMaps* maps, const void* q, long long total_q, int hq, int hkv, int q_tokens);
 
 // Per-sequence launch plan, built on the host from the host lengths.
 struct SeqPlan {
@@ -36,6 +42,10 @@ struct SeqPlan {
     int chunk_major;   // order of the work items: 0 = KV head outermost, 1 = row chunk outermost (row chunks last to first in both)
 };
 
+// Split partials: fp32 rows | fp16 rows in slots | fp16 rows in tiles (256-row tensor-core schedule): the 64 KB of a sequence's (KV head, row
+// chunk, split) from part_base * 512 bytes on, splits innermost, 256 bytes per row, 16-byte unit u of row r at u ^ (r & 15).
+enum PartHalf { PART_F32 = 0, PART_HALF_SLOTS = 1, PART_HALF_TILES = 2 };
+
 struct AttnParams {
     const void* q;
     const void* k_pool;
@@ -44,11 +54,11 @@ struct AttnParams {
     void* out;
     float* lse;
     float* part_o;   // [entries][head_dim] fp32, un-normalised, relative to part_ml.x; or, with part_half, rows NORMALISED by their
-                     // own sum and stored as fp16 in the first 256 bytes of the same 512-byte slots
+                     // own sum as fp16: in the first 256 bytes of the same 512-byte slots, or in the tiles of the CTAs that made them (PartHalf)
     float2* part_ml; // [entries] (running max in log2 units, sum)
     int* status;
     unsigned long long row_div_magic;   // ceil(2^32 / G), G = hq / hkv: (row * magic) >> 32 == row / G for rows < 2^22
-    int part_half;       // != 0: split partials of this launch are normalised fp16 rows (256-row tensor-core schedule)
+    int part_half;       // how the split partials of this launch are stored, a PartHalf
     int cluster_size;    // > 1: the launch's CTAs form clusters of this size = the KV splits of one (sequence, KV head), merged in-kernel
     const void* k_new;   // fused append (agx_attn_prefixed_append): the block's K/V rows [total_q][hkv][d], or NULL
     const void* v_new;

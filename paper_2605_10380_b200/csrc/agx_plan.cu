@@ -464,10 +464,12 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 sp.item0 = ln.num_items;
                 sp.part_base = 0;
                 if (sp.nsplit > 1 && !cluster) {
-                    if (plan.part_entries + (long long)Q[s] * c.num_q_heads * sp.nsplit > 0x7FFFFFFFll)
-                        return fail(AGX_E_RANGE, "split partials exceed 2^31 entries");
+                    long long entries = (long long)Q[s] * c.num_q_heads * sp.nsplit;
+                    // (a tile of fp16 partials is 128 slots: more than the slots of its rows only where one chunk has fewer than 128 of them)
+                    if (k == KIND_TILE) entries = std::max(entries, per_seq_items[n] * sp.nsplit * 128);
+                    if (plan.part_entries + entries > 0x7FFFFFFFll) return fail(AGX_E_RANGE, "split partials exceed 2^31 entries");
                     sp.part_base = (int)plan.part_entries;
-                    plan.part_entries += (long long)Q[s] * c.num_q_heads * sp.nsplit;
+                    plan.part_entries += entries;
                     plan.any_split = true;
                 }
                 const long long items = per_seq_items[n] * sp.nsplit;

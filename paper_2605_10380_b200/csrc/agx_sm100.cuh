@@ -22,6 +22,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {   // (no arrival)
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -74,6 +77,19 @@ __device__ __forceinline__ void tma_load_rows128(uint32_t dst, const CUtensorMap
     tma_load_rows8(dst, map, row, head, bar);   // (the map's box is 16 row groups)
 }
 
+// Eight rows of one KV head, as they lie in a K or V tile, to half a page of the pool (RowsMaps::k_pool8 / v_pool8); `group` as above.
+__device__ __forceinline__ void tma_store_group(const CUtensorMap* map, int group, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %1, %1, %2}], [%3];\n" ::"l"(map), "r"(0), "r"(group), "r"(src) : "memory");
+}
+
+// One half (64 dims) of Q rows of KV head g through RowsMaps::q_box (all heads of q_tokens tokens from `token` on) or q_row (head `hh` of the
+// group, one token), one 128-byte line per row.  The 128-byte swizzle goes by the address in shared memory, so that a copy may start at any row
+// of a tile.  Past the end zeros arrive.
+__device__ __forceinline__ void tma_load_q(uint32_t dst, const CUtensorMap* map, int hh, int token, int half, int g, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n"
+                 ::"r"(dst), "l"(map), "r"(0), "r"(hh), "r"(token), "r"(half), "r"(g), "r"(bar) : "memory");
+}
+
 // One lane of a converged warp.  Unlike `lane == 0` this tells the compiler that a single thread takes the branch, so the
 // instructions that want their operands in uniform registers (tcgen05.mma, TMA copies) are issued without a loop over lanes.
 __device__ __forceinline__ bool elect_one() {
@@ -91,8 +107,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 // Fused KV append (bf16, d = 128): the block's rows [i_lo, i_hi) of KV head g go into the sequence's pages (Sec. 2.3: the block's KV
 // joins the cache).  Nothing in the same launch reads them there: the attention CTAs take the block's own rows from k_new / v_new,
 // so there is nothing to wait for.
+template <int kBatch>   // 16-byte units in flight per thread: idx0, idx0 + nthreads, ...
 struct BlockRows {
-    static constexpr int kBatch = 4;   // 16-byte units in flight per thread: idx0, idx0 + nthreads, ...
     uint4 v[kBatch];
     int id[kBatch];
     __device__ __forceinline__ void load(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int idx0, int nthreads) {
