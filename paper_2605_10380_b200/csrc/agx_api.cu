@@ -37,6 +37,8 @@ struct agx_handle {
     long long wait_limit_cycles;   // AGX_OPT_WAIT_LIMIT_CYCLES
     int early_prefix;       // AGX_OPT_EARLY_PREFIX_LOADS
     int drop_stage;         // AGX_OPT_TEST_DROP_STAGE (-1 = none)
+    const char* last_out;   // `out` of the last attention call: kernels that write it may still be running when the next call's start
+    size_t last_out_bytes;
     std::vector<int32_t> cu_host;  // staging for agx_verify_step_host (lives until its final sync)
     // Large attention-only host steps run as a pipeline of row chunks: uploads on one stream of the handle's own, the
     // attention calls on the caller's stream, downloads on a third (env AGX_HOST_PIPELINE_ROWS: rows per chunk, 0 = off).
@@ -147,6 +149,8 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     env = getenv("AGX_HOST_PIPELINE_ROWS");
     h->pipe_rows = env ? std::max(0, atoi(env)) : 384;   // measured on the long-context step: 256 / 384 / 512 / 768 / 1024 rows -> 1.54 / 1.43 / 1.57 / 1.56 / 1.72 ms
     h->pipe_in = h->pipe_out = nullptr;
+    h->last_out = nullptr;
+    h->last_out_bytes = 0;
     env = getenv("AGX_ZERO_COPY");
     h->zero_copy = env ? atoi(env) : 3;
     h->wait_limit_cycles = kWaitLimitCycles;
@@ -269,6 +273,8 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         else if (plan.tensor_core) memset(&maps_new, 0, sizeof maps_new);
         if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
+    h->last_out = (const char*)out;
+    h->last_out_bytes = (size_t)plan.total_rows * p.hq * p.head_dim * elem_size(h->cfg.dtype);
     for (const Launch& ln : plan.launches) {
         p.num_seqs = (int)ln.seqs.size();
         p.num_items = ln.num_items;
@@ -644,6 +650,9 @@ static agx_status verify_step_host_impl(agx_handle* h, void* k_pool, void* v_poo
         sc.src[0] = (const uint4*)mq; sc.src[1] = (const uint4*)mk; sc.src[2] = (const uint4*)mv;
         sc.dst[0] = (uint4*)(ws + L.q); sc.dst[1] = (uint4*)(ws + L.k); sc.dst[2] = (uint4*)(ws + L.v);
         sc.units[0] = (unsigned)(L.q_bytes / 16); sc.units[1] = sc.units[2] = (unsigned)(L.kv_bytes / 16);
+        // the inputs are read ahead of the stream's order, unless they are what the step in front still writes
+        auto written = [&](const void* p, size_t bytes) { return (const char*)p < h->last_out + h->last_out_bytes && h->last_out < (const char*)p + bytes; };
+        sc.src_in_order = written(mq, L.q_bytes) || written(mk, L.kv_bytes) || written(mv, L.kv_bytes);
         e = launch_stage_in(sc, stream);
         if (e == cudaSuccess) ++launches;
     } else {
