@@ -35,3 +35,17 @@ def test_accept_against_the_oracle(dtype, vocab, q):
     ref = oracle.accept_greedy(aw.logits, dtype, aw.vocab, aw.drafts, aw.cu_q, aw.prefix_len)
     for g, r in zip(got, ref):
         assert np.array_equal(g, r)
+
+
+@pytest.mark.parametrize("dtype,vocab", [("f32", 2), ("f32", 517), ("f32", 4096), ("f32", 4100), ("bf16", 8192), ("bf16", 8200), ("bf16", 60000)])
+@pytest.mark.parametrize("q", [[2], [2, 1], [3, 2], [1, 1, 4], [7], [1] * 8, [8], [4, 5]], ids=["2", "3", "5", "6", "7", "8x1", "8", "9"])
+def test_few_rows_on_both_sides_of_one_cluster(dtype, vocab, q):
+    """Up to eight rows of at most 16 KB a CTA are one cluster's, more or longer ones are not; longest matches of drafts in both."""
+    import oracle
+    from paper_2605_10380_b200 import agx
+    from tests.gpu_util import run_accept
+    aw = W.make_planted_accept("few", vocab + sum(q), dtype, vocab, q, [50 + i for i in range(len(q))], row_stride=(vocab + 7) // 8 * 8)
+    got = run_accept(agx.Handle(32, 8, 128, "bf16"), aw)
+    ref = oracle.accept_greedy(aw.logits, dtype, aw.vocab, aw.drafts, aw.cu_q, aw.prefix_len)
+    for g, r in zip(got, ref):
+        assert np.array_equal(g, r)
