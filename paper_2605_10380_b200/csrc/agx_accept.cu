@@ -130,9 +130,13 @@ accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, 
               int* __restrict__ seq_lens, unsigned long long* row_keys, int* tokens_global, unsigned int* ticket) {
     constexpr int kVecElems = kBf16 ? 8 : 4;
     pdl_launch_dependents();
-    pdl_wait();
     const int row = blockIdx.y;
     const int chunk = blockIdx.x;
+    const char* row_ptr = (const char*)logits + (size_t)row * row_stride * (kBf16 ? 2 : 4);
+    unsigned long long* row_key = row_keys + row;
+    hold(row_ptr); hold(row_key); hold(cu_q); hold(drafts); hold(seq_lens); hold(ticket); hold(vocab); hold(B);
+    asm volatile("" ::"l"(accept_len), "l"(next_token), "l"(argmax), "r"(total_q), "l"(tokens_global));   // (in the constant cache for the last block)
+    pdl_wait();
     const unsigned int begin = (unsigned int)chunk * (unsigned int)chunk_elems;
     const unsigned int end = min((unsigned int)vocab, begin + (unsigned int)chunk_elems);
 
@@ -143,7 +147,6 @@ accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, 
     head.load_rows(warp, B, cu_q, seq_lens);
     unsigned long long best = 0ull;  // "no element": loses to every real element
     if (kVec) {
-        const char* row_ptr = (const char*)logits + (size_t)row * row_stride * (kBf16 ? 2 : 4);
         VecMax<kBf16> vm;
         // two independent 16-byte loads in flight per thread per trip
         unsigned int i = begin + threadIdx.x * kVecElems;
@@ -162,8 +165,8 @@ accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, 
     } else {
         for (unsigned int e = begin + threadIdx.x; e < end; e += 256) {
             float x;
-            if (kBf16) x = bf16_bits_to_float(((const unsigned short*)logits)[(size_t)row * row_stride + e]);
-            else x = ((const float*)logits)[(size_t)row * row_stride + e];
+            if (kBf16) x = bf16_bits_to_float(((const unsigned short*)row_ptr)[e]);
+            else x = ((const float*)row_ptr)[e];
             const unsigned long long k = pack_key(ordered_key(x), e);
             best = k > best ? k : best;
         }
@@ -179,7 +182,7 @@ accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, 
         unsigned long long b = warp_best[0];
 #pragma unroll
         for (int w = 1; w < 8; ++w) b = warp_best[w] > b ? warp_best[w] : b;
-        if (b) atomicMax(row_keys + row, b);   // (0: no number in this chunk)
+        if (b) atomicMax(row_key, b);   // (0: no number in this chunk)
         __threadfence();
         const unsigned int total = gridDim.x * gridDim.y;
         const unsigned int t = atomicAdd(ticket, 1u);
@@ -226,12 +229,13 @@ accept_cluster_kernel(const void* __restrict__ logits, long long row_stride, int
     pdl_launch_dependents();
     const int rank = blockIdx.x, row = rank / chunks, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned int begin = (unsigned int)(rank - row * chunks) * (unsigned int)chunk_elems, end = min((unsigned int)vocab, begin + (unsigned int)chunk_elems);
+    const char* row_ptr = (const char*)logits + (size_t)row * row_stride * (kBf16 ? 2 : 4);
+    hold(row_ptr); hold(cu_q); hold(drafts); hold(seq_lens); hold(accept_len); hold(next_token); hold(argmax); hold(B); hold(total_q);
     pdl_wait();
     SeqHead head;
     if (rank == 0) head.load_rows(warp, B, cu_q, seq_lens);
     VecMax<kBf16> vm;
     if (row < total_q) {
-        const char* row_ptr = (const char*)logits + (size_t)row * row_stride * (kBf16 ? 2 : 4);
         for (unsigned int i = begin + threadIdx.x * kVecElems; i < end; i += 256 * kVecElems) {
             if (i + kVecElems <= end) vm.take(__ldg((const uint4*)(row_ptr + (size_t)i * (kBf16 ? 2 : 4))), i);
             else vm.take_partial(row_ptr, i, end);

@@ -80,8 +80,10 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
     const int nsplit = sp.nsplit, split = local % nsplit;
     local /= nsplit;
     const int rc = local % sp.row_chunks, g = local / sp.row_chunks;
-    const int G = p.hq / p.hkv, P = sp.prefix_len, q = sp.q_len, L = P + q, rows = q * G, row0 = rc * kR;
-    const int vis_end = P + min(q - 1, (row0 + kR - 1) / G) + 1;
+    const int G = p.gqa, P = sp.prefix_len, q = sp.q_len, L = P + q, rows = q * G, row0 = rc * kR;
+    auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div_magic) >> 32); };   // r / G without the division
+    auto row_of = [&](int r) { const int i = div_g(r); return (long long)(sp.q_row0 + i) * p.hq + g * G + r - i * G; };   // of q and out
+    const int vis_end = P + min(q - 1, div_g(row0 + kR - 1)) + 1;
     const int tok_begin = split * sp.split_tokens, tok_end = min(vis_end, tok_begin + sp.split_tokens);
     const int pool_end = p.k_new ? P : L;
     const bool writer = p.k_new && rc == sp.row_chunks - 1;
@@ -96,18 +98,34 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
 #pragma unroll
         for (int j = 0; j < kPer; ++j) id[j] = page_id(tok_begin + (tid + j * kThreads) / kUnits);
     }
+    // what the parameters are needed for behind the wait, worked out before it (the kernel is a chain of latencies; with this and without
+    // divisions behind the wait 256 cached tokens, q = 4, 4/2 heads, fp32 with its acceptance 8.8 -> 8.1 us)
+    static_assert(kR * kUnits <= kThreads, "one unit of Q per thread");
+    const bool has_q = tid < kR * kUnits && row0 + tid / kUnits < rows;
+    const unsigned char* q_at = (const unsigned char*)p.q + (row_of(has_q ? row0 + tid / kUnits : 0) * D + (tid % kUnits) * 4) * (kBf16 ? 2 : 4);
+    const void *k_pool = p.k_pool, *v_pool = p.v_pool, *k_new = p.k_new, *v_new = p.v_new;
+    int num_pages = (int)min(p.num_pages, 0x7FFFFFFFll), hkv = p.hkv;
+    float scale = p.scale_log2;
+    hold(q_at); hold(k_pool); hold(v_pool); hold(k_new); hold(v_new); hold(num_pages); hold(hkv); hold(scale);
+    // the first result of this thread (of its cluster's share where there is one)
+    const bool in_cluster = p.cluster_size > 1;
+    const int out0 = in_cluster ? split + nsplit * tid : tid;
+    unsigned char* out_at = nullptr;
+    float* lse_at = nullptr;
+    if (out0 < kR * kUnits && row0 + out0 / kUnits < rows && (in_cluster || nsplit == 1)) {
+        const long long at = row_of(row0 + out0 / kUnits);
+        out_at = (unsigned char*)p.out + (at * D + (out0 % kUnits) * 4) * (kBf16 ? 2 : 4);
+        if (p.lse && out0 % kUnits == 0) lse_at = p.lse + at;
+    }
+    hold(out_at); hold(lse_at);
     pdl_wait();
     if (!p.early_prefix) {
 #pragma unroll
         for (int j = 0; j < kPer; ++j) id[j] = page_id(tok_begin + (tid + j * kThreads) / kUnits);
     }
     // Q (a unit per thread), scaled so that the scores are in log2 units; rows past q * G are zeros
-    static_assert(kR * kUnits <= kThreads, "one unit of Q per thread");
     float4 qx = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < kR * kUnits && row0 + tid / kUnits < rows) {
-        const int r = row0 + tid / kUnits;
-        qx = load4<kBf16>(p.q, ((long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G) * D + (tid % kUnits) * 4);
-    }
+    if (has_q) qx = load4<kBf16>(q_at, 0);
     float acc[kR][kCols];
 #pragma unroll
     for (int r = 0; r < kR; ++r)
@@ -115,9 +133,9 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
         for (int c = 0; c < kCols; ++c) acc[r][c] = 0.f;
     float m_run = -INFINITY, l_run = 0.f;                      // of row `warp`
     const int st = tid & (kT - 1), sr = (tid / kT) * 2;        // this thread's token and first row in the scoring step
-    const int lim0 = P + min((row0 + sr) / G, q - 1), lim1 = P + min((row0 + sr + 1) / G, q - 1);
+    const int lim0 = P + min(div_g(row0 + sr), q - 1), lim1 = P + min(div_g(row0 + sr + 1), q - 1);
 
-    const int hidden = P + row0 / G + 1;                       // the first token that not every row sees
+    const int hidden = P + div_g(row0) + 1;                       // the first token that not every row sees
     if (tid == 0) sm.odd = 0;
     for (int t0 = tok_begin; t0 < tok_end; t0 += kT) {
         float4 kv[2][kPer];
@@ -127,20 +145,20 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
             kv[0][j] = kv[1][j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (tok >= tok_end) continue;
             const long long page = id[j];
-            const bool ok = page >= 0 && page < p.num_pages;
+            const bool ok = page >= 0 && page < num_pages;
             if (!ok) atomicOr(p.status, AGX_DEV_BAD_PAGE);
-            const long long slot = ((page * p.hkv + g) * kPage + (tok & 15)) * (long long)D + c;
+            const long long slot = ((page * hkv + g) * kPage + (tok & 15)) * (long long)D + c;
             if (tok < pool_end) {
-                if (ok) { kv[0][j] = load4<kBf16>(p.k_pool, slot); kv[1][j] = load4<kBf16>(p.v_pool, slot); }
+                if (ok) { kv[0][j] = load4<kBf16>(k_pool, slot); kv[1][j] = load4<kBf16>(v_pool, slot); }
             } else {
-                const long long at = ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * D + c;
-                kv[0][j] = load4<kBf16>(p.k_new, at); kv[1][j] = load4<kBf16>(p.v_new, at);
-                if (writer && ok) { store4<kBf16>((void*)p.k_pool, slot, kv[0][j]); store4<kBf16>((void*)p.v_pool, slot, kv[1][j]); }
+                const long long at = ((long long)(sp.q_row0 + tok - P) * hkv + g) * D + c;
+                kv[0][j] = load4<kBf16>(k_new, at); kv[1][j] = load4<kBf16>(v_new, at);
+                if (writer && ok) { store4<kBf16>((void*)k_pool, slot, kv[0][j]); store4<kBf16>((void*)v_pool, slot, kv[1][j]); }
             }
         }
         __syncthreads();                                       // the tile before this one has been used
         if (t0 == tok_begin && tid < kR * kUnits)
-            *(float4*)&sm.q[tid / kUnits][(tid % kUnits) * 4] = make_float4(qx.x * p.scale_log2, qx.y * p.scale_log2, qx.z * p.scale_log2, qx.w * p.scale_log2);
+            *(float4*)&sm.q[tid / kUnits][(tid % kUnits) * 4] = make_float4(qx.x * scale, qx.y * scale, qx.z * scale, qx.w * scale);
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int u = tid + j * kThreads;
@@ -235,8 +253,7 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
         for (int c = 0; c < kCols; ++c) part[(warp * kR + r) * D + c * 32 + lane] = acc[r][c];
     if (lane == 0) sm.ml[warp] = make_float2(m_run, l_run);
     __syncthreads();
-    const bool in_cluster = p.cluster_size > 1;
-    for (int i = tid; i < kR * kUnits; i += kThreads) {
+    for (int i = tid; i < kR * kUnits; i += kThreads) {   // (once: kR * kUnits <= kThreads)
         const int rl = i / kUnits, c = (i % kUnits) * 4, r = row0 + rl;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -248,12 +265,11 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
         if (in_cluster) {
             *(float4*)&sm.o[rl][c] = o;
         } else if (r < rows) {
-            const long long at = (long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G;
             if (nsplit == 1) {
-                store4<kBf16>(p.out, at * D + c, make_float4(o.x / ml.y, o.y / ml.y, o.z / ml.y, o.w / ml.y));
-                if (p.lse && c == 0) p.lse[at] = (ml.x + log2f(ml.y)) * 0.6931471805599453f;
+                store4<kBf16>(out_at, 0, make_float4(o.x / ml.y, o.y / ml.y, o.z / ml.y, o.w / ml.y));
+                if (lse_at) *lse_at = (ml.x + log2f(ml.y)) * 0.6931471805599453f;
             } else {
-                const long long e = (long long)sp.part_base + ((long long)(r / G) * p.hq + g * G + r % G) * nsplit + split;
+                const long long e = (long long)sp.part_base + (row_of(r) - (long long)sp.q_row0 * p.hq) * nsplit + split;
                 *(float4*)(p.part_o + e * D + c) = o;
                 if (c == 0) p.part_ml[e] = ml;
             }
@@ -262,9 +278,9 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
     if (in_cluster) {
         cluster_sync();
         // groups of four columns are dealt round-robin to the cluster's CTAs
-        for (int i = split + nsplit * tid; i < kR * kUnits; i += nsplit * kThreads) {
-            const int rl = i / kUnits, c = (i % kUnits) * 4, r = row0 + rl;
-            if (r >= rows) continue;
+        for (int i = out0; i < kR * kUnits; i += nsplit * kThreads) {   // (once)
+            const int rl = i / kUnits, c = (i % kUnits) * 4;
+            if (!out_at) continue;
             const uint32_t ml_addr = smem_u32(&sm.ml[rl]), o_addr = smem_u32(&sm.o[rl][c]);
             float2 ml[16];
             float4 x[16];
@@ -282,9 +298,8 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
                     l += ml[k].y * w;
                     o.x += x[k].x * w; o.y += x[k].y * w; o.z += x[k].z * w; o.w += x[k].w * w;
                 }
-            const long long at = (long long)(sp.q_row0 + r / G) * p.hq + g * G + r % G;
-            store4<kBf16>(p.out, at * D + c, make_float4(o.x / l, o.y / l, o.z / l, o.w / l));
-            if (p.lse && c == 0) p.lse[at] = (m + log2f(l)) * 0.6931471805599453f;
+            store4<kBf16>(out_at, 0, make_float4(o.x / l, o.y / l, o.z / l, o.w / l));
+            if (lse_at) *lse_at = (m + log2f(l)) * 0.6931471805599453f;
         }
         cluster_sync();   // no CTA leaves while its rows may still be read
     }

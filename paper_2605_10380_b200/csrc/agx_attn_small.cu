@@ -633,20 +633,26 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     const int c4 = lane * 4;               // each lane owns 4 output columns
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m_all, l_all;
+    const float2* ml_at = p.part_ml + e0 + lane;
+    const float* row_at = p.part_o + e0 * D + c4;
+    const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
+    unsigned char* out_at = (unsigned char*)p.out + (out_row * D + c4) * (kBf16Out ? 2 : 4);
+    float* lse_at = p.lse ? p.lse + out_row : nullptr;
+    hold(ml_at); hold(row_at); hold(out_at); hold(lse_at);
     pdl_wait();   // the partials are complete
     // One round trip to memory: lane k fetches (m, l) of split k while every lane already fetches its
     // columns of every split's O row; the weights then travel by shuffle, splits in index order.
     // (volatile loads: the compiler leaves them in this order, ahead of the first use of any of them)
     float2 ml = make_float2(-INFINITY, 0.f);
-    if (lane < ns) ml = ld_volatile_f2(p.part_ml + e0 + lane);
+    if (lane < ns) ml = ld_volatile_f2(ml_at);
     float4 v[kInFlight], v2[kFew ? 1 : 16];
 #pragma unroll
     for (int j = 0; j < kInFlight; ++j)
-        if (j < ns && c4 < D) v[j] = ld_volatile_f4(p.part_o + (e0 + j) * D + c4);
+        if (j < ns && c4 < D) v[j] = ld_volatile_f4(row_at + j * D);
     if (!kFew && ns > 16) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-            if (16 + j < ns && c4 < D) v2[j] = ld_volatile_f4(p.part_o + (e0 + 16 + j) * D + c4);
+            if (16 + j < ns && c4 < D) v2[j] = ld_volatile_f4(row_at + (16 + j) * D);
     }
     m_all = ml.x;
 #pragma unroll
@@ -673,18 +679,17 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         }
     }
     const float inv = 1.f / l_all;
-    const long long off = ((long long)(sp.q_row0 + i) * p.hq + h) * D + c4;
     if (c4 < D) {
         if (kBf16Out) {
             uint2 packed;
             packed.x = pack_bf16(acc.x * inv, acc.y * inv);
             packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-            *(uint2*)((__nv_bfloat16*)p.out + off) = packed;
+            *(uint2*)out_at = packed;
         } else {
-            *(float4*)((float*)p.out + off) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+            *(float4*)out_at = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
         }
     }
-    if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+    if (lse_at && lane == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
 // The same merge where a sequence has more than 32 splits (long contexts over few KV heads): one CTA per (row, head), whose warps take
@@ -710,14 +715,20 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     const int ns = sp.nsplit, D = p.head_dim, c4 = lane * 4, i = lrow - acc_rows;
     if (ns == 1) return;   // written directly by the attention kernel
     const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
-    const HalfRows rows(p, sp, i, h, lane);
+    HalfRows rows(p, sp, i, h, lane);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m = -INFINITY, l = 0.f;
+    const float2* ml_at = p.part_ml + e0 + lane;
+    const float* row_at = p.part_o + e0 * D + c4;
+    const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
+    unsigned char* out_at = (unsigned char*)p.out + (out_row * D + c4) * (kBf16Out ? 2 : 4);
+    float* lse_at = p.lse ? p.lse + out_row : nullptr;
+    hold(ml_at); hold(row_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride);
     pdl_wait();   // the partials are complete
     for (int k0 = warp * kManyBatch; k0 < ns; k0 += warps * kManyBatch) {
         const int n = min(kManyBatch, ns - k0);
         float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < n) ml = ld_volatile_f2(p.part_ml + e0 + k0 + lane);
+        if (lane < n) ml = ld_volatile_f2(ml_at + k0);
         float4 v[kManyBatch];
 #pragma unroll
         for (int j = 0; j < kManyBatch; ++j)
@@ -727,7 +738,7 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
                     const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
                     v[j] = make_float4(a.x, a.y, b.x, b.y);
                 } else {
-                    v[j] = ld_volatile_f4(p.part_o + (e0 + k0 + j) * D + c4);
+                    v[j] = ld_volatile_f4(row_at + (long long)(k0 + j) * D);
                 }
             }
         float m_new = ml.x;
@@ -765,16 +776,15 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         acc.x += a.x * e; acc.y += a.y * e; acc.z += a.z * e; acc.w += a.w * e;
     }
     const float inv = 1.f / l_all;
-    const long long off = ((long long)(sp.q_row0 + i) * p.hq + h) * D + c4;
     if (kBf16Out) {
         uint2 packed;
         packed.x = pack_bf16(acc.x * inv, acc.y * inv);
         packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-        *(uint2*)((__nv_bfloat16*)p.out + off) = packed;
+        *(uint2*)out_at = packed;
     } else {
-        *(float4*)((float*)p.out + off) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        *(float4*)out_at = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     }
-    if (p.lse && lane == 0) p.lse[(long long)(sp.q_row0 + i) * p.hq + h] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+    if (lse_at && lane == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
 // The same merge for the partials of the 256-row tensor-core schedule (fp16 rows divided by their own sums, at most 4
@@ -791,13 +801,15 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
     const int n_pairs = total_rows * p.hq;
     const int stride = gridDim.x * 4;
     const int rh0 = blockIdx.x * 4 + (threadIdx.x >> 5);
-    long long e0[kCombineRows], out_off[kCombineRows];
+    const float2* ml_at[kCombineRows];
+    unsigned char* out_at[kCombineRows];
+    float* lse_at[kCombineRows];
     const unsigned char* rows[kCombineRows];
     int ns[kCombineRows], stride_bytes[kCombineRows];
 #pragma unroll
     for (int j = 0; j < kCombineRows; ++j) {
         const int rh = rh0 + j * stride;
-        ns[j] = 0; e0[j] = 0; out_off[j] = 0; rows[j] = nullptr; stride_bytes[j] = 0;
+        ns[j] = 0; ml_at[j] = nullptr; out_at[j] = nullptr; lse_at[j] = nullptr; rows[j] = nullptr; stride_bytes[j] = 0;
         if (rh < n_pairs) {
             const int lrow = rh / p.hq, h = rh - lrow * p.hq;
             int si = 0, acc_rows = 0;
@@ -810,12 +822,15 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
             if (sp.nsplit > 1) {   // (a single split was written directly by the attention kernel)
                 const int i = lrow - acc_rows;
                 ns[j] = sp.nsplit;
-                e0[j] = (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit;
-                out_off[j] = (long long)(sp.q_row0 + i) * p.hq + h;
+                const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
+                ml_at[j] = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + lane;
+                out_at[j] = (unsigned char*)p.out + out_row * (kD * 2) + lane * 8;
+                lse_at[j] = p.lse ? p.lse + out_row : nullptr;
                 const HalfRows hr(p, sp, i, h, lane);
                 rows[j] = hr.at; stride_bytes[j] = hr.stride;
             }
         }
+        hold(ns[j]); hold(ml_at[j]); hold(out_at[j]); hold(lse_at[j]); hold(rows[j]); hold(stride_bytes[j]);
     }
     pdl_wait();   // the partials are complete
     float2 ml[kCombineRows];
@@ -823,7 +838,7 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
 #pragma unroll
     for (int j = 0; j < kCombineRows; ++j) {
         ml[j] = make_float2(-INFINITY, 0.f);
-        if (lane < ns[j]) ml[j] = ld_volatile_f2(p.part_ml + e0[j] + lane);
+        if (lane < ns[j]) ml[j] = ld_volatile_f2(ml_at[j]);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k < ns[j]) v[j][k] = ld_volatile_u2(rows[j] + k * stride_bytes[j]);
@@ -854,8 +869,8 @@ attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) 
         uint2 packed;
         packed.x = pack_bf16(acc.x * inv, acc.y * inv);
         packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-        *(uint2*)((__nv_bfloat16*)p.out + out_off[j] * kD + lane * 4) = packed;
-        if (p.lse && lane == 0) p.lse[out_off[j]] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+        *(uint2*)out_at[j] = packed;
+        if (lse_at[j] && lane == 0) *lse_at[j] = (m_all + log2f(l_all)) * 0.6931471805599453f;
     }
 }
 
@@ -882,9 +897,12 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
     if (ns > 1) {   // (a single split was written directly by the attention kernel)
         const SeqPlan& sp = p.seq[si];
         const int i = lrow - acc_rows;
-        const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
-        const long long out_off = (long long)(sp.q_row0 + i) * p.hq + h;
-        const HalfRows rows(p, sp, i, h, lane);
+        const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
+        const float2* ml_at = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * ns + lane;
+        unsigned char* out_at = (unsigned char*)p.out + out_row * (kD * 2) + lane * 8;
+        float* lse_at = p.lse ? p.lse + out_row : nullptr;
+        HalfRows rows(p, sp, i, h, lane);
+        hold(ml_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride); hold(ns);
         pdl_wait();   // the partials are complete
         // Every load is issued before the first use of any of them: volatile loads keep their place in the instruction stream
         // (left to itself the compiler moved the row loads behind the reduction of the maxima, i.e. behind a first trip to
@@ -894,7 +912,7 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
 #pragma unroll
         for (int k = 0; k < kNsMax; ++k) v[k] = rows.load(min(k, ns - 1));
         float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < ns) ml = ld_volatile_f2(p.part_ml + e0 + lane);
+        if (lane < ns) ml = ld_volatile_f2(ml_at);
         float m_all = ml.x;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
@@ -916,8 +934,8 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
         uint2 packed;
         packed.x = pack_bf16(acc.x * inv, acc.y * inv);
         packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-        *(uint2*)((__nv_bfloat16*)p.out + out_off * kD + lane * 4) = packed;
-        if (p.lse && lane == 0) p.lse[out_off] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+        *(uint2*)out_at = packed;
+        if (lse_at && lane == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
     }
 }
 

@@ -108,23 +108,28 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
     const int own_units = (n_pages - own_pg) * 512;   // 16-byte units, [page][K, V][16 rows][16 units]
     constexpr int kOwn = (512 + kThreads - 1) / kThreads;   // a thread's units of the first own page
+    // A unit's place in the pool but for its page, and its source where it is a block row's (held in registers for the first page).
+    auto own_tok = [&](int u) { return tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15); };
+    auto own_pool = [&](int u) {
+        return (unsigned char*)(((u >> 8) & 1) ? p.v_pool : p.k_pool) + (g * kPage + (own_tok(u) & 15)) * 256 + (u & 15) * 16;
+    };
+    auto own_new = [&](int u) {
+        const int tok = own_tok(u);
+        return (const unsigned char*)(((u >> 8) & 1) ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * 256 + (u & 15) * 16;
+    };
+    int num_pages = (int)min(p.num_pages, 0x7FFFFFFFll), page_bytes = p.hkv * kPage * 256;
     auto own_id = [&](int u) { const int slot = page0 + own_pg + (u >> 9); return slot < p.pt_stride ? __ldg(pt_row + slot) : -1; };
-    auto own_load = [&](int u, int id) {
-        const int tok = tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15), is_v = (u >> 8) & 1, ch = u & 15;
+    auto own_load = [&](int u, int id, unsigned char* in_pool, const unsigned char* in_new) {
+        const int tok = own_tok(u);
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (tok < pool_end) {
-            const long long page = (id < 0 || id >= p.num_pages) ? 0 : id;   // (reported below)
-            v = __ldcg((const uint4*)((const unsigned char*)(is_v ? p.v_pool : p.k_pool) + ((page * p.hkv + g) * kPage + (tok & 15)) * 256 + ch * 16));
-        } else if (tok < L) {
-            v = __ldg((const uint4*)((const unsigned char*)(is_v ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * 256 + ch * 16));
-        }
+        if (tok < pool_end) v = __ldcg((const uint4*)(in_pool + (long long)((id < 0 || id >= num_pages) ? 0 : id) * page_bytes));   // (reported below)
+        else if (tok < L) v = __ldg((const uint4*)in_new);
         return v;
     };
-    auto own_store = [&](int u, int id, const uint4 v) {
-        const int pg = own_pg + (u >> 9), r = (u >> 4) & 15, is_v = (u >> 8) & 1, ch = u & 15, tok = tok_begin + pg * kPage + r;
+    auto own_store = [&](int u, int id, unsigned char* in_pool, const uint4 v) {
+        const int pg = own_pg + (u >> 9), r = (u >> 4) & 15, is_v = (u >> 8) & 1, ch = u & 15, tok = own_tok(u);
         *(uint4*)(smem + (is_v ? S::kV : S::kK) + pg * 4096 + (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v;
-        if (tok >= pool_end && tok < L && id >= 0 && id < p.num_pages)
-            *(uint4*)((unsigned char*)(is_v ? p.v_pool : p.k_pool) + (((long long)id * p.hkv + g) * kPage + (tok & 15)) * 256 + ch * 16) = v;
+        if (tok >= pool_end && tok < L && id >= 0 && id < num_pages) *(uint4*)(in_pool + (long long)id * page_bytes) = v;
     };
     int first_id[kOwn];   // issuer: the id of page `lane`
     auto fetch_ids = [&]() {
@@ -135,6 +140,52 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 if (tid + j * kThreads < own_units) first_id[j] = own_id(tid + j * kThreads);
     };
     if (pre) fetch_ids();
+    // what the parameters are needed for behind the wait, worked out before it: sources of Q and of the own page, destinations of the result rows
+    constexpr int kUnits = NC * 16, kPer = (kUnits + kThreads - 1) / kThreads;
+    const uint4* q_at[kPer];
+    unsigned char* own_pool_at[kOwn];
+    const unsigned char* own_new_at[kOwn];
+    float2* ml_at = nullptr;
+    float* lse_at = nullptr;
+    float scale = p.scale_log2;
+    int half_rows = sp.nsplit == 1 || p.part_half;   // 16-bit result rows
+    const int my_row = lane & (NR - 1);
+    const bool merged_here = p.cluster_size > 1 && sp.nsplit > 1;
+    unsigned long long* const row_dst = (unsigned long long*)(smem + S::kDst) + warp * NR;
+    if (!issuer) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int c = tid + j * kThreads, r = c >> 4;
+            q_at[j] = nullptr;
+            if (c < kUnits && r < n_rows) {
+                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
+                q_at[j] = (const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16);
+            }
+            hold(q_at[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j) {
+            own_pool_at[j] = own_pool(tid + j * kThreads); own_new_at[j] = own_new(tid + j * kThreads);
+            hold(own_pool_at[j]); hold(own_new_at[j]);
+        }
+        if (tile < 2) {   // row my_row's, for all lanes of the warp through shared memory
+            unsigned long long dst = 0;
+            if (my_row < n_rows && !merged_here) {
+                const int i = div_g(row0 + my_row), hd = g * G + (row0 + my_row) - i * G;
+                if (sp.nsplit == 1) {
+                    const long long at = (long long)(sp.q_row0 + i) * p.hq + hd;
+                    dst = (unsigned long long)((unsigned char*)p.out + at * 256);
+                    if (p.lse && warp == 0 && lane < NR) lse_at = p.lse + at;
+                } else {
+                    const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
+                    dst = (unsigned long long)(p.part_o + e * 128);
+                    if (warp == 0 && lane < NR) ml_at = p.part_ml + e;
+                }
+            }
+            row_dst[my_row] = dst;
+        }
+    }
+    hold(ml_at); hold(lse_at); hold(scale); hold(half_rows); hold(num_pages); hold(page_bytes);
     if (issuer && lane == 0) {
         for (int i = 0; i < 3 * NT + 1; ++i) mbar_init(base + S::kBar + 8u * i, 1);
         *abort_flag = 0;
@@ -170,20 +221,15 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         if (!waited) pdl_wait();
     } else {
         // Q: [half of 64 dims][NC rows][128 B], 128-byte swizzle; rows past q * G are zeros.  (All loads are issued before the first store.)
-        constexpr int kUnits = NC * 16, kPer = (kUnits + kThreads - 1) / kThreads;
         uint4 v[kPer], w[kOwn];
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
-            const int c = tid + j * kThreads, r = c >> 4;
             v[j] = make_uint4(0, 0, 0, 0);
-            if (c < kUnits && r < n_rows) {
-                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
-                v[j] = __ldg((const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16));
-            }
+            if (q_at[j]) v[j] = __ldg(q_at[j]);
         }
 #pragma unroll
         for (int j = 0; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, first_id[j]);
+            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, first_id[j], own_pool_at[j], own_new_at[j]);
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int c = tid + j * kThreads, r = c >> 4, ch = c & 15;
@@ -191,8 +237,11 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
 #pragma unroll
         for (int j = 0; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, first_id[j], w[j]);
-        for (int u = tid + kOwn * kThreads; u < own_units; u += kThreads) { const int id = own_id(u); own_store(u, id, own_load(u, id)); }
+            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, first_id[j], own_pool_at[j], w[j]);
+        for (int u = tid + kOwn * kThreads; u < own_units; u += kThreads) {
+            const int id = own_id(u);
+            own_store(u, id, own_pool(u), own_load(u, id, own_pool(u), own_new(u)));
+        }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
     tc_fence_before();
@@ -245,7 +294,6 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         __syncwarp();
     }
 
-    const bool merged_here = p.cluster_size > 1 && sp.nsplit > 1;
     float* cl_o = (float*)(smem + S::kO);
     float2* cl_ml = (float2*)(smem + S::kO + NR * 512);
     if (!issuer) {
@@ -269,11 +317,10 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     }
     float* x_max = (float*)(smem + S::kMax);
     float* x_sum = (float*)(smem + S::kSum);
-    const int my_row = lane & (NR - 1);
 #pragma unroll
     for (int r = 0; r < NR; ++r) x[r] = s[r];
     const float w_max = across_lanes<NR>(x, [](float a, float b) { return fmaxf(a, b); });
-    x_max[warp * NR + my_row] = w_max * p.scale_log2;   // (NR < 32: several lanes write the same)
+    x_max[warp * NR + my_row] = w_max * scale;   // (NR < 32: several lanes write the same)
     tc_fence_before();
     asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");   // every warp's maxima; all scores are in registers, so K is dead
     tc_fence_after();
@@ -297,7 +344,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int r = r4 + k;
-                x[r] = ex2(fmaf(s[r], p.scale_log2, n[k]));
+                x[r] = ex2(fmaf(s[r], scale, n[k]));
                 *(__nv_bfloat16*)(pt + r * 128 + ((c ^ (r & 7)) << 4)) = __float2bfloat16_rn(x[r]);
             }
         }
@@ -319,23 +366,10 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
 
     // ---- epilogue: lane = head dim, column = row; the first two warpgroups take half of the rows each
     constexpr int kHalf = NR / 2;
-    // weight and destination of row my_row, for all lanes of the warp through shared memory (its copy of the row references is dead)
-    unsigned long long* row_dst = (unsigned long long*)(smem + S::kDst) + warp * NR;
+    // weight of row my_row, for all lanes of the warp through shared memory (its copy of the row references is dead)
     if (tile < 2) {
-        unsigned long long dst = 0;
-        if (my_row < n_rows && !merged_here) {
-            const int i = div_g(row0 + my_row), hd = g * G + (row0 + my_row) - i * G;
-            if (sp.nsplit == 1) {
-                const long long at = (long long)(sp.q_row0 + i) * p.hq + hd;
-                dst = (unsigned long long)((unsigned char*)p.out + at * 256);
-                if (p.lse && warp == 0 && lane < NR) p.lse[at] = (m_row + log2f(l_row)) * 0.6931471805599453f;
-            } else {
-                const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
-                dst = (unsigned long long)(p.part_o + e * 128);
-                if (warp == 0 && lane < NR) p.part_ml[e] = make_float2(m_row, l_row);
-            }
-        }
-        row_dst[my_row] = dst;
+        if (lse_at) *lse_at = (m_row + log2f(l_row)) * 0.6931471805599453f;
+        if (ml_at) *ml_at = make_float2(m_row, l_row);
         ref[my_row] = (l_row > 0.f) ? 1.f / l_row : 0.f;
         __syncwarp();
     }
@@ -355,7 +389,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             if (warp == 0 && lane < NR) cl_ml[lane] = make_float2(m_row, l_row);
 #pragma unroll
             for (int j = 0; j < kHalf; ++j) cl_o[(tile * kHalf + j) * 128 + d] = o[j];
-        } else if (sp.nsplit > 1 && !p.part_half) {   // the un-normalised fp32 rows
+        } else if (!half_rows) {   // the un-normalised fp32 rows
 #pragma unroll
             for (int j = 0; j < kHalf; ++j) {
                 const unsigned long long at = row_dst[tile * kHalf + j];

@@ -98,6 +98,19 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
+// Holds a value in a register from here on.  Kernel parameters are read through the constant cache where they are used, and the cache is cold at the
+// start of a launch: what is needed behind the dependency wait is worked out and held before it.  (A decode layer over 4096 tokens, launched as
+// a stream of kernels: 7.7 -> 7.25 us with it in the merge kernel, whose addresses come from six parameters, 6.8 with the attention kernel's; in
+// a graph, where the cache is warm, 6.15.  The warp-MMA and the tensor-core kernel gain nothing: the addresses are not on their critical path.)
+__device__ __forceinline__ void hold(int& x) { asm volatile("" : "+r"(x)); }
+__device__ __forceinline__ void hold(unsigned& x) { asm volatile("" : "+r"(x)); }
+__device__ __forceinline__ void hold(float& x) { asm volatile("" : "+f"(x)); }
+__device__ __forceinline__ void hold(long long& x) { asm volatile("" : "+l"(x)); }
+template <typename T>
+__device__ __forceinline__ void hold(T*& x) { asm volatile("" : "+l"(x)); }
+template <typename T>
+__device__ __forceinline__ void hold(T* __restrict__& x) { asm volatile("" : "+l"(x)); }
+
 // Programmatic dependent launch: a kernel lets the next launch in the stream start early (its CTAs then run
 // their set-up and block in pdl_wait), and itself waits, before it touches global memory, until the launch
 // before it has completed and its writes are visible.  Both are no-ops for launches without the attribute.
