@@ -107,8 +107,11 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int pool_end = p.k_new ? P : L;
     const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
     const int own_units = (n_pages - own_pg) * 512;   // 16-byte units, [page][K, V][16 rows][16 units]
-    constexpr int kOwn = (512 + kThreads - 1) / kThreads;   // a thread's units of the first own page
-    // A unit's place in the pool but for its page, and its source where it is a block row's (held in registers for the first page).
+    // a thread's units of the first own page, and of the second where there is one (a block of up to 16 rows lies in two at most; with the second
+    // page behind the first one's trip to memory 8 rows from token 2750 on took 10.0 us a layer, from 2752 on 8.1)
+    constexpr int kOwn1 = (512 + kThreads - 1) / kThreads, kOwn = (1024 + kThreads - 1) / kThreads;
+    const bool more_own = own_units > kOwn1 * kThreads;
+    // A unit's place in the pool but for its page, and its source where it is a block row's (held in registers for the first two pages).
     auto own_tok = [&](int u) { return tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15); };
     auto own_pool = [&](int u) {
         return (unsigned char*)(((u >> 8) & 1) ? p.v_pool : p.k_pool) + (g * kPage + (own_tok(u) & 15)) * 256 + (u & 15) * 16;
@@ -131,13 +134,13 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         *(uint4*)(smem + (is_v ? S::kV : S::kK) + pg * 4096 + (r >> 3) * 2048 + (ch >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v;
         if (tok >= pool_end && tok < L && id >= 0 && id < num_pages) *(uint4*)(in_pool + (long long)id * page_bytes) = v;
     };
-    int first_id[kOwn];   // issuer: the id of page `lane`
+    int first_id = 0, second_id = 0;   // of the own pages; issuer: first_id is that of page `lane`
     auto fetch_ids = [&]() {
-        if (issuer) first_id[0] = lane < n_pages ? __ldg(pt_row + page0 + lane) : 0;
-        else
-#pragma unroll
-            for (int j = 0; j < kOwn; ++j)
-                if (tid + j * kThreads < own_units) first_id[j] = own_id(tid + j * kThreads);
+        if (issuer) { if (lane < n_pages) first_id = __ldg(pt_row + page0 + lane); }
+        else if (own_units) {
+            first_id = own_id(0);
+            if (own_units > 512) second_id = own_id(512);
+        }
     };
     if (pre) fetch_ids();
     // what the parameters are needed for behind the wait, worked out before it: sources of Q and of the own page, destinations of the result rows
@@ -164,10 +167,11 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             hold(q_at[j]);
         }
 #pragma unroll
-        for (int j = 0; j < kOwn; ++j) {
-            own_pool_at[j] = own_pool(tid + j * kThreads); own_new_at[j] = own_new(tid + j * kThreads);
-            hold(own_pool_at[j]); hold(own_new_at[j]);
-        }
+        for (int j = 0; j < kOwn; ++j)
+            if (j < kOwn1 || more_own) {
+                own_pool_at[j] = own_pool(tid + j * kThreads); own_new_at[j] = own_new(tid + j * kThreads);
+                hold(own_pool_at[j]); hold(own_new_at[j]);
+            }
         if (tile < 2) {   // row my_row's, for all lanes of the warp through shared memory
             unsigned long long dst = 0;
             if (my_row < n_rows && !merged_here) {
@@ -202,7 +206,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (!pre) fetch_ids();
     if (issuer) {
         __syncwarp();
-        int id = first_id[0];
+        int id = first_id;
         if (lane < n_pages && (id < 0 || id >= p.num_pages)) { id = 0; atomicOr(p.status, AGX_DEV_BAD_PAGE); }
         bool waited = !pre;
         if (!waited && !p.k_new && tok_end > (P & ~(kPage - 1))) { pdl_wait(); waited = true; }
@@ -228,16 +232,24 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             if (q_at[j]) v[j] = __ldg(q_at[j]);
         }
 #pragma unroll
-        for (int j = 0; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, first_id[j], own_pool_at[j], own_new_at[j]);
+        for (int j = 0; j < kOwn1; ++j)
+            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
+        if (more_own)
+#pragma unroll
+        for (int j = kOwn1; j < kOwn; ++j)
+            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int c = tid + j * kThreads, r = c >> 4, ch = c & 15;
             if (c < kUnits) *(uint4*)(smem + S::kQ + (ch >> 3) * (NC * 128) + r * 128 + (((ch & 7) ^ (r & 7)) << 4)) = v[j];
         }
 #pragma unroll
-        for (int j = 0; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, first_id[j], own_pool_at[j], w[j]);
+        for (int j = 0; j < kOwn1; ++j)
+            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
+        if (more_own)
+#pragma unroll
+        for (int j = kOwn1; j < kOwn; ++j)
+            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
         for (int u = tid + kOwn * kThreads; u < own_units; u += kThreads) {
             const int id = own_id(u);
             own_store(u, id, own_pool(u), own_load(u, id, own_pool(u), own_new(u)));
