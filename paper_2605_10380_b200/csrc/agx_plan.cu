@@ -391,6 +391,22 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 if (c.debug_plan) fprintf(stderr, "agx plan: clusters of %d: %d fit the device, %lld needed\n", common, fit, base_items);
             }
         }
+        // One block in splits that an SM holds whole: as long as two or three KV tiles allow, and the last one a tile shorter than the others, since its
+        // CTA also puts the block's own pages together by hand.  At most 16 of them, with fp32 partials; two tiles up to 12 splits at 8 KV heads, where the
+        // launch leaves SMs to the next one's CTAs.  32/8 heads, a layer, equal splits / these: 8 rows over 700 tokens 7.2 / 6.6 us, 1550 7.1 / 6.6, 2750
+        // 7.7 / 7.2, 3500 9.2 / 7.8, 4096 8.3 / 8.1, 5100 11.0 / 9.0; one row over 4096 6.6 / 6.4, 5100 8.0 / 6.8.  (Up to 16 rows over 3100 to 3840
+        // tokens 15 equal splits of two tiles are faster: three rows over 3660 6.4 / 7.3.  From 17 splits of three tiles on nothing is gained.)
+        bool last_shorter = false;
+        if (whole && !cluster && seqs.size() == 1 && c.merge_sms) {
+            const int L = P[seqs[0]] + Q[seqs[0]], twos = ceil_div(L, 256) * c.num_kv_heads, tiles = twos * 10 <= c.sm_count * 7 ? 2 : 3;
+            const bool equal_twos = tiles == 3 && k == KIND_SMALL1 && twos * 6 <= c.sm_count * 5;
+            for (int t = tiles * 128; t > tiles * 128 - 128 && !last_shorter && !equal_twos; t -= unit) {
+                const int n = ceil_div(L, t);
+                if (n < 2 || n > 16 || n * c.num_kv_heads > c.sm_count || L - (n - 1) * t > (tiles - 1) * 128) continue;
+                C = t;
+                last_shorter = memory_merge = true;
+            }
+        }
         // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, with fp32 partials, are faster than 17 to 24 with SMs left to
         // the merge of fp16 rows (32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
         // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).  (All of it from 14 shapes.)
@@ -453,7 +469,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 sp.q_row0 = row0[s];
                 sp.seq_index = s;
                 sp.nsplit = ceil_div(L, C);
-                sp.split_tokens = round_up(ceil_div(L, sp.nsplit), unit);
+                sp.split_tokens = last_shorter ? C : round_up(ceil_div(L, sp.nsplit), unit);
                 sp.nsplit = ceil_div(L, sp.split_tokens);
                 if (cluster) { sp.nsplit = cluster; sp.split_tokens = round_up(ceil_div(L, cluster), kPage); }
                 sp.row_chunks = (Q[s] * G + rows_per_chunk - 1) / rows_per_chunk;

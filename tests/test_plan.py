@@ -108,3 +108,17 @@ def test_chains_of_the_fp32_kernel_are_bounded():
         return max(s.split_tokens for l in plan(P, Q, dtype="f32", hq=32, hkv=8).launches for s in l.seqs)
     assert longest([20000] + [40] * 30, [1] * 31) <= 256 and longest([8000] * 6, [1] * 6) <= 256 and longest([1000] * 16, [1] * 16) == 512
     assert plan([0], [4000], dtype="f32", hq=32, hkv=8).launches[0].seqs[0].nsplit == 1
+
+
+@pytest.mark.parametrize("q", [3, 8])
+def test_one_block_has_a_shorter_last_split(q):
+    """Blocks of one sequence in splits that an SM holds whole: at most 16, the last one with a KV tile less than the others."""
+    shorter = 0
+    for L in range(270, 6200, 37):
+        ln = plan([L - q], [q]).launches[0]
+        s = ln.seqs[0]
+        if ln.kind in ("small1", "small2") and s.split_tokens <= 384 and not ln.cluster and not ln.lean:
+            last = L - (s.nsplit - 1) * s.split_tokens
+            assert 2 <= s.nsplit <= 16 and 0 < last <= s.split_tokens
+            shorter += -(-last // 128) < -(-s.split_tokens // 128)
+    assert shorter > 100
