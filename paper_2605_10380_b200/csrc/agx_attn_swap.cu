@@ -22,6 +22,7 @@ namespace agx {
 namespace {
 
 constexpr int kTileTok = 128;
+constexpr unsigned kSuspendNs = 20000;   // see mbar_try_wait
 constexpr uint32_t kTile = 128 * 256;   // 8 pages of K or V
 constexpr uint32_t kCols = 128;         // TMEM: O^T at column 0, S^T of tile t at 32 + 32 t
 
@@ -267,7 +268,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         if (elect_one()) {
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
-                ok = mbar_wait(k_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
+                ok = mbar_wait<kSuspendNs>(k_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t kd = make_desc(base + S::kK + t * kTile, 16, 2048), qd = make_desc(base + S::kQ, 16, 1024);
@@ -285,7 +286,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         if (elect_one()) {
             bool ok = !*abort_flag;
             for (int t = 0; t < n_tiles && ok; ++t) {
-                ok = mbar_wait(v_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
+                ok = mbar_wait<kSuspendNs>(v_bar(t), 0, abort_flag, p.status, p.wait_limit_cycles);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t vd = make_desc(base + S::kV + t * kTile, 1024, 2048), pd = make_desc(base + S::kP + t * (2 * NC * 128), 16, 1024);
@@ -312,7 +313,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // ---- one token per thread: mask, row maxima, P = 2^(S * scale - m)
     const uint32_t lanes = (uint32_t)((warp & 3) << 5) << 16;
     const int t_warp = tile * kTileTok + (warp & 3) * 32, tok = tok_begin + t_warp + lane;   // (t_warp: first token of the warp, from tok_begin)
-    bool live = tile < n_tiles && __all_sync(0xFFFFFFFFu, mbar_wait(s_bar(min(tile, NT - 1)), 0, abort_flag, p.status, p.wait_limit_cycles));
+    bool live = tile < n_tiles && __all_sync(0xFFFFFFFFu, mbar_wait<kSuspendNs>(s_bar(min(tile, NT - 1)), 0, abort_flag, p.status, p.wait_limit_cycles));
     float s[NR], x[NR];
     if (live) {
         tc_fence_after();
@@ -385,7 +386,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         ref[my_row] = (l_row > 0.f) ? 1.f / l_row : 0.f;
         __syncwarp();
     }
-    const bool done = __all_sync(0xFFFFFFFFu, mbar_wait(o_bar, 0, abort_flag, p.status, p.wait_limit_cycles));
+    const bool done = __all_sync(0xFFFFFFFFu, mbar_wait<kSuspendNs>(o_bar, 0, abort_flag, p.status, p.wait_limit_cycles));
     if (tile < 2) {
         float o[kHalf];
         if (done && n_tiles > 0) {
