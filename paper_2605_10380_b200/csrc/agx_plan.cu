@@ -25,18 +25,24 @@ struct SplitModel {
     double merge, merge_mb, merge_mb_beyond_16;   // merge launch, per MB of partials up to 16 (they stay in L2) and beyond
     int part_row_bytes;
     double lean;            // > 0: one-wave launches with few (row, head) pairs leave SMs to their merge kernel, which costs this and 0.2 per MB
+    bool in_order;          // up to 16 waves: CTAs dealt out as the grid has them instead of longest first
 };
+// Fitted to 340 launches of one to eight blocks, each in all splits that make sense: the split chosen is 1.0 % slower than the best of them on
+// average (with 1.9 us a tile, 2.2 + 0.38 us per MB: 1.4 %).  The grid's order counts where a launch is little more than
+// one wave: 152 CTAs dealt out longest first fit 148 SMs as if the short ones were stacked, but the last ones to start are long ones (256 tokens behind
+// 3000, 32/8 heads, 5 / 4 splits: 31.1 / 21.7 us a layer; 931 behind 3086, 24/8: 66.7 -> 60.2; 598 behind 5293: 76 -> 68.3; verify blocks with three to
+// eight prefills 5 to 10 %).  (Planning a new batch of 1 / 8 / 48 prefills takes 21 / 57 / 102 us instead of 16 / 30 / 95.)
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
-SplitModel tile_model(const PlanConfig& c) { return {128, c.sm_count, 3, 5.7, 0, 1.9, 0, 2.2, 0.38, 0.3, 264, 0}; }
+SplitModel tile_model(const PlanConfig& c) { return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.5, 0.45, 0.3, 264, 0, true}; }
 // (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them.  40 rows over 300 / 450 / 600
 // tokens, 40/8 heads, take 9.0 / 9.8 / 10.5 us whole and 10.5 / 10.1 / 9.9 in splits of 256 tokens: the merge behind two tiles costs as much as two)
 SplitModel stream_model(const PlanConfig& c, bool wide) {
-    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, wide ? 2.2 : 1.0};
+    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, wide ? 2.2 : 1.0, false};
 }
 // warp-MMA kernel with 4-page stages, two CTAs per SM: HBM-bound with one 16-row tile, bounded by its own chain with two (mma.sync)
 SplitModel small4_model(const PlanConfig& c, int mt) {
-    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, 0};
+    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, 0, false};
 }
 
 // Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time, and that time.  A server's lengths change with every
@@ -89,7 +95,8 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
             }
         }
     };
-    struct Cand { int tiles, longest; double bound, merge; long long sum; };
+    struct Cand { int tiles, longest; double bound, merge; long long sum, count; };
+    struct Chunks { long long n; int per, full, rest; };
     std::vector<Cand> cands;
     const int n_max = (int)std::min<long long>((max_tiles + min_tiles - 1) / min_tiles, std::max<long long>(32, 2 * sms / std::max<long long>(base_items, 1)));
     cands.reserve(n_max);
@@ -115,6 +122,7 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         cd.tiles = t;
         cd.longest = longest;
         cd.sum = sum;
+        cd.count = count;
         cd.merge = mb == 0 ? 0 : md.lean > 0 && count <= sms * 15 / 16 && pairs <= 3 * sms ? md.lean + 0.2 * mb
                    : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
                    : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
@@ -126,19 +134,15 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
     SplitChoice best;
     std::vector<int> load;
     std::vector<long long> of_size;   // CTAs with that many tiles
+    std::vector<Chunks> in_order;
     for (const Cand& cd : cands) {
         if (best.tiles && cd.bound >= best.time) break;   // (bounds ascend)
-        of_size.assign(cd.longest + 1, 0);
-        deal(cd.tiles, [&](const Seen& v, int per, int full, int rest) {
-            if (full) of_size[per] += v.n * full;
-            of_size[rest] += v.n;   // (of_size[0] is not looked at)
-        });
         // load[x]: SMs with x tiles (and starts) so far; a CTA goes to an SM with the least
         load.assign((size_t)(cd.sum / sms) + cd.longest + kOverhead + 2, 0);
         load[0] = sms;
         size_t lo = 0, hi = 0;
-        for (int size = cd.longest; size > 0; --size)
-            for (long long left = of_size[size]; left > 0;) {
+        auto place = [&](int size, long long left) {
+            while (left > 0) {
                 while (load[lo] == 0) ++lo;
                 const int k = (int)std::min<long long>(load[lo], left);
                 load[lo] -= k;
@@ -146,6 +150,27 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
                 hi = std::max(hi, lo + size + kOverhead);
                 left -= k;
             }
+        };
+        if (md.in_order && cd.count <= 16 * sms) {
+            in_order.clear();
+            deal(cd.tiles, [&](const Seen& v, int per, int full, int rest) { in_order.push_back({v.n, per, full, rest}); });
+            size_t at = 0, first = 0;
+            for (const Seq& w : work) {   // a sequence's row chunks last to first, a chunk's splits first to last
+                for (at = w.seen_end; at-- > first;)
+                    for (long long n = 0; n < in_order[at].n; ++n) {
+                        place(in_order[at].per, in_order[at].full);
+                        if (in_order[at].rest) place(in_order[at].rest, 1);
+                    }
+                first = w.seen_end;
+            }
+        } else {
+            of_size.assign(cd.longest + 1, 0);
+            deal(cd.tiles, [&](const Seen& v, int per, int full, int rest) {
+                if (full) of_size[per] += v.n * full;
+                of_size[rest] += v.n;   // (of_size[0] is not looked at)
+            });
+            for (int size = cd.longest; size > 0; --size) place(size, of_size[size]);
+        }
         double t = md.base;
         size_t prev = kOverhead;
         int busy = sms;

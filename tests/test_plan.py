@@ -122,3 +122,15 @@ def test_one_block_has_a_shorter_last_split(q):
             assert 2 <= s.nsplit <= 16 and 0 < last <= s.split_tokens
             shorter += -(-last // 128) < -(-s.split_tokens // 128)
     assert shorter > 100
+
+
+@pytest.mark.parametrize("P,q,hq,hkv", [(3000, 256, 32, 8), (2364, 308, 24, 8), (875, 225, 32, 8), (1500, 200, 32, 8), (5000, 256, 16, 2)])
+def test_a_few_long_splits_are_not_left_for_a_second_wave(P, q, hq, hkv):
+    """A split prefill of about one wave: the CTAs with tokens fit the SMs at once, or all of them take part in the second wave."""
+    ln, = plan([P], [q], hq, hkv).launches
+    assert ln.kind == "tile"
+    s, G, busy = ln.seqs[0], hq // hkv, 0
+    for rc in range(s.row_chunks):
+        seen = P + min(q - 1, (256 * rc + 255) // G) + 1
+        busy += hkv * min(s.nsplit, -(-seen // s.split_tokens))
+    assert busy <= 148 or busy >= 1.5 * 148
