@@ -22,6 +22,8 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "agx_internal.cuh"
 
 #include <algorithm>
@@ -606,6 +608,23 @@ struct HalfRows {
     }
     __device__ __forceinline__ uint2 load(int split) const { return ld_volatile_u2(at + (long long)split * stride); }   // (written by other SMs just before: past the L1)
 };
+// The same of the fp32 partials (columns [4 lane, 4 lane + 4)).
+struct F32Rows {
+    const unsigned char* at;
+    int stride;
+    __device__ __forceinline__ F32Rows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane) {
+        if (p.part_half == PART_F32_TILES) {
+            const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rows = sp.q_len * p.gqa;
+            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + (long long)g * sp.nsplit * rows) * 512 + ((lane >> 4) * rows + r) * 256 +
+                 (((lane & 15) ^ (r & 15)) << 4);
+            stride = rows * 512;
+        } else {
+            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * (p.head_dim * 4) + lane * 16;
+            stride = p.head_dim * 4;
+        }
+    }
+    __device__ __forceinline__ float4 load(int split) const { return ld_volatile_f4((const float*)(at + (long long)split * stride)); }
+};
 template <bool kBf16Out, int kMaxNs>
 __global__ void __launch_bounds__(128, kMaxNs <= 4 ? 10 : kMaxNs <= 16 ? 5 : 3)
 attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
@@ -634,11 +653,11 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m_all, l_all;
     const float2* ml_at = p.part_ml + e0 + lane;
-    const float* row_at = p.part_o + e0 * D + c4;
+    F32Rows rows(p, sp, i, h, lane);
     const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
     unsigned char* out_at = (unsigned char*)p.out + (out_row * D + c4) * (kBf16Out ? 2 : 4);
     float* lse_at = p.lse ? p.lse + out_row : nullptr;
-    hold(ml_at); hold(row_at); hold(out_at); hold(lse_at);
+    hold(ml_at); hold(rows.at); hold(rows.stride); hold(out_at); hold(lse_at);
     pdl_wait();   // the partials are complete
     // One round trip to memory: lane k fetches (m, l) of split k while every lane already fetches its
     // columns of every split's O row; the weights then travel by shuffle, splits in index order.
@@ -648,11 +667,11 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     float4 v[kInFlight], v2[kFew ? 1 : 16];
 #pragma unroll
     for (int j = 0; j < kInFlight; ++j)
-        if (j < ns && c4 < D) v[j] = ld_volatile_f4(row_at + j * D);
+        if (j < ns && c4 < D) v[j] = rows.load(j);
     if (!kFew && ns > 16) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-            if (16 + j < ns && c4 < D) v2[j] = ld_volatile_f4(row_at + (16 + j) * D);
+            if (16 + j < ns && c4 < D) v2[j] = rows.load(16 + j);
     }
     m_all = ml.x;
 #pragma unroll
@@ -715,15 +734,14 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     const int ns = sp.nsplit, D = p.head_dim, c4 = lane * 4, i = lrow - acc_rows;
     if (ns == 1) return;   // written directly by the attention kernel
     const long long e0 = (long long)sp.part_base + ((long long)i * p.hq + h) * ns;
-    HalfRows rows(p, sp, i, h, lane);
+    std::conditional_t<kHalfPart, HalfRows, F32Rows> rows(p, sp, i, h, lane);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float m = -INFINITY, l = 0.f;
     const float2* ml_at = p.part_ml + e0 + lane;
-    const float* row_at = p.part_o + e0 * D + c4;
     const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
     unsigned char* out_at = (unsigned char*)p.out + (out_row * D + c4) * (kBf16Out ? 2 : 4);
     float* lse_at = p.lse ? p.lse + out_row : nullptr;
-    hold(ml_at); hold(row_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride);
+    hold(ml_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride);
     pdl_wait();   // the partials are complete
     for (int k0 = warp * kManyBatch; k0 < ns; k0 += warps * kManyBatch) {
         const int n = min(kManyBatch, ns - k0);
@@ -733,12 +751,12 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
 #pragma unroll
         for (int j = 0; j < kManyBatch; ++j)
             if (j < n && c4 < D) {
-                if (kHalfPart) {
+                if constexpr (kHalfPart) {
                     const uint2 raw = rows.load(k0 + j);
                     const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
                     v[j] = make_float4(a.x, a.y, b.x, b.y);
                 } else {
-                    v[j] = ld_volatile_f4(row_at + (long long)(k0 + j) * D);
+                    v[j] = rows.load(k0 + j);
                 }
             }
         float m_new = ml.x;
@@ -1058,7 +1076,7 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
     int ns_max = 1;
     for (int i = 0; i < p.num_seqs; ++i) ns_max = p.seq[i].nsplit > ns_max ? p.seq[i].nsplit : ns_max;
     const int many_threads = 32 * std::min(kManyWarps, (ns_max + kManyBatch - 1) / kManyBatch);
-    if (dtype == AGX_BF16 && p.part_half) {
+    if (dtype == AGX_BF16 && (p.part_half == PART_HALF_SLOTS || p.part_half == PART_HALF_TILES)) {
         if (ns_max <= 4) {
             // CTAs whose warps take kCombineRows pairs each
             const int want = (int)((n + 4 * kCombineRows - 1) / (4 * kCombineRows));

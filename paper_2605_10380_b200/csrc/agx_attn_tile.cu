@@ -176,7 +176,7 @@ struct EpiCtx {
     TileItem it;
     int part_base, hq;
     int part_half;   // a PartHalf
-    unsigned char* part_tile;   // 256-row schedule: this CTA's tile of fp16 partials
+    unsigned char* part_tile;   // 256-row schedule: this CTA's tile of partials, or the first 64 columns of its rows
     void* out;
     float* part_o;
     float2* part_ml;
@@ -215,7 +215,7 @@ __device__ __forceinline__ TileItem locate_item(const AttnParams& p, int block) 
 // With a single KV split the rows are normalised and written as bf16; otherwise partials and (m, l) go to the
 // workspace for the combine kernel.  Kept out of line, and re-deriving its indices from the block index,
 // so that nothing but its few arguments has to stay alive across the register-hungry main loop.
-template <bool kStreams>
+template <bool kStreams, bool kF32Part>
 __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, float m_ref, float l_run, bool ok) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     {   // the context is written by another warp at kernel start: wait for its arrival (long complete, normally)
@@ -301,7 +301,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                 }
             }
             const bool half_part = kStreams && !single && cx.part_half != PART_F32;
-            if (single || !kStreams || half_part) {   // (the 256-row schedule normalises its split partials too: they leave as fp16)
+            if (single || (!kStreams && !kF32Part) || half_part) {   // (the 256-row schedule normalises its fp16 partials too)
 #pragma unroll
                 for (int c = 0; c < 64; ++c) oreg[c] = __float_as_uint(__uint_as_float(oreg[c]) * inv);
             }
@@ -327,6 +327,22 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                         }
                     }
                 }
+            } else if (kF32Part && !single) {
+                // fp32 partials: these 64 columns of the warp's rows go through the staging area
+                if (c8) {
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int v = 0; v < 16; ++v)
+                    *(uint4*)(stage + lane * 256 + ((v ^ (lane & 15)) << 4)) = make_uint4(oreg[4 * v], oreg[4 * v + 1], oreg[4 * v + 2], oreg[4 * v + 3]);
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(cx.part_tile + (long long)(c8 >> 1) * it.rows * 256 + (warp - 4) * 8192),
+                                 "r"(smem_u32(stage)), "r"(min(32, it.rows - r_warp0) * 256) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                }
             } else {
                 // pack to the 16-bit output format first (bf16 results, fp16 split partials): 256 bytes per row go through
                 // the staging area, 16-byte units XOR-swizzled by row
@@ -351,8 +367,12 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     }
     if (kStreams) return;
     const int n_valid = min(32, it.rows - r_warp0);
+    if (kF32Part && !single) {
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
+        return;
+    }
     if (!single) {
-        // Split partials leave as they lie in the staging area, one bulk copy a warp: they are in a layout of their own, that of the staging
+        // fp16 split partials leave as they lie in the staging area, one bulk copy a warp: they are in a layout of their own, that of the staging
         // area.  Row by row through the LSU to a slot per (row, head, split) took 1.4 us instead of 0.1.
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncwarp();
@@ -472,7 +492,7 @@ struct QTile {
 
 }  // namespace
 
-template <bool kStreams>
+template <bool kStreams, bool kF32Part>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k,
                       const __grid_constant__ CUtensorMap map_v, const __grid_constant__ RowsMaps maps_new) {
@@ -779,7 +799,9 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cx->magic = p.row_div_magic; cx->status = p.status;
             cx->part_half = p.part_half;
             const int rc = row0 / kRowsPerCta;
-            cx->part_tile = (unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536;
+            cx->part_tile = (unsigned char*)p.part_o + (long long)sp.part_base * 512 +
+                            (kF32Part ? ((long long)g * sp.nsplit + split) * rows * 512 + row0 * 256
+                                      : (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536);
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }
         // what of the fused append is no whole row group of a tile that stays in shared memory (see the end of warp 0)
@@ -931,7 +953,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             if (lane == 0) mbar_arrive(bar(BAR_P_TAIL + x));
         }
         if (kStreams && ok) ok = mbar_wait(bar(BAR_O_FULL), 0, abort_flag, p.status, p.wait_limit_cycles);   // (else waited for in the epilogue)
-        if (ok || kStreams) tile_epilogue<kStreams>(smem, tO, m_ref, l_run, ok);
+        if (ok || kStreams) tile_epilogue<kStreams, kF32Part>(smem, tO, m_ref, l_run, ok);
     }
     // ---- teardown
     tc_fence_before();
@@ -1016,7 +1038,7 @@ bool make_q_maps(RowsMaps* m, const void* q, long long total_q, int hq, int hkv,
 }
 
 namespace {
-template <bool kStreams>
+template <bool kStreams, bool kF32Part>
 cudaError_t launch_tile(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, const RowsMaps& maps_new,
                         cudaStream_t stream) {
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
@@ -1025,18 +1047,20 @@ cudaError_t launch_tile(const AttnParams& p, const CUtensorMap& map_k, const CUt
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
     bool& configured = configured_on[device];
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(attn_tile_bf16_kernel<kStreams>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(attn_tile_bf16_kernel<kStreams, kF32Part>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_chained(attn_tile_bf16_kernel<kStreams>, dim3(p.num_items), dim3(kThreads), kSmemBytes, stream, p, map_k, map_v, maps_new);
+    return launch_chained(attn_tile_bf16_kernel<kStreams, kF32Part>, dim3(p.num_items), dim3(kThreads), kSmemBytes, stream, p, map_k, map_v, maps_new);
 }
 }  // namespace
 
 cudaError_t launch_attn_tile_bf16(const AttnParams& p, bool streams, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                   const RowsMaps& maps_new, cudaStream_t stream) {
     if (p.num_items == 0) return cudaSuccess;
-    return streams ? launch_tile<true>(p, map_k, map_v, maps_new, stream) : launch_tile<false>(p, map_k, map_v, maps_new, stream);
+    if (streams) return launch_tile<true, false>(p, map_k, map_v, maps_new, stream);
+    // (fp32 partials as a case of the same kernel: 512-row prefills 0.8 % slower, for the code at the end of a CTA)
+    return p.part_half == PART_F32_TILES ? launch_tile<false, true>(p, map_k, map_v, maps_new, stream) : launch_tile<false, false>(p, map_k, map_v, maps_new, stream);
 }
 
 }  // namespace agx

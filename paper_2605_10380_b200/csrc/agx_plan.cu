@@ -34,7 +34,9 @@ struct SplitModel {
 // eight prefills 5 to 10 %).  (Planning a new batch of 1 / 8 / 48 prefills takes 21 / 57 / 102 us instead of 16 / 30 / 95.)
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
-SplitModel tile_model(const PlanConfig& c) { return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.5, 0.45, 0.3, 264, 0, true}; }
+SplitModel tile_model(const PlanConfig& c, bool f32_partials = false) {
+    return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, f32_partials ? 1.9 : 1.5, f32_partials ? 0.3 : 0.45, 0.3, f32_partials ? 520 : 264, 0, true};
+}
 // (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them.  40 rows over 300 / 450 / 600
 // tokens, 40/8 heads, take 9.0 / 9.8 / 10.5 us whole and 10.5 / 10.1 / 9.9 in splits of 256 tokens: the merge behind two tiles costs as much as two)
 SplitModel stream_model(const PlanConfig& c, bool wide) {
@@ -219,6 +221,7 @@ PlanConfig plan_config(const agx_config& cfg, int sm_count, int (*max_clusters)(
     c.merge_sms = number("AGX_MERGE_SMS", 1) != 0;
     c.cluster_merge = !getenv("AGX_CLUSTER_MERGE") ? 1 : number("AGX_CLUSTER_MERGE", 0) ? 2 : 0;
     c.stream_max_rows = number("AGX_STREAM_MAX_ROWS", 384);
+    c.stream_rows_estimated = getenv("AGX_STREAM_MAX_ROWS") == nullptr;
     c.stream_min_tokens = number("AGX_STREAM_MIN_TOKENS", -1);
     return c;
 }
@@ -255,8 +258,23 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             if (rows <= 32) { small_k += (P[s] + Q[s]) * 1e-3 * c.num_kv_heads / 8; small_rows = std::max(small_rows, rows); small_seqs.push_back(s); }
             else if (rows <= c.stream_max_rows) wide_seqs.push_back(s);
         }
+    // One block of 65 to 384 rows: the 256-row schedule reads K/V half as often as 128-row chunks do and takes fewer splits, but one KV tile at a
+    // time, so that it loses where HBM is the bound.  By the estimates of both, with a margin for what they miss; its partials are fp32 here, as
+    // those of the other schedule.  120 such blocks, up to 384 rows over 200 to 16000 tokens: 10 % faster together than all of them in 128-row chunks, single
+    // ones up to 5 % slower.  A layer in us: (693, 37) 14.4 -> 9.1, (1687, 70) 19.5 -> 12.6 with 24/8 heads, (2110, 42) 16.7 -> 11.7 with 32/8.
+    // (Batches: gains and losses of 20 %, which the estimates do not tell apart.  One query head per KV head: not measured.)
+    bool wide_tiles = false;
+    SplitChoice tile_choice, stream_choice, small_choice[2];   // splits that the estimates were made with, where they were
+    if (c.stream_rows_estimated && B == 1 && wide_seqs.size() == 1 && Q[0] * G > kSmallRowsMax && G > 1 && !c.force_mma_sync) {
+        auto estimate = [&](const SplitModel& md, int chunk, int min_tiles) {
+            return choose_split(c, md, wide_seqs, P, Q, G, chunk, min_tiles, (long long)c.num_kv_heads * ((Q[0] * G + chunk - 1) / chunk));
+        };
+        tile_choice = estimate(tile_model(c, true), 256, 1);
+        stream_choice = estimate(stream_model(c, true), 128, 2);
+        wide_tiles = tile_choice.time < (Q[0] * G <= 128 ? 0.86 : 0.89) * stream_choice.time;
+        if (c.debug_plan) fprintf(stderr, "agx plan: %d rows, 256-row schedule %.1f us, 128-row chunks %.1f us\n", Q[0] * G, tile_choice.time, stream_choice.time);
+    }
     bool batch_streams = false;
-    SplitChoice stream_choice, small_choice[2];   // splits that the estimates below were made with, where they were
     if (!small_seqs.empty()) {
         if (c.batch_stream_tokens >= 0) {
             batch_streams = small_seqs.size() >= 2 && small_k * 1e3 >= c.batch_stream_tokens;
@@ -306,7 +324,8 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             // (with the batch rule forced the estimates are not asked, and a sequence of its own keeps the cross-over between the two kernels)
             const int cross = c.stream_min_tokens >= 0 ? c.stream_min_tokens : c.batch_stream_tokens < 0 ? INT_MAX : rows > 8 ? 7168 : 10240;
             const bool forced = P[s] + Q[s] >= cross;
-            if (tile_ok && rows <= c.stream_max_rows && (rows > 32 || batch_streams || forced)) k = KIND_STREAM;
+            if (wide_tiles) k = KIND_TILE;
+            else if (tile_ok && rows <= c.stream_max_rows && (rows > 32 || batch_streams || forced)) k = KIND_STREAM;
             else if (rows <= 16) k = KIND_SMALL1;
             else if (rows <= 32) k = KIND_SMALL2;
             else if (rows <= kSmallRowsMax || c.force_mma_sync) k = KIND_SMALL4;
@@ -366,7 +385,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         if (k == KIND_TILE || k == KIND_STREAM) {
             int max_len = 0;
             for (int s : seqs) max_len = std::max(max_len, P[s] + Q[s]);
-            SplitChoice choice = k == KIND_STREAM ? stream_choice : SplitChoice();
+            SplitChoice choice = k == KIND_STREAM ? stream_choice : tile_choice;
             if (!choice.tiles) {
                 const bool wide = std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; });
                 choice = choose_split(c, k == KIND_STREAM ? stream_model(c, wide) : tile_model(c), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
@@ -484,6 +503,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             ln.num_items = 0;
             ln.cluster = cluster;
             ln.lean_merge = lean_merge;
+            ln.f32_partials = wide_tiles;
             ln.kw = kw;
             for (size_t n = a; n < std::min(seqs.size(), a + kMaxSeqs); ++n) {
                 const int s = seqs[n];
@@ -507,7 +527,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 if (sp.nsplit > 1 && !cluster) {
                     long long entries = (long long)Q[s] * c.num_q_heads * sp.nsplit;
                     // (a tile of fp16 partials is 128 slots: more than the slots of its rows only where one chunk has fewer than 128 of them)
-                    if (k == KIND_TILE) entries = std::max(entries, per_seq_items[n] * sp.nsplit * 128);
+                    if (k == KIND_TILE && !wide_tiles) entries = std::max(entries, per_seq_items[n] * sp.nsplit * 128);
                     if (plan.part_entries + entries > 0x7FFFFFFFll) return fail(AGX_E_RANGE, "split partials exceed 2^31 entries");
                     sp.part_base = (int)plan.part_entries;
                     plan.part_entries += entries;
