@@ -847,7 +847,7 @@ def run_agx(args):
     dom = dict(head["roofline"]["prefill_blocks"])   # the dominant kernel of the step: the 256-row tensor-core schedule
     traffic, traffic_src = ncu_traffic("attn_tile_bf16_c5_long_context_prefill.txt", TILE_SOURCES)
     dom.update({"traffic": traffic, "traffic_source": traffic_src,
-                "kernel": "attn_tile_bf16_kernel<false> (+ attn_combine_kernel where the planner splits the KV axis): the "
+                "kernel": "attn_tile_bf16_kernel<false, false> (+ attn_combine_kernel where the planner splits the KV axis): the "
                           "agx_attn_prefixed call on the 2048-row prefill block",
                 "us_per_launch": dom["us"], "share_of_step": dom["us"] * 1e-3 / head["ms_per_step"]})
     line = {
