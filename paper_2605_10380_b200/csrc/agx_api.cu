@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <exception>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -23,6 +24,44 @@ struct CallRange {
 };
 }  // namespace
 
+// `out` of the last attention call on a stream, of whatever handle: kernels that write it may still be running when the next call's first one starts (of
+// calls further in front none is).  At most 16 streams are kept; of one that had to make room nothing is known, and it may write anything.
+class LastOuts {
+    struct Entry { int device; const void* stream; const char* at; size_t bytes; };
+    std::mutex lock;
+    Entry entries[16];
+    int used = 0, next = 0;
+    bool full = false;
+    static const void* key(cudaStream_t s) {
+        static thread_local char own;
+        return s == cudaStreamPerThread ? &own : (const void*)s;
+    }
+    Entry* find(int device, const void* k) {
+        for (int i = 0; i < used; ++i)
+            if (entries[i].device == device && entries[i].stream == k) return &entries[i];
+        return nullptr;
+    }
+
+public:
+    void set(int device, cudaStream_t s, const void* at, size_t bytes) {
+        const std::lock_guard<std::mutex> hold(lock);
+        Entry* e = find(device, key(s));
+        if (!e) {
+            full |= used == 16;
+            e = &entries[next];
+            next = (next + 1) % 16;
+            used = std::max(used, (int)(e - entries) + 1);
+        }
+        *e = {device, key(s), (const char*)at, bytes};
+    }
+    bool may_write(int device, cudaStream_t s, const void* p, size_t bytes) {
+        const std::lock_guard<std::mutex> hold(lock);
+        const Entry* e = find(device, key(s));
+        return e ? (const char*)p < e->at + e->bytes && e->at < (const char*)p + bytes : full;
+    }
+};
+static LastOuts g_last_outs;
+
 struct agx_handle {
     agx_config cfg;
     float scale;
@@ -37,8 +76,6 @@ struct agx_handle {
     long long wait_limit_cycles;   // AGX_OPT_WAIT_LIMIT_CYCLES
     int early_prefix;       // AGX_OPT_EARLY_PREFIX_LOADS
     int drop_stage;         // AGX_OPT_TEST_DROP_STAGE (-1 = none)
-    const char* last_out;   // `out` of the last attention call: kernels that write it may still be running when the next call's start
-    size_t last_out_bytes;
     std::vector<int32_t> cu_host;  // staging for agx_verify_step_host (lives until its final sync)
     // Large attention-only host steps run as a pipeline of row chunks: uploads on one stream of the handle's own, the
     // attention calls on the caller's stream, downloads on a third (env AGX_HOST_PIPELINE_ROWS: rows per chunk, 0 = off).
@@ -149,8 +186,6 @@ agx_status agx_create(const agx_config* cfg, agx_handle** out) {
     env = getenv("AGX_HOST_PIPELINE_ROWS");
     h->pipe_rows = env ? std::max(0, atoi(env)) : 384;   // measured on the long-context step: 256 / 384 / 512 / 768 / 1024 rows -> 1.54 / 1.43 / 1.57 / 1.56 / 1.72 ms
     h->pipe_in = h->pipe_out = nullptr;
-    h->last_out = nullptr;
-    h->last_out_bytes = 0;
     env = getenv("AGX_ZERO_COPY");
     h->zero_copy = env ? atoi(env) : 3;
     h->wait_limit_cycles = kWaitLimitCycles;
@@ -273,8 +308,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         else if (plan.tensor_core) memset(&maps_new, 0, sizeof maps_new);
         if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
-    h->last_out = (const char*)out;
-    h->last_out_bytes = (size_t)plan.total_rows * p.hq * p.head_dim * elem_size(h->cfg.dtype);
+    g_last_outs.set(h->device, stream, out, (size_t)plan.total_rows * p.hq * p.head_dim * elem_size(h->cfg.dtype));
     for (const Launch& ln : plan.launches) {
         p.num_seqs = (int)ln.seqs.size();
         p.num_items = ln.num_items;
@@ -651,7 +685,7 @@ static agx_status verify_step_host_impl(agx_handle* h, void* k_pool, void* v_poo
         sc.dst[0] = (uint4*)(ws + L.q); sc.dst[1] = (uint4*)(ws + L.k); sc.dst[2] = (uint4*)(ws + L.v);
         sc.units[0] = (unsigned)(L.q_bytes / 16); sc.units[1] = sc.units[2] = (unsigned)(L.kv_bytes / 16);
         // the inputs are read ahead of the stream's order, unless they are what the step in front still writes
-        auto written = [&](const void* p, size_t bytes) { return (const char*)p < h->last_out + h->last_out_bytes && h->last_out < (const char*)p + bytes; };
+        auto written = [&](const void* p, size_t bytes) { return g_last_outs.may_write(h->device, stream, p, bytes); };
         sc.src_in_order = written(mq, L.q_bytes) || written(mk, L.kv_bytes) || written(mv, L.kv_bytes);
         e = launch_stage_in(sc, stream);
         if (e == cudaSuccess) ++launches;
