@@ -108,10 +108,12 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int pool_end = p.k_new ? P : L;
     const int own_pg = min(n_pages, max(0, (pool_end >> 4) - page0));
     const int own_units = (n_pages - own_pg) * 512;   // 16-byte units, [page][K, V][16 rows][16 units]
-    // a thread's units of the first own page, and of the second where there is one (a block of up to 16 rows lies in two at most; with the second
-    // page behind the first one's trip to memory 8 rows from token 2750 on took 10.0 us a layer, from 2752 on 8.1)
+    // a thread's units of the first own page, and of the second where there is one (with the second page behind the first one's trip to
+    // memory 8 rows from token 2750 on took 10.0 us a layer, from 2752 on 8.1).  A block of 18 to 32 rows (one head a group) may lie in three
+    // pages: units from 1024 on have an id of their own and come behind the others.
     constexpr int kOwn1 = (512 + kThreads - 1) / kThreads, kOwn = (1024 + kThreads - 1) / kThreads;
     const bool more_own = own_units > kOwn1 * kThreads;
+    const int two_pages = min(own_units, 1024);
     // A unit's place in the pool but for its page, and its source where it is a block row's (held in registers for the first two pages).
     auto own_tok = [&](int u) { return tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15); };
     auto own_pool = [&](int u) {
@@ -234,11 +236,11 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
 #pragma unroll
         for (int j = 0; j < kOwn1; ++j)
-            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
+            if (tid + j * kThreads < two_pages) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
         if (more_own)
 #pragma unroll
         for (int j = kOwn1; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
+            if (tid + j * kThreads < two_pages) w[j] = own_load(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], own_new_at[j]);
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const int c = tid + j * kThreads, r = c >> 4, ch = c & 15;
@@ -246,12 +248,12 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
 #pragma unroll
         for (int j = 0; j < kOwn1; ++j)
-            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
+            if (tid + j * kThreads < two_pages) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
         if (more_own)
 #pragma unroll
         for (int j = kOwn1; j < kOwn; ++j)
-            if (tid + j * kThreads < own_units) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
-        for (int u = tid + kOwn * kThreads; u < own_units; u += kThreads) {
+            if (tid + j * kThreads < two_pages) own_store(tid + j * kThreads, tid + j * kThreads < 512 ? first_id : second_id, own_pool_at[j], w[j]);
+        for (int u = tid + 1024; u < own_units; u += kThreads) {
             const int id = own_id(u);
             own_store(u, id, own_pool(u), own_load(u, id, own_pool(u), own_new(u)));
         }
