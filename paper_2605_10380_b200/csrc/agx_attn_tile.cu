@@ -538,7 +538,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (warp == 0 && early_ids && lane < n_pool_pages) first_id = __ldg(first_id_at);
     if (tid == 0) {
         for (int i = 0; i < BAR_COUNT; ++i)
-            if (i != BAR_Q_FULL && i != BAR_Q_FULL_B) mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : 1u);
+            if (i != BAR_Q_FULL && i != BAR_Q_FULL_B && i != BAR_CTX) mbar_init(bar(i), (i == BAR_P_READY || i == BAR_P_READY + 1 || i == BAR_P_TAIL || i == BAR_P_TAIL + 1 || i == BAR_S_FREE) ? 4u : 1u);
         *abort_flag = 0;
         *(long long*)(smem + kOffBar + BAR_COUNT * 8 + 16) = p.wait_limit_cycles;   // for the out-of-line epilogue
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -558,6 +558,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (warp == 3 && elect_one()) {
         mbar_init(bar(BAR_Q_FULL), 1);
         mbar_init(bar(BAR_Q_FULL_B), 1);
+        mbar_init(bar(BAR_CTX), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(maps_new.q_tokens ? &maps_new.q_box : &maps_new.q_row) : "memory");
     }
@@ -571,8 +572,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    // Barriers initialised, TMEM address published.  Warps 0 and 3, which set the barriers up and need nothing from the others, only signal and
-    // go straight to their first copies.  No warp has waited for the launch in front yet: what follows such a wait (warps 0, 2 and 3 have one
+    // Barriers initialised, TMEM address published.  Warps 0 and 3 only signal and go straight to their first copies: each of them has set up
+    // all the barriers that it uses itself, and needs nothing else from the others.  No warp has waited for the launch in front yet: what follows such a wait (warps 0, 2 and 3 have one
     // each; whatever else the CTA reads or writes comes behind the Q tiles) is a chain of latencies with as little code as can be.
     tc_fence_before();
     if (warp == 0 || warp == 3) { __syncwarp(); asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory"); }
