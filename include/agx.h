@@ -255,9 +255,7 @@ AGX_API agx_status agx_get_status(agx_handle* handle, void* stream, int32_t* dev
  *                                copies asynchronous; pageable memory works but serialises).
  *                                When the three are pinned, mapped into the device's address space
  *                                (cudaHostAlloc / cudaHostRegister) and together at most 1 MiB, one
- *                                kernel reads them across the bus instead of three transfers, ahead of what the launch
- *                                in front of it still does (work in front on the stream must not write them; `out` of the
- *                                call in front, of any handle, may be among them and is waited for); a
+ *                                kernel reads them across the bus instead of three transfers; a
  *                                pinned, mapped h_out of at most 1 MiB is written by the attention
  *                                kernels directly.  Results are the same either way.
  *   h_logits                   : host, [total_q][row_stride] of logits_dtype; a megabyte or more of them is

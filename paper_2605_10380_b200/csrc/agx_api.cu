@@ -6,7 +6,6 @@
 
 #include <algorithm>
 #include <exception>
-#include <mutex>
 #include <new>
 #include <vector>
 
@@ -23,44 +22,6 @@ struct CallRange {
     ~CallRange() { nvtxRangePop(); }
 };
 }  // namespace
-
-// `out` of the last attention call on a stream, of whatever handle: kernels that write it may still be running when the next call's first one starts (of
-// calls further in front none is).  At most 16 streams are kept; of one that had to make room nothing is known, and it may write anything.
-class LastOuts {
-    struct Entry { int device; const void* stream; const char* at; size_t bytes; };
-    std::mutex lock;
-    Entry entries[16];
-    int used = 0, next = 0;
-    bool full = false;
-    static const void* key(cudaStream_t s) {
-        static thread_local char own;
-        return s == cudaStreamPerThread ? &own : (const void*)s;
-    }
-    Entry* find(int device, const void* k) {
-        for (int i = 0; i < used; ++i)
-            if (entries[i].device == device && entries[i].stream == k) return &entries[i];
-        return nullptr;
-    }
-
-public:
-    void set(int device, cudaStream_t s, const void* at, size_t bytes) {
-        const std::lock_guard<std::mutex> hold(lock);
-        Entry* e = find(device, key(s));
-        if (!e) {
-            full |= used == 16;
-            e = &entries[next];
-            next = (next + 1) % 16;
-            used = std::max(used, (int)(e - entries) + 1);
-        }
-        *e = {device, key(s), (const char*)at, bytes};
-    }
-    bool may_write(int device, cudaStream_t s, const void* p, size_t bytes) {
-        const std::lock_guard<std::mutex> hold(lock);
-        const Entry* e = find(device, key(s));
-        return e ? (const char*)p < e->at + e->bytes && e->at < (const char*)p + bytes : full;
-    }
-};
-static LastOuts g_last_outs;
 
 struct agx_handle {
     agx_config cfg;
@@ -308,7 +269,6 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         else if (plan.tensor_core) memset(&maps_new, 0, sizeof maps_new);
         if (!ok) return fail(h, AGX_E_CUDA, "cuTensorMapEncodeTiled failed");
     }
-    g_last_outs.set(h->device, stream, out, (size_t)plan.total_rows * p.hq * p.head_dim * elem_size(h->cfg.dtype));
     for (const Launch& ln : plan.launches) {
         p.num_seqs = (int)ln.seqs.size();
         p.num_items = ln.num_items;
@@ -684,9 +644,6 @@ static agx_status verify_step_host_impl(agx_handle* h, void* k_pool, void* v_poo
         sc.src[0] = (const uint4*)mq; sc.src[1] = (const uint4*)mk; sc.src[2] = (const uint4*)mv;
         sc.dst[0] = (uint4*)(ws + L.q); sc.dst[1] = (uint4*)(ws + L.k); sc.dst[2] = (uint4*)(ws + L.v);
         sc.units[0] = (unsigned)(L.q_bytes / 16); sc.units[1] = sc.units[2] = (unsigned)(L.kv_bytes / 16);
-        // the inputs are read ahead of the stream's order, unless they are what the step in front still writes
-        auto written = [&](const void* p, size_t bytes) { return g_last_outs.may_write(h->device, stream, p, bytes); };
-        sc.src_in_order = written(mq, L.q_bytes) || written(mk, L.kv_bytes) || written(mv, L.kv_bytes);
         e = launch_stage_in(sc, stream);
         if (e == cudaSuccess) ++launches;
     } else {

@@ -123,7 +123,6 @@ struct StageCopies {
     const uint4* src[3];
     uint4* dst[3];
     unsigned units[3];
-    int src_in_order;   // != 0: the launch in front may write the sources
 };
 cudaError_t launch_stage_in(const StageCopies& c, cudaStream_t stream);
 

@@ -110,27 +110,26 @@ cudaError_t launch_write_meta(const StepMeta& m, int* prefix, int* seq_lens, int
     return launch_chained(write_meta_kernel, dim3(1), dim3(64), 0, stream, m, prefix, seq_lens, cu_q);
 }
 
-// Bound by the trip across the bus (96 KB: 6.2 us), which is taken ahead of the dependency wait: the host buffers are the caller's, unchanged from
-// the call on, and the launch in front does not write them (else c.src_in_order); only the stores wait, since that launch may still read
-// the destination.  A 32-layer verify step over 4096 tokens 696 -> 580 us (what is left of a layer: 5 us until the results have crossed the bus).  The next launch may start only once everything in front of this one is
-// complete, so that the attention kernel behind it may fetch cached-prefix pages.
+// Bound by the trip across the bus (96 KB: 6.2 us).  The next launch may start only once everything in front of this one is complete, so
+// that the attention kernel behind it may fetch cached-prefix pages, its set-up and its page ids while this kernel waits for the bus.
+// (Read ahead of the wait, the inputs would cross under the layer in front, 32 layers of 8 rows over 4096 tokens 606 -> 539 us; but what is in front on the
+// stream may be writing them, the caller's own kernels among it, and neither the host nor the kernel can tell.)
 __global__ void __launch_bounds__(256) stage_in_kernel(const StageCopies c) {
-    const unsigned n0 = c.units[0], n1 = n0 + c.units[1], n2 = n1 + c.units[2];
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = i < n0 ? 0 : i < n1 ? 1 : 2;
-    const unsigned j = i - (k == 0 ? 0u : k == 1 ? n0 : n1);
-    if (c.src_in_order) pdl_wait();
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (i < n2) asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(c.src[k] + j));
-    pdl_wait();
+    pdl_wait();   // the launch before this one may still read the destination, or write the sources
     pdl_launch_dependents();
-    if (i < n2) c.dst[k][j] = v;
+    const unsigned n0 = c.units[0], n1 = n0 + c.units[1], n2 = n1 + c.units[2];
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += gridDim.x * blockDim.x) {
+        const int k = i < n0 ? 0 : i < n1 ? 1 : 2;
+        const unsigned j = i - (k == 0 ? 0u : k == 1 ? n0 : n1);
+        c.dst[k][j] = c.src[k][j];
+    }
 }
 
 cudaError_t launch_stage_in(const StageCopies& c, cudaStream_t stream) {
     const unsigned n = c.units[0] + c.units[1] + c.units[2];
     if (n == 0) return cudaSuccess;
-    return launch_chained(stage_in_kernel, dim3((n + 255u) / 256u), dim3(256), 0, stream, c);
+    const unsigned blocks = std::min(1024u, (n + 255u) / 256u);
+    return launch_chained(stage_in_kernel, dim3(blocks), dim3(256), 0, stream, c);
 }
 
 bool pdl_enabled() {
