@@ -439,12 +439,13 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         // CTA also puts the block's own pages together by hand.  At most 16 of them, with fp32 partials; two tiles up to 12 splits at 8 KV heads, where the
         // launch leaves SMs to the next one's CTAs.  32/8 heads, a layer, equal splits / these: 8 rows over 700 tokens 7.2 / 6.6 us, 1550 7.1 / 6.6, 2750
         // 7.7 / 7.2, 3500 9.2 / 7.8, 4096 8.3 / 8.1, 5100 11.0 / 9.0; one row over 4096 6.6 / 6.4, 5100 8.0 / 6.8.  (Up to 16 rows over 3100 to 3840
-        // tokens 15 equal splits of two tiles are faster: three rows over 3660 6.4 / 7.3.  From 17 splits of three tiles on nothing is gained.)
+        // tokens 15 equal splits of two tiles are faster: three rows over 3660 6.4 / 7.3.  From 17 splits of three tiles on nothing is gained.
+        // Up to 256 tokens are one CTA's, without a merge: one row over 160 / 200 / 250 tokens 3.9 / 4.0 / 4.0 us, in two splits 5.6; 8 rows 5.3 / 6.0.)
         bool last_shorter = false;
         if (whole && !cluster && seqs.size() == 1 && c.merge_sms) {
             const int L = P[seqs[0]] + Q[seqs[0]], twos = ceil_div(L, 256) * c.num_kv_heads, tiles = twos * 10 <= c.sm_count * 7 ? 2 : 3;
-            const bool equal_twos = tiles == 3 && k == KIND_SMALL1 && twos * 6 <= c.sm_count * 5;
-            for (int t = tiles * 128; t > tiles * 128 - 128 && !last_shorter && !equal_twos; t -= unit) {
+            const bool equal_twos = tiles == 3 && k == KIND_SMALL1 && twos * 6 <= c.sm_count * 5, is_split = L > C;
+            for (int t = tiles * 128; t > tiles * 128 - 128 && !last_shorter && !equal_twos && is_split; t -= unit) {
                 const int n = ceil_div(L, t);
                 if (n < 2 || n > 16 || n * c.num_kv_heads > c.sm_count || L - (n - 1) * t > (tiles - 1) * 128) continue;
                 C = t;

@@ -134,3 +134,13 @@ def test_a_few_long_splits_are_not_left_for_a_second_wave(P, q, hq, hkv):
         seen = P + min(q - 1, (256 * rc + 255) // G) + 1
         busy += hkv * min(s.nsplit, -(-seen // s.split_tokens))
     assert busy <= 148 or busy >= 1.5 * 148
+
+
+@pytest.mark.parametrize("hq,hkv", [(32, 8), (24, 8), (40, 8), (16, 2), (8, 8), (4, 1)])
+def test_one_block_is_split_from_257_tokens_on(hq, hkv):
+    """What one CTA holds whole in two KV tiles needs no second launch."""
+    for q in range(1, 17):
+        for L in range(130, 300, 3):
+            ln, = plan([L - q], [q], hq, hkv).launches
+            if ln.kind in ("small1", "small2"):
+                assert (ln.seqs[0].nsplit > 1) == (L > 256), (L, q)
