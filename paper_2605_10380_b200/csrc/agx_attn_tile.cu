@@ -70,7 +70,12 @@ constexpr uint32_t kOffBar = kOffV + 2 * kTileBytes;
 // V stage s: the first two at kOffV, the third behind two K stages, or (kStreams: three K stages) in the unused second Q tile
 template <bool kStreams>
 __host__ __device__ constexpr uint32_t v_stage_off(int s) { return s < 2 ? kOffV + s * kTileBytes : kStreams ? kOffQ + kTileBytes : kOffK + 2 * kTileBytes; }
-constexpr uint32_t kOffPark = kOffK + 2 * kTileBytes;   // kStreams epilogue: stream 1's O rows (64 KB), then its (m, l)
+// kStreams epilogue: where stream 1's O row `rt` (512 bytes) waits for stream 0: in the K and the V stage that neither of the last two tiles is in, from
+// which the block's own rows may still be on their way to the pool.
+__device__ __forceinline__ uint32_t park_off(int rt, int n_tiles) {
+    const int s = n_tiles % 3;
+    return (rt < 64 ? kOffK + s * kTileBytes : v_stage_off<true>(s)) + (rt & 63) * 512;
+}
 constexpr uint32_t kOffCtx = kOffBar + 256;            // what the epilogue needs to know, parked at kernel start
 constexpr uint32_t kOffPages = kOffBar + 512;          // row-group coordinates of the pages of up to 16 tiles
 constexpr uint32_t kSmemBytes = kOffPages + 512 + 1024;   // + alignment slack
@@ -230,8 +235,8 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     if (kStreams) {
         // Stream 1 (warps 8-11) parks its rows in shared memory; stream 0 (warps 4-7) adds them to its own.
         const int rt = ((warp & 3) << 5) + lane;
-        unsigned char* park = smem + kOffPark + rt * 512;
-        float2* park_ml = (float2*)(smem + kOffPark + 128 * 512);
+        unsigned char* park = smem + park_off(rt, it.n_tiles);
+        float2* park_ml = (float2*)(smem + kOffQ);   // (Q is dead)
         if (warp >= 8 && ok && warp_has_rows) {
             tc_fence_after();
             uint32_t oreg[32];
@@ -290,7 +295,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             tmem_ld_x32(tO + c8 * 32 + 32, oreg + 32);
             tmem_wait_ld();
             if (kStreams) {
-                const unsigned char* park = smem + kOffPark + ((((warp & 3) << 5) + lane) * 512);
+                const unsigned char* park = smem + park_off(((warp & 3) << 5) + lane, it.n_tiles);
 #pragma unroll
                 for (int v = 0; v < 16; ++v) {
                     const float4 o1 = *(const float4*)(park + (((c8 * 8 + v) ^ lane) << 4));
@@ -459,6 +464,19 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
     __syncwarp();
 }
 
+// The block's own row groups of K tile `tok0` ahead of its stage's next tile: a chunk of 256 tokens (one head a group) lies in up to three tiles, and K
+// has two stages.  Row groups from `lo` on, see the end of warp 0.
+__device__ __noinline__ void store_k_groups(const AttnParams& p, const CUtensorMap* map, const int* pt_row, int g, int L, int lo, int tok0, uint32_t tile) {
+    const int lane = threadIdx.x & 31, tok = tok0 + lane * 8;
+    if (lane < kBN / 8 && tok >= lo && tok + 8 <= L) {
+        const int id = tok / kPage < p.pt_stride ? __ldg(pt_row + tok / kPage) : -1;   // (a bad one is reported with V's)
+        if (id >= 0 && id < p.num_pages) tma_store_group(map, (id * p.hkv + g) * (kPage / 8) + ((tok >> 3) & 1), tile + lane * 8 * 256);
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+    }
+    __syncwarp();
+}
+
 // A Q tile's rows [row0, row0 + n) of KV head g, n <= 128, by one thread: single rows up to the next whole token, boxes of q_tokens tokens
 // while they fit the tile (the last one may bring rows nobody looks at), single rows again.  Where G divides 128 that is one box per half.
 struct QTile {
@@ -581,10 +599,11 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = (warp == 0 || warp == 3) ? 0u : *tmem_slot;
     // Fused append: a row group (eight tokens of half a page) is stored by the CTA whose row chunk's first query rows and whose split its first
-    // block token lies in.  That CTA has the group in its last K and V tiles, and a whole one leaves from there by TMA (by_tma).
+    // block token lies in.  That CTA has the group in one of its last K and V tiles, and a whole one leaves from there by TMA (by_tma).
     const int own_lo = max(kv_begin, P + (int)(((uint64_t)(uint32_t)(row0 + G - 1) * p.row_div_magic) >> 32));
     const int own_hi = p.k_new ? min(kv_end, kv_begin + sp.split_tokens) : 0;
-    auto by_tma = [&](int tok) { return !kStreams && tok >= P && tok + 8 <= L && tok >= kv_begin + (n_tiles - kStagesK) * kBN; };
+    auto by_tma = [&](int tok) { return tok >= P && tok + 8 <= L; };
+    const int own_group0 = (max(own_lo, P) + 7) & ~7;   // the first that may be a whole one
     auto pages_in_tile = [&](int t) { return min(8, (kv_end - (kv_begin + t * kBN) + kPage - 1) / kPage); };
 
     // the softmax warpgroups keep a whole score row in registers: warps 0-3 hand registers over to them
@@ -646,6 +665,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 ok = mbar_wait(empty, is_v ? vph : kph, abort_flag, p.status, p.wait_limit_cycles);
                 if (!ok) continue;
                 if (is_v) last_v = t; else last_k = t;
+                if (!kStreams && !is_v && p.k_new && p.drop_stage < 0 && tok0 - (kStagesK - 1) * kBN > own_group0)
+                    store_k_groups(p, &maps_new.k_pool8, pt_row, g, L, own_group0, tok0 - kStagesK * kBN, smem_base + off);
                 if (whole) {
                     if (elect_one()) {
                         const int4 c0 = *(const int4*)(page_ring + ((t * 8) & 127)), c1 = *(const int4*)(page_ring + ((t * 8) & 127) + 4);
@@ -671,31 +692,36 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 if (is_v) { if (++vs == kStagesV) { vs = 0; vph ^= 1; } } else if (++ks == kStagesK) { ks = 0; kph ^= 1; }
             }
         }
+        // The block's own row groups go from the tiles into the pool, a lane per group (a chunk has 32 at most).  Through registers it was 85 tokens' worth of
+        // loads and stores a CTA (3584 uncached tokens, 24/8 heads): in front of the softmax warps' loop 3 us of their way to the first scores; on warp 3
+        // beside the loop its instructions slowed the softmax warps of its scheduler, and with them the CTA, by a quarter.
+        // With one Q tile they went through registers of warp 3, eight tokens a trip to memory: 8/8 heads, 128 rows over 100 tokens 27.3 us, now 12.8 (12.5
+        // by ten warps in front of their loops).
+        const int own_tok = own_group0 + lane * 8, own_t = (own_tok - kv_begin) / kBN;
+        const bool leaves = ok && p.drop_stage < 0 && own_tok < own_hi && by_tma(own_tok);
+        int own_id = -1;
+        if (leaves) {
+            if (own_tok / kPage < p.pt_stride) own_id = __ldg(pt_row + own_tok / kPage);   // (under the last copies)
+            if (own_id >= p.num_pages) own_id = -1;
+            if (own_id < 0) atomicOr(p.status, AGX_DEV_BAD_PAGE);
+        }
+        const int own_at = ((own_tok - kv_begin) & (kBN - 1)) * 256, own_group = (own_id * p.hkv + g) * (kPage / 8) + ((own_tok >> 3) & 1);
         // drain: the copies this warp started must land before the CTA's shared memory goes away.  Bounded by the
         // clock alone: after a time-out elsewhere in the CTA the abort flag is up, and the copies still have to land.
-        if (lane == 0) {
+        if (lane == 0)
             for (int t = max(0, last_k - kStagesK + 1); t <= last_k; ++t)
                 if (t != p.drop_stage) mbar_drain(bar(BAR_K_FULL + t % kStagesK), (t / kStagesK) & 1, p.wait_limit_cycles);
+        __syncwarp();
+        if (own_id >= 0 && own_t >= n_tiles - kStagesK) tma_store_group(&maps_new.k_pool8, own_group, smem_base + kOffK + (own_t % kStagesK) * kTileBytes + own_at);
+        __syncwarp();
+        if (lane == 0)
             for (int t = max(0, last_v - kStagesV + 1); t <= last_v; ++t)
                 if (t != p.drop_stage) mbar_drain(bar(BAR_V_FULL + t % kStagesV), (t / kStagesV) & 1, p.wait_limit_cycles);
-        }
         __syncwarp();
-        // The block's own row groups go from the tiles into the pool, a lane per group.  Through registers it was 85 tokens' worth of loads
-        // and stores a CTA (3584 uncached tokens, 24/8 heads): in front of the softmax warps' loop 3 us of their way to the first scores; on warp 3
-        // beside the loop its instructions slowed the softmax warps of its scheduler, and with them the CTA, by a quarter.
-        if (!kStreams && ok && p.drop_stage < 0)
-            for (int tok = ((max(own_lo, P) + 7) & ~7) + lane * 8; tok < own_hi; tok += 256) {
-                if (!by_tma(tok)) continue;
-                const int id = tok / kPage < p.pt_stride ? __ldg(pt_row + tok / kPage) : -1, t = (tok - kv_begin) / kBN;
-                if (id < 0 || id >= p.num_pages) { atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
-                const int group = (id * p.hkv + g) * (kPage / 8) + ((tok >> 3) & 1), at = ((tok - kv_begin) & (kBN - 1)) * 256;
-                tma_store_group(&maps_new.k_pool8, group, smem_base + kOffK + (t % kStagesK) * kTileBytes + at);
-                tma_store_group(&maps_new.v_pool8, group, smem_base + v_stage_off<kStreams>(t % kStagesV) + at);
-            }
-        if (!kStreams) {   // (they are read before the CTA's shared memory goes away)
-            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-        }
+        if (own_id >= 0) tma_store_group(&maps_new.v_pool8, own_group, smem_base + v_stage_off<kStreams>(own_t % kStagesV) + own_at);
+        // (they are read before the CTA's shared memory goes away)
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
         __syncwarp();
     } else if (warp == 1 || warp == 2) {
         // ================= MMA issuers: one thread of warp 1 for S = Q K^T, one of warp 2 for O += P V =================
