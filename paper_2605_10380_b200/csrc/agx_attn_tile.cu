@@ -444,19 +444,16 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
         if (base == rows0) base = rows1;
         if (base >= own1 || (!is_v && base >= rows1)) break;   // (K rows beyond the last token are masked, whatever they are)
         by_hand = true;
+        // a lane takes 64 bytes of a row
+        const int r = lane >> 2, tok = base + r;
+        const unsigned char* src = tok < pool_end ? pool + ((long long)own_group * 8 + (tok & 15)) * 256
+                                   : tok < L ? rows + ((long long)(q_row0 + tok - P) * hkv + g) * 256 : nullptr;
         uint4 u[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int tok = base + (lane >> 4) + 2 * j;
-            u[j] = make_uint4(0, 0, 0, 0);
-            if (tok < pool_end) u[j] = __ldcg((const uint4*)(pool + ((long long)own_group * 8 + (tok & 15)) * 256 + (lane & 15) * 16));
-            else if (tok < L) u[j] = __ldg((const uint4*)(rows + ((long long)(q_row0 + tok - P) * hkv + g) * 256 + (lane & 15) * 16));
-        }
+        for (int j = 0; j < 4; ++j) u[j] = src ? __ldcg((const uint4*)(src + (lane & 3) * 64) + j) : make_uint4(0, 0, 0, 0);
+        unsigned char* at = dst + (base - tok0) * 256 + ((lane & 2) >> 1) * 1024 + r * 128;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = (lane >> 4) + 2 * j;
-            *(uint4*)(dst + (base - tok0) * 256 + ((lane & 15) >> 3) * 1024 + r * 128 + (((lane & 7) ^ r) << 4)) = u[j];
-        }
+        for (int j = 0; j < 4; ++j) *(uint4*)(at + ((((lane & 1) * 4 + j) ^ r) << 4)) = u[j];
     }
     if (by_hand) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncwarp();
@@ -695,8 +692,8 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // The block's own row groups go from the tiles into the pool, a lane per group (a chunk has 32 at most).  Through registers it was 85 tokens' worth of
         // loads and stores a CTA (3584 uncached tokens, 24/8 heads): in front of the softmax warps' loop 3 us of their way to the first scores; on warp 3
         // beside the loop its instructions slowed the softmax warps of its scheduler, and with them the CTA, by a quarter.
-        // With one Q tile they went through registers of warp 3, eight tokens a trip to memory: 8/8 heads, 128 rows over 100 tokens 27.3 us, now 12.8 (12.5
-        // by ten warps in front of their loops).
+        // With one Q tile they went through registers of warp 3, eight tokens a trip to memory: 8/8 heads, 128 rows over 100 tokens 27.3 us, now 10.8 (12.5 by
+        // ten warps in front of their loops).
         const int own_tok = own_group0 + lane * 8, own_t = (own_tok - kv_begin) / kBN;
         const bool leaves = ok && p.drop_stage < 0 && own_tok < own_hi && by_tma(own_tok);
         int own_id = -1;
@@ -831,16 +828,31 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                                       : (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536);
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }
-        // what of the fused append is no whole row group of a tile that stays in shared memory (see the end of warp 0)
+        // what of the fused append is no whole row group (see the end of warp 0): the groups that the block begins and ends in, a lane 64 bytes of K and V
         if (p.k_new) {
             pdl_wait();
-            for (int tok = own_lo & ~7; tok < own_hi; tok += 8) {
-                const int first = max(tok, P);
-                if (first < own_lo || by_tma(tok)) continue;
-                BlockRows<8> own;
-                own.load(p, sp, g, first - P, min(tok + 8, L) - P, lane, 32);
-                own.store(p, sp, g, first - P, min(tok + 8, L) - P, lane, 32);
+#pragma unroll 1
+            for (int end = 0; end < 2; ++end) {
+                const int t0 = (end ? L : P) & ~7, first = max(t0, P), tok = t0 + (lane >> 2);
+                if (t0 == (end ? L : P) || (end && t0 < P) || first < own_lo || first >= own_hi) continue;   // (whole, the other one's, or another CTA's)
+                const int id = t0 / kPage < p.pt_stride ? __ldg(p.page_table + (long long)sp.seq_index * p.pt_stride + t0 / kPage) : -1;
+                if (id < 0 || id >= p.num_pages) { atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
+                if (tok < P || tok >= L) continue;
+                const long long from = ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * 256 + (lane & 3) * 64;
+                const long long to = (((long long)id * p.hkv + g) * kPage + (tok & 15)) * 256 + (lane & 3) * 64;
+                uint4 k[4], v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    k[j] = __ldg((const uint4*)((const unsigned char*)p.k_new + from) + j);
+                    v[j] = __ldg((const uint4*)((const unsigned char*)p.v_new + from) + j);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    *((uint4*)((unsigned char*)p.k_pool + to) + j) = k[j];
+                    *((uint4*)((unsigned char*)p.v_pool + to) + j) = v[j];
+                }
             }
+            __syncwarp();
         }
         // (the copies must land before the CTA's shared memory goes away, also after a time-out elsewhere)
         if (lane == 0) mbar_drain(bar(BAR_Q_FULL), 0, p.wait_limit_cycles);

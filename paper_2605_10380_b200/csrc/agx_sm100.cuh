@@ -128,37 +128,6 @@ __device__ __forceinline__ void hold(T* __restrict__& x) { asm volatile("" : "+l
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
-// Fused KV append (bf16, d = 128): the block's rows [i_lo, i_hi) of KV head g go into the sequence's pages (Sec. 2.3: the block's KV
-// joins the cache).  Nothing in the same launch reads them there: the attention CTAs take the block's own rows from k_new / v_new,
-// so there is nothing to wait for.
-template <int kBatch>   // 16-byte units in flight per thread: idx0, idx0 + nthreads, ...
-struct BlockRows {
-    uint4 v[kBatch];
-    int id[kBatch];
-    __device__ __forceinline__ void load(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int idx0, int nthreads) {
-        const int* pt_row = p.page_table + (long long)sp.seq_index * p.pt_stride;
-        const int units = (i_hi - i_lo) * 32;
-#pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            const int idx = idx0 + j * nthreads, i = i_lo + (idx >> 5), slot = (sp.prefix_len + i) >> 4;
-            id[j] = -2;
-            if (idx < units) {
-                id[j] = slot < p.pt_stride ? __ldg(pt_row + slot) : -1;
-                v[j] = __ldg((const uint4*)((const unsigned char*)((idx & 16) ? p.v_new : p.k_new) + (((long long)(sp.q_row0 + i) * p.hkv + g) * 256 + (idx & 15) * 16)));
-            }
-        }
-    }
-    __device__ __forceinline__ void store(const AttnParams& p, const SeqPlan& sp, int g, int i_lo, int i_hi, int idx0, int nthreads) {
-#pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            const int idx = idx0 + j * nthreads, tok = sp.prefix_len + i_lo + (idx >> 5);
-            if (id[j] >= 0 && id[j] < p.num_pages)
-                *(uint4*)((unsigned char*)((idx & 16) ? p.v_pool : p.k_pool) + ((((long long)id[j] * p.hkv + g) * kPage + (tok & 15)) * 256 + (idx & 15) * 16)) = v[j];
-            else if (id[j] != -2) atomicOr(p.status, AGX_DEV_BAD_PAGE);
-        }
-    }
-};
-
 // The sequence plan of a work item.
 __device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
     int s = 0;
