@@ -31,7 +31,8 @@ struct SplitModel {
 // average (with 1.9 us a tile, 2.2 + 0.38 us per MB: 1.4 %).  The grid's order counts where a launch is little more than
 // one wave: 152 CTAs dealt out longest first fit 148 SMs as if the short ones were stacked, but the last ones to start are long ones (256 tokens behind
 // 3000, 32/8 heads, 5 / 4 splits: 31.1 / 21.7 us a layer; 931 behind 3086, 24/8: 66.7 -> 60.2; 598 behind 5293: 76 -> 68.3; verify blocks with three to
-// eight prefills 5 to 10 %).  (Planning a new batch of 1 / 8 / 48 prefills takes 21 / 57 / 102 us instead of 16 / 30 / 95.)
+// eight prefills 5 to 10 %).  (Sequences whose K/V exceed 48 MB have the KV head outermost in the grid and are dealt out here like the others: 50 plans that
+// the order makes different were 0.2 % slower together with it, single ones 13 % faster to 13 % slower.)
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
 SplitModel tile_model(const PlanConfig& c, bool f32_partials = false) {
@@ -128,8 +129,9 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         cd.merge = mb == 0 ? 0 : md.lean > 0 && count <= sms * 15 / 16 && pairs <= 3 * sms ? md.lean + 0.2 * mb
                    : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
                    : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
-        cd.bound = md.base + cd.merge + std::max((load - kOverhead) * (md.per_add + md.per_min),
-                                                 (sum - (double)kOverhead * std::min<long long>(count, sms)) * md.per_busy);
+        // (a step takes per_add, and beyond it per_min or what all CTAs at work share of per_busy)
+        cd.bound = md.base + cd.merge + (load - kOverhead) * md.per_add +
+                   std::max((load - kOverhead) * md.per_min, (sum - (double)kOverhead * std::min<long long>(count, sms)) * md.per_busy);
         cands.push_back(cd);
     }
     std::stable_sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.bound < b.bound; });
@@ -156,13 +158,24 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         if (md.in_order && cd.count <= 16 * sms) {
             in_order.clear();
             deal(cd.tiles, [&](const Seen& v, int per, int full, int rest) { in_order.push_back({v.n, per, full, rest}); });
-            size_t at = 0, first = 0;
+            size_t first = 0;
             for (const Seq& w : work) {   // a sequence's row chunks last to first, a chunk's splits first to last
-                for (at = w.seen_end; at-- > first;)
-                    for (long long n = 0; n < in_order[at].n; ++n) {
-                        place(in_order[at].per, in_order[at].full);
-                        if (in_order[at].rest) place(in_order[at].rest, 1);
+                for (size_t at = w.seen_end; at-- > first;) {
+                    const Chunks& v = in_order[at];
+                    if (v.rest == 0) place(v.per, v.full * v.n);
+                    else if (v.full == 0) place(v.rest, v.n);
+                    else for (long long left = v.n; left > 0;) {
+                        // as many (chunk, head) pairs as the SMs of the least load can take whole go there together, one that they cannot by itself
+                        while (load[lo] == 0) ++lo;
+                        const int k = (int)std::min<long long>(load[lo] / (v.full + 1), left);
+                        load[lo] -= k * (v.full + 1);
+                        load[lo + v.per + kOverhead] += k * v.full;
+                        load[lo + v.rest + kOverhead] += k;
+                        if (k > 0) hi = std::max(hi, lo + v.per + kOverhead);   // (the rest is shorter)
+                        left -= k;
+                        if (k == 0) { place(v.per, v.full); place(v.rest, 1); --left; }
                     }
+                }
                 first = w.seen_end;
             }
         } else {
