@@ -256,7 +256,10 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.hq = h->cfg.num_q_heads; p.hkv = h->cfg.num_kv_heads; p.head_dim = h->cfg.head_dim;
     p.scale_log2 = h->scale * 1.4426950408889634f;
     p.gqa = p.hq / p.hkv;
-    p.row_div_magic = (0x100000000ull + (unsigned)(p.hq / p.hkv) - 1) / (unsigned)(p.hq / p.hkv);
+    p.row_div_magic = (0x100000000ull + (unsigned)p.gqa - 1) / (unsigned)p.gqa;
+    p.row_div_shift = 31;
+    while ((1ll << (p.row_div_shift - 31)) < p.gqa) ++p.row_div_shift;
+    p.row_div31 = (unsigned)(((1ull << p.row_div_shift) + (unsigned)p.gqa - 1) / (unsigned)p.gqa);
     p.wait_limit_cycles = h->wait_limit_cycles;
     p.early_prefix = early_prefix;
     p.drop_stage = h->drop_stage;

@@ -81,7 +81,7 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
     local /= nsplit;
     const int rc = local % sp.row_chunks, g = local / sp.row_chunks;
     const int G = p.gqa, P = sp.prefix_len, q = sp.q_len, L = P + q, rows = q * G, row0 = rc * kR;
-    auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div_magic) >> 32); };   // r / G without the division
+    auto div_g = [&](int r) { return (int)(((uint64_t)(uint32_t)r * p.row_div31) >> p.row_div_shift); };   // r / G without the division
     auto row_of = [&](int r) { const int i = div_g(r); return (long long)(sp.q_row0 + i) * p.hq + g * G + r - i * G; };   // of q and out
     const int vis_end = P + min(q - 1, div_g(row0 + kR - 1)) + 1;
     const int tok_begin = split * sp.split_tokens, tok_end = min(vis_end, tok_begin + sp.split_tokens);

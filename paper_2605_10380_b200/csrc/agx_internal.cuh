@@ -59,6 +59,8 @@ struct AttnParams {
     float2* part_ml; // [entries] (running max in log2 units, sum)
     int* status;
     unsigned long long row_div_magic;   // ceil(2^32 / G), G = hq / hkv: (row * magic) >> 32 == row / G for rows < 2^22
+    unsigned row_div31;                 // ceil(2^row_div_shift / G), row_div_shift = 31 + ceil(log2 G): (row * row_div31) >> row_div_shift == row / G
+    int row_div_shift;                  // for all rows < 2^31
     int part_half;       // how the split partials of this launch are stored, a PartHalf
     int cluster_size;    // > 1: the launch's CTAs form clusters of this size = the KV splits of one (sequence, KV head), merged in-kernel
     const void* k_new;   // fused append (agx_attn_prefixed_append): the block's K/V rows [total_q][hkv][d], or NULL

@@ -54,3 +54,23 @@ def test_what_a_row_does_not_see_does_not_reach_it(dtype, d, value):
         assert bool(torch.isfinite(outs[1][0][:q - 1]).all()), (P, q)
         assert torch.equal(outs[0][0][:q - 1], outs[1][0][:q - 1]) and torch.equal(outs[0][1], outs[1][1])
         assert not bool(torch.isfinite(outs[1][0][q - 1]).any())
+
+
+def test_rows_of_very_many_heads():
+    """65793 query heads over one KV head: the last row of the first token is the first where row * ceil(2^32 / heads) >> 32 is one too many."""
+    import torch
+
+    from tests.gpu_util import DeviceBatch
+    heads, P, q = 65793, 20, 3
+    assert ((heads - 1) * -(-2 ** 32 // heads)) >> 32 == 1
+    b = DeviceBatch(W.make_attn_workload("heads", 11, "f32", heads, 1, 64, [P], [q], spare_pages=1))
+    out, lse = (torch.from_numpy(a).cuda() for a in b.attend_append())
+    assert b.status() == 0
+    table = b.page_table[0].long()
+    k, v = (pool[table][:, 0].reshape(-1, 64)[:P + q].double() for pool in (b.k_pool, b.v_pool))   # (with the block's rows)
+    s = b.q_block.double() @ k.T / 8
+    hidden = torch.arange(P + q, device="cuda")[None, :] > P + torch.arange(q, device="cuda")[:, None]
+    s = s.masked_fill(hidden[:, None, :], float("-inf"))
+    # (the bounds of test_simt_kernel_against_the_oracle)
+    assert float((torch.softmax(s, -1) @ v - out).abs().max()) < 2e-4
+    assert float((torch.logsumexp(s, -1) - lse).abs().max()) < 1e-4
