@@ -141,7 +141,8 @@ AGX_API int64_t agx_attn_workspace_bytes(agx_handle* handle, int32_t B, const in
  * per KV head (q_len * G) run a split-KV kernel (latency-bound; tcgen05 with swapped operands where one wave of KV splits of at most 384 tokens
  * covers the launch, warp MMAs otherwise) or, all of a batch together, the tensor-core kernel with one padded Q tile whose KV tiles alternate
  * between two softmax warpgroups (HBM-bound), whichever an estimate of the launch gives the shorter time; 33..384 rows run the latter in
- * chunks of 128 rows, longer blocks the tensor-core kernel with 256-row tiles (tensor-bound).  Sequences of all kinds may share a batch.
+ * chunks of 128 rows, longer blocks the tensor-core kernel with 256-row tiles (tensor-bound), and so does one block of 65..384 rows where the estimates
+ * of both say that it is clearly faster.  Sequences of all kinds may share a batch.
  * Errors: AGX_E_INVAL (null/misaligned, q_len < 1, prefix_len < 0, workspace too small),
  * AGX_E_RANGE ((P + q) exceeds 16 * page_table_stride), AGX_E_CUDA.  Page ids outside
  * [0, num_pages) set AGX_DEV_BAD_PAGE and read as zeros.

@@ -82,7 +82,10 @@ struct AttnParams {
 
 // Launch with programmatic stream serialisation: the kernel may start while the launch before it in the
 // stream is still draining, so its launch latency and set-up overlap that kernel's tail.  Every kernel
-// launched this way calls pdl_wait() before its first global-memory access.  AGX_NO_PDL=1 turns it off.
+// launched this way calls pdl_wait() before its first global-memory access, except that with early_prefix the attention kernels read
+// page ids and pool pages below the cached-prefix length before it (the caller, or a kernel in front that waits before it lets the next
+// launch start, vouches that nothing in flight writes them).  Most kernels let the next launch start before they wait themselves, so that launches
+// further in front than the last one may still be running when a kernel starts.  AGX_NO_PDL=1 turns it off.
 bool pdl_enabled();
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
