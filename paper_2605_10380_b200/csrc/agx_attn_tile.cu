@@ -444,16 +444,21 @@ __device__ __noinline__ void load_mixed(const AttnParams& p, const CUtensorMap* 
         if (base == rows0) base = rows1;
         if (base >= own1 || (!is_v && base >= rows1)) break;   // (K rows beyond the last token are masked, whatever they are)
         by_hand = true;
-        // a lane takes 64 bytes of a row
-        const int r = lane >> 2, tok = base + r;
-        const unsigned char* src = tok < pool_end ? pool + ((long long)own_group * 8 + (tok & 15)) * 256
-                                   : tok < L ? rows + ((long long)(q_row0 + tok - P) * hkv + g) * 256 : nullptr;
+        // half a warp a row, rows r0, r0 + 2, r0 + 4, r0 + 6 of the group
+        const int r0 = lane >> 4, u0 = lane & 15;
+        const unsigned char* in_pool = pool + ((long long)own_group * 8 + (base & 15) + r0) * 256 + u0 * 16;
+        const unsigned char* in_rows = rows + ((long long)(q_row0 + base + r0 - P) * hkv + g) * 256 + u0 * 16;
         uint4 u[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) u[j] = src ? __ldcg((const uint4*)(src + (lane & 3) * 64) + j) : make_uint4(0, 0, 0, 0);
-        unsigned char* at = dst + (base - tok0) * 256 + ((lane & 2) >> 1) * 1024 + r * 128;
+        for (int j = 0; j < 4; ++j) {
+            const int tok = base + r0 + 2 * j;
+            const unsigned char* src = tok < pool_end ? in_pool + j * 512 : in_rows + j * hkv * 512;
+            u[j] = make_uint4(0, 0, 0, 0);
+            if (tok < L) u[j] = __ldcg((const uint4*)src);
+        }
+        unsigned char* at = dst + (base - tok0) * 256 + (u0 >> 3) * 1024;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) *(uint4*)(at + ((((lane & 1) * 4 + j) ^ r) << 4)) = u[j];
+        for (int j = 0; j < 4; ++j) { const int r = r0 + 2 * j; *(uint4*)(at + r * 128 + (((u0 & 7) ^ r) << 4)) = u[j]; }
     }
     if (by_hand) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncwarp();
@@ -470,6 +475,36 @@ __device__ __noinline__ void store_k_groups(const AttnParams& p, const CUtensorM
         if (id >= 0 && id < p.num_pages) tma_store_group(map, (id * p.hkv + g) * (kPage / 8) + ((tok >> 3) & 1), tile + lane * 8 * 256);
         asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+    }
+    __syncwarp();
+}
+
+// Rows of the block that are in no whole group of eight, from k_new / v_new to the pool by one warp, half a warp a row: of the groups that the block
+// begins and ends in those whose first block row is in [own_lo, own_hi).
+__device__ __forceinline__ void store_ends(const AttnParams& p, const SeqPlan& sp, int g, int L, int own_lo, int own_hi) {
+    const int lane = threadIdx.x & 31, r0 = lane >> 4, P = sp.prefix_len;
+#pragma unroll 1
+    for (int end = 0; end < 2; ++end) {
+        const int t0 = (end ? L : P) & ~7, first = max(t0, P);
+        if (t0 == (end ? L : P) || (end && t0 < P) || first < own_lo || first >= own_hi) continue;   // (whole, the other one's, or another CTA's)
+        const int id = t0 / kPage < p.pt_stride ? __ldg(p.page_table + (long long)sp.seq_index * p.pt_stride + t0 / kPage) : -1;
+        const long long from = ((long long)(sp.q_row0 + t0 + r0 - P) * p.hkv + g) * 256 + (lane & 15) * 16;
+        auto mine = [&](int j) { const int tok = t0 + r0 + 2 * j; return tok >= P && tok < L; };
+        uint4 k[4], v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)   // (in one trip with the page id)
+            if (mine(j)) {
+                k[j] = __ldg((const uint4*)((const unsigned char*)p.k_new + from + j * p.hkv * 512));
+                v[j] = __ldg((const uint4*)((const unsigned char*)p.v_new + from + j * p.hkv * 512));
+            }
+        if (id < 0 || id >= p.num_pages) { atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
+        const long long to = (((long long)id * p.hkv + g) * kPage + (t0 & 15) + r0) * 256 + (lane & 15) * 16;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (mine(j)) {
+                *(uint4*)((unsigned char*)p.k_pool + to + j * 512) = k[j];
+                *(uint4*)((unsigned char*)p.v_pool + to + j * 512) = v[j];
+            }
     }
     __syncwarp();
 }
@@ -828,31 +863,10 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                                       : (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536);
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }
-        // what of the fused append is no whole row group (see the end of warp 0): the groups that the block begins and ends in, a lane 64 bytes of K and V
+        // what of the fused append is no whole row group (see the end of warp 0): the groups that the block begins and ends in
         if (p.k_new) {
             pdl_wait();
-#pragma unroll 1
-            for (int end = 0; end < 2; ++end) {
-                const int t0 = (end ? L : P) & ~7, first = max(t0, P), tok = t0 + (lane >> 2);
-                if (t0 == (end ? L : P) || (end && t0 < P) || first < own_lo || first >= own_hi) continue;   // (whole, the other one's, or another CTA's)
-                const int id = t0 / kPage < p.pt_stride ? __ldg(p.page_table + (long long)sp.seq_index * p.pt_stride + t0 / kPage) : -1;
-                if (id < 0 || id >= p.num_pages) { atomicOr(p.status, AGX_DEV_BAD_PAGE); continue; }
-                if (tok < P || tok >= L) continue;
-                const long long from = ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * 256 + (lane & 3) * 64;
-                const long long to = (((long long)id * p.hkv + g) * kPage + (tok & 15)) * 256 + (lane & 3) * 64;
-                uint4 k[4], v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    k[j] = __ldg((const uint4*)((const unsigned char*)p.k_new + from) + j);
-                    v[j] = __ldg((const uint4*)((const unsigned char*)p.v_new + from) + j);
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    *((uint4*)((unsigned char*)p.k_pool + to) + j) = k[j];
-                    *((uint4*)((unsigned char*)p.v_pool + to) + j) = v[j];
-                }
-            }
-            __syncwarp();
+            store_ends(p, sp, g, L, own_lo, own_hi);
         }
         // (the copies must land before the CTA's shared memory goes away, also after a time-out elsewhere)
         if (lane == 0) mbar_drain(bar(BAR_Q_FULL), 0, p.wait_limit_cycles);
