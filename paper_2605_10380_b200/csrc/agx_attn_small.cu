@@ -63,6 +63,11 @@ __device__ __forceinline__ uint2 ld_volatile_u2(const void* p) {
     asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint4 ld_volatile_u4(const void* p) {
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ float4 ld_volatile_f4(const void* p) {
     float4 v;
     asm volatile("ld.volatile.global.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
@@ -591,21 +596,19 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 // One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
 // kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel takes more).  Four O rows per
 // warp instead of 32 keep the register count low enough for ten CTAs per SM, which is what the partials of a split prefill need.
-// Where the fp16 partials of row i, head h lie: split 0's, at this lane's four columns, and the bytes from split to split.
+// Where 16-byte unit u of split 0's fp16 partial of row i, head h lies.
+__device__ __forceinline__ const unsigned char* half_row(const AttnParams& p, const SeqPlan& sp, int i, int h, int u) {
+    if (p.part_half != PART_HALF_TILES) return (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + u * 16;
+    const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rl = r & 255;
+    return (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 + rl * 256 +
+           ((u ^ (rl & 15)) << 4);
+}
+// The fp16 partials of row i, head h, four columns a lane: split 0's, and the bytes from split to split.
 struct HalfRows {
     const unsigned char* at;
     int stride;
-    __device__ __forceinline__ HalfRows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane) {
-        if (p.part_half == PART_HALF_TILES) {
-            const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rl = r & 255;
-            at = (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 +
-                 rl * 256 + (((lane >> 1) ^ (rl & 15)) << 4) + (lane & 1) * 8;
-            stride = 65536;
-        } else {
-            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + lane * 8;
-            stride = 512;
-        }
-    }
+    __device__ __forceinline__ HalfRows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane)
+        : at(half_row(p, sp, i, h, lane >> 1) + (lane & 1) * 8), stride(p.part_half == PART_HALF_TILES ? 65536 : 512) {}
     __device__ __forceinline__ uint2 load(int split) const { return ld_volatile_u2(at + (long long)split * stride); }   // (written by other SMs just before: past the L1)
 };
 // The same of the fp32 partials (columns [4 lane, 4 lane + 4)).
@@ -805,91 +808,84 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     if (lse_at && lane == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
-// The same merge for the partials of the 256-row tensor-core schedule (fp16 rows divided by their own sums, at most 4
-// splits): each warp takes two (row, head) pairs with all their loads in flight at once, so that the merge of a split
-// prefill (12288 pairs, 9 MB of partials) is about one wave of CTAs and one memory round trip per warp instead of several
-// waves of short-lived CTAs, and a larger merge has half the CTAs with twice the bytes in flight each.  (Measured: one /
-// two / three / four pairs per warp give 29.1 / 19.8 / 20.5-21.6 / - us for the 65536 pairs of the long prefill under
-// ncu; c3 29.9 / 29.9 / 31.0 us and (1500, 200) 17.8 / 18.3 / 19.3 us per call for two / three / four.)
-constexpr int kCombineRows = 2;
-__global__ void __launch_bounds__(128, 8)
-attn_combine_half4_kernel(const __grid_constant__ AttnParams p, int total_rows) {
+// The same merge for fp16 partials (rows divided by their own sums) of at most kNs <= 8 splits: half a warp merges a (row, head) pair, a lane eight
+// columns, lane k of the half holding split k's (m, l), all loads in flight at once.  Bound by instructions and by the CTAs of a wave before anything
+// else: the merge of a split prefill is thousands of pairs (12288 and 9 MB for 512 tokens of 24 heads), each with its row's address to work out.  16 bytes
+// a lane are half the loads and half the address arithmetic of a warp a pair.
+// (One layer, one warp a pair and four columns a lane / this: 512 rows over 3072 tokens, 24/8 heads 27.3 / 26.0 us, 128 over 1000 13.2 / 11.8, 200 over
+// 1500 17.7 / 17.1, 300 over 2000, 40/8, 22.3 / 20.7, 700 over 8000 90.3 / 88.0, six decode blocks over 1000 8.06 / 7.79.  Two pairs a half-warp with
+// their loads in flight together: 128 over 1000 as fast, 512 over 3072 26.3.)
+template <int kNs>
+__global__ void __launch_bounds__(128, kNs <= 4 ? 12 : 8)
+attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31;
-    const int n_pairs = total_rows * p.hq;
-    const int stride = gridDim.x * 4;
-    const int rh0 = blockIdx.x * 4 + (threadIdx.x >> 5);
-    const float2* ml_at[kCombineRows];
-    unsigned char* out_at[kCombineRows];
-    float* lse_at[kCombineRows];
-    const unsigned char* rows[kCombineRows];
-    int ns[kCombineRows], stride_bytes[kCombineRows];
-#pragma unroll
-    for (int j = 0; j < kCombineRows; ++j) {
-        const int rh = rh0 + j * stride;
-        ns[j] = 0; ml_at[j] = nullptr; out_at[j] = nullptr; lse_at[j] = nullptr; rows[j] = nullptr; stride_bytes[j] = 0;
-        if (rh < n_pairs) {
-            const int lrow = rh / p.hq, h = rh - lrow * p.hq;
-            int si = 0, acc_rows = 0;
+    const int u = threadIdx.x & 15;
+    const int rh = blockIdx.x * 8 + (threadIdx.x >> 4);
+    const float2* ml_at = nullptr;
+    unsigned char* out_at = nullptr;
+    float* lse_at = nullptr;
+    const unsigned char* rows = nullptr;
+    int ns = 0, stride = p.part_half == PART_HALF_TILES ? 65536 : 512;
+    if (rh < total_rows * p.hq) {
+        const int lrow = rh / p.hq, h = rh - lrow * p.hq;
+        int si = 0, acc_rows = 0;
 #pragma unroll 1
-            for (int s = 0; s < p.num_seqs; ++s) {
-                if (lrow >= acc_rows && lrow < acc_rows + p.seq[s].q_len) { si = s; break; }
-                acc_rows += p.seq[s].q_len;
-            }
-            const SeqPlan& sp = p.seq[si];
-            if (sp.nsplit > 1) {   // (a single split was written directly by the attention kernel)
-                const int i = lrow - acc_rows;
-                ns[j] = sp.nsplit;
-                const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
-                ml_at[j] = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + lane;
-                out_at[j] = (unsigned char*)p.out + out_row * (kD * 2) + lane * 8;
-                lse_at[j] = p.lse ? p.lse + out_row : nullptr;
-                const HalfRows hr(p, sp, i, h, lane);
-                rows[j] = hr.at; stride_bytes[j] = hr.stride;
-            }
+        for (int s = 0; s < p.num_seqs; ++s) {
+            if (lrow >= acc_rows && lrow < acc_rows + p.seq[s].q_len) { si = s; break; }
+            acc_rows += p.seq[s].q_len;
         }
-        hold(ns[j]); hold(ml_at[j]); hold(out_at[j]); hold(lse_at[j]); hold(rows[j]); hold(stride_bytes[j]);
+        const SeqPlan& sp = p.seq[si];
+        if (sp.nsplit > 1) {   // (a single split was written directly by the attention kernel)
+            const int i = lrow - acc_rows;
+            ns = sp.nsplit;
+            const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
+            ml_at = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + u;
+            out_at = (unsigned char*)p.out + out_row * (kD * 2) + u * 16;
+            lse_at = p.lse ? p.lse + out_row : nullptr;
+            rows = half_row(p, sp, i, h, u);
+        }
     }
+    hold(ns); hold(ml_at); hold(out_at); hold(lse_at); hold(rows); hold(stride);
     pdl_wait();   // the partials are complete
-    float2 ml[kCombineRows];
-    uint2 v[kCombineRows][4];
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (u < ns) ml = ld_volatile_f2(ml_at);
+    uint4 v[kNs];
 #pragma unroll
-    for (int j = 0; j < kCombineRows; ++j) {
-        ml[j] = make_float2(-INFINITY, 0.f);
-        if (lane < ns[j]) ml[j] = ld_volatile_f2(ml_at[j]);
+    for (int k = 0; k < kNs; ++k)
+        if (k < ns) v[k] = ld_volatile_u4(rows + k * stride);
+    float m_all = ml.x;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (k < ns[j]) v[j][k] = ld_volatile_u2(rows[j] + k * stride_bytes[j]);
-    }
+    for (int off = kNs / 2; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));   // splits sit in lanes 0 .. kNs - 1
+    const float w_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * ml.y;
+    float l_all = w_mine;
 #pragma unroll
-    for (int j = 0; j < kCombineRows; ++j) {
-        if (ns[j] == 0) continue;   // (uniform over the warp)
-        float m_all = ml[j].x;
+    for (int off = kNs / 2; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);   // (a fixed order: reproducible)
+    m_all = __shfl_sync(0xFFFFFFFFu, m_all, 0, 16);
+    l_all = __shfl_sync(0xFFFFFFFFu, l_all, 0, 16);
+    float acc[8];
 #pragma unroll
-        for (int off = 2; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));   // splits sit in lanes 0..3
-        const float w_mine = (ml[j].x == -INFINITY) ? 0.f : exp2f(ml[j].x - m_all) * ml[j].y;
-        float l_all = w_mine;
+    for (int c = 0; c < 8; ++c) acc[c] = 0.f;
 #pragma unroll
-        for (int off = 2; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);
-        m_all = __shfl_sync(0xFFFFFFFFu, m_all, 0);
-        l_all = __shfl_sync(0xFFFFFFFFu, l_all, 0);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < kNs; ++k) {
+        const float w = __shfl_sync(0xFFFFFFFFu, w_mine, k, 16);
+        if (k < ns && w != 0.f) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0): its row may hold anything, NaN included
+            const uint32_t x[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float w = __shfl_sync(0xFFFFFFFFu, w_mine, k);
-            if (k < ns[j] && w != 0.f) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0)
-                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v[j][k].x));
-                const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&v[j][k].y));
-                acc.x += a.x * w; acc.y += a.y * w; acc.z += b.x * w; acc.w += b.y * w;
+            for (int c = 0; c < 4; ++c) {
+                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&x[c]));
+                acc[2 * c] += a.x * w; acc[2 * c + 1] += a.y * w;
             }
         }
-        const float inv = 1.f / l_all;
-        uint2 packed;
-        packed.x = pack_bf16(acc.x * inv, acc.y * inv);
-        packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-        *(uint2*)out_at[j] = packed;
-        if (lse_at[j] && lane == 0) *lse_at[j] = (m_all + log2f(l_all)) * 0.6931471805599453f;
     }
+    if (ns == 0) return;
+    const float inv = 1.f / l_all;
+    uint4 packed;
+    packed.x = pack_bf16(acc[0] * inv, acc[1] * inv);
+    packed.y = pack_bf16(acc[2] * inv, acc[3] * inv);
+    packed.z = pack_bf16(acc[4] * inv, acc[5] * inv);
+    packed.w = pack_bf16(acc[6] * inv, acc[7] * inv);
+    *(uint4*)out_at = packed;
+    if (lse_at && u == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
 // The same merge for the fp16 partials of the small-q kernel (5 to 32 KV splits): one (row, head) pair per warp, lane k
@@ -1077,13 +1073,9 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
     for (int i = 0; i < p.num_seqs; ++i) ns_max = p.seq[i].nsplit > ns_max ? p.seq[i].nsplit : ns_max;
     const int many_threads = 32 * std::min(kManyWarps, (ns_max + kManyBatch - 1) / kManyBatch);
     if (dtype == AGX_BF16 && (p.part_half == PART_HALF_SLOTS || p.part_half == PART_HALF_TILES)) {
-        if (ns_max <= 4) {
-            // CTAs whose warps take kCombineRows pairs each
-            const int want = (int)((n + 4 * kCombineRows - 1) / (4 * kCombineRows));
-            return launch_chained(attn_combine_half4_kernel, dim3(want > 0 ? want : 1), dim3(128), 0, stream, p, total_rows);
-        }
+        if (ns_max <= 8)
+            return launch_chained(ns_max <= 4 ? attn_combine_few_kernel<4> : attn_combine_few_kernel<8>, dim3((unsigned)((n + 7) / 8)), dim3(128), 0, stream, p, total_rows);
         if (ns_max <= 32) {
-            if (ns_max <= 8) return launch_chained(attn_combine_half32_kernel<8>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 12) return launch_chained(attn_combine_half32_kernel<12>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 20) return launch_chained(attn_combine_half32_kernel<20>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             return launch_chained(attn_combine_half32_kernel<32>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
