@@ -6,7 +6,7 @@
 // (mma.sync over 16-row tiles, or tcgen05 over 128 mostly empty rows) that chain is the matrix instructions.  Here the tokens take the M
 // side, S^T = K Q^T, and the head dimension in the second product, O^T = V^T P^T: the query rows are the N side, 16 or 32 columns, so
 // that both products of a split are some 25 to 50 instructions of one thread.  TMEM then holds a token per lane and a query row per
-// column: every thread owns one token's scores, row maxima and row sums are butterflies over lanes that leave row r in lane r, and P goes
+// column: every thread owns one token's scores (RH = 2: those of half of the rows), row maxima and row sums are butterflies over lanes that leave row r in lane r, and P goes
 // back through shared memory (dead K) as the B operand.  All of a split's K, V and scores are on the SM at once: one softmax, no rescaling.
 // A CTA of one verify layer over 4096 tokens, from Q's arrival: scores 0.6 us behind it, P 1.6, O 2.6, stored 3.2 (mma.sync kernel: 4.3).
 // What is left is the chain itself: three barriers, two MMA round trips (a 128 x 16 operand tile takes the MMA unit about 64 clocks to
@@ -26,15 +26,16 @@ constexpr unsigned kSuspendNs = 20000;   // see mbar_try_wait
 constexpr uint32_t kTile = 128 * 256;   // 8 pages of K or V
 constexpr uint32_t kCols = 128;         // TMEM: O^T at column 0, S^T of tile t at 32 + 32 t
 
-// NR query rows that a CTA works on (4, 8, 16 or 32), NC columns of the MMAs (the rows behind NR are zeros nobody reads)
-template <int NR, int NT>
+// NR query rows that a CTA works on (4, 8, 16 or 32), NC columns of the MMAs (the rows behind NR are zeros nobody reads); RH threads a token, each
+// with NR / RH of its rows
+template <int NR, int NT, int RH>
 struct Lay {
     static constexpr int NC = NR < 16 ? 16 : NR;
     static constexpr uint32_t kK = 0, kV = NT * kTile, kQ = 2 * NT * kTile, kBar = kQ + NC * 256;
-    static constexpr uint32_t kMax = kBar + 128;                       // [warp][NR] row maxima
-    static constexpr uint32_t kRef = kMax + NT * 4 * NR * 4;           // [warp][NR] the row references, a copy per warp
-    static constexpr uint32_t kSum = kRef + NT * 4 * NR * 4;           // [warp][NR]
-    static constexpr uint32_t kDst = kSum + NT * 4 * NR * 4;           // [warp][NR] where the rows go
+    static constexpr uint32_t kMax = kBar + 128;                       // [token warp][NR] row maxima
+    static constexpr uint32_t kRef = kMax + NT * 4 * NR * 4;           // [warp][NR / RH] the row references, a copy per warp
+    static constexpr uint32_t kSum = kRef + NT * 4 * NR * 4;           // [token warp][NR]
+    static constexpr uint32_t kDst = kSum + NT * 4 * NR * 4;           // [warp][NR / RH] where the rows go
     static constexpr uint32_t kBytes = kDst + NT * 4 * NR * 8 + 1024;  // + alignment slack
     static constexpr uint32_t kP = kK;                                 // P: [64-token block][NC rows][128 B], 128-byte swizzle
     static constexpr uint32_t kO = kV;                                 // cluster merge: [NR][128] floats, then [NR] (m, l)
@@ -64,12 +65,12 @@ __device__ __forceinline__ float across_lanes(float (&v)[NR], Op op) {
 
 }  // namespace
 
-template <int NR, int NT>
-__global__ void __launch_bounds__(NT * 128 + 32, 1)
+template <int NR, int NT, int RH>
+__global__ void __launch_bounds__(NT * 128 * RH + 32, 1)
 attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
-    using S = Lay<NR, NT>;
-    constexpr int NC = S::NC;
-    constexpr int kThreads = NT * 128, kWarps = NT * 4;   // of the softmax warps; one more warp issues the copies and the MMAs
+    using S = Lay<NR, NT, RH>;
+    constexpr int NC = S::NC, NH = NR / RH;   // NH: rows of a softmax warp
+    constexpr int kTokenWarps = NT * 4, kWarps = kTokenWarps * RH, kThreads = kWarps * 32;   // of the softmax warps; one more warp issues the copies and the MMAs
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -80,7 +81,8 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     volatile int* abort_flag = (volatile int*)(smem + S::kBar + 8 * (3 * NT + 1));
     uint32_t* tmem_slot = (uint32_t*)(smem + S::kBar + 8 * (3 * NT + 2));
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tile = warp >> 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int part = RH == 1 ? 0 : warp / kTokenWarps, tw = warp - part * kTokenWarps, tile = tw >> 2, row_off = part * NH;   // (issuer: not used)
     const bool issuer = warp == kWarps;
     const SeqPlan& sp = p.seq[find_seq(p, blockIdx.x)];
     // Items are ((g * row_chunks) + rc) * nsplit + split.  The planner sends blocks of one row chunk only, but the kernel keeps the general form:
@@ -155,9 +157,9 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     float* lse_at = nullptr;
     float scale = p.scale_log2;
     int half_rows = sp.nsplit == 1 || p.part_half;   // 16-bit result rows
-    const int my_row = lane & (NR - 1);
-    const bool merged_here = p.cluster_size > 1 && sp.nsplit > 1;
-    unsigned long long* const row_dst = (unsigned long long*)(smem + S::kDst) + warp * NR;
+    const int my_row = lane & (NH - 1), my_r = row_off + my_row;
+    const bool merged_here = RH == 1 && p.cluster_size > 1 && sp.nsplit > 1;
+    unsigned long long* const row_dst = (unsigned long long*)(smem + S::kDst) + warp * NH;
     if (!issuer) {
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
@@ -177,16 +179,16 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             }
         if (tile < 2) {   // row my_row's, for all lanes of the warp through shared memory
             unsigned long long dst = 0;
-            if (my_row < n_rows && !merged_here) {
-                const int i = div_g(row0 + my_row), hd = g * G + (row0 + my_row) - i * G;
+            if (my_r < n_rows && !merged_here) {
+                const int i = div_g(row0 + my_r), hd = g * G + (row0 + my_r) - i * G;
                 if (sp.nsplit == 1) {
                     const long long at = (long long)(sp.q_row0 + i) * p.hq + hd;
                     dst = (unsigned long long)((unsigned char*)p.out + at * 256);
-                    if (p.lse && warp == 0 && lane < NR) lse_at = p.lse + at;
+                    if (p.lse && tw == 0 && lane < NH) lse_at = p.lse + at;
                 } else {
                     const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
                     dst = (unsigned long long)(p.part_o + e * 128);
-                    if (warp == 0 && lane < NR) ml_at = p.part_ml + e;
+                    if (tw == 0 && lane < NH) ml_at = p.part_ml + e;
                 }
             }
             row_dst[my_row] = dst;
@@ -314,43 +316,43 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     if (!issuer) {
     // ---- one token per thread: mask, row maxima, P = 2^(S * scale - m)
     const uint32_t lanes = (uint32_t)((warp & 3) << 5) << 16;
-    const int t_warp = tile * kTileTok + (warp & 3) * 32, tok = tok_begin + t_warp + lane;   // (t_warp: first token of the warp, from tok_begin)
+    const int t_warp = tw * 32, tok = tok_begin + t_warp + lane;   // (t_warp: first token of the warp, from tok_begin)
     bool live = tile < n_tiles && __all_sync(0xFFFFFFFFu, mbar_wait<kSuspendNs>(s_bar(min(tile, NT - 1)), 0, abort_flag, p.status, p.wait_limit_cycles));
-    float s[NR], x[NR];
+    float s[NH], x[NH];
     if (live) {
         tc_fence_after();
-        tmem_ld<NR>(tmem + lanes + 32 + 32 * tile, (uint32_t*)s);
+        tmem_ld<NH>(tmem + lanes + 32 + 32 * tile + row_off, (uint32_t*)s);
         tmem_wait_ld();
         if (tok_begin + t_warp + 31 > P || tok_begin + t_warp + 32 > tok_end) {   // rows below `lo` do not see this token
-            const int lo = tok >= tok_end ? NR : (tok - P) * G - row0;
+            const int lo = tok >= tok_end ? NR : (tok - P) * G - row0 - row_off;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) if (r < lo) s[r] = -INFINITY;
+            for (int r = 0; r < NH; ++r) if (r < lo) s[r] = -INFINITY;
         }
     } else {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) s[r] = -INFINITY;
+        for (int r = 0; r < NH; ++r) s[r] = -INFINITY;
     }
     float* x_max = (float*)(smem + S::kMax);
     float* x_sum = (float*)(smem + S::kSum);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) x[r] = s[r];
-    const float w_max = across_lanes<NR>(x, [](float a, float b) { return fmaxf(a, b); });
-    x_max[warp * NR + my_row] = w_max * scale;   // (NR < 32: several lanes write the same)
+    for (int r = 0; r < NH; ++r) x[r] = s[r];
+    const float w_max = across_lanes<NH>(x, [](float a, float b) { return fmaxf(a, b); });
+    x_max[tw * NR + my_r] = w_max * scale;   // (NH < 32: several lanes write the same)
     tc_fence_before();
     asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");   // every warp's maxima; all scores are in registers, so K is dead
     tc_fence_after();
     float m_row = -INFINITY;   // of row my_row
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) m_row = fmaxf(m_row, x_max[w * NR + my_row]);
-    float* ref = (float*)(smem + S::kRef) + warp * NR;
+    for (int w = 0; w < kTokenWarps; ++w) m_row = fmaxf(m_row, x_max[w * NR + my_r]);
+    float* ref = (float*)(smem + S::kRef) + warp * NH;
     ref[my_row] = (m_row == -INFINITY) ? 0.f : -m_row;
     __syncwarp();
     if (tile < n_tiles) {
         const int t = t_warp + lane, c = (t & 63) >> 3;
-        unsigned char* pt = smem + S::kP + (t >> 6) * (NC * 128) + (t & 7) * 2;
+        unsigned char* pt = smem + S::kP + (t >> 6) * (NC * 128) + row_off * 128 + (t & 7) * 2;
 #pragma unroll
-        for (int r4 = 0; r4 < NR; r4 += 4) {
-            if (r4 >= n_rows) {   // (padding: the columns of O^T that come of it are not stored, whatever P holds)
+        for (int r4 = 0; r4 < NH; r4 += 4) {
+            if (row_off + r4 >= n_rows) {   // (padding: the columns of O^T that come of it are not stored, whatever P holds)
                 x[r4] = x[r4 + 1] = x[r4 + 2] = x[r4 + 3] = 0.f;
                 continue;
             }
@@ -360,27 +362,27 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             for (int k = 0; k < 4; ++k) {
                 const int r = r4 + k;
                 x[r] = ex2(fmaf(s[r], scale, n[k]));
-                *(__nv_bfloat16*)(pt + r * 128 + ((c ^ (r & 7)) << 4)) = __float2bfloat16_rn(x[r]);
+                *(__nv_bfloat16*)(pt + r * 128 + ((c ^ ((row_off + r) & 7)) << 4)) = __float2bfloat16_rn(x[r]);
             }
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     } else {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) x[r] = 0.f;
+        for (int r = 0; r < NH; ++r) x[r] = 0.f;
     }
     tc_fence_before();
     asm volatile("bar.arrive 1, %0;\n" ::"n"(kThreads + 32) : "memory");   // P is in place
 
     // ---- row sums, while O^T is under way
-    const float w_sum = across_lanes<NR>(x, [](float a, float b) { return a + b; });
-    x_sum[warp * NR + my_row] = w_sum;
+    const float w_sum = across_lanes<NH>(x, [](float a, float b) { return a + b; });
+    x_sum[tw * NR + my_r] = w_sum;
     asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");   // every warp's sums
     float l_row = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) l_row += x_sum[w * NR + my_row];
+    for (int w = 0; w < kTokenWarps; ++w) l_row += x_sum[w * NR + my_r];
 
-    // ---- epilogue: lane = head dim, column = row; the first two warpgroups take half of the rows each
-    constexpr int kHalf = NR / 2;
+    // ---- epilogue: lane = head dim, column = row; the warpgroups of the first two tiles take half of their rows each
+    constexpr int kHalf = NH / 2;
     // weight of row my_row, for all lanes of the warp through shared memory (its copy of the row references is dead)
     if (tile < 2) {
         if (lse_at) *lse_at = (m_row + log2f(l_row)) * 0.6931471805599453f;
@@ -393,7 +395,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         float o[kHalf];
         if (done && n_tiles > 0) {
             tc_fence_after();
-            tmem_ld<kHalf>(tmem + lanes + tile * kHalf, (uint32_t*)o);
+            tmem_ld<kHalf>(tmem + lanes + row_off + tile * kHalf, (uint32_t*)o);
             tmem_wait_ld();
         } else {
 #pragma unroll
@@ -401,9 +403,9 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         }
         const int d = (warp & 3) * 32 + lane;
         if (merged_here) {
-            if (warp == 0 && lane < NR) cl_ml[lane] = make_float2(m_row, l_row);
+            if (tw == 0 && lane < NH) cl_ml[my_r] = make_float2(m_row, l_row);
 #pragma unroll
-            for (int j = 0; j < kHalf; ++j) cl_o[(tile * kHalf + j) * 128 + d] = o[j];
+            for (int j = 0; j < kHalf; ++j) cl_o[(row_off + tile * kHalf + j) * 128 + d] = o[j];
         } else if (!half_rows) {   // the un-normalised fp32 rows
 #pragma unroll
             for (int j = 0; j < kHalf; ++j) {
@@ -437,34 +439,44 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
     }
-    if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
+    if constexpr (RH == 1)
+        if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
 }
 
 namespace {
-template <int NR, int NT>
+template <int NR, int NT, int RH>
 cudaError_t launch_swap(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    constexpr int kSmem = (int)Lay<NR, NT>::kBytes;
+    constexpr int kSmem = (int)Lay<NR, NT, RH>::kBytes;
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
     static bool configured_on[64] = {false};
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!configured_on[device]) {
-        cudaError_t e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        cudaError_t e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+        e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
         if (e != cudaSuccess) return e;
         configured_on[device] = true;
     }
     if (p.cluster_size > 1)
-        return launch_chained_cluster(attn_swap_bf16_kernel<NR, NT>, dim3(p.num_items), dim3(NT * 128 + 32), kSmem, (unsigned)p.cluster_size, stream, p, map_k, map_v);
-    return launch_chained(attn_swap_bf16_kernel<NR, NT>, dim3(p.num_items), dim3(NT * 128 + 32), kSmem, stream, p, map_k, map_v);
+        return launch_chained_cluster(attn_swap_bf16_kernel<NR, NT, RH>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, (unsigned)p.cluster_size, stream, p, map_k, map_v);
+    return launch_chained(attn_swap_bf16_kernel<NR, NT, RH>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, stream, p, map_k, map_v);
 }
 
 template <int NT>
 cudaError_t launch_rows(const AttnParams& p, int rows, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    if (rows <= 4) return launch_swap<4, NT>(p, map_k, map_v, stream);
-    if (rows <= 8) return launch_swap<8, NT>(p, map_k, map_v, stream);
-    return rows <= 16 ? launch_swap<16, NT>(p, map_k, map_v, stream) : launch_swap<32, NT>(p, map_k, map_v, stream);
+    if (rows <= 4) return launch_swap<4, NT, 1>(p, map_k, map_v, stream);
+    // More than four rows and two tiles: two threads a token, each with half of its rows, so that butterflies, exponentials and stores are half as long.  One
+    // layer, one thread a token / two: 8 rows of 32/8 heads over 3 x 700 tokens 8.46 / 6.80 us, 5 over 2 x 1500 8.47 / 7.04, 4 over 8 x 300 7.49 / 6.60, 8 over
+    // 3000 7.64 / 7.01, 2 over 1000 7.08 / 6.48.  Not for three tiles, whose 800 threads are slower (8 rows
+    // over 4096 tokens 7.84 / 8.38: the third tile's scores, a third of a microsecond behind the first's, set the pace), nor for splits merged in
+    // clusters (one row or two; not compiled: the merge's loads want 64 registers).
+    if constexpr (NT == 2) {
+        if (p.cluster_size <= 1)
+            return rows <= 8 ? launch_swap<8, NT, 2>(p, map_k, map_v, stream)
+                             : rows <= 16 ? launch_swap<16, NT, 2>(p, map_k, map_v, stream) : launch_swap<32, NT, 2>(p, map_k, map_v, stream);
+    }
+    return rows <= 8 ? launch_swap<8, NT, 1>(p, map_k, map_v, stream) : rows <= 16 ? launch_swap<16, NT, 1>(p, map_k, map_v, stream) : launch_swap<32, NT, 1>(p, map_k, map_v, stream);
 }
 }  // namespace
 

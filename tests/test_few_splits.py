@@ -1,5 +1,6 @@
 """Merge of fp16 partials of two to eight KV splits, a half-warp a (row, head) pair: partials in tiles (256-row schedule; row groups of whole and of
-cut tiles, a batch of sequences with different and with no splits) and in slots, odd numbers of pairs."""
+cut tiles, a batch of sequences with different and with no splits) and in slots, odd numbers of pairs; and the swapped-operand kernel with two threads
+a token, at the row counts where its halves begin and end."""
 import numpy as np
 import pytest
 
@@ -53,3 +54,12 @@ def test_partials_in_slots(n, tokens, q, hq, hkv, kind, splits):
     ln, = plan([tokens] * n, [q] * n, hq, hkv).launches
     assert ln.lean and ln.kind == kind and ln.seqs[0].nsplit == splits
     check([tokens] * n, [q] * n, hq, hkv, "slots")
+
+
+@pytest.mark.parametrize("rows", [5, 8, 9, 12, 13, 16, 17, 20, 24, 25, 31, 32])
+@pytest.mark.parametrize("tokens", [40, 129, 250, 300, 511])
+def test_two_threads_a_token(rows, tokens):
+    """Rows of one head a group, so that any number of them may be there."""
+    ln, = plan([tokens], [rows], 2, 2).launches
+    assert ln.kind in ("small1", "small2") and ln.seqs[0].split_tokens <= 256 and not ln.cluster
+    check([tokens], [rows], 2, 2, f"{rows} rows")
