@@ -202,6 +202,20 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
             if (tid >= 32 && tid - 32 + j * kLoaders < own_units) first_id[j] = own_id(tid - 32 + j * kLoaders);
     };
     if (kByHand && pre) fetch_own_ids();         // (the caller vouches for the page table too)
+    // Q and the block's own rows, on their way to L2 before the wait (one row: 4 x 2500 tokens 11.07 -> 10.82 us, 12 x 1000 13.79 -> 13.38, 12000
+    // 12.43 -> 12.32)
+    if (tid >= 32) {
+        for (int c = tid - 32; c < MT * 256; c += kLoaders) {
+            const int r = row0 + (c >> 4), i = div_g(r);
+            if (r < rows) prefetch_l2((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + g * G + r - i * G) * kRowBytes + (c & 15) * 16);
+        }
+        if (kByHand && p.k_new)
+            for (int u = tid - 32; u < own_units; u += kLoaders) {
+                const int tok = tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15);
+                if (tok >= P && tok < L)
+                    prefetch_l2((const unsigned char*)(((u >> 8) & 1) ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * kRowBytes + (u & 15) * 16);
+            }
+    }
     if (!(warp == 0 && pre)) pdl_wait();   // from here on global memory written by the launch before this one is read
     if (kByHand && !pre) fetch_own_ids();
     // ---- producer state (warp 0; lane 0 issues the TMA copies).  Page ids are fetched 32 at a time,

@@ -170,12 +170,21 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 q_at[j] = (const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16);
             }
             hold(q_at[j]);
+            if (q_at[j]) prefetch_l2(q_at[j]);   // (8 rows over 1000 / 4096 tokens with Q in memory 7.17 / 7.77 -> 6.70 / 7.68 us a layer)
         }
 #pragma unroll
         for (int j = 0; j < kOwn; ++j)
             if (j < kOwn1 || more_own) {
                 own_pool_at[j] = own_pool(tid + j * kThreads); own_new_at[j] = own_new(tid + j * kThreads);
                 hold(own_pool_at[j]); hold(own_new_at[j]);
+                const int u = tid + j * kThreads, tok = own_tok(u);
+                if (u < two_pages && tok < L) {
+                    if (tok >= pool_end) prefetch_l2(own_new_at[j]);
+                    else if (pre) {
+                        const int id = u < 512 ? first_id : second_id;
+                        if (id >= 0 && id < num_pages) prefetch_l2(own_pool_at[j] + (long long)id * page_bytes);
+                    }
+                }
             }
         if (tile < 2) {   // row my_row's, for all lanes of the warp through shared memory
             unsigned long long dst = 0;
@@ -468,7 +477,7 @@ cudaError_t launch_rows(const AttnParams& p, int rows, const CUtensorMap& map_k,
     if (rows <= 4) return launch_swap<4, NT, 1>(p, map_k, map_v, stream);
     // More than four rows and two tiles: two threads a token, each with half of its rows, so that butterflies, exponentials and stores are half as long.  One
     // layer, one thread a token / two: 8 rows of 32/8 heads over 3 x 700 tokens 8.46 / 6.80 us, 5 over 2 x 1500 8.47 / 7.04, 4 over 8 x 300 7.49 / 6.60, 8 over
-    // 3000 7.64 / 7.01, 2 over 1000 7.08 / 6.48.  Not for three tiles, whose 800 threads are slower (8 rows
+    // 3000 7.64 / 7.01, 2 over 1000 7.08 / 6.48 (with Q on its way to L2 ahead of the wait, below).  Not for three tiles, whose 800 threads are slower (8 rows
     // over 4096 tokens 7.84 / 8.38: the third tile's scores, a third of a microsecond behind the first's, set the pace), nor for splits merged in
     // clusters (one row or two; not compiled: the merge's loads want 64 registers).
     if constexpr (NT == 2) {

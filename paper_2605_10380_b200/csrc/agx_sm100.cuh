@@ -128,6 +128,9 @@ __device__ __forceinline__ void hold(T* __restrict__& x) { asm volatile("" : "+l
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
+// On its way to L2 before the dependency wait: a hint that moves no data to the SM, so that it may run ahead of the launch that writes the line.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p) : "memory"); }
+
 // The sequence plan of a work item.
 __device__ __forceinline__ int find_seq(const AttnParams& p, int item) {
     int s = 0;
