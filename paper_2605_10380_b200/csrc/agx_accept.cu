@@ -78,12 +78,8 @@ struct VecMax {
 };
 
 __device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        v = o > v ? o : v;
-    }
-    return v;
+    const unsigned int hi = (unsigned int)(v >> 32), top = __reduce_max_sync(0xFFFFFFFFu, hi);
+    return ((unsigned long long)top << 32) | __reduce_max_sync(0xFFFFFFFFu, hi == top ? (unsigned int)v : 0u);
 }
 
 // What the comparison of a sequence needs besides the winners, fetched by a warp ahead of them: its rows, and of its drafts the first 32.

@@ -192,9 +192,7 @@ attn_simt_kernel(const __grid_constant__ AttnParams p) {
         __syncthreads();
         {   // warp r: softmax of row r
             const float2 x = *(const float2*)&sm.s[warp][2 * lane];
-            float mx = fmaxf(x.x, x.y);
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, d));
+            const float mx = warp_max(fmaxf(x.x, x.y));
             const float m_new = fmaxf(m_run, mx), m_ref = m_new == -INFINITY ? 0.f : m_new;
             const float corr = exp2f(m_run - m_ref);
             const float2 w = make_float2(exp2f(x.x - m_ref), exp2f(x.y - m_ref));

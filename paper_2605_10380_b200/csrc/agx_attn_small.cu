@@ -691,8 +691,7 @@ attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {
             if (16 + j < ns && c4 < D) v2[j] = rows.load(16 + j);
     }
     m_all = ml.x;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
+    m_all = warp_max(m_all);
     const float e_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
     l_all = ml.y * e_mine;
     const float w_mine = e_mine;   // weight of this lane's split's O row
@@ -776,9 +775,7 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
                     v[j] = rows.load(k0 + j);
                 }
             }
-        float m_new = ml.x;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xFFFFFFFFu, m_new, off));
+        float m_new = warp_max(ml.x);
         m_new = fmaxf(m, m_new);
         const float e = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_new), keep = (m == -INFINITY) ? 0.f : exp2f(m - m_new);
         float sum = ml.y * e;
@@ -941,9 +938,7 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
         for (int k = 0; k < kNsMax; ++k) v[k] = rows.load(min(k, ns - 1));
         float2 ml = make_float2(-INFINITY, 0.f);
         if (lane < ns) ml = ld_volatile_f2(ml_at);
-        float m_all = ml.x;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));
+        const float m_all = warp_max(ml.x);
         const float w_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * ml.y;   // 0 in lanes past the last split
         float l_all = w_mine;
 #pragma unroll

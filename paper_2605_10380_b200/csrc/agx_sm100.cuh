@@ -212,6 +212,14 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
     return v;
 }
 
+// Maximum over the warp, in every lane, by one instruction (a NaN loses, as with fmaxf).  Five steps of shuffles and maxima in its place are a chain of
+// some 130 clocks.
+__device__ __forceinline__ float warp_max(float x) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;\n" : "=f"(m) : "f"(x));
+    return m;
+}
+
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
@@ -234,9 +242,7 @@ __device__ __forceinline__ void merge_cluster_rows(const AttnParams& p, const Se
     for (int r = split + warp * cs; r < n_rows; r += kWarps * cs) {
         float2 ml = make_float2(-INFINITY, 0.f);
         if (lane < cs) ml = ld_cluster_f2(cluster_map(smem_u32(cl_ml + r), lane));
-        float m_all = ml.x;
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, d));
+        const float m_all = warp_max(ml.x);
         const float w = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all);
         float l_all = ml.y * w;
 #pragma unroll
