@@ -9,6 +9,8 @@
 // block to finish (ticket counter) reads the row keys back, leaves them and the ticket at zero for
 // the next launch, compares drafts and writes the results, so no second launch and no host round
 // trip is needed.
+#include <algorithm>
+
 #include "agx_internal.cuh"
 #include "agx_sm100.cuh"
 
@@ -116,10 +118,11 @@ __device__ __forceinline__ void commit_sequence(int s, const SeqHead& h, const i
     }
 }
 
+constexpr int kAcceptCtas = 6;               // CTAs per SM
 constexpr int kTokSmem = 2048;               // winners of up to this many rows stay in shared memory for the draft comparison
 
 template <bool kBf16, bool kVec>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kAcceptCtas)
 accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, int chunk_elems,
               const int* __restrict__ drafts, const int* __restrict__ cu_q, int B, int total_q,
               int* __restrict__ accept_len, int* __restrict__ next_token, int* __restrict__ argmax,
@@ -144,18 +147,19 @@ accept_kernel(const void* __restrict__ logits, long long row_stride, int vocab, 
     unsigned long long best = 0ull;  // "no element": loses to every real element
     if (kVec) {
         VecMax<kBf16> vm;
-        // two independent 16-byte loads in flight per thread per trip
-        unsigned int i = begin + threadIdx.x * kVecElems;
+        // four independent 16-byte loads in flight per thread and trip, also in the last one
         const unsigned int stride = 256 * kVecElems;
-        for (; i + stride + kVecElems <= end; i += 2 * stride) {
-            const uint4 a = __ldg((const uint4*)(row_ptr + (size_t)i * (kBf16 ? 2 : 4)));
-            const uint4 b = __ldg((const uint4*)(row_ptr + (size_t)(i + stride) * (kBf16 ? 2 : 4)));
-            vm.take(a, i);
-            vm.take(b, i + stride);
-        }
-        for (; i < end; i += stride) {
-            if (i + kVecElems <= end) vm.take(__ldg((const uint4*)(row_ptr + (size_t)i * (kBf16 ? 2 : 4))), i);
-            else vm.take_partial(row_ptr, i, end);
+        for (unsigned int i = begin + threadIdx.x * kVecElems; i < end; i += 4 * stride) {
+            uint4 a[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i + u * stride + kVecElems <= end) a[u] = __ldg((const uint4*)(row_ptr + (size_t)(i + u * stride) * (kBf16 ? 2 : 4)));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned int at = i + u * stride;
+                if (at + kVecElems <= end) vm.take(a[u], at);
+                else if (at < end) vm.take_partial(row_ptr, at, end);
+            }
         }
         best = vm.key();
     } else {
@@ -260,6 +264,18 @@ accept_cluster_kernel(const void* __restrict__ logits, long long row_stride, int
     cluster_sync();   // no CTA leaves while its keys may still be read
 }
 
+// Chunks per row: one wave of CTAs, as long as every thread has two 16-byte loads to do.  (Rounded up the last CTAs were a second wave: rows of 128256 bf16,
+// eight CTAs of two loads a thread per SM rounded up / eight rounded down / six of four loads rounded down, us: 64 rows 9.5 / 7.6 / 7.8, 128 13.3 / 10.6 /
+// 10.3, 256 22.3 / 17.8 / 16.5, 512 - / 33.3 / 31.7, 33 6.2 / 6.2 / 6.0, 16 5.6 / - / 5.4; eight of four or five of six are as good.)
+int accept_chunks(int sm_count, int total_q, int vocab, int elem_bytes) {
+    const int vec = 16 / elem_bytes;
+    const int max_chunks = (vocab + 256 * vec * 2 - 1) / (256 * vec * 2);
+    const int want = std::max(1, std::min(kAcceptCtas * sm_count / std::max(total_q, 1), max_chunks));
+    int chunk_elems = (vocab + want - 1) / want;
+    chunk_elems = (chunk_elems + vec - 1) / vec * vec;
+    return (vocab + chunk_elems - 1) / chunk_elems;
+}
+
 cudaError_t launch_accept(const void* logits, int logits_dtype, long long row_stride, int vocab, const int* drafts,
                           const int* cu_q, int B, int total_q, int* accept_len, int* next_token, int* argmax,
                           int* seq_lens, unsigned long long* row_keys, int* tokens_global, int chunks, unsigned int* ticket,
@@ -362,17 +378,7 @@ extern "C" AGX_API agx_status agx_accept_greedy_static(const void* logits, int32
             scratch = ptr;
         }
     }
-    // Chunks per row: enough CTAs that every thread needs a single trip of two 16-byte loads (8 per SM, as the workspace
-    // variant aims for).
-    const int vec = logits_dtype == AGX_BF16 ? 8 : 4;
-    int want = (8 * st.sm_count + total_q - 1) / total_q;
-    const int max_chunks = (vocab + 256 * vec * 2 - 1) / (256 * vec * 2);   // >= 2 vectors per thread
-    if (want > max_chunks) want = max_chunks;
-    if (want < 1) want = 1;
-    int chunk_elems = (vocab + want - 1) / want;
-    chunk_elems = (chunk_elems + vec - 1) / vec * vec;
-    const int chunks = (vocab + chunk_elems - 1) / chunk_elems;   // <= want
-
+    const int chunks = accept_chunks(st.sm_count, total_q, vocab, logits_dtype == AGX_BF16 ? 2 : 4);
     unsigned char* base = (unsigned char*)scratch;
     // the array keeps whatever the previous call left: the ticket counter and the rows' keys must start at zero (the
     // kernel leaves them at zero itself; the clear makes the call independent of how an earlier one ended)

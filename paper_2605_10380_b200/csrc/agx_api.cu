@@ -341,17 +341,6 @@ agx_status agx_attn_prefixed_append(agx_handle* h, const void* q_block, const vo
                      workspace, workspace_bytes, stream, h && h->early_prefix);
 }
 
-static int accept_chunks(const agx_handle* h, int total_q, int vocab, int dtype) {
-    const int vec = 16 / elem_size(dtype);
-    const int target = 8 * h->sm_count;   // enough CTAs that every thread needs a single trip of two 16-byte loads
-    int want = std::max(1, (target + total_q - 1) / total_q);
-    const int max_chunks = std::max(1, (vocab + 256 * vec * 2 - 1) / (256 * vec * 2));  // >= 2 vectors per thread
-    want = std::min(want, max_chunks);
-    int chunk_elems = (vocab + want - 1) / want;
-    chunk_elems = (chunk_elems + vec - 1) / vec * vec;
-    return (vocab + chunk_elems - 1) / chunk_elems;
-}
-
 int64_t agx_accept_workspace_bytes(agx_handle* h, int32_t total_q, int32_t vocab) {
     if (!h) return AGX_E_INVAL;
     if (total_q < 0 || vocab < 1) return fail(h, AGX_E_RANGE, "total_q < 0 or vocab < 1");
@@ -377,7 +366,7 @@ agx_status agx_accept_greedy(agx_handle* h, const void* logits, int32_t logits_d
     const int64_t need = agx_accept_workspace_bytes(h, total_q, vocab);
     if (!workspace || !aligned(workspace, 8) || (int64_t)workspace_bytes < need)
         return fail(h, AGX_E_INVAL, "accept workspace missing, misaligned or too small (%lld needed)", (long long)need);
-    const int chunks = accept_chunks(h, total_q, vocab, logits_dtype);
+    const int chunks = accept_chunks(h->sm_count, total_q, vocab, elem_size(logits_dtype));
     cudaError_t e = launch_accept(logits, logits_dtype, row_stride, vocab, drafts, cu_q, B, total_q, accept_len,
                                   next_token, argmax, seq_lens, h->d_row_keys, (int*)workspace, chunks, h->d_ticket,
                                   (cudaStream_t)stream);
