@@ -26,6 +26,8 @@ struct SplitModel {
     int part_row_bytes;
     double lean;            // > 0: one-wave launches with few (row, head) pairs leave SMs to their merge kernel, which costs this and 0.2 per MB
     bool in_order;          // up to 16 waves: CTAs dealt out as the grid has them instead of longest first
+    double crowd;           // launches of one wave and more: the next call's CTAs find no free SMs to start on (all of it; nothing up to half of the SMs)
+    double merge_many;      // a merge of more than four splits
 };
 // Fitted to 340 launches of one to eight blocks, each in all splits that make sense: the split chosen is 1.0 % slower than the best of them on
 // average (with 1.9 us a tile, 2.2 + 0.38 us per MB: 1.4 %).  The grid's order counts where a launch is little more than
@@ -33,19 +35,22 @@ struct SplitModel {
 // 3000, 32/8 heads, 5 / 4 splits: 31.1 / 21.7 us a layer; 931 behind 3086, 24/8: 66.7 -> 60.2; 598 behind 5293: 76 -> 68.3; verify blocks with three to
 // eight prefills 5 to 10 %).  (Sequences whose K/V exceed 48 MB have the KV head outermost in the grid and are dealt out here like the others: 50 plans that
 // the order makes different were 0.2 % slower together with it, single ones 13 % faster to 13 % slower.)
+// The last four constants are from 185 lone blocks of 97 to 1500 rows, each in all splits that make sense, with the merge of half a warp a pair: the split
+// chosen is 0.75 % slower than the best of them on average (1.5 % with a merge of 1.5 + 0.45 us per MB and neither of the two others).
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
 SplitModel tile_model(const PlanConfig& c, bool f32_partials = false) {
-    return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, f32_partials ? 1.9 : 1.5, f32_partials ? 0.3 : 0.45, 0.3, f32_partials ? 520 : 264, 0, true};
+    if (f32_partials) return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.9, 0.3, 0.3, 520, 0, true, 0, 0};
+    return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.1, 0.35, 0.3, 264, 0, true, 0.5, 0.4};
 }
 // (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them.  40 rows over 300 / 450 / 600
 // tokens, 40/8 heads, take 9.0 / 9.8 / 10.5 us whole and 10.5 / 10.1 / 9.9 in splits of 256 tokens: the merge behind two tiles costs as much as two)
 SplitModel stream_model(const PlanConfig& c, bool wide) {
-    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, wide ? 2.2 : 1.0, false};
+    return {128, c.sm_count, 7, 7.5, 0, wide ? 1.25 : 0.85, 0.0093, wide ? 2.5 : 4.5, wide ? 0.4 : 0.6, 0.3, 520, wide ? 2.2 : 1.0, false, 0, 0};
 }
 // warp-MMA kernel with 4-page stages, two CTAs per SM: HBM-bound with one 16-row tile, bounded by its own chain with two (mma.sync)
 SplitModel small4_model(const PlanConfig& c, int mt) {
-    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, 0, false};
+    return {64, 2 * c.sm_count, mt == 1 ? 3 : 2, 4.0, 0, mt == 1 ? 1.1 : 1.6, mt == 1 ? 0.00537 : 0.0055, 3.0, 0.38, 0.3, 520, 0, false, 0, 0};
 }
 
 // Steps (of md.unit tokens) per KV split: the candidate with the smallest estimated time, and that time.  A server's lengths change with every
@@ -98,7 +103,7 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
             }
         }
     };
-    struct Cand { int tiles, longest; double bound, merge; long long sum, count; };
+    struct Cand { int tiles, longest; double bound, merge; long long sum, count; };   // merge: what follows the last tile, and what the next call waits for
     struct Chunks { long long n; int per, full, rest; };
     std::vector<Cand> cands;
     const int n_max = (int)std::min<long long>((max_tiles + min_tiles - 1) / min_tiles, std::max<long long>(32, 2 * sms / std::max<long long>(base_items, 1)));
@@ -108,10 +113,11 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         if (t == last) continue;
         last = t;
         long long sum = 0, count = 0;
-        int longest = 0;
+        int longest = 0, ns_max = 1;
         double mb = 0;
         for (const Seq& w : work) {
             const int ns = (w.tiles + t - 1) / t;
+            ns_max = std::max(ns_max, ns);
             if (ns > 1) mb += w.rows_heads * ns * md.part_row_bytes * 1e-6;
         }
         deal(t, [&](const Seen& v, int per, int full, int rest) {
@@ -129,6 +135,7 @@ SplitChoice choose_split(const PlanConfig& c, const SplitModel& md, const std::v
         cd.merge = mb == 0 ? 0 : md.lean > 0 && count <= sms * 15 / 16 && pairs <= 3 * sms ? md.lean + 0.2 * mb
                    : md.unit == 64 && equal && n <= 16 ? (count <= sms ? 0.5 : 4.0)   // (merged inside clusters)
                    : md.merge + md.merge_mb * std::min(mb, 16.0) + md.merge_mb_beyond_16 * std::max(mb - 16.0, 0.0);
+        cd.merge += md.crowd * std::min(1.0, std::max(0.0, (double)(count - sms / 2) / (sms / 2))) + (ns_max > 4 ? md.merge_many : 0.0);
         // (a step takes per_add, and beyond it per_min or what all CTAs at work share of per_busy)
         cd.bound = md.base + cd.merge + (load - kOverhead) * md.per_add +
                    std::max((load - kOverhead) * md.per_min, (sum - (double)kOverhead * std::min<long long>(count, sms)) * md.per_busy);
