@@ -616,8 +616,8 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 __device__ __forceinline__ const unsigned char* half_row(const AttnParams& p, const SeqPlan& sp, int i, int h, int u) {
     if (p.part_half != PART_HALF_TILES) return (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + u * 16;
     const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rl = r & 255;
-    return (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 + rl * 256 +
-           ((u ^ (rl & 15)) << 4);
+    return (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 + (u >> 3) * 32768 + rl * 128 +
+           (((u ^ rl) & 7) << 4);
 }
 // The fp16 partials of row i, head h, four columns a lane: split 0's, and the bytes from split to split.
 struct HalfRows {
@@ -634,8 +634,8 @@ struct F32Rows {
     __device__ __forceinline__ F32Rows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane) {
         if (p.part_half == PART_F32_TILES) {
             const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rows = sp.q_len * p.gqa;
-            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + (long long)g * sp.nsplit * rows) * 512 + ((lane >> 4) * rows + r) * 256 +
-                 (((lane & 15) ^ (r & 15)) << 4);
+            at = (const unsigned char*)p.part_o + ((long long)sp.part_base + (long long)g * sp.nsplit * rows) * 512 + ((lane >> 3) * rows + r) * 128 +
+                 (((lane ^ r) & 7) << 4);
             stride = rows * 512;
         } else {
             at = (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * (p.head_dim * 4) + lane * 16;

@@ -287,6 +287,15 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     if (!kStreams && !mbar_wait(smem_u32(smem) + kOffBar + 8u * (warp < 8 ? BAR_O_FULL : BAR_O_FULL_B), 0, (volatile int*)(smem + kOffBar + BAR_COUNT * 8), cx.status,
                                 *(const long long*)(smem + kOffBar + BAR_COUNT * 8 + 16))) return;
     tc_fence_after();
+    // 128 bytes of each of the warp's rows, as they lie in a half of the staging area, to `at` of this CTA's partials
+    auto leave = [&](const unsigned char* half, long long at) {
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(cx.part_tile + at + (warp - 4) * 4096), "r"(smem_u32(half)), "r"(min(32, it.rows - r_warp0) * 128) : "memory");
+            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+        }
+    };
     {
         uint32_t oreg[64];   // two 32-column chunks per TMEM round trip
 #pragma unroll 1
@@ -333,38 +342,43 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                     }
                 }
             } else if (kF32Part && !single) {
-                // fp32 partials: these 64 columns of the warp's rows go through the staging area
-                if (c8) {
-                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-                    __syncwarp();
-                }
+                // fp32 partials the same way, 32 columns at a time through either half of the staging area
 #pragma unroll
-                for (int v = 0; v < 16; ++v)
-                    *(uint4*)(stage + lane * 256 + ((v ^ (lane & 15)) << 4)) = make_uint4(oreg[4 * v], oreg[4 * v + 1], oreg[4 * v + 2], oreg[4 * v + 3]);
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(cx.part_tile + (long long)(c8 >> 1) * it.rows * 256 + (warp - 4) * 8192),
-                                 "r"(smem_u32(stage)), "r"(min(32, it.rows - r_warp0) * 256) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                for (int c4 = 0; c4 < 2; ++c4) {
+                    unsigned char* half = stage + c4 * 4096;
+                    if (c8) {
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int v = 0; v < 8; ++v)
+                        *(uint4*)(half + lane * 128 + ((v ^ (lane & 7)) << 4)) = make_uint4(oreg[32 * c4 + 4 * v], oreg[32 * c4 + 4 * v + 1], oreg[32 * c4 + 4 * v + 2], oreg[32 * c4 + 4 * v + 3]);
+                    leave(half, (long long)(c8 + c4) * it.rows * 128);
                 }
-            } else {
-                // pack to the 16-bit output format first (bf16 results, fp16 split partials): 256 bytes per row go through
-                // the staging area, 16-byte units XOR-swizzled by row
+            } else if (!single) {
+                // fp16 split partials, 64 columns of the warp's rows at a time: 128 bytes per row through the staging area, 16-byte units XOR-swizzled by row, and
+                // on their way as they lie there, one bulk copy, while the other columns are read (128 rows
+                // over 1000 tokens 11.5 -> 11.1 us, 250 over 900 with 16/2 heads 11.4 -> 11.0, 512 over 3072 with 24/8 25.7 -> 25.5 against one copy at the end)
+                unsigned char* half = stage + (c8 >> 1) * 4096;
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
                     uint4 pk;
-                    if (single) {
-                        pk.x = pack_bf16(__uint_as_float(oreg[8 * v + 0]), __uint_as_float(oreg[8 * v + 1]));
-                        pk.y = pack_bf16(__uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
-                        pk.z = pack_bf16(__uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
-                        pk.w = pack_bf16(__uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
-                    } else {
-                        pk.x = pack_f16(__uint_as_float(oreg[8 * v + 0]), __uint_as_float(oreg[8 * v + 1]));
-                        pk.y = pack_f16(__uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
-                        pk.z = pack_f16(__uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
-                        pk.w = pack_f16(__uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
-                    }
+                    pk.x = pack_f16(__uint_as_float(oreg[8 * v + 0]), __uint_as_float(oreg[8 * v + 1]));
+                    pk.y = pack_f16(__uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
+                    pk.z = pack_f16(__uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
+                    pk.w = pack_f16(__uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
+                    *(uint4*)(half + lane * 128 + ((v ^ (lane & 7)) << 4)) = pk;
+                }
+                leave(half, (c8 >> 1) * 32768);
+            } else {
+                // bf16 results: 256 bytes per row go through the staging area, 16-byte units XOR-swizzled by row
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                    uint4 pk;
+                    pk.x = pack_bf16(__uint_as_float(oreg[8 * v + 0]), __uint_as_float(oreg[8 * v + 1]));
+                    pk.y = pack_bf16(__uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
+                    pk.z = pack_bf16(__uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
+                    pk.w = pack_bf16(__uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
                     *(uint4*)(stage + lane * 256 + ((((c8 >> 1) * 8 + v) ^ (lane & 15)) << 4)) = pk;
                 }
             }
@@ -372,20 +386,8 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     }
     if (kStreams) return;
     const int n_valid = min(32, it.rows - r_warp0);
-    if (kF32Part && !single) {
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
-        return;
-    }
     if (!single) {
-        // fp16 split partials leave as they lie in the staging area, one bulk copy a warp: they are in a layout of their own, that of the staging
-        // area.  Row by row through the LSU to a slot per (row, head, split) took 1.4 us instead of 0.1.
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(cx.part_tile + (warp - 4) * 8192), "r"(smem_u32(stage)), "r"(n_valid * 256) : "memory");
-            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
-        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
         return;
     }
     __syncwarp();
@@ -863,7 +865,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cx->part_half = p.part_half;
             const int rc = row0 / kRowsPerCta;
             cx->part_tile = (unsigned char*)p.part_o + (long long)sp.part_base * 512 +
-                            (kF32Part ? ((long long)g * sp.nsplit + split) * rows * 512 + row0 * 256
+                            (kF32Part ? ((long long)g * sp.nsplit + split) * rows * 512 + row0 * 128
                                       : (((long long)g * sp.row_chunks + rc) * sp.nsplit + split) * 65536);
             mbar_arrive(bar(BAR_CTX));   // (release) the epilogue waits on this before it reads the context
         }

@@ -42,9 +42,9 @@ struct SeqPlan {
     int chunk_major;   // order of the work items: 0 = KV head outermost, 1 = row chunk outermost (row chunks last to first in both)
 };
 
-// Split partials: fp32 rows in slots | fp16 rows in slots | fp16 or fp32 rows in tiles (256-row tensor-core schedule), 256 bytes of a row side by side and
-// their 16-byte unit u at u ^ (r & 15), from part_base * 512 bytes on.  fp16: 64 KB per (KV head, row chunk, split) of a sequence, splits innermost.
-// fp32: per (KV head, split) the first 64 columns of all rows, then the others.
+// Split partials: fp32 rows in slots | fp16 rows in slots | fp16 or fp32 rows in tiles (256-row tensor-core schedule), from part_base * 512 bytes on.  In tiles
+// the first 128 bytes of all rows come first, then the second ones and so on; 16-byte unit u of 128 bytes lies at u ^ (r & 7).  fp16: two times 256 rows,
+// 64 KB, per (KV head, row chunk, split) of a sequence, splits innermost.  fp32: four times all rows per (KV head, split).
 enum PartHalf { PART_F32 = 0, PART_HALF_SLOTS = 1, PART_HALF_TILES = 2, PART_F32_TILES = 3 };
 
 struct AttnParams {
