@@ -611,7 +611,8 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 // Combine: out[row, h] = sum_k O_k 2^(m_k - m) / sum_k l_k 2^(m_k - m), splits in index order.
 // One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
 // kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel takes more).  Four O rows per
-// warp instead of 32 keep the register count low enough for ten CTAs per SM, which is what the partials of a split prefill need.
+// warp instead of 32 keep the register count low enough for ten CTAs per SM.
+
 // Where 16-byte unit u of split 0's fp16 partial of row i, head h lies.
 __device__ __forceinline__ const unsigned char* half_row(const AttnParams& p, const SeqPlan& sp, int i, int h, int u) {
     if (p.part_half != PART_HALF_TILES) return (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + u * 16;
@@ -901,7 +902,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     if (lse_at && u == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
-// The same merge for the fp16 partials of the small-q kernel (5 to 32 KV splits): one (row, head) pair per warp, lane k
+// The same merge for the fp16 partials of more splits (9 to 32): one (row, head) pair per warp, lane k
 // holding split k's (m, l) and every lane four columns of every split's row, all loads in flight at once.  CTAs of two
 // warps with few registers (12 or 8 CTAs per SM), so that the merge of a one-wave launch fits the few SMs the planner
 // leaves out of the attention grid for it.

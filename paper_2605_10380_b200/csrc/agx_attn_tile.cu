@@ -29,7 +29,7 @@
 //               operand of the P V MMA comes from TMEM), O rescaled in TMEM only when the row maximum
 //               grew by more than 2^8.
 // The Q tiles arrive by TMA (warps 3 and 2) while warp 0 already streams K/V; results leave through a per-warp shared-memory staging area (the
-// Q tiles, dead by then): split partials as they lie there, one bulk copy a warp, finished rows as whole-row stores.  The block's own K/V rows go
+// Q tiles, dead by then): split partials as they lie there, in bulk copies of 64 or 32 columns, finished rows as whole-row stores.  The block's own K/V rows go
 // from the tiles into the pool by TMA.  What a CTA does once runs at five clocks and more an instruction and counts as much as its tiles where these
 // are few (from the dependency wait to the first scores 3.1 -> 2.3 us, c3 29.2 -> 27.2 us, 3584 uncached tokens, 24/8 heads, 85.7 -> 79.9).
 // TMEM columns: S [0,128) P_A [128,192) P_B [192,256) O_A [256,384) O_B [384,512).

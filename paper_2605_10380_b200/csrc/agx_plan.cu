@@ -493,7 +493,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         //      An attention CTA takes a whole SM, so merge CTAs that find no free SM sit on SMs the next call's attention CTAs
         //      need, and those CTAs then start (and fetch their K/V) only after the merge instead of under it.  With a few SMs
         //      left out of the attention grid the merge CTAs are resident there from the start and the next call's grid
-        //      follows this one without a gap.  A two-warp merge CTA handles two (row, head) pairs; 12 (up to 20 splits) or 8
+        //      follows this one without a gap.  A two-warp merge CTA of 9 and more splits handles two (row, head) pairs; 12 (up to 20 splits) or 8
         //      of them fit an SM.
         bool lean_merge = false;   // fp16 partials and the two-warp merge kernel (slower than fp32 partials and the four-warp
                                    // one where the attention grid fills every SM twice over, e.g. four verify blocks of 4096)
