@@ -766,18 +766,11 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         const int n = min(kManyBatch, ns - k0);
         float2 ml = make_float2(-INFINITY, 0.f);
         if (lane < n) ml = ld_volatile_f2(ml_at + k0);
-        float4 v[kManyBatch];
+        // (the rows as they come: converted where they are loaded, one load waited for the other, one row over 12000 tokens with 16/2 heads 7.5 -> 11.1 us)
+        std::conditional_t<kHalfPart, uint2, float4> v[kManyBatch];
 #pragma unroll
         for (int j = 0; j < kManyBatch; ++j)
-            if (j < n && c4 < D) {
-                if constexpr (kHalfPart) {
-                    const uint2 raw = rows.load(k0 + j);
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-                    v[j] = make_float4(a.x, a.y, b.x, b.y);
-                } else {
-                    v[j] = rows.load(k0 + j);
-                }
-            }
+            if (j < n && c4 < D) v[j] = rows.load(k0 + j);
         float m_new = warp_max(ml.x);
         m_new = fmaxf(m, m_new);
         const float e = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_new), keep = (m == -INFINITY) ? 0.f : exp2f(m - m_new);
@@ -791,7 +784,14 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         for (int j = 0; j < kManyBatch; ++j) {
             const float w = __shfl_sync(0xFFFFFFFFu, w_mine, j);
             if (j < n && w != 0.f && c4 < D) {   // a split that saw no token for this row publishes only (m, l) = (-inf, 0)
-                acc.x += v[j].x * w; acc.y += v[j].y * w; acc.z += v[j].z * w; acc.w += v[j].w * w;
+                float4 x;
+                if constexpr (kHalfPart) {
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&v[j].x)), b = __half22float2(*reinterpret_cast<const __half2*>(&v[j].y));
+                    x = make_float4(a.x, a.y, b.x, b.y);
+                } else {
+                    x = v[j];
+                }
+                acc.x += x.x * w; acc.y += x.y * w; acc.z += x.z * w; acc.w += x.w * w;
             }
         }
         m = m_new;
