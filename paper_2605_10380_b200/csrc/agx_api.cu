@@ -316,7 +316,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         if (e != cudaSuccess) return cuda_fail(h, e, "attention launch");
         h->last_launches++;
         if (split) {
-            e = launch_attn_combine(p, h->cfg.dtype, ln.total_rows, stream);
+            e = launch_attn_combine(p, h->cfg.dtype, ln.total_rows, ln.kind == KIND_STREAM, stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "combine launch");
             h->last_launches++;
         }

@@ -902,7 +902,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     if (lse_at && u == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
-// The same merge for the fp16 partials of more splits (9 to 32): one (row, head) pair per warp, lane k
+// The same merge for the fp16 partials of more splits (9 to 32, behind the one-Q-tile schedule 5 to 32): one (row, head) pair per warp, lane k
 // holding split k's (m, l) and every lane four columns of every split's row, all loads in flight at once.  CTAs of two
 // warps with few registers (12 or 8 CTAs per SM), so that the merge of a one-wave launch fits the few SMs the planner
 // leaves out of the attention grid for it.
@@ -1077,7 +1077,7 @@ cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CU
     }
 }
 
-cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, cudaStream_t stream) {
+cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, bool behind_streams, cudaStream_t stream) {
     const long long n = (long long)total_rows * p.hq;
     if (n == 0) return cudaSuccess;
     const int blocks = (int)((n + 3) / 4);
@@ -1085,9 +1085,13 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
     for (int i = 0; i < p.num_seqs; ++i) ns_max = p.seq[i].nsplit > ns_max ? p.seq[i].nsplit : ns_max;
     const int many_threads = 32 * std::min(kManyWarps, (ns_max + kManyBatch - 1) / kManyBatch);
     if (dtype == AGX_BF16 && (p.part_half == PART_HALF_SLOTS || p.part_half == PART_HALF_TILES)) {
-        if (ns_max <= 8)
+        // (five to eight splits behind the one-Q-tile schedule, a few hundred pairs: its CTAs leave nothing of an SM, and the merge's small CTAs of a warp a
+        // pair find room sooner, 7 rows over 1500 tokens with 40/8 heads 10.5 us a layer, half a warp a pair 10.8, 12 over 1200 with 24/8 9.3 / 9.75; behind
+        // the small-q kernels 3 x (1500, 1) 7.4 / 6.8, 3 x (1500, 3) 7.8 / 7.7)
+        if (ns_max <= 4 || (ns_max <= 8 && !behind_streams))
             return launch_chained(ns_max <= 4 ? attn_combine_few_kernel<4> : attn_combine_few_kernel<8>, dim3((unsigned)((n + 7) / 8)), dim3(128), 0, stream, p, total_rows);
         if (ns_max <= 32) {
+            if (ns_max <= 8) return launch_chained(attn_combine_half32_kernel<8>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 12) return launch_chained(attn_combine_half32_kernel<12>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 20) return launch_chained(attn_combine_half32_kernel<20>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             return launch_chained(attn_combine_half32_kernel<32>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);

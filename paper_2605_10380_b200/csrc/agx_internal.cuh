@@ -153,7 +153,7 @@ cudaError_t launch_attn_swap(const AttnParams& p, int rows, int longest, const C
 // fp32-math kernel (agx_attn_simt.cu) for AGX_F32 pools (any q, d in {64, 128}) and for AGX_BF16 pools with d = 64.
 cudaError_t launch_attn_simt(const AttnParams& p, int dtype, cudaStream_t stream);
 // Merge of split partials into out / lse.
-cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, cudaStream_t stream);   // honours p.part_half
+cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, bool behind_streams, cudaStream_t stream);   // honours p.part_half; behind the one-Q-tile schedule or another kernel
 
 // Tensor-core tile kernel (bf16, d = 128, tcgen05 + TMEM + TMA).  streams = false: 256 query rows per CTA
 // (two Q tiles); streams = true: 128 rows per CTA whose KV tiles alternate between two softmax warpgroups
