@@ -107,7 +107,11 @@ agx_status make_plan(agx_handle* h, int B, const int32_t* P, const int32_t* Q, i
     return AGX_OK;
 }
 
+// Split partials: (max, sum) of every entry, the rows, and the exponents of rows beyond fp16's range.
 inline size_t part_ml_bytes(long long entries) { return (size_t)((entries * sizeof(float2) + 255) / 256 * 256); }
+inline size_t part_bytes(long long entries, int head_dim) {
+    return entries == 0 ? 0 : part_ml_bytes(entries) + (size_t)entries * head_dim * sizeof(float) + (size_t)(entries + 255) / 256 * 256;
+}
 
 }  // namespace
 
@@ -211,7 +215,7 @@ int64_t agx_attn_workspace_bytes(agx_handle* h, int32_t B, const int32_t* P, con
     if (st != AGX_OK) return st;
     const Plan& plan = *plan_ptr;
     if (plan.part_entries == 0) return 0;
-    return (int64_t)(part_ml_bytes(plan.part_entries) + (size_t)plan.part_entries * h->cfg.head_dim * sizeof(float));
+    return (int64_t)part_bytes(plan.part_entries, h->cfg.head_dim);
 }
 
 // Attention, optionally with the append of the block's own K/V rows (k_new != NULL): the attention kernels take the block's rows from
@@ -236,8 +240,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     agx_status st = make_plan(h, B, P, Q, pt_stride, plan_ptr);
     if (st != AGX_OK) return st;
     const Plan& plan = *plan_ptr;
-    const size_t need = plan.part_entries == 0 ? 0
-        : part_ml_bytes(plan.part_entries) + (size_t)plan.part_entries * h->cfg.head_dim * sizeof(float);
+    const size_t need = part_bytes(plan.part_entries, h->cfg.head_dim);
     if (need > 0) {
         if (!workspace || !aligned(workspace, 256)) return fail(h, AGX_E_INVAL, "workspace missing or not 256-byte aligned");
         if (workspace_bytes < need) return fail(h, AGX_E_INVAL, "workspace too small: %zu < %zu", workspace_bytes, need);
@@ -249,6 +252,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
     p.out = out; p.lse = lse;
     p.part_ml = (float2*)workspace;
     p.part_o = need ? (float*)((char*)workspace + part_ml_bytes(plan.part_entries)) : nullptr;
+    p.part_exp = need ? (signed char*)(p.part_o + plan.part_entries * h->cfg.head_dim) : nullptr;
     p.status = h->d_status;
     p.num_pages = num_pages;
     p.total_rows = (int)plan.total_rows;

@@ -541,6 +541,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     const bool in_cluster = p.cluster_size > 1;
     float* cl_o = (float*)ring;                              // [MT*16][kD]
     float2* cl_ml = (float2*)(ring + MT * 16 * kD * 4);      // [MT*16]
+    bool beyond = false;   // some fp16 row does not fit (fp16_exponent), by this lane's 16 columns of it
 #pragma unroll
     for (int wh = 0; wh < 2 * MW; ++wh) {
         const int w = wh >> 1, h = wh & 1;
@@ -584,8 +585,11 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                     unsigned char* orow = (unsigned char*)p.part_o + e * 512;
 #pragma unroll
                     for (int c = 0; c < kCG; ++c) {
-                        const __half2 lo = __floats2half2_rn(o[w][2 * c][2 * h] * inv, o[w][2 * c][2 * h + 1] * inv);
-                        const __half2 hi = __floats2half2_rn(o[w][2 * c + 1][2 * h] * inv, o[w][2 * c + 1][2 * h + 1] * inv);
+                        const float x0 = o[w][2 * c][2 * h] * inv, x1 = o[w][2 * c][2 * h + 1] * inv, x2 = o[w][2 * c + 1][2 * h] * inv, x3 = o[w][2 * c + 1][2 * h + 1] * inv;
+                        const float top = max3_abs(max3_abs(0.f, x0, x1), x2, x3);
+                        const unsigned int large = __ballot_sync(row_lanes, top >= kFp16Least);   // (all lanes of a row)
+                        beyond |= top > kFp16Most || !(large >> (lane & 28) & 15);
+                        const __half2 lo = __floats2half2_rn(x0, x1), hi = __floats2half2_rn(x2, x3);
                         const unsigned int mine_lo = *reinterpret_cast<const unsigned int*>(&lo);
                         const unsigned int mine_hi = *reinterpret_cast<const unsigned int*>(&hi);
                         const bool odd = lane & 1;
@@ -605,6 +609,41 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
         }
     }
     if (in_cluster && sp.nsplit > 1) merge_cluster_rows<kWarps>(p, sp, cl_o, cl_ml, g, split, row0, min(rows - row0, MT * 16));
+    // fp16 rows beyond its range: each row's largest value, through the row sums' place, and the rows once more
+    if (p.part_half && !in_cluster && sp.nsplit > 1 && __syncthreads_or(beyond && !*abort_flag)) {
+        auto each_row = [&](auto act) {   // act(row of the CTA, its partial, 1 / sum, m-tile, half)
+#pragma unroll
+            for (int wh = 0; wh < 2 * MW; ++wh) {
+                const int w = wh >> 1, h = wh & 1, r = (mt0 + w) * 16 + rg + 8 * h;
+                if (row0 + r >= rows) continue;
+                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
+                const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
+                const float l_all = fabsf(((volatile float2*)p.part_ml)[e].y);   // (written above)
+                act(r, e, (l_all > 0.f) ? 1.f / l_all : 0.f, w, h);
+            }
+        };
+        each_row([&](int r, long long, float inv, int w, int h) {
+            float top = 0.f;
+#pragma unroll
+            for (int n = 0; n < 2 * kCG; ++n) top = fmaxf(top, fmaxf(finite_abs(o[w][n][2 * h] * inv), finite_abs(o[w][n][2 * h + 1] * inv)));
+            const unsigned row_lanes = 15u << (lane & 28);
+            top = fmaxf(top, __shfl_xor_sync(row_lanes, top, 1));
+            top = fmaxf(top, __shfl_xor_sync(row_lanes, top, 2));
+            if ((lane & 3) == 0) x_l[r * KW + kg] = top;
+        });
+        __syncthreads();   // (every sum has been read as well)
+        each_row([&](int r, long long e, float inv, int w, int h) {
+            float top = 0.f;
+            for (int k = 0; k < KW; ++k) top = fmaxf(top, x_l[r * KW + k]);
+            const int ex = fp16_exponent(top);
+            if (ex == 0) return;
+            if (kg == 0 && (lane & 3) == 0) { p.part_ml[e].y = -p.part_ml[e].y; p.part_exp[e] = (signed char)ex; }
+#pragma unroll
+            for (int n = 0; n < 2 * kCG; ++n)
+                *(uint32_t*)((unsigned char*)p.part_o + e * 512 + ((kg * kCG * 2 + n) * 8 + 2 * (lane & 3)) * 2) =
+                    pack_f16(o[w][n][2 * h] * inv * pow2(-ex), o[w][n][2 * h + 1] * inv * pow2(-ex));
+        });
+    }
 }
 
 // --------------------------------------------------------------------------------------------
@@ -628,6 +667,15 @@ struct HalfRows {
         : at(half_row(p, sp, i, h, lane >> 1) + (lane & 1) * 8), stride(p.part_half == PART_HALF_TILES ? 65536 : 512) {}
     __device__ __forceinline__ uint2 load(int split) const { return ld_volatile_u2(at + (long long)split * stride); }   // (written by other SMs just before: past the L1)
 };
+// What an fp16 row was divided by, where it was: its sum is negative then, and `exp` is not whatever was there.  (The merges of up to 32
+// splits read it with the sum in any case: a branch on the way to the weights costs them 0.1 to 0.3 us, the load a third of that; the merge of more splits
+// reads it where it is needed, one row over 34704 tokens with 16/2 heads 10.65 us a layer, 11.1 the other way, 10.5 without either.)
+__device__ __forceinline__ float row_scale(float sum, int exp) { return sum < 0.f ? pow2(exp) : 1.f; }
+__device__ __forceinline__ int ld_volatile_s8(const signed char* p) {
+    int v;
+    asm volatile("ld.volatile.global.s8 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 // The same of the fp32 partials (columns [4 lane, 4 lane + 4)).
 struct F32Rows {
     const unsigned char* at;
@@ -774,8 +822,9 @@ attn_combine_many_kernel(const __grid_constant__ AttnParams p, int total_rows) {
         float m_new = warp_max(ml.x);
         m_new = fmaxf(m, m_new);
         const float e = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_new), keep = (m == -INFINITY) ? 0.f : exp2f(m - m_new);
-        float sum = ml.y * e;
-        const float w_mine = kHalfPart ? sum : e;
+        float sum = (kHalfPart ? fabsf(ml.y) : ml.y) * e;
+        float w_mine = kHalfPart ? sum : e;
+        if (kHalfPart && ml.y < 0.f) w_mine *= pow2(ld_volatile_s8(p.part_exp + (ml_at - p.part_ml) + k0));
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
         l = l * keep + sum;
@@ -836,6 +885,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     const int u = threadIdx.x & 15;
     const int rh = blockIdx.x * 8 + (threadIdx.x >> 4);
     const float2* ml_at = nullptr;
+    const signed char* exp_at = nullptr;
     unsigned char* out_at = nullptr;
     float* lse_at = nullptr;
     const unsigned char* rows = nullptr;
@@ -853,16 +903,18 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
             const int i = lrow - acc_rows;
             ns = sp.nsplit;
             const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
-            ml_at = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + u;
+            const long long e = (long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit + u;
+            ml_at = p.part_ml + e; exp_at = p.part_exp + e;
             out_at = (unsigned char*)p.out + out_row * (kD * 2) + u * 16;
             lse_at = p.lse ? p.lse + out_row : nullptr;
             rows = half_row(p, sp, i, h, u);
         }
     }
-    hold(ns); hold(ml_at); hold(out_at); hold(lse_at); hold(rows); hold(stride);
+    hold(ns); hold(ml_at); hold(exp_at); hold(out_at); hold(lse_at); hold(rows); hold(stride);
     pdl_wait();   // the partials are complete
     float2 ml = make_float2(-INFINITY, 0.f);
-    if (u < ns) ml = ld_volatile_f2(ml_at);
+    int exp = 0;
+    if (u < ns) { ml = ld_volatile_f2(ml_at); exp = ld_volatile_s8(exp_at); }
     uint4 v[kNs];
 #pragma unroll
     for (int k = 0; k < kNs; ++k)
@@ -870,8 +922,8 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     float m_all = ml.x;
 #pragma unroll
     for (int off = kNs / 2; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));   // splits sit in lanes 0 .. kNs - 1
-    const float w_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * ml.y;
-    float l_all = w_mine;
+    float l_all = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * fabsf(ml.y);
+    const float w_mine = l_all * row_scale(ml.y, exp);
 #pragma unroll
     for (int off = kNs / 2; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);   // (a fixed order: reproducible)
     m_all = __shfl_sync(0xFFFFFFFFu, m_all, 0, 16);
@@ -926,11 +978,13 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
         const SeqPlan& sp = p.seq[si];
         const int i = lrow - acc_rows;
         const long long out_row = (long long)(sp.q_row0 + i) * p.hq + h;
-        const float2* ml_at = p.part_ml + (long long)sp.part_base + ((long long)i * p.hq + h) * ns + lane;
+        const long long e = (long long)sp.part_base + ((long long)i * p.hq + h) * ns + lane;
+        const float2* ml_at = p.part_ml + e;
+        const signed char* exp_at = p.part_exp + e;
         unsigned char* out_at = (unsigned char*)p.out + out_row * (kD * 2) + lane * 8;
         float* lse_at = p.lse ? p.lse + out_row : nullptr;
         HalfRows rows(p, sp, i, h, lane);
-        hold(ml_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride); hold(ns);
+        hold(ml_at); hold(exp_at); hold(out_at); hold(lse_at); hold(rows.at); hold(rows.stride); hold(ns);
         pdl_wait();   // the partials are complete
         // Every load is issued before the first use of any of them: volatile loads keep their place in the instruction stream
         // (left to itself the compiler moved the row loads behind the reduction of the maxima, i.e. behind a first trip to
@@ -940,10 +994,11 @@ attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows)
 #pragma unroll
         for (int k = 0; k < kNsMax; ++k) v[k] = rows.load(min(k, ns - 1));
         float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < ns) ml = ld_volatile_f2(ml_at);
+        int exp = 0;
+        if (lane < ns) { ml = ld_volatile_f2(ml_at); exp = ld_volatile_s8(exp_at); }
         const float m_all = warp_max(ml.x);
-        const float w_mine = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * ml.y;   // 0 in lanes past the last split
-        float l_all = w_mine;
+        float l_all = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - m_all) * fabsf(ml.y);   // 0 in lanes past the last split
+        const float w_mine = l_all * row_scale(ml.y, exp);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xFFFFFFFFu, l_all, off);   // (a fixed order: reproducible)
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);

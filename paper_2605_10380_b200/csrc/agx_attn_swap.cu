@@ -322,6 +322,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         __syncwarp();
     }
 
+    bool beyond = false;   // some fp16 row does not fit
     float* cl_o = (float*)(smem + S::kO);
     float2* cl_ml = (float2*)(smem + S::kO + NR * 512);
     if (!issuer) {
@@ -427,14 +428,24 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             // 16-bit rows (bf16 results, normalised fp16 partials): lane pairs swap so that the even lane stores two columns of the first
             // row of a pair, the odd lane two of the second
             const bool odd = lane & 1;
+            unsigned seen = 0;   // fp16: bit j: a value of row j is not below what it needs
+            float top = 0.f;
 #pragma unroll
             for (int j = 0; j < kHalf; j += 2) {
                 const float a = o[j] * ref[tile * kHalf + j], b = o[j + 1] * ref[tile * kHalf + j + 1];
+                if (fabsf(a) >= kFp16Least) seen |= 1u << j;
+                if (fabsf(b) >= kFp16Least) seen |= 2u << j;
+                top = max3_abs(top, a, b);
                 const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1);
                 const float lo = odd ? got : a, hi = odd ? b : got;
                 unsigned char* const at = (unsigned char*)row_dst[tile * kHalf + j + odd];
                 if (sp.nsplit == 1) { if (at) *(uint32_t*)(at + (d & ~1) * 2) = pack_bf16(lo, hi); }
                 else if (at) __stcg((uint32_t*)(at + (d & ~1) * 2), pack_f16(lo, hi));
+            }
+            if (sp.nsplit > 1) {
+                const int n = min(max(n_rows - row_off - tile * kHalf, 0), kHalf);   // rows here that are not padding
+                seen = __reduce_or_sync(0xFFFFFFFFu, seen | (0x7FFFFFFFu & ~((1u << n) - 1)) | (top > kFp16Most ? 0x80000000u : 0u));
+                beyond = done && n_tiles > 0 && seen != 0x7FFFFFFFu;
             }
         }
     }
@@ -445,13 +456,60 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         for (int t = 0; t < n_tiles; ++t)
             if (t != p.drop_stage) { mbar_drain(k_bar(t), 0, p.wait_limit_cycles); mbar_drain(v_bar(t), 0, p.wait_limit_cycles); }
     tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+    const bool again = __syncthreads_or(beyond);
+    auto release = [&]() {
+        if (warp == 1) {
+            tc_fence_after();
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+        }
+    };
+    if (!again) {
+        release();
+        if constexpr (RH == 1)
+            if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
+        return;
     }
-    if constexpr (RH == 1)
-        if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
+    // fp16 rows beyond its range (a warp has seen it in its 32 columns of one): the warps find each row's largest value, and store the rows again
+    if (!issuer) {
+        tc_fence_after();
+        const uint32_t t_rows = tmem + ((uint32_t)((warp & 3) << 5) << 16) + row_off + tile * (NH / 2);
+        float* const ref = (float*)(smem + S::kRef) + warp * NH;
+        float* const tops = (float*)(smem + S::kMax);   // [quarter of the columns][NR] (the maxima are dead)
+        float x[2];
+        if (tile < 2)
+#pragma unroll 1
+            for (int j = 0; j < NH / 2; j += 2) {
+                tmem_ld<2>(t_rows + j, (uint32_t*)x);
+                tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int r = tile * (NH / 2) + j + k;
+                    const float t = warp_max(finite_abs(x[k] * ref[r]));
+                    if (lane == 0) tops[(warp & 3) * NR + row_off + r] = t;
+                }
+            }
+        asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
+        auto exponent = [&](int r) { return fp16_exponent(fmaxf(fmaxf(tops[r], tops[NR + r]), fmaxf(tops[2 * NR + r], tops[3 * NR + r]))); };
+        if (ml_at) {
+            const int e = exponent(my_r);
+            if (e) { ml_at->y = -ml_at->y; p.part_exp[ml_at - p.part_ml] = (signed char)e; }   // (this lane wrote it)
+        }
+        if (tile < 2)
+#pragma unroll 1
+            for (int j = 0; j < NH / 2; j += 2) {
+                tmem_ld<2>(t_rows + j, (uint32_t*)x);
+                tmem_wait_ld();
+                const bool odd = lane & 1;
+                const int r = tile * (NH / 2) + j;
+                const float a = x[0] * ref[r] * pow2(-exponent(row_off + r)), b = x[1] * ref[r + 1] * pow2(-exponent(row_off + r + 1));
+                const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1);
+                unsigned char* const at = (unsigned char*)row_dst[r + odd];
+                if (at) __stcg((uint32_t*)(at + ((warp & 3) * 32 + (lane & ~1)) * 2), pack_f16(odd ? got : a, odd ? b : got));
+            }
+        tc_fence_before();
+    }
+    __syncthreads();
+    release();
 }
 
 namespace {

@@ -185,6 +185,7 @@ struct EpiCtx {
     void* out;
     float* part_o;
     float2* part_ml;
+    signed char* part_exp;
     float* lse;
     int* status;
     unsigned long long magic;   // (row * magic) >> 32 == row / G exactly for rows < 2^22
@@ -269,6 +270,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     // per-row scalars, and the row's destination: lane j works them out for row j once, the copy loop below fetches
     // them by shuffle (a single warp doing the index arithmetic row by row took longer than the copies themselves)
     unsigned long long row_dst = 0;
+    long long entry = -1;   // of this lane's partial
     {
         const int r = r_warp0 + lane;
         if (r < it.rows) {
@@ -279,6 +281,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             } else {
                 const long long e = (long long)cx.part_base + ((long long)i * cx.hq + h) * it.nsplit + it.split;
                 cx.part_ml[e] = make_float2(m_ref, l_run);
+                entry = e;
                 if (kStreams) row_dst = (unsigned long long)(cx.part_o + e * kD);
             }
         }
@@ -296,6 +299,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
     };
+    float top = 0.f;   // fp16: the row's largest value
     {
         uint32_t oreg[64];   // two 32-column chunks per TMEM round trip
 #pragma unroll 1
@@ -334,6 +338,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                             uint2 pk;
                             pk.x = pack_f16(__uint_as_float(oreg[4 * v]), __uint_as_float(oreg[4 * v + 1]));
                             pk.y = pack_f16(__uint_as_float(oreg[4 * v + 2]), __uint_as_float(oreg[4 * v + 3]));
+                            top = max3_abs(max3_abs(top, __uint_as_float(oreg[4 * v]), __uint_as_float(oreg[4 * v + 1])), __uint_as_float(oreg[4 * v + 2]), __uint_as_float(oreg[4 * v + 3]));
                             __stcg((uint2*)((unsigned char*)row_dst + (c8 * 8 + v) * 8), pk);
                         } else {
                             __stcg((uint4*)((unsigned char*)row_dst + (c8 * 8 + v) * 16),
@@ -360,6 +365,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                 // on their way as they lie there, one bulk copy, while the other columns are read (128 rows
                 // over 1000 tokens 11.5 -> 11.1 us, 250 over 900 with 16/2 heads 11.4 -> 11.0, 512 over 3072 with 24/8 25.7 -> 25.5 against one copy at the end)
                 unsigned char* half = stage + (c8 >> 1) * 4096;
+                float top1 = 0.f;
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
                     uint4 pk;
@@ -367,8 +373,13 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                     pk.y = pack_f16(__uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
                     pk.z = pack_f16(__uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
                     pk.w = pack_f16(__uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
+                    top = max3_abs(top, __uint_as_float(oreg[8 * v]), __uint_as_float(oreg[8 * v + 1]));
+                    top1 = max3_abs(top1, __uint_as_float(oreg[8 * v + 2]), __uint_as_float(oreg[8 * v + 3]));
+                    top = max3_abs(top, __uint_as_float(oreg[8 * v + 4]), __uint_as_float(oreg[8 * v + 5]));
+                    top1 = max3_abs(top1, __uint_as_float(oreg[8 * v + 6]), __uint_as_float(oreg[8 * v + 7]));
                     *(uint4*)(half + lane * 128 + ((v ^ (lane & 7)) << 4)) = pk;
                 }
+                top = fmaxf(top, top1);
                 leave(half, (c8 >> 1) * 32768);
             } else {
                 // bf16 results: 256 bytes per row go through the staging area, 16-byte units XOR-swizzled by row
@@ -384,29 +395,81 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             }
         }
     }
-    if (kStreams) return;
+    // fp16 rows that need more than its range.  (The loops are rolled up: in line and unrolled, never taken, this cost 0.2 to 0.5 us.)
+    const bool half_rows = !kF32Part && !single && (!kStreams || cx.part_half != PART_F32);
+    const bool again = half_rows && __any_sync(0xFFFFFFFFu, entry >= 0 && (top < kFp16Least || top > kFp16Most));
     const int n_valid = min(32, it.rows - r_warp0);
-    if (!single) {
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
+    if (!again) {
+        if (kStreams) return;
+        if (!single) {
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // (the staging area is read before the CTA ends)
+            return;
+        }
+        __syncwarp();
+        // a half-warp writes one 256-byte row per instruction (lane j moves 16-byte unit j % 16 of row 2 u + j / 16); eight
+        // row pairs' loads are in flight before the first store
+        for (int rl0 = 0; rl0 < n_valid; rl0 += 16) {
+            uint4 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int rl = rl0 + 2 * u + (lane >> 4);
+                v[u] = *(const uint4*)(stage + rl * 256 + (((lane & 15) ^ (rl & 15)) << 4));
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int rl = rl0 + 2 * u + (lane >> 4);
+                const unsigned long long dst = __shfl_sync(0xFFFFFFFFu, row_dst, rl & 31);
+                if (rl < n_valid) *(uint4*)((unsigned char*)dst + (lane & 15) * 16) = v[u];
+            }
+        }
         return;
     }
-    __syncwarp();
-    // a half-warp writes one 256-byte row per instruction (lane j moves 16-byte unit j % 16 of row 2 u + j / 16); eight
-    // row pairs' loads are in flight before the first store
-    for (int rl0 = 0; rl0 < n_valid; rl0 += 16) {
-        uint4 v[8];
+    auto piece = [&](int c, float (&x)[16]) {   // columns [c, c + 16)
+        tmem_ld<16>(tO + c, (uint32_t*)x);
+        tmem_wait_ld();
+        if (kStreams) {
+            const unsigned char* park = smem + park_off(((warp & 3) << 5) + lane, it.n_tiles);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int rl = rl0 + 2 * u + (lane >> 4);
-            v[u] = *(const uint4*)(stage + rl * 256 + (((lane & 15) ^ (rl & 15)) << 4));
+            for (int k = 0; k < 16; ++k) {
+                const float o1 = *(const float*)(park + (((c / 4 + k / 4) ^ lane) << 4) + (k & 3) * 4);
+                x[k] = x[k] * w_own + (w_other != 0.f ? o1 * w_other : 0.f);
+            }
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int rl = rl0 + 2 * u + (lane >> 4);
-            const unsigned long long dst = __shfl_sync(0xFFFFFFFFu, row_dst, rl & 31);
-            if (rl < n_valid) *(uint4*)((unsigned char*)dst + (lane & 15) * 16) = v[u];
-        }
+        for (int k = 0; k < 16; ++k) x[k] *= inv;
+    };
+    float x[16];
+    top = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < kD; c += 16) {
+        piece(c, x);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) top = fmaxf(top, finite_abs(x[k]));
     }
+    const int e = entry >= 0 ? fp16_exponent(top) : 0;
+    if (__any_sync(0xFFFFFFFFu, e)) {
+        if (!kStreams && lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // (the rows are on their way as they were)
+        __syncwarp();
+        if (e) {
+            cx.part_ml[entry] = make_float2(m_ref, -l_run);
+            cx.part_exp[entry] = (signed char)e;
+        }
+        const float f = pow2(-e);
+#pragma unroll 1
+        for (int c = 0; c < kD; c += 16) {
+            piece(c, x);
+#pragma unroll
+            for (int k = 0; k < 16; k += 8) {
+                const uint4 pk = make_uint4(pack_f16(x[k] * f, x[k + 1] * f), pack_f16(x[k + 2] * f, x[k + 3] * f), pack_f16(x[k + 4] * f, x[k + 5] * f),
+                                            pack_f16(x[k + 6] * f, x[k + 7] * f));
+                const int unit = (c + k) / 8;
+                if (!kStreams) *(uint4*)(stage + (unit >> 3) * 4096 + lane * 128 + (((unit ^ lane) & 7) << 4)) = pk;
+                else if (row_dst) __stcg((uint4*)((unsigned char*)row_dst + unit * 16), pk);
+            }
+        }
+        if (!kStreams) { leave(stage, 0); leave(stage + 4096, 32768); }
+    }
+    if (!kStreams && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
 // K or V of a tile that holds block rows or ends inside a page, by the whole producer warp.  Tokens [0, pool_end) come from the pool,
@@ -860,7 +923,7 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             EpiCtx* cx = (EpiCtx*)(smem + kOffCtx);
             cx->it = locate_item<kStreams>(p, blockIdx.x);
             cx->part_base = sp.part_base; cx->hq = p.hq;
-            cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->lse = p.lse;
+            cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->part_exp = p.part_exp; cx->lse = p.lse;
             cx->magic = p.row_div_magic; cx->status = p.status;
             cx->part_half = p.part_half;
             const int rc = row0 / kRowsPerCta;

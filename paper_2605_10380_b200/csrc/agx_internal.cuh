@@ -56,7 +56,8 @@ struct AttnParams {
     float* lse;
     float* part_o;   // [entries][head_dim] fp32, un-normalised, relative to part_ml.x; or, with part_half, rows NORMALISED by their
                      // own sum as fp16: in the first 256 bytes of the same 512-byte slots, or in the tiles of the CTAs that made them (PartHalf)
-    float2* part_ml; // [entries] (running max in log2 units, sum)
+    float2* part_ml; // [entries] (running max in log2 units, sum); a negative sum: the fp16 row was divided by 2^part_exp
+    signed char* part_exp;   // [entries], see fp16_exponent
     int* status;
     unsigned long long row_div_magic;   // ceil(2^32 / G), G = hq / hkv: (row * magic) >> 32 == row / G for rows < 2^22
     unsigned row_div31;                 // ceil(2^row_div_shift / G), row_div_shift = 31 + ceil(log2 G): (row * row_div31) >> row_div_shift == row / G

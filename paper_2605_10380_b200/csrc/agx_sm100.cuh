@@ -220,6 +220,22 @@ __device__ __forceinline__ float warp_max(float x) {
     return m;
 }
 
+// Partials in fp16.  A row divided by its own sum is of V's magnitude, which may be anything that bf16 holds.  One whose largest magnitude `top` is above fp16's
+// range or below 2^-11 is stored divided by 2^fp16_exponent(top), to at most 2^15, with the sum's sign as the mark of it, and the merge multiplies it back;
+// others are stored as they are.  So a value is rounded to 11 bits or to 2^-14 of the row's largest, whichever is more (2^-25, half of fp16's smallest step, is
+// 2^-14 of 2^-11).  The kernels store every row as it is and look at it on the way; what does not fit is stored once more.
+constexpr float kFp16Least = 0x1p-11f, kFp16Most = 65504.f;
+__device__ __forceinline__ int fp16_exponent(float top) {   // (top finite; not below -110, so that 2^-e times any value is finite: fp16 holds 2^-126 times 2^110)
+    return (top >= kFp16Least && top <= kFp16Most) || top == 0.f ? 0 : max((__float_as_int(top) >> 23) - 127 - 14, -110);
+}
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }   // |e| <= 126
+__device__ __forceinline__ float finite_abs(float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.f; }   // (infinities and NaN stay what they are and do not count)
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
