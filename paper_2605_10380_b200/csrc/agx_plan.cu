@@ -35,12 +35,16 @@ struct SplitModel {
 // 3000, 32/8 heads, 5 / 4 splits: 31.1 / 21.7 us a layer; 931 behind 3086, 24/8: 66.7 -> 60.2; 598 behind 5293: 76 -> 68.3; verify blocks with three to
 // eight prefills 5 to 10 %).  (Sequences whose K/V exceed 48 MB have the KV head outermost in the grid and are dealt out here like the others: 50 plans that
 // the order makes different were 0.2 % slower together with it, single ones 13 % faster to 13 % slower.)
-// The last four constants are from 185 lone blocks of 97 to 1500 rows, each in all splits that make sense, with the merge of half a warp a pair: the split
-// chosen is 0.75 % slower than the best of them on average (1.5 % with a merge of 1.5 + 0.45 us per MB and neither of the two others).
+// For one block or two, merge, merge_mb, crowd and merge_many are from 185 lone blocks of 97 to 1500 rows, each in all splits that make sense, with the merge of half
+// a warp a pair: the split chosen is 0.75 % slower than the best of them on average (1.5 % with a merge of 1.5 + 0.45 us per MB and neither of the two others;
+// 72 drawn blocks whose plans the two make different: 3.3 % faster together, single ones 18 % faster to 11 % slower; 23 drawn batches with one or two prefills
+// beside decode and verify blocks 3.5 %, 11 % faster to 1 % slower).  Three and more blocks keep the other constants: with these 50 drawn batches were 1.6 %
+// slower together, 10 % faster to 10 % slower.
 // It replaced waves x (tiles + 3), which took every CTA of a launch for as long as its longest: 48 decode blocks over 700-6000 tokens 129 ->
 // 101 us (no split at all), 400 uncached tokens 15.8 -> 13.3, 4 x (32768, 8) 98 -> 93, a ragged prefill batch 512 -> 473.
-SplitModel tile_model(const PlanConfig& c, bool f32_partials = false) {
+SplitModel tile_model(const PlanConfig& c, size_t blocks, bool f32_partials = false) {
     if (f32_partials) return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.9, 0.3, 0.3, 520, 0, true, 0, 0};
+    if (blocks > 2) return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.5, 0.45, 0.3, 264, 0, true, 0, 0};
     return {128, c.sm_count, 3, 6.0, 1.3, 0.17, 0.0047, 1.1, 0.35, 0.3, 264, 0, true, 0.5, 0.4};
 }
 // (a tile of 64 KB takes 0.85 us and more per SM, 1.25 with more than 32 rows; HBM is busy with about 90 of them.  40 rows over 300 / 450 / 600
@@ -289,7 +293,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         auto estimate = [&](const SplitModel& md, int chunk, int min_tiles) {
             return choose_split(c, md, wide_seqs, P, Q, G, chunk, min_tiles, (long long)c.num_kv_heads * ((Q[0] * G + chunk - 1) / chunk));
         };
-        tile_choice = estimate(tile_model(c, true), 256, 1);
+        tile_choice = estimate(tile_model(c, 1, true), 256, 1);
         stream_choice = estimate(stream_model(c, true), 128, 2);
         wide_tiles = tile_choice.time < (Q[0] * G <= 128 ? 0.86 : 0.89) * stream_choice.time;
         if (c.debug_plan) fprintf(stderr, "agx plan: %d rows, 256-row schedule %.1f us, 128-row chunks %.1f us\n", Q[0] * G, tile_choice.time, stream_choice.time);
@@ -408,7 +412,7 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
             SplitChoice choice = k == KIND_STREAM ? stream_choice : tile_choice;
             if (!choice.tiles) {
                 const bool wide = std::any_of(seqs.begin(), seqs.end(), [&](int s) { return Q[s] * G > 32; });
-                choice = choose_split(c, k == KIND_STREAM ? stream_model(c, wide) : tile_model(c), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
+                choice = choose_split(c, k == KIND_STREAM ? stream_model(c, wide) : tile_model(c, seqs.size()), seqs, P, Q, G, rows_per_chunk, min_split / unit, base_items);
             }
             C = unit * choice.tiles;
             if (const char* force = getenv("AGX_TILE_SPLIT_TOKENS")) { if (atoi(force) >= unit) C = atoi(force) / unit * unit; }

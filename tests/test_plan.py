@@ -144,3 +144,16 @@ def test_one_block_is_split_from_257_tokens_on(hq, hkv):
             ln, = plan([L - q], [q], hq, hkv).launches
             if ln.kind in ("small1", "small2"):
                 assert (ln.seqs[0].nsplit > 1) == (L > 256), (L, q)
+
+
+@pytest.mark.parametrize("prefix,q,hq,splits", [
+    ([4000, 4000, 8000], [1000, 500, 400], 32, [1, 1, 1]),
+    ([8000, 6000, 1000], [700, 400, 200], 24, [1, 1, 1]),
+    ([3000, 2000, 0], [400, 400, 700], 24, [2, 2, 1]),
+    ([6000, 1000, 3000, 8000, 4000], [200, 200, 700, 500, 500], 32, [1, 1, 1, 1, 1]),
+    ([3178], [958], 24, [3]),                               # (one block: what it saves to split is more, 62.6 / 52.4 us a layer)
+])
+def test_splits_of_several_prefills(prefix, q, hq, splits):
+    """Three and more blocks of the 256-row schedule keep each other's SMs busy: a merge behind them costs what it did before its costs were fitted to lone blocks."""
+    ln, = plan(prefix, q, hq, 8).launches
+    assert ln.kind == "tile" and [s.nsplit for s in sorted(ln.seqs, key=lambda s: s.index)] == splits
