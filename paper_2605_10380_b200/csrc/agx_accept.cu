@@ -118,7 +118,6 @@ __device__ __forceinline__ void commit_sequence(int s, const SeqHead& h, const i
     }
 }
 
-constexpr int kAcceptCtas = 6;               // CTAs per SM
 constexpr int kTokSmem = 2048;               // winners of up to this many rows stay in shared memory for the draft comparison
 
 template <bool kBf16, bool kVec>
@@ -264,27 +263,13 @@ accept_cluster_kernel(const void* __restrict__ logits, long long row_stride, int
     cluster_sync();   // no CTA leaves while its keys may still be read
 }
 
-// Chunks per row: one wave of CTAs, as long as every thread has two 16-byte loads to do.  (Rounded up the last CTAs were a second wave: rows of 128256 bf16,
-// eight CTAs of two loads a thread per SM rounded up / eight rounded down / six of four loads rounded down, us: 64 rows 9.5 / 7.6 / 7.8, 128 13.3 / 10.6 /
-// 10.3, 256 22.3 / 17.8 / 16.5, 512 - / 33.3 / 31.7, 33 6.2 / 6.2 / 6.0, 16 5.6 / - / 5.4; eight of four or five of six are as good.)
-int accept_chunks(int sm_count, int total_q, int vocab, int elem_bytes) {
-    const int vec = 16 / elem_bytes;
-    const int max_chunks = (vocab + 256 * vec * 2 - 1) / (256 * vec * 2);
-    const int want = std::max(1, std::min(kAcceptCtas * sm_count / std::max(total_q, 1), max_chunks));
-    int chunk_elems = (vocab + want - 1) / want;
-    chunk_elems = (chunk_elems + vec - 1) / vec * vec;
-    return (vocab + chunk_elems - 1) / chunk_elems;
-}
-
 cudaError_t launch_accept(const void* logits, int logits_dtype, long long row_stride, int vocab, const int* drafts,
                           const int* cu_q, int B, int total_q, int* accept_len, int* next_token, int* argmax,
-                          int* seq_lens, unsigned long long* row_keys, int* tokens_global, int chunks, unsigned int* ticket,
+                          int* seq_lens, unsigned long long* row_keys, int* tokens_global, int sm_count, unsigned int* ticket,
                           cudaStream_t stream) {
     const bool bf16 = logits_dtype == AGX_BF16;
     const int esz = bf16 ? 2 : 4;
     const int vec_elems = 16 / esz;
-    int chunk_elems = (vocab + chunks - 1) / chunks;
-    chunk_elems = (chunk_elems + vec_elems - 1) / vec_elems * vec_elems;  // chunk starts stay 16-byte aligned
     const bool vec = ((uintptr_t)logits % 16 == 0) && ((row_stride * esz) % 16 == 0);
     // up to 8 rows whose CTAs have at most four vectors a thread each
     const int cluster_chunks = total_q <= kClusterCtas ? kClusterCtas / total_q : 0;
@@ -294,7 +279,10 @@ cudaError_t launch_accept(const void* logits, int logits_dtype, long long row_st
         return launch_chained(bf16 ? accept_cluster_kernel<true> : accept_cluster_kernel<false>, dim3(kClusterCtas), dim3(256), 0, stream, logits, row_stride, vocab,
                               cluster_chunks, elems, drafts, cu_q, B, total_q, accept_len, next_token, argmax, seq_lens);
     }
-    dim3 grid(chunks, total_q);
+    const int chunks = accept_chunks(sm_count, total_q, vocab, esz, vec);
+    int chunk_elems = (vocab + chunks - 1) / chunks;
+    chunk_elems = (chunk_elems + vec_elems - 1) / vec_elems * vec_elems;  // chunk starts stay 16-byte aligned
+    dim3 grid((vocab + chunk_elems - 1) / chunk_elems, total_q);
     cudaError_t err = cudaSuccess;
 #define AGX_LAUNCH_ACCEPT(BF, VEC)                                                                              \
     err = launch_chained(accept_kernel<BF, VEC>, grid, dim3(256), 0, stream, logits, row_stride, vocab, chunk_elems,  \
@@ -378,13 +366,12 @@ extern "C" AGX_API agx_status agx_accept_greedy_static(const void* logits, int32
             scratch = ptr;
         }
     }
-    const int chunks = accept_chunks(st.sm_count, total_q, vocab, logits_dtype == AGX_BF16 ? 2 : 4);
     unsigned char* base = (unsigned char*)scratch;
     // the array keeps whatever the previous call left: the ticket counter and the rows' keys must start at zero (the
     // kernel leaves them at zero itself; the clear makes the call independent of how an earlier one ended)
     if (cudaMemsetAsync(base, 0, 256 + (size_t)total_q * 8, (cudaStream_t)stream) != cudaSuccess) return AGX_E_CUDA;
     cudaError_t e = launch_accept(logits, logits_dtype, row_stride, vocab, drafts, cu_q, B, total_q, accept_len,
-                                  next_token, argmax, seq_lens, (unsigned long long*)(base + 256), nullptr, chunks,
+                                  next_token, argmax, seq_lens, (unsigned long long*)(base + 256), nullptr, st.sm_count,
                                   (unsigned int*)base, (cudaStream_t)stream);
     return e == cudaSuccess ? AGX_OK : AGX_E_CUDA;
 }

@@ -370,9 +370,8 @@ agx_status agx_accept_greedy(agx_handle* h, const void* logits, int32_t logits_d
     const int64_t need = agx_accept_workspace_bytes(h, total_q, vocab);
     if (!workspace || !aligned(workspace, 8) || (int64_t)workspace_bytes < need)
         return fail(h, AGX_E_INVAL, "accept workspace missing, misaligned or too small (%lld needed)", (long long)need);
-    const int chunks = accept_chunks(h->sm_count, total_q, vocab, elem_size(logits_dtype));
     cudaError_t e = launch_accept(logits, logits_dtype, row_stride, vocab, drafts, cu_q, B, total_q, accept_len,
-                                  next_token, argmax, seq_lens, h->d_row_keys, (int*)workspace, chunks, h->d_ticket,
+                                  next_token, argmax, seq_lens, h->d_row_keys, (int*)workspace, h->sm_count, h->d_ticket,
                                   (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "accept launch");
     h->last_launches = 1;

@@ -163,10 +163,11 @@ cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, 
 cudaError_t launch_attn_tile_bf16(const AttnParams& p, bool streams, const CUtensorMap& map_k, const CUtensorMap& map_v,
                                   const RowsMaps& maps_new, cudaStream_t stream);
 
-int accept_chunks(int sm_count, int total_q, int vocab, int elem_bytes);
+constexpr int kAcceptCtas = 6;   // CTAs of the accept kernel per SM
+int accept_chunks(int sm_count, int total_q, int vocab, int elem_bytes, bool aligned);   // (agx_plan.cu)
 cudaError_t launch_accept(const void* logits, int logits_dtype, long long row_stride, int vocab, const int* drafts,
                           const int* cu_q, int B, int total_q, int* accept_len, int* next_token, int* argmax,
-                          int* seq_lens, unsigned long long* row_keys, int* tokens_global, int chunks, unsigned int* ticket,
+                          int* seq_lens, unsigned long long* row_keys, int* tokens_global, int sm_count, unsigned int* ticket,
                           cudaStream_t stream);
 
 // Private copies of KV pages (a reused prefix that is cut inside a page, Sec. 4.2).

@@ -229,6 +229,27 @@ int one_wave_split(const PlanConfig& c, const std::vector<int>& seqs, const int3
 
 }  // namespace
 
+// Chunks that the accept kernel cuts a row of logits into, a CTA each.
+// Rows read 16 bytes a load: one wave of CTAs, as long as every thread has two loads to do.  (Rounded up, the last CTAs were a second wave: rows of 128256 bf16,
+// eight CTAs of two loads a thread per SM rounded up / six of four loads rounded down, us: 33 rows 6.3 / 6.0, 64 9.0 / 7.8, 128 12.6 / 10.4, 256 20.1 / 16.5, 300
+// 20.8 / 16.8, 445 26.5 / 23.6, 512 33.7 / 31.7, 600 43.8 / 35.4, 800 49.3 / 44.3, 888 52.5 / 48.8.)  More whole rows than a wave holds are cut in two where the last
+// wave is half empty or more: 128256 bf16, one chunk / two, 889 rows 49.5 / 44.8, 1000 61.9 / 57.3, 1184 67.4 / 64.4, 2000 109 / 106, but 1500 64.1 / 67.1;
+// 32000 f32 889 27.9 / 24.8, 2000 71.3 / 69.9; shorter rows, 32000 bf16, 1000 25.5 / 25.5, 2000 51.1 / 52.2, 3000 84 / 89.
+// Other rows, one element a load, wait longer for each and want the CTAs that an SM can hold, rounded up (one wave as above / this, us: 32003 bf16, 256 rows 18.0
+// / 14.5, 445 34.7 / 19.1, 600 41.8 / 30.3, 889 39.4 / 34.3; 128257 bf16 300 61.7 / 45.1, 600 113 / 92; 32003 f32 256 17.9 / 14.7, 64 7.2 / 7.4).
+int accept_chunks(int sm_count, int total_q, int vocab, int elem_bytes, bool aligned) {
+    const int vec = 16 / elem_bytes, rows = std::max(total_q, 1);
+    const int max_chunks = (vocab + 256 * vec * 2 - 1) / (256 * vec * 2);
+    const int wave = kAcceptCtas * sm_count;
+    int want = wave / rows;
+    if (!aligned) want = (8 * sm_count + rows - 1) / rows;
+    else if (want == 0 && rows % wave * 2 <= wave && (long long)vocab * elem_bytes >= 128000) want = 2;
+    want = std::max(1, std::min(want, max_chunks));
+    int chunk_elems = (vocab + want - 1) / want;
+    chunk_elems = (chunk_elems + vec - 1) / vec * vec;
+    return (vocab + chunk_elems - 1) / chunk_elems;
+}
+
 PlanConfig plan_config(const agx_config& cfg, int sm_count, int (*max_clusters)(int mt, int kw, int cluster)) {
     auto number = [](const char* name, int otherwise) { const char* v = getenv(name); return v ? atoi(v) : otherwise; };
     PlanConfig c;

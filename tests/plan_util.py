@@ -22,6 +22,7 @@ static int clusters(int mt, int kw, int n) {
     static const int one[] = {74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7}, two[] = {148, 93, 71, 56, 45, 37, 33, 30, 26, 21, 21, 17, 14, 14, 14};
     return n < 2 || n > 16 ? 0 : (kw == 4 && mt < 4 ? two : one)[n - 2];
 }
+extern "C" int accept_chunks(int sms, int rows, int vocab, int elem_bytes, int aligned) { return agx::accept_chunks(sms, rows, vocab, elem_bytes, aligned != 0); }
 extern "C" int plan(int hq, int hkv, int d, int dtype, int sms, int B, const int* P, const int* Q, int stride, char* out, int out_bytes) {
     const agx_config cfg = {hq, hkv, d, 16, dtype, 0.f};
     agx::Plan pl;
@@ -94,3 +95,7 @@ def plan(P, Q, hq=32, hkv=8, d=128, dtype="bf16", sms=148, stride=-1) -> Plan:
         v = [int(x) for x in line.split()]
         launches.append(Launch(KINDS[v[0]], v[1], v[2], bool(v[3]), v[4], v[5], [Seq(*v[i:i + 6]) for i in range(6, len(v), 6)]))
     return Plan(int(status), int(entries), error, launches)
+
+
+def accept_chunks(rows, vocab, elem_bytes=2, aligned=True, sms=148) -> int:
+    return _lib().accept_chunks(sms, rows, vocab, elem_bytes, int(aligned))

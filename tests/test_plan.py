@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from tests.plan_util import plan
+from tests.plan_util import accept_chunks, plan
 
 ROWS = {"small1": 16, "small2": 32, "small4": 64, "stream": 128, "tile": 256, "simt": 8}
 UNIT = {"small1": 16, "small2": 16, "small4": 16, "stream": 128, "tile": 128, "simt": 16}
@@ -157,3 +157,14 @@ def test_splits_of_several_prefills(prefix, q, hq, splits):
     """Three and more blocks of the 256-row schedule keep each other's SMs busy: a merge behind them costs what it did before its costs were fitted to lone blocks."""
     ln, = plan(prefix, q, hq, 8).launches
     assert ln.kind == "tile" and [s.nsplit for s in sorted(ln.seqs, key=lambda s: s.index)] == splits
+
+
+@pytest.mark.parametrize("rows,vocab,elem_bytes,aligned,chunks", [
+    (64, 128256, 2, True, 13), (444, 128256, 2, True, 2), (445, 128256, 2, True, 1), (888, 128256, 2, True, 1), (64, 4096, 2, True, 1),   # one wave
+    (889, 128256, 2, True, 2), (1332, 128256, 2, True, 2), (1333, 128256, 2, True, 1), (1776, 128256, 2, True, 2),                        # and the one that is left
+    (889, 32000, 4, True, 2), (889, 32000, 2, True, 1),
+    (445, 32003, 2, False, 3), (256, 128257, 2, False, 5), (889, 128257, 2, False, 2), (4000, 128257, 2, False, 1), (33, 2000, 2, False, 1),
+])
+def test_chunks_of_a_logits_row(rows, vocab, elem_bytes, aligned, chunks):
+    """One wave of CTAs where rows are read 16 bytes a load, eight CTAs an SM rounded up where an element a load."""
+    assert accept_chunks(rows, vocab, elem_bytes, aligned) == chunks
