@@ -518,9 +518,11 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         //      An attention CTA takes a whole SM, so merge CTAs that find no free SM sit on SMs the next call's attention CTAs
         //      need, and those CTAs then start (and fetch their K/V) only after the merge instead of under it.  With a few SMs
         //      left out of the attention grid the merge CTAs are resident there from the start and the next call's grid
-        //      follows this one without a gap.  A two-warp merge CTA of 9 and more splits handles two (row, head) pairs; 12 (up to 20 splits) or 8
-        //      of them fit an SM.
-        bool lean_merge = false;   // fp16 partials and the two-warp merge kernel (slower than fp32 partials and the four-warp
+        //      follows this one without a gap.  24 (row, head) pairs an SM, 16 with more than 20 splits, are what the two-warp merge CTAs of nine and more splits
+        //      take there.  The half-warp CTAs of fewer splits take 96 or 64, but are counted the same: what they leave is where the next call's CTAs start.
+        //      (Counted as 96 and 64, up to 8 splits, 70 batches of one to eight blocks whose plans that changes: 2.9 % slower together, 9 % faster to 15 % slower;
+        //      4 verify blocks 7.7 -> 8.9 us, five of 800 to 2700 tokens 14.5 -> 16.6.)
+        bool lean_merge = false;   // fp16 partials and the merges of small CTAs (slower than fp32 partials and the four-warp
                                    // one where the attention grid fills every SM twice over, e.g. four verify blocks of 4096)
         const bool small_one_per_sm = k == KIND_SMALL4 || (small_kind && kw == 8);
         // (the one-Q-tile tensor-core schedule as well: a single long sequence is one wave of whole-SM CTAs too)
