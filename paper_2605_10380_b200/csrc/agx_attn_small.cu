@@ -203,16 +203,16 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     };
     if (kByHand && pre) fetch_own_ids();         // (the caller vouches for the page table too)
     // Q and the block's own rows, on their way to L2 before the wait (one row: 4 x 2500 tokens 11.07 -> 10.82 us, 12 x 1000 13.79 -> 13.38, 12000
-    // 12.43 -> 12.32), by the CTAs of the first wave: for others the wait is over.
+    // 12.43 -> 12.32), a line of 128 bytes each, by about the CTAs of the first wave: for others the wait is over.
     unsigned sms;
     asm("mov.u32 %0, %%nsmid;\n" : "=r"(sms));
-    if (tid >= 32 && blockIdx.x < 2 * sms) {
-        for (int c = tid - 32; c < MT * 256; c += kLoaders) {
+    if (tid >= 32 && blockIdx.x < (KW == 4 && MT < 4 ? 2 : 1) * sms) {
+        for (int c = 8 * (tid - 32); c < MT * 256; c += 8 * kLoaders) {
             const int r = row0 + (c >> 4), i = div_g(r);
             if (r < rows) prefetch_l2((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + g * G + r - i * G) * kRowBytes + (c & 15) * 16);
         }
         if (kByHand && p.k_new)
-            for (int u = tid - 32; u < own_units; u += kLoaders) {
+            for (int u = 8 * (tid - 32); u < own_units; u += 8 * kLoaders) {
                 const int tok = tok_begin + (own_pg + (u >> 9)) * kPage + ((u >> 4) & 15);
                 if (tok >= P && tok < L)
                     prefetch_l2((const unsigned char*)(((u >> 8) & 1) ? p.v_new : p.k_new) + ((long long)(sp.q_row0 + tok - P) * p.hkv + g) * kRowBytes + (u & 15) * 16);

@@ -172,7 +172,8 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 q_at[j] = (const uint4*)((const unsigned char*)p.q + ((long long)(sp.q_row0 + i) * p.hq + hd) * 256 + (c & 15) * 16);
             }
             hold(q_at[j]);
-            if (q_at[j]) prefetch_l2(q_at[j]);   // (8 rows over 1000 / 4096 tokens with Q in memory 7.17 / 7.77 -> 6.70 / 7.68 us a layer)
+            // (8 rows over 1000 / 4096 tokens with Q in memory 7.17 / 7.77 -> 6.70 / 7.68 us a layer; a line of 128 bytes each: by every thread 3 x 700 tokens 6.30 -> 6.22)
+            if (q_at[j] && (tid & 7) == 0) prefetch_l2(q_at[j]);
         }
 #pragma unroll
         for (int j = 0; j < kOwn; ++j)
@@ -180,7 +181,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 own_pool_at[j] = own_pool(tid + j * kThreads); own_new_at[j] = own_new(tid + j * kThreads);
                 hold(own_pool_at[j]); hold(own_new_at[j]);
                 const int u = tid + j * kThreads, tok = own_tok(u);
-                if (u < two_pages && tok < L) {
+                if ((tid & 7) == 0 && u < two_pages && tok < L) {
                     if (tok >= pool_end) prefetch_l2(own_new_at[j]);
                     else if (pre) {
                         const int id = u < 512 ? first_id : second_id;
