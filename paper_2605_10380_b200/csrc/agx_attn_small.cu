@@ -647,10 +647,7 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 }
 
 // --------------------------------------------------------------------------------------------
-// Combine: out[row, h] = sum_k O_k 2^(m_k - m) / sum_k l_k 2^(m_k - m), splits in index order.
-// One warp per (row, head); lanes own 4 consecutive floats of each 128-wide chunk.
-// kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel takes more).  Four O rows per
-// warp instead of 32 keep the register count low enough for ten CTAs per SM.
+// Merges of split partials: out[row, h] = sum_k O_k 2^(m_k - m) / sum_k l_k 2^(m_k - m), splits in index order.
 
 // Where 16-byte unit u of split 0's fp16 partial of row i, head h lies.
 __device__ __forceinline__ const unsigned char* half_row(const AttnParams& p, const SeqPlan& sp, int i, int h, int u) {
@@ -693,6 +690,8 @@ struct F32Rows {
     }
     __device__ __forceinline__ float4 load(int split) const { return ld_volatile_f4((const float*)(at + (long long)split * stride)); }
 };
+// fp32 partials, one warp per (row, head), a lane 4 columns.  kMaxNs: no sequence of the launch has more splits than this (4, 16 or 32; attn_combine_many_kernel
+// takes more).  Four O rows per warp instead of 32 keep the register count low enough for ten CTAs per SM.
 template <bool kBf16Out, int kMaxNs>
 __global__ void __launch_bounds__(128, kMaxNs <= 4 ? 10 : kMaxNs <= 16 ? 5 : 3)
 attn_combine_kernel(const __grid_constant__ AttnParams p, int total_rows) {

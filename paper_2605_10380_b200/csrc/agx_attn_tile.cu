@@ -181,7 +181,7 @@ struct EpiCtx {
     TileItem it;
     int part_base, hq;
     int part_half;   // a PartHalf
-    unsigned char* part_tile;   // 256-row schedule: this CTA's tile of partials, or the first 64 columns of its rows
+    unsigned char* part_tile;   // 256-row schedule: this CTA's tile of partials, or the first 32 columns of its rows (fp32)
     void* out;
     float* part_o;
     float2* part_ml;

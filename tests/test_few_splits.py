@@ -22,8 +22,8 @@ def check(prefix, q, hq, hkv, what):
     kp, vp = oracle_pools_after_append(w)
     ref, ref_lse = oracle.attn_paged_batch(w.q_block, kp, vp, w.page_table, w.dtype, w.prefix_len, w.q_len, w.cu_q)
     check_attention(out, ref, what)
-    # (scores of bf16 inputs are exact products summed in fp32: 128 terms of magnitude 1 at 2^-24 each, far below this)
-    assert np.abs(lse - ref_lse).max() <= 2e-3
+    # (fp32 results of 2 to 9, half an ulp 2^-22, behind scores of exact products, sums and logarithms in fp32: at most 1.1e-6 measured over all of these shapes)
+    assert np.abs(lse - ref_lse).max() <= 5e-6
 
 
 @pytest.mark.parametrize("splits", [2, 3, 4, 5, 7, 8])
@@ -61,5 +61,14 @@ def test_partials_in_slots(n, tokens, q, hq, hkv, kind, splits):
 def test_two_threads_a_token(rows, tokens):
     """Rows of one head a group, so that any number of them may be there."""
     ln, = plan([tokens], [rows], 2, 2).launches
-    assert ln.kind in ("small1", "small2") and ln.seqs[0].split_tokens <= 256 and not ln.cluster
+    assert ln.kind in ("small1", "small2") and ln.kw == 8 and ln.seqs[0].split_tokens <= 256 and not ln.cluster
     check([tokens], [rows], 2, 2, f"{rows} rows")
+
+
+@pytest.mark.parametrize("q,G", [(3, 3), (4, 3), (5, 3), (7, 3), (10, 3), (3, 4), (4, 4), (5, 4), (6, 4), (8, 4)])
+@pytest.mark.parametrize("tokens", [29, 127, 128, 252, 255, 300, 511])
+def test_two_threads_a_token_of_a_group(q, G, tokens):
+    """Several heads a group: a token's rows lie on both sides of the halves, and so does the edge up to which the block's rows see."""
+    ln, = plan([tokens], [q], 2 * G, 2).launches
+    assert ln.kind in ("small1", "small2") and ln.kw == 8 and ln.seqs[0].split_tokens <= 256 and not ln.cluster
+    check([tokens], [q], 2 * G, 2, f"{q} x {G} rows")

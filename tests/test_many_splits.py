@@ -3,6 +3,7 @@ sequences with few splits or one; 16-bit and fp32 partials, bf16 and fp32 result
 import pytest
 
 from paper_2605_10380_b200 import workloads as W
+from tests.plan_util import plan
 
 pytestmark = pytest.mark.gpu
 
@@ -22,6 +23,26 @@ def test_many_splits(dtype, hq, d, lengths, q, lean, monkeypatch):
     assert b.status() == 0
     again, _ = b.attend_append()
     assert (again == out).all()   # splits are added in order
+    kp, vp = oracle_pools_after_append(w)
+    ref, _ = oracle.attn_paged_batch(w.q_block, kp, vp, w.page_table, w.dtype, w.prefix_len, w.q_len, w.cu_q)
+    check_attention(out, ref, "many")
+
+
+@pytest.mark.parametrize("tokens,q,hq,hkv,kind,splits", [(9000, 1, 8, 2, "small1", 36), (9000, 8, 8, 2, "small2", 36), (12000, 1, 16, 2, "small1", 47), (4058, 129, 8, 2, "tile", 33)])
+def test_many_splits_of_fp16_rows(tokens, q, hq, hkv, kind, splits, monkeypatch):
+    import oracle
+    from tests.gpu_util import DeviceBatch, check_attention, oracle_pools_after_append
+    if kind == "tile":
+        monkeypatch.setenv("AGX_TILE_SPLIT_TOKENS", "128")
+        monkeypatch.setenv("AGX_STREAM_MAX_ROWS", "32")
+    ln, = plan([tokens], [q], hq, hkv).launches
+    assert ln.kind == kind and ln.seqs[0].nsplit == splits and (ln.lean or kind == "tile")
+    w = W.make_attn_workload("many", tokens, "bf16", hq, hkv, 128, [tokens], [q], spare_pages=1)
+    b = DeviceBatch(w)
+    out, lse = b.attend_append()
+    assert b.status() == 0
+    again, _ = b.attend_append()
+    assert (again == out).all()
     kp, vp = oracle_pools_after_append(w)
     ref, _ = oracle.attn_paged_batch(w.q_block, kp, vp, w.page_table, w.dtype, w.prefix_len, w.q_len, w.cu_q)
     check_attention(out, ref, "many")

@@ -1,6 +1,6 @@
 """Values far from 1: split partials are fp16 rows in many launches, and whatever magnitude V has must come through them as it does through fp32.
 Each kernel that writes such partials with each merge that reads them, V scaled by powers of two: all of it, differently by column, by token (so
-that the splits of a row differ), and with an infinite value in it."""
+that the splits of a row differ), every other KV head, and with an infinite value in it."""
 import numpy as np
 import pytest
 
@@ -25,11 +25,11 @@ SHAPES = [
 def scales(what, tokens):
     """Powers of two by which V is scaled: [tokens][128]."""
     tok, col = np.arange(tokens)[:, None], np.arange(128)[None, :]
-    e = {"tiny": -20, "huge": 20, "least": -100, "most": 100, "infinite": 24, "columns": 4 * (col // 16) - 60, "tokens": 20 * (tok // 64 % 3) - 24}[what]
+    e = {"tiny": -20, "huge": 20, "least": -100, "most": 100, "infinite": 24, "heads": 0, "columns": 4 * (col // 16) - 60, "tokens": 20 * (tok // 64 % 3) - 24}[what]
     return np.exp2(np.broadcast_to(np.asarray(e, np.float32), (tokens, 128)))
 
 
-@pytest.mark.parametrize("what", ["tiny", "huge", "least", "most", "columns", "tokens", "infinite"])
+@pytest.mark.parametrize("what", ["tiny", "huge", "least", "most", "columns", "tokens", "heads", "infinite"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[6]}-{s[7]}")
 def test_any_magnitude(shape, what, monkeypatch):
     import oracle
@@ -51,6 +51,9 @@ def test_any_magnitude(shape, what, monkeypatch):
             page[w.page_table[s, 0], :, 0, 37] = np.inf
             if P == 0:
                 new[s * q, :, 37] = np.inf
+    if what == "heads":
+        page[:, 1::2] *= 2.0 ** -30
+        new[:, 1::2] *= 2.0 ** -30
     w.v_pool, w.v_new = W.to_storage(page, "bf16"), W.to_storage(new, "bf16")
     b = DeviceBatch(w)
     out, lse = b.attend_append()
@@ -64,4 +67,4 @@ def test_any_magnitude(shape, what, monkeypatch):
     out, ref = out.reshape(-1, 8, 16), ref.reshape(-1, 8, 16)
     assert np.isfinite(out).all() and np.isfinite(ref).all()
     assert (np.abs(out - ref).max(-1) <= RTOL * np.abs(ref).max(-1)).all(), np.max(np.abs(out - ref).max(-1) / np.abs(ref).max(-1))
-    assert np.abs(lse - ref_lse).max() <= 2e-3
+    assert np.abs(lse - ref_lse).max() <= 5e-6   # (V is not in it: as in test_few_splits.py)
