@@ -666,7 +666,7 @@ struct HalfRows {
 };
 // What an fp16 row was divided by, where it was: its sum is negative then, and `exp` is not whatever was there.  (The merges of up to 32
 // splits read it with the sum in any case: a branch on the way to the weights costs them 0.1 to 0.3 us, the load a third of that; the merge of more splits
-// reads it where it is needed, one row over 34704 tokens with 16/2 heads 10.65 us a layer, 11.1 the other way, 10.5 without either.)
+// reads it where it is needed.)
 __device__ __forceinline__ float row_scale(float sum, int exp) { return sum < 0.f ? pow2(exp) : 1.f; }
 __device__ __forceinline__ int ld_volatile_s8(const signed char* p) {
     int v;

@@ -541,6 +541,9 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 if (whole && C + unit > kSwapMaxTokens) break;   // (6 x 1000 tokens, one row, 10.1 -> 8.1 us; 8 rows over 6700 12.7 -> 11.5)
                 C += unit;
             }
+            // More than 32 splits, which another kernel merges: fp32 rows.  (fp16 rows were 1.5 % faster there while nobody looked at their range; since then 14 blocks
+            // over 9000 to 50000 tokens, one to three KV heads, are 2.5 % faster with fp32 rows: one row over 15000 tokens 16/2 heads 7.0 / 6.8 us, 8 over 9000, 8/2 7.7 / 7.15.)
+            for (int s : seqs) lean_merge &= ceil_div(P[s] + Q[s], C) <= 32;
         }
         // ---- emit launches of at most kMaxSeqs sequences
         for (size_t a = 0; a < seqs.size(); a += kMaxSeqs) {

@@ -38,7 +38,7 @@ def test_any_magnitude(shape, what, monkeypatch):
     for k, v in env.items():
         monkeypatch.setenv(k, v)
     ln, = plan([P] * n, [q] * n, hq, hkv).launches
-    assert ln.kind == kind and ln.seqs[0].nsplit == splits and not ln.cluster and (ln.lean or kind == "tile")
+    assert ln.kind == kind and ln.seqs[0].nsplit == splits and not ln.cluster and (ln.lean or kind == "tile" or splits > 32)   # (more than 32 in slots are fp32 rows)
     w = W.make_attn_workload("range", P + q, "bf16", hq, hkv, 128, [P] * n, [q] * n, spare_pages=1)
     f = scales(what, P + q)
     page, new = W.storage_to_f32(w.v_pool, "bf16").copy(), W.storage_to_f32(w.v_new, "bf16").copy()   # [pages][hkv][16][128], [rows][hkv][128]
