@@ -137,7 +137,7 @@ AGX_API int64_t agx_attn_workspace_bytes(agx_handle* handle, int32_t B, const in
  *                  scaled scores
  *   workspace    : device, >= agx_attn_workspace_bytes(...) bytes, 256-byte aligned (may be NULL
  *                  when that figure is 0)
- * Range: V may be of any magnitude whose sum over a row's tokens float holds.  Parts of a bf16 row's tokens may be merged from fp16 rows, which
+ * Range: V may be of any magnitude whose sum over a row's tokens float holds.  Parts of a row's tokens may, for the blocks of the 256-row kernel below, be merged from fp16 rows, which
  * carry a power of two of their own where fp16's range is too narrow: before it is rounded to bf16, an element is off by at most 2^-11 of itself or 2^-14 of
  * its row's largest element, whichever is more, beside what fp32 sums and bf16 weights leave.
  * Dispatch (G = num_q_heads / num_kv_heads; bf16 handles with head_dim 128 - other handles run the fp32-arithmetic kernel): up to 32 query rows

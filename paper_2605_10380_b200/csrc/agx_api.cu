@@ -288,7 +288,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         }
         cudaError_t e;
         p.cluster_size = ln.cluster;
-        p.part_half = ln.kind == KIND_TILE ? (ln.f32_partials ? PART_F32_TILES : PART_HALF_TILES) : ln.lean_merge ? PART_HALF_SLOTS : PART_F32;
+        p.part_half = ln.kind != KIND_TILE ? PART_F32 : ln.f32_partials ? PART_F32_TILES : PART_HALF_TILES;
         p.k_new = p.v_new = nullptr;
         if (k_new) {
             p.k_new = k_new; p.v_new = v_new;
@@ -320,7 +320,7 @@ static agx_status attn_impl(agx_handle* h, const void* q_block, const void* k_ne
         if (e != cudaSuccess) return cuda_fail(h, e, "attention launch");
         h->last_launches++;
         if (split) {
-            e = launch_attn_combine(p, h->cfg.dtype, ln.total_rows, ln.kind == KIND_STREAM, stream);
+            e = launch_attn_combine(p, h->cfg.dtype, ln.total_rows, stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "combine launch");
             h->last_launches++;
         }

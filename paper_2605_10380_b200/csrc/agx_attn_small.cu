@@ -541,12 +541,10 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
     const bool in_cluster = p.cluster_size > 1;
     float* cl_o = (float*)ring;                              // [MT*16][kD]
     float2* cl_ml = (float2*)(ring + MT * 16 * kD * 4);      // [MT*16]
-    bool beyond = false;   // some fp16 row does not fit (fp16_exponent), by this lane's 16 columns of it
 #pragma unroll
     for (int wh = 0; wh < 2 * MW; ++wh) {
         const int w = wh >> 1, h = wh & 1;
         const int r = (mt0 + w) * 16 + rg + 8 * h;           // row of the CTA's chunk
-        const unsigned int row_lanes = __ballot_sync(0xFFFFFFFFu, row0 + r < rows);   // (the four lanes of a row go together)
         if (row0 + r >= rows) continue;
         float l_all = 0.f;
 #pragma unroll
@@ -573,77 +571,17 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
                 for (int n = 0; n < 2 * kCG; ++n)
                     *(float2*)(orow + (kg * kCG * 2 + n) * 8 + 2 * (lane & 3)) = make_float2(o[w][n][2 * h], o[w][n][2 * h + 1]);
             } else {
-                // split partial for the merge kernel, written past the L1 (read next by other SMs)
+                // split partial for the merge kernel, the un-normalised fp32 row, written past the L1 (read next by other SMs)
                 const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
                 if (first) p.part_ml[e] = make_float2(m_all, l_all);
-                if (p.part_half) {
-                    // the row divided by its own sum, as fp16 in the first 256 bytes of the entry's 512-byte slot (the merge
-                    // weighs split k by l_k 2^(m_k - m)).  A lane holds two columns of each of two neighbouring 8-column
-                    // tiles: lane pairs swap one pair each, so that every lane stores four consecutive columns (8 bytes) and
-                    // the four lanes of a row write a whole 32-byte sector
-                    const float inv = (l_all > 0.f) ? 1.f / l_all : 0.f;
-                    unsigned char* orow = (unsigned char*)p.part_o + e * 512;
+                float* orow = p.part_o + e * kD;
 #pragma unroll
-                    for (int c = 0; c < kCG; ++c) {
-                        const float x0 = o[w][2 * c][2 * h] * inv, x1 = o[w][2 * c][2 * h + 1] * inv, x2 = o[w][2 * c + 1][2 * h] * inv, x3 = o[w][2 * c + 1][2 * h + 1] * inv;
-                        const float top = max3_abs(max3_abs(0.f, x0, x1), x2, x3);
-                        const unsigned int large = __ballot_sync(row_lanes, top >= kFp16Least);   // (all lanes of a row)
-                        beyond |= top > kFp16Most || !(large >> (lane & 28) & 15);
-                        const __half2 lo = __floats2half2_rn(x0, x1), hi = __floats2half2_rn(x2, x3);
-                        const unsigned int mine_lo = *reinterpret_cast<const unsigned int*>(&lo);
-                        const unsigned int mine_hi = *reinterpret_cast<const unsigned int*>(&hi);
-                        const bool odd = lane & 1;
-                        const unsigned int got = __shfl_xor_sync(row_lanes, odd ? mine_lo : mine_hi, 1);
-                        // even lane: its own columns of the first tile, then its partner's; odd lane: the same in the second tile
-                        const uint2 pk = odd ? make_uint2(got, mine_hi) : make_uint2(mine_lo, got);
-                        const int col = (kg * kCG + c) * 16 + (odd ? 8 : 0) + 4 * ((lane & 3) >> 1);
-                        __stcg((uint2*)(orow + col * 2), pk);
-                    }
-                } else {   // the un-normalised fp32 row
-                    float* orow = p.part_o + e * kD;
-#pragma unroll
-                    for (int n = 0; n < 2 * kCG; ++n)
-                        __stcg((float2*)(orow + (kg * kCG * 2 + n) * 8 + 2 * (lane & 3)), make_float2(o[w][n][2 * h], o[w][n][2 * h + 1]));
-                }
+                for (int n = 0; n < 2 * kCG; ++n)
+                    __stcg((float2*)(orow + (kg * kCG * 2 + n) * 8 + 2 * (lane & 3)), make_float2(o[w][n][2 * h], o[w][n][2 * h + 1]));
             }
         }
     }
     if (in_cluster && sp.nsplit > 1) merge_cluster_rows<kWarps>(p, sp, cl_o, cl_ml, g, split, row0, min(rows - row0, MT * 16));
-    // fp16 rows beyond its range: each row's largest value, through the row sums' place, and the rows once more
-    if (p.part_half && !in_cluster && sp.nsplit > 1 && __syncthreads_or(beyond && !*abort_flag)) {
-        auto each_row = [&](auto act) {   // act(row of the CTA, its partial, 1 / sum, m-tile, half)
-#pragma unroll
-            for (int wh = 0; wh < 2 * MW; ++wh) {
-                const int w = wh >> 1, h = wh & 1, r = (mt0 + w) * 16 + rg + 8 * h;
-                if (row0 + r >= rows) continue;
-                const int i = div_g(row0 + r), hd = g * G + (row0 + r) - i * G;
-                const long long e = (long long)sp.part_base + ((long long)i * p.hq + hd) * sp.nsplit + split;
-                const float l_all = fabsf(((volatile float2*)p.part_ml)[e].y);   // (written above)
-                act(r, e, (l_all > 0.f) ? 1.f / l_all : 0.f, w, h);
-            }
-        };
-        each_row([&](int r, long long, float inv, int w, int h) {
-            float top = 0.f;
-#pragma unroll
-            for (int n = 0; n < 2 * kCG; ++n) top = fmaxf(top, fmaxf(finite_abs(o[w][n][2 * h] * inv), finite_abs(o[w][n][2 * h + 1] * inv)));
-            const unsigned row_lanes = 15u << (lane & 28);
-            top = fmaxf(top, __shfl_xor_sync(row_lanes, top, 1));
-            top = fmaxf(top, __shfl_xor_sync(row_lanes, top, 2));
-            if ((lane & 3) == 0) x_l[r * KW + kg] = top;
-        });
-        __syncthreads();   // (every sum has been read as well)
-        each_row([&](int r, long long e, float inv, int w, int h) {
-            float top = 0.f;
-            for (int k = 0; k < KW; ++k) top = fmaxf(top, x_l[r * KW + k]);
-            const int ex = fp16_exponent(top);
-            if (ex == 0) return;
-            if (kg == 0 && (lane & 3) == 0) { p.part_ml[e].y = -p.part_ml[e].y; p.part_exp[e] = (signed char)ex; }
-#pragma unroll
-            for (int n = 0; n < 2 * kCG; ++n)
-                *(uint32_t*)((unsigned char*)p.part_o + e * 512 + ((kg * kCG * 2 + n) * 8 + 2 * (lane & 3)) * 2) =
-                    pack_f16(o[w][n][2 * h] * inv * pow2(-ex), o[w][n][2 * h + 1] * inv * pow2(-ex));
-        });
-    }
 }
 
 // --------------------------------------------------------------------------------------------
@@ -651,7 +589,6 @@ attn_small_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_consta
 
 // Where 16-byte unit u of split 0's fp16 partial of row i, head h lies.
 __device__ __forceinline__ const unsigned char* half_row(const AttnParams& p, const SeqPlan& sp, int i, int h, int u) {
-    if (p.part_half != PART_HALF_TILES) return (const unsigned char*)p.part_o + ((long long)sp.part_base + ((long long)i * p.hq + h) * sp.nsplit) * 512 + u * 16;
     const int g = (int)(((uint64_t)(uint32_t)h * p.row_div_magic) >> 32), r = i * p.gqa + h - g * p.gqa, rl = r & 255;
     return (const unsigned char*)p.part_o + (long long)sp.part_base * 512 + (((long long)g * sp.row_chunks + (r >> 8)) * sp.nsplit) * 65536 + (u >> 3) * 32768 + rl * 128 +
            (((u ^ rl) & 7) << 4);
@@ -661,7 +598,7 @@ struct HalfRows {
     const unsigned char* at;
     int stride;
     __device__ __forceinline__ HalfRows(const AttnParams& p, const SeqPlan& sp, int i, int h, int lane)
-        : at(half_row(p, sp, i, h, lane >> 1) + (lane & 1) * 8), stride(p.part_half == PART_HALF_TILES ? 65536 : 512) {}
+        : at(half_row(p, sp, i, h, lane >> 1) + (lane & 1) * 8), stride(65536) {}
     __device__ __forceinline__ uint2 load(int split) const { return ld_volatile_u2(at + (long long)split * stride); }   // (written by other SMs just before: past the L1)
 };
 // What an fp16 row was divided by, where it was: its sum is negative then, and `exp` is not whatever was there.  (The merges of up to 32
@@ -888,7 +825,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     unsigned char* out_at = nullptr;
     float* lse_at = nullptr;
     const unsigned char* rows = nullptr;
-    int ns = 0, stride = p.part_half == PART_HALF_TILES ? 65536 : 512;
+    int ns = 0;
     if (rh < total_rows * p.hq) {
         const int lrow = rh / p.hq, h = rh - lrow * p.hq;
         int si = 0, acc_rows = 0;
@@ -909,7 +846,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
             rows = half_row(p, sp, i, h, u);
         }
     }
-    hold(ns); hold(ml_at); hold(exp_at); hold(out_at); hold(lse_at); hold(rows); hold(stride);
+    hold(ns); hold(ml_at); hold(exp_at); hold(out_at); hold(lse_at); hold(rows);
     pdl_wait();   // the partials are complete
     float2 ml = make_float2(-INFINITY, 0.f);
     int exp = 0;
@@ -917,7 +854,7 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     uint4 v[kNs];
 #pragma unroll
     for (int k = 0; k < kNs; ++k)
-        if (k < ns) v[k] = ld_volatile_u4(rows + k * stride);
+        if (k < ns) v[k] = ld_volatile_u4(rows + k * 65536);
     float m_all = ml.x;
 #pragma unroll
     for (int off = kNs / 2; off > 0; off >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, off));   // splits sit in lanes 0 .. kNs - 1
@@ -953,12 +890,10 @@ attn_combine_few_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     if (lse_at && u == 0) *lse_at = (m_all + log2f(l_all)) * 0.6931471805599453f;
 }
 
-// The same merge for the fp16 partials of more splits (9 to 32, behind the one-Q-tile schedule 5 to 32): one (row, head) pair per warp, lane k
-// holding split k's (m, l) and every lane four columns of every split's row, all loads in flight at once.  CTAs of two
-// warps with few registers (12 or 8 CTAs per SM), so that the merge of a one-wave launch fits the few SMs the planner
-// leaves out of the attention grid for it.
+// The same merge for the fp16 partials of more splits (9 to 32): one (row, head) pair per warp, lane k holding split k's (m, l) and every lane four columns
+// of every split's row, all loads in flight at once.  CTAs of two warps with few registers, 12 or 7 of them per SM.
 template <int kNsMax>
-__global__ void __launch_bounds__(64, kNsMax <= 20 ? 12 : 8)
+__global__ void __launch_bounds__(64, kNsMax <= 20 ? 12 : 7)
 attn_combine_half32_kernel(const __grid_constant__ AttnParams p, int total_rows) {
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
@@ -1131,21 +1066,17 @@ cudaError_t launch_attn_small_bf16(const AttnParams& p, int mt, int kw, const CU
     }
 }
 
-cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, bool behind_streams, cudaStream_t stream) {
+cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, cudaStream_t stream) {
     const long long n = (long long)total_rows * p.hq;
     if (n == 0) return cudaSuccess;
     const int blocks = (int)((n + 3) / 4);
     int ns_max = 1;
     for (int i = 0; i < p.num_seqs; ++i) ns_max = p.seq[i].nsplit > ns_max ? p.seq[i].nsplit : ns_max;
     const int many_threads = 32 * std::min(kManyWarps, (ns_max + kManyBatch - 1) / kManyBatch);
-    if (dtype == AGX_BF16 && (p.part_half == PART_HALF_SLOTS || p.part_half == PART_HALF_TILES)) {
-        // (five to eight splits behind the one-Q-tile schedule, a few hundred pairs: its CTAs leave nothing of an SM, and the merge's small CTAs of a warp a
-        // pair find room sooner, 7 rows over 1500 tokens with 40/8 heads 10.5 us a layer, half a warp a pair 10.8, 12 over 1200 with 24/8 9.3 / 9.75; behind
-        // the small-q kernels 3 x (1500, 1) 7.4 / 6.8, 3 x (1500, 3) 7.8 / 7.7)
-        if (ns_max <= 4 || (ns_max <= 8 && !behind_streams))
+    if (p.part_half == PART_HALF_TILES) {
+        if (ns_max <= 8)
             return launch_chained(ns_max <= 4 ? attn_combine_few_kernel<4> : attn_combine_few_kernel<8>, dim3((unsigned)((n + 7) / 8)), dim3(128), 0, stream, p, total_rows);
         if (ns_max <= 32) {
-            if (ns_max <= 8) return launch_chained(attn_combine_half32_kernel<8>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 12) return launch_chained(attn_combine_half32_kernel<12>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             if (ns_max <= 20) return launch_chained(attn_combine_half32_kernel<20>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);
             return launch_chained(attn_combine_half32_kernel<32>, dim3((int)((n + 1) / 2)), dim3(64), 0, stream, p, total_rows);

@@ -13,7 +13,6 @@
 // P 1.4, O 2.0, stored 2.3; over 4096 (three tiles) 0.45, 1.2, 2.0, 3.0, 3.3.
 // What is left is the chain itself: three barriers, two MMA round trips (a 128 x 16 operand tile takes the MMA unit about 64 clocks to
 // read whatever N is), and around it the launch, the dependency waits and the merge of the splits.
-#include <cuda_fp16.h>
 
 #include <algorithm>
 
@@ -67,8 +66,7 @@ __device__ __forceinline__ float sum_across_lanes(float (&v)[NR]) {
 
 }  // namespace
 
-// kF16: split partials are fp16 rows.  A kernel of its own: what their range asks for cost the others 1 % (one row over 4096 tokens 5.78 -> 5.88 us a layer).
-template <int NR, int NT, int RH, bool kF16>
+template <int NR, int NT, int RH>
 __global__ void __launch_bounds__(NT * 128 * RH + 32, 1)
 attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
     using S = Lay<NR, NT, RH>;
@@ -159,9 +157,9 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     float2* ml_at = nullptr;
     float* lse_at = nullptr;
     float scale = p.scale_log2;
-    int half_rows = kF16 || sp.nsplit == 1;   // 16-bit result rows
+    int whole_rows = sp.nsplit == 1;   // results, not partials
     const int my_row = lane & (NH - 1), my_r = row_off + my_row;
-    const bool merged_here = RH == 1 && !kF16 && p.cluster_size > 1 && sp.nsplit > 1;
+    const bool merged_here = RH == 1 && p.cluster_size > 1 && sp.nsplit > 1;
     unsigned long long* const row_dst = (unsigned long long*)(smem + S::kDst) + warp * NH;
     if (!issuer) {
 #pragma unroll
@@ -207,7 +205,7 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             row_dst[my_row] = dst;
         }
     }
-    hold(ml_at); hold(lse_at); hold(scale); hold(half_rows); hold(num_pages); hold(page_bytes);
+    hold(ml_at); hold(lse_at); hold(scale); hold(whole_rows); hold(num_pages); hold(page_bytes);
     if (issuer && lane == 0) {
         for (int i = 0; i < 3 * NT + 1; ++i) mbar_init(base + S::kBar + 8u * i, 1);
         *abort_flag = 0;
@@ -324,7 +322,6 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         __syncwarp();
     }
 
-    bool beyond = false;   // some fp16 row does not fit
     float* cl_o = (float*)(smem + S::kO);
     float2* cl_ml = (float2*)(smem + S::kO + NR * 512);
     if (!issuer) {
@@ -420,36 +417,23 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             if (tw == 0 && lane < NH) cl_ml[my_r] = make_float2(m_row, l_row);
 #pragma unroll
             for (int j = 0; j < kHalf; ++j) cl_o[(row_off + tile * kHalf + j) * 128 + d] = o[j];
-        } else if (!half_rows) {   // the un-normalised fp32 rows
+        } else if (!whole_rows) {   // the un-normalised fp32 rows
 #pragma unroll
             for (int j = 0; j < kHalf; ++j) {
                 const unsigned long long at = row_dst[tile * kHalf + j];
                 if (at) __stcg((float*)at + d, o[j]);
             }
         } else {
-            // 16-bit rows (bf16 results, normalised fp16 partials): lane pairs swap so that the even lane stores two columns of the first
+            // bf16 results: lane pairs swap so that the even lane stores two columns of the first
             // row of a pair, the odd lane two of the second
             const bool odd = lane & 1;
-            unsigned seen = 0;   // fp16: bit j: a value of row j is not below what it needs
-            float top = 0.f;
 #pragma unroll
             for (int j = 0; j < kHalf; j += 2) {
                 const float a = o[j] * ref[tile * kHalf + j], b = o[j + 1] * ref[tile * kHalf + j + 1];
-                if constexpr (kF16) {
-                    if (fabsf(a) >= kFp16Least) seen |= 1u << j;
-                    if (fabsf(b) >= kFp16Least) seen |= 2u << j;
-                    top = max3_abs(top, a, b);
-                }
                 const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1);
                 const float lo = odd ? got : a, hi = odd ? b : got;
                 unsigned char* const at = (unsigned char*)row_dst[tile * kHalf + j + odd];
-                if (!kF16 || sp.nsplit == 1) { if (at) *(uint32_t*)(at + (d & ~1) * 2) = pack_bf16(lo, hi); }
-                else if (at) __stcg((uint32_t*)(at + (d & ~1) * 2), pack_f16(lo, hi));
-            }
-            if (kF16 && sp.nsplit > 1) {
-                const int n = min(max(n_rows - row_off - tile * kHalf, 0), kHalf);   // rows here that are not padding
-                seen = __reduce_or_sync(0xFFFFFFFFu, seen | (0x7FFFFFFFu & ~((1u << n) - 1)) | (top > kFp16Most ? 0x80000000u : 0u));
-                beyond = done && n_tiles > 0 && seen != 0x7FFFFFFFu;
+                if (at) *(uint32_t*)(at + (d & ~1) * 2) = pack_bf16(lo, hi);
             }
         }
     }
@@ -460,68 +444,17 @@ attn_swap_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         for (int t = 0; t < n_tiles; ++t)
             if (t != p.drop_stage) { mbar_drain(k_bar(t), 0, p.wait_limit_cycles); mbar_drain(v_bar(t), 0, p.wait_limit_cycles); }
     tc_fence_before();
-    auto release = [&]() {
-        if (warp == 1) {
-            tc_fence_after();
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
-        }
-    };
-    if constexpr (!kF16) {
-        __syncthreads();
-        release();
-        if constexpr (RH == 1)
-            if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
-    } else {
-        if (!__syncthreads_or(beyond)) {
-            release();
-            return;
-        }
-        // fp16 rows beyond its range (a warp has seen it in its 32 columns of one): the warps find each row's largest value, and store the rows again
-        if (!issuer) {
-            tc_fence_after();
-            const uint32_t t_rows = tmem + ((uint32_t)((warp & 3) << 5) << 16) + row_off + tile * (NH / 2);
-            float* const ref = (float*)(smem + S::kRef) + warp * NH;
-            float* const tops = (float*)(smem + S::kMax);   // [quarter of the columns][NR] (the maxima are dead)
-            float x[2];
-            if (tile < 2)
-#pragma unroll 1
-                for (int j = 0; j < NH / 2; j += 2) {
-                    tmem_ld<2>(t_rows + j, (uint32_t*)x);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int r = tile * (NH / 2) + j + k;
-                        const float t = warp_max(finite_abs(x[k] * ref[r]));
-                        if (lane == 0) tops[(warp & 3) * NR + row_off + r] = t;
-                    }
-                }
-            asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
-            auto exponent = [&](int r) { return fp16_exponent(fmaxf(fmaxf(tops[r], tops[NR + r]), fmaxf(tops[2 * NR + r], tops[3 * NR + r]))); };
-            if (ml_at) {
-                const int e = exponent(my_r);
-                if (e) { ml_at->y = -ml_at->y; p.part_exp[ml_at - p.part_ml] = (signed char)e; }   // (this lane wrote it)
-            }
-            if (tile < 2)
-#pragma unroll 1
-                for (int j = 0; j < NH / 2; j += 2) {
-                    tmem_ld<2>(t_rows + j, (uint32_t*)x);
-                    tmem_wait_ld();
-                    const bool odd = lane & 1;
-                    const int r = tile * (NH / 2) + j;
-                    const float a = x[0] * ref[r] * pow2(-exponent(row_off + r)), b = x[1] * ref[r + 1] * pow2(-exponent(row_off + r + 1));
-                    const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? a : b, 1);
-                    unsigned char* const at = (unsigned char*)row_dst[r + odd];
-                    if (at) __stcg((uint32_t*)(at + ((warp & 3) * 32 + (lane & ~1)) * 2), pack_f16(odd ? got : a, odd ? b : got));
-                }
-            tc_fence_before();
-        }
-        __syncthreads();
-        release();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
     }
+    if constexpr (RH == 1)
+        if (merged_here) merge_cluster_rows<kWarps + 1>(p, sp, cl_o, cl_ml, g, split, row0, n_rows);   // (uniform over the cluster)
 }
 
 namespace {
-template <int NR, int NT, int RH, bool kF16>
+template <int NR, int NT, int RH>
 cudaError_t launch_swap(const AttnParams& p, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
     constexpr int kSmem = (int)Lay<NR, NT, RH>::kBytes;
     // the attribute is per device: remember which devices have it (a process normally drives one GPU)
@@ -529,32 +462,31 @@ cudaError_t launch_swap(const AttnParams& p, const CUtensorMap& map_k, const CUt
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!configured_on[device]) {
-        cudaError_t e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH, kF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        cudaError_t e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH, kF16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
+        e = cudaFuncSetAttribute(attn_swap_bf16_kernel<NR, NT, RH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of up to 16
         if (e != cudaSuccess) return e;
         configured_on[device] = true;
     }
     if (p.cluster_size > 1)
-        return launch_chained_cluster(attn_swap_bf16_kernel<NR, NT, RH, kF16>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, (unsigned)p.cluster_size, stream, p, map_k, map_v);
-    return launch_chained(attn_swap_bf16_kernel<NR, NT, RH, kF16>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, stream, p, map_k, map_v);
+        return launch_chained_cluster(attn_swap_bf16_kernel<NR, NT, RH>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, (unsigned)p.cluster_size, stream, p, map_k, map_v);
+    return launch_chained(attn_swap_bf16_kernel<NR, NT, RH>, dim3(p.num_items), dim3(NT * 128 * RH + 32), kSmem, stream, p, map_k, map_v);
 }
 
-template <int NT, bool kF16>
+template <int NT>
 cudaError_t launch_rows(const AttnParams& p, int rows, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    if (rows <= 4) return launch_swap<4, NT, 1, kF16>(p, map_k, map_v, stream);
+    if (rows <= 4) return launch_swap<4, NT, 1>(p, map_k, map_v, stream);
     // More than four rows and two tiles: two threads a token, each with half of its rows, so that butterflies, exponentials and stores are half as long.  One
     // layer, one thread a token / two: 8 rows of 32/8 heads over 3 x 700 tokens 8.46 / 6.80 us, 5 over 2 x 1500 8.47 / 7.04, 4 over 8 x 300 7.49 / 6.60, 8 over
     // 3000 7.64 / 7.01, 2 over 1000 7.08 / 6.48 (with Q on its way to L2 ahead of the wait, below).  Not for three tiles, whose 800 threads are slower (8 rows
     // over 4096 tokens 7.84 / 8.38: the third tile's scores, a third of a microsecond behind the first's, set the pace), nor for splits merged in
     // clusters (one row or two; not compiled: the merge's loads want 64 registers).
     if constexpr (NT == 2) {
-        if (kF16 || p.cluster_size <= 1)
-            return rows <= 8 ? launch_swap<8, NT, 2, kF16>(p, map_k, map_v, stream)
-                             : rows <= 16 ? launch_swap<16, NT, 2, kF16>(p, map_k, map_v, stream) : launch_swap<32, NT, 2, kF16>(p, map_k, map_v, stream);
+        if (p.cluster_size <= 1)
+            return rows <= 8 ? launch_swap<8, NT, 2>(p, map_k, map_v, stream)
+                             : rows <= 16 ? launch_swap<16, NT, 2>(p, map_k, map_v, stream) : launch_swap<32, NT, 2>(p, map_k, map_v, stream);
     }
-    if constexpr (NT == 2 && kF16) return cudaErrorInvalidValue;   // (not reached)
-    else return rows <= 8 ? launch_swap<8, NT, 1, kF16>(p, map_k, map_v, stream) : rows <= 16 ? launch_swap<16, NT, 1, kF16>(p, map_k, map_v, stream) : launch_swap<32, NT, 1, kF16>(p, map_k, map_v, stream);
+    return rows <= 8 ? launch_swap<8, NT, 1>(p, map_k, map_v, stream) : rows <= 16 ? launch_swap<16, NT, 1>(p, map_k, map_v, stream) : launch_swap<32, NT, 1>(p, map_k, map_v, stream);
 }
 }  // namespace
 
@@ -564,8 +496,7 @@ cudaError_t launch_rows(const AttnParams& p, int rows, const CUtensorMap& map_k,
 // In 32 layers launched eagerly over 4096 tokens, with the merge, since then: one row 7.7 -> 6.3 us a layer, 8 rows 9.1 -> 8.0 (parameters held ahead of the
 // dependency wait, own pages in one trip, a shorter last split, long suspensions).
 cudaError_t launch_attn_swap(const AttnParams& p, int rows, int longest, const CUtensorMap& map_k, const CUtensorMap& map_v, cudaStream_t stream) {
-    if (p.part_half) return longest <= 2 * kTileTok ? launch_rows<2, true>(p, rows, map_k, map_v, stream) : launch_rows<3, true>(p, rows, map_k, map_v, stream);
-    return longest <= 2 * kTileTok ? launch_rows<2, false>(p, rows, map_k, map_v, stream) : launch_rows<3, false>(p, rows, map_k, map_v, stream);
+    return longest <= 2 * kTileTok ? launch_rows<2>(p, rows, map_k, map_v, stream) : launch_rows<3>(p, rows, map_k, map_v, stream);
 }
 
 }  // namespace agx

@@ -180,7 +180,6 @@ struct TileItem {
 struct EpiCtx {
     TileItem it;
     int part_base, hq;
-    int part_half;   // a PartHalf
     unsigned char* part_tile;   // 256-row schedule: this CTA's tile of partials, or the first 32 columns of its rows (fp32)
     void* out;
     float* part_o;
@@ -299,7 +298,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
         }
     };
-    float top = 0.f;   // fp16: the row's largest value
+    float top = 0.f;   // fp16 partials: the row's largest value
     {
         uint32_t oreg[64];   // two 32-column chunks per TMEM round trip
 #pragma unroll 1
@@ -318,8 +317,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                     oreg[4 * v + 3] = __float_as_uint(__uint_as_float(oreg[4 * v + 3]) * w_own + (w_other != 0.f ? o1.w * w_other : 0.f));
                 }
             }
-            const bool half_part = kStreams && !single && cx.part_half != PART_F32;
-            if (single || (!kStreams && !kF32Part) || half_part) {   // (the 256-row schedule normalises its fp16 partials too)
+            if (single || (!kStreams && !kF32Part)) {   // (the 256-row schedule normalises its fp16 partials too)
 #pragma unroll
                 for (int c = 0; c < 64; ++c) oreg[c] = __float_as_uint(__uint_as_float(oreg[c]) * inv);
             }
@@ -334,12 +332,6 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                             pk.x = pack_bf16(__uint_as_float(oreg[4 * v]), __uint_as_float(oreg[4 * v + 1]));
                             pk.y = pack_bf16(__uint_as_float(oreg[4 * v + 2]), __uint_as_float(oreg[4 * v + 3]));
                             *(uint2*)((unsigned char*)row_dst + (c8 * 8 + v) * 8) = pk;
-                        } else if (half_part) {
-                            uint2 pk;
-                            pk.x = pack_f16(__uint_as_float(oreg[4 * v]), __uint_as_float(oreg[4 * v + 1]));
-                            pk.y = pack_f16(__uint_as_float(oreg[4 * v + 2]), __uint_as_float(oreg[4 * v + 3]));
-                            top = max3_abs(max3_abs(top, __uint_as_float(oreg[4 * v]), __uint_as_float(oreg[4 * v + 1])), __uint_as_float(oreg[4 * v + 2]), __uint_as_float(oreg[4 * v + 3]));
-                            __stcg((uint2*)((unsigned char*)row_dst + (c8 * 8 + v) * 8), pk);
                         } else {
                             __stcg((uint4*)((unsigned char*)row_dst + (c8 * 8 + v) * 16),
                                    make_uint4(oreg[4 * v], oreg[4 * v + 1], oreg[4 * v + 2], oreg[4 * v + 3]));
@@ -396,8 +388,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
         }
     }
     // fp16 rows that need more than its range.  (The loops are rolled up: in line and unrolled, never taken, this cost 0.2 to 0.5 us.)
-    const bool half_rows = !kF32Part && !single && (!kStreams || cx.part_half != PART_F32);
-    const bool again = half_rows && __any_sync(0xFFFFFFFFu, entry >= 0 && (top < kFp16Least || top > kFp16Most));
+    const bool again = !kStreams && !kF32Part && !single && __any_sync(0xFFFFFFFFu, entry >= 0 && (top < kFp16Least || top > kFp16Most));
     const int n_valid = min(32, it.rows - r_warp0);
     if (!again) {
         if (kStreams) return;
@@ -427,14 +418,6 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     auto piece = [&](int c, float (&x)[16]) {   // columns [c, c + 16)
         tmem_ld<16>(tO + c, (uint32_t*)x);
         tmem_wait_ld();
-        if (kStreams) {
-            const unsigned char* park = smem + park_off(((warp & 3) << 5) + lane, it.n_tiles);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float o1 = *(const float*)(park + (((c / 4 + k / 4) ^ lane) << 4) + (k & 3) * 4);
-                x[k] = x[k] * w_own + (w_other != 0.f ? o1 * w_other : 0.f);
-            }
-        }
 #pragma unroll
         for (int k = 0; k < 16; ++k) x[k] *= inv;
     };
@@ -448,7 +431,7 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
     }
     const int e = entry >= 0 ? fp16_exponent(top) : 0;
     if (__any_sync(0xFFFFFFFFu, e)) {
-        if (!kStreams && lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // (the rows are on their way as they were)
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // (the rows are on their way as they were)
         __syncwarp();
         if (e) {
             cx.part_ml[entry] = make_float2(m_ref, -l_run);
@@ -463,13 +446,13 @@ __device__ __noinline__ void tile_epilogue(unsigned char* smem, uint32_t tO, flo
                 const uint4 pk = make_uint4(pack_f16(x[k] * f, x[k + 1] * f), pack_f16(x[k + 2] * f, x[k + 3] * f), pack_f16(x[k + 4] * f, x[k + 5] * f),
                                             pack_f16(x[k + 6] * f, x[k + 7] * f));
                 const int unit = (c + k) / 8;
-                if (!kStreams) *(uint4*)(stage + (unit >> 3) * 4096 + lane * 128 + (((unit ^ lane) & 7) << 4)) = pk;
-                else if (row_dst) __stcg((uint4*)((unsigned char*)row_dst + unit * 16), pk);
+                *(uint4*)(stage + (unit >> 3) * 4096 + lane * 128 + (((unit ^ lane) & 7) << 4)) = pk;
             }
         }
-        if (!kStreams) { leave(stage, 0); leave(stage + 4096, 32768); }
+        leave(stage, 0);
+        leave(stage + 4096, 32768);
     }
-    if (!kStreams && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
 // K or V of a tile that holds block rows or ends inside a page, by the whole producer warp.  Tokens [0, pool_end) come from the pool,
@@ -925,7 +908,6 @@ attn_tile_bf16_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             cx->part_base = sp.part_base; cx->hq = p.hq;
             cx->out = p.out; cx->part_o = p.part_o; cx->part_ml = p.part_ml; cx->part_exp = p.part_exp; cx->lse = p.lse;
             cx->magic = p.row_div_magic; cx->status = p.status;
-            cx->part_half = p.part_half;
             const int rc = row0 / kRowsPerCta;
             cx->part_tile = (unsigned char*)p.part_o + (long long)sp.part_base * 512 +
                             (kF32Part ? ((long long)g * sp.nsplit + split) * rows * 512 + row0 * 128

@@ -42,10 +42,10 @@ struct SeqPlan {
     int chunk_major;   // order of the work items: 0 = KV head outermost, 1 = row chunk outermost (row chunks last to first in both)
 };
 
-// Split partials: fp32 rows in slots | fp16 rows in slots | fp16 or fp32 rows in tiles (256-row tensor-core schedule), from part_base * 512 bytes on.  In tiles
+// Split partials: fp32 rows in slots | fp16 or fp32 rows in tiles (256-row tensor-core schedule), from part_base * 512 bytes on.  In tiles
 // the first 128 bytes of all rows come first, then the second ones and so on; 16-byte unit u of 128 bytes lies at u ^ (r & 7).  fp16: two times 256 rows,
 // 64 KB, per (KV head, row chunk, split) of a sequence, splits innermost.  fp32: four times all rows per (KV head, split).
-enum PartHalf { PART_F32 = 0, PART_HALF_SLOTS = 1, PART_HALF_TILES = 2, PART_F32_TILES = 3 };
+enum PartHalf { PART_F32 = 0, PART_HALF_TILES = 1, PART_F32_TILES = 2 };
 
 struct AttnParams {
     const void* q;
@@ -54,8 +54,8 @@ struct AttnParams {
     const int* page_table;
     void* out;
     float* lse;
-    float* part_o;   // [entries][head_dim] fp32, un-normalised, relative to part_ml.x; or, with part_half, rows NORMALISED by their
-                     // own sum as fp16: in the first 256 bytes of the same 512-byte slots, or in the tiles of the CTAs that made them (PartHalf)
+    float* part_o;   // [entries][head_dim] fp32, un-normalised, relative to part_ml.x; or, with PART_HALF_TILES, rows NORMALISED by their own sum as fp16, in the
+                     // tiles of the CTAs that made them (PartHalf)
     float2* part_ml; // [entries] (running max in log2 units, sum); a negative sum: the fp16 row was divided by 2^part_exp
     signed char* part_exp;   // [entries], see fp16_exponent
     int* status;
@@ -154,7 +154,7 @@ cudaError_t launch_attn_swap(const AttnParams& p, int rows, int longest, const C
 // fp32-math kernel (agx_attn_simt.cu) for AGX_F32 pools (any q, d in {64, 128}) and for AGX_BF16 pools with d = 64.
 cudaError_t launch_attn_simt(const AttnParams& p, int dtype, cudaStream_t stream);
 // Merge of split partials into out / lse.
-cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, bool behind_streams, cudaStream_t stream);   // honours p.part_half; behind the one-Q-tile schedule or another kernel
+cudaError_t launch_attn_combine(const AttnParams& p, int dtype, int total_rows, cudaStream_t stream);   // honours p.part_half
 
 // Tensor-core tile kernel (bf16, d = 128, tcgen05 + TMEM + TMA).  streams = false: 256 query rows per CTA
 // (two Q tiles); streams = true: 128 rows per CTA whose KV tiles alternate between two softmax warpgroups

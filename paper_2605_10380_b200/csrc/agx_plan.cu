@@ -497,8 +497,8 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 last_shorter = memory_merge = true;
             }
         }
-        // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, with fp32 partials, are faster than 17 to 24 with SMs left to
-        // the merge of fp16 rows (32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
+        // One block over more than 16 such splits: 16 or fewer, of 320 tokens or more, are faster than 17 to 24 with SMs left to
+        // the merge (of fp16 rows when this was measured; 32/8 heads, 8 rows over 4096 / 4400 / 6000 tokens 8.05 -> 7.66 / 9.43 -> 7.89 / 10.07 -> 9.32 us, one row
         // 6.14 -> 5.91 over 4096, 7.82 -> 7.36 over 6000); not for few rows on a third of the SMs (16/2, one row over 6000 5.71 -> 5.96).  (All of it from 14 shapes.)
         if (whole && !cluster && !memory_merge && seqs.size() == 1 && c.merge_sms && (k == KIND_SMALL2 || count_items(C) * 2 > c.sm_count)) {
             const int L = P[seqs[0]] + Q[seqs[0]], longer = std::max(320, round_up((L + 15) / 16, unit));
@@ -518,12 +518,10 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
         //      An attention CTA takes a whole SM, so merge CTAs that find no free SM sit on SMs the next call's attention CTAs
         //      need, and those CTAs then start (and fetch their K/V) only after the merge instead of under it.  With a few SMs
         //      left out of the attention grid the merge CTAs are resident there from the start and the next call's grid
-        //      follows this one without a gap.  24 (row, head) pairs an SM, 16 with more than 20 splits, are what the two-warp merge CTAs of nine and more splits
-        //      take there.  The half-warp CTAs of fewer splits take 96 or 64, but are counted the same: what they leave is where the next call's CTAs start.
-        //      (Counted as 96 and 64, up to 8 splits, 70 batches of one to eight blocks whose plans that changes: 2.9 % slower together, 9 % faster to 15 % slower;
-        //      4 verify blocks 7.7 -> 8.9 us, five of 800 to 2700 tokens 14.5 -> 16.6.)
-        bool lean_merge = false;   // fp16 partials and the merges of small CTAs (slower than fp32 partials and the four-warp
-                                   // one where the attention grid fills every SM twice over, e.g. four verify blocks of 4096)
+        //      follows this one without a gap.  24 (row, head) pairs an SM, 16 with more than 20 splits.  More of them fit, but what the merge leaves is where
+        //      the next call's CTAs start (counted as 96 and 64 pairs, up to 8 splits, 70 batches of one to eight blocks whose plans that changes: 2.9 % slower
+        //      together, 9 % faster to 15 % slower; 4 verify blocks 7.7 -> 8.9 us, five of 800 to 2700 tokens 14.5 -> 16.6).
+        bool lean_merge = false;
         const bool small_one_per_sm = k == KIND_SMALL4 || (small_kind && kw == 8);
         // (the one-Q-tile tensor-core schedule as well: a single long sequence is one wave of whole-SM CTAs too)
         if (!cluster && !memory_merge && (small_one_per_sm || k == KIND_STREAM) && seqs.size() <= (size_t)kMaxSeqs && c.merge_sms) {
@@ -541,9 +539,6 @@ agx_status build_plan(const PlanConfig& c, int B, const int32_t* P, const int32_
                 if (whole && C + unit > kSwapMaxTokens) break;   // (6 x 1000 tokens, one row, 10.1 -> 8.1 us; 8 rows over 6700 12.7 -> 11.5)
                 C += unit;
             }
-            // More than 32 splits, which another kernel merges: fp32 rows.  (fp16 rows were 1.5 % faster there while nobody looked at their range; since then 14 blocks
-            // over 9000 to 50000 tokens, one to three KV heads, are 2.5 % faster with fp32 rows: one row over 15000 tokens 16/2 heads 7.0 / 6.8 us, 8 over 9000, 8/2 7.7 / 7.15.)
-            for (int s : seqs) lean_merge &= ceil_div(P[s] + Q[s], C) <= 32;
         }
         // ---- emit launches of at most kMaxSeqs sequences
         for (size_t a = 0; a < seqs.size(); a += kMaxSeqs) {

@@ -37,7 +37,7 @@ struct Launch {
     int num_items;
     int kw;          // small-q kernel: pages per pipeline stage (KV groups), 4 or 8
     int cluster;     // > 1: CTAs per cluster = KV splits of every sequence of the launch, merged in-kernel (no partials)
-    bool lean_merge; // small-q kernel or one-Q-tile schedule: fp16 partials, merged by the two-warp merge kernel on SMs left out of the attention grid
+    bool lean_merge; // small-q kernel or one-Q-tile schedule: one wave, its merge on SMs left out of the attention grid
     bool f32_partials = false;   // 256-row schedule: fp32 partials
     std::vector<SeqPlan> seqs;
 };

@@ -1,5 +1,5 @@
-"""Merge of fp16 partials of two to eight KV splits, a half-warp a (row, head) pair: partials in tiles (256-row schedule; row groups of whole and of
-cut tiles, a batch of sequences with different and with no splits) and in slots, odd numbers of pairs; and the swapped-operand kernel with two threads
+"""Merge of the partials of two to eight KV splits: fp16 rows in tiles (256-row schedule; row groups of whole and of cut tiles, a batch of sequences with
+different and with no splits), a half-warp a (row, head) pair, and fp32 rows in slots, odd numbers of pairs; and the swapped-operand kernel with two threads
 a token, at the row counts where its halves begin and end."""
 import numpy as np
 import pytest

@@ -39,7 +39,7 @@ def test_many_splits_of_each_kernel(tokens, q, hq, hkv, kind, splits, monkeypatc
         monkeypatch.setenv("AGX_TILE_SPLIT_TOKENS", "128")
         monkeypatch.setenv("AGX_STREAM_MAX_ROWS", "32")
     ln, = plan([tokens], [q], hq, hkv).launches
-    assert ln.kind == kind and ln.seqs[0].nsplit == splits and not ln.lean
+    assert ln.kind == kind and ln.seqs[0].nsplit == splits
     w = W.make_attn_workload("many", tokens, "bf16", hq, hkv, 128, [tokens], [q], spare_pages=1)
     b = DeviceBatch(w)
     out, lse = b.attend_append()

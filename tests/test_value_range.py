@@ -1,6 +1,6 @@
-"""Values far from 1: split partials are fp16 rows in many launches, and whatever magnitude V has must come through them as it does through fp32.
-Each kernel that writes such partials with each merge that reads them, V scaled by powers of two: all of it, differently by column, by token (so
-that the splits of a row differ), every other KV head, and with an infinite value in it."""
+"""Values far from 1: split partials of the 256-row schedule are fp16 rows, and whatever magnitude V has must come through them as it does through the fp32
+rows of the other kernels.  Each kernel that leaves partials with each merge that reads them, V scaled by powers of two: all of it, differently by column, by
+token (so that the splits of a row differ), every other KV head, and with an infinite value in it."""
 import numpy as np
 import pytest
 
@@ -38,7 +38,7 @@ def test_any_magnitude(shape, what, monkeypatch):
     for k, v in env.items():
         monkeypatch.setenv(k, v)
     ln, = plan([P] * n, [q] * n, hq, hkv).launches
-    assert ln.kind == kind and ln.seqs[0].nsplit == splits and not ln.cluster and (ln.lean or kind == "tile" or splits > 32)   # (more than 32 in slots are fp32 rows)
+    assert ln.kind == kind and ln.seqs[0].nsplit == splits and not ln.cluster
     w = W.make_attn_workload("range", P + q, "bf16", hq, hkv, 128, [P] * n, [q] * n, spare_pages=1)
     f = scales(what, P + q)
     page, new = W.storage_to_f32(w.v_pool, "bf16").copy(), W.storage_to_f32(w.v_new, "bf16").copy()   # [pages][hkv][16][128], [rows][hkv][128]
